@@ -60,7 +60,8 @@ enum hpsi_option {
   HPSI_OPT_KERNEL_TIMING = 3, /* 1: bracket every launch of the library's kernels with CUDA events */
   HPSI_OPT_NL_TERMS = 4,      /* mixed path: bf16 terms per nonlocal operand, 3 (six products,
                                  default) or 2 (three products); re-splits the projectors */
-  HPSI_OPT_LOCAL_PATH = 5,    /* 0 (default): register-codelet kernels where the box allows them;
+  HPSI_OPT_LOCAL_PATH = 5,    /* 0 (default): where the box allows them, register-codelet kernels (float32)
+                                 or 64-bit fixed-point kernels (float64);
                                  1: always the generic radix-2/3/4/5 kernels */
   HPSI_OPT_TC_KSPLIT = 6,     /* mixed path: at most this many 64-wide K steps accumulate in one
                                  tensor-memory accumulator of <beta|psi> before the partial sums
@@ -76,10 +77,10 @@ enum hpsi_option {
   HPSI_OPT_BASIS = 8,         /* davidson_solve: the reduced basis grows to this many times N
                                  vectors (2: the basic 2N form, 3 or 4) before a restart; 0
                                  (default): 3 in a mixed context, 4 in a float64 one */
-  HPSI_OPT_AUTOTUNE = 9,      /* 1 (default): the first hpsi_apply of a problem with >= 4 bands at a
-                                 precision times every shared-memory plan of the register-codelet
+  HPSI_OPT_AUTOTUNE = 9,      /* 1 (default): the first hpsi_apply of a problem with >= 4 bands at
+                                 HPSI_MIXED times every shared-memory plan of the register-codelet
                                  kernels and three band-block sizes on its own bands and keeps the
-                                 fastest (results do not depend on the choice); at HPSI_MIXED it
+                                 fastest (results do not depend on the choice); it
                                  also times caps of 4, 8 and 16 K-steps per float32 accumulation of
                                  the tensor-core calbec (unless HPSI_OPT_TC_KSPLIT is set; results
                                  differ at float32 rounding level).  That call synchronizes.

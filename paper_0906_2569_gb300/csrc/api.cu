@@ -187,8 +187,25 @@ static int upload_potential(Context& c, const int n[3], const double* vr, int* s
   rc = upload(c, &d32, t32.data(), nr);
   if (rc) return rc;
   c.vbufs.push_back(d32);
-  *slot = (int)c.vbufs.size() - 2;
+  c.vbufs.push_back(nullptr);   // made by the first problem whose local term can run in fixed point
+  c.vbufs.push_back(nullptr);
+  *slot = (int)c.vbufs.size() - 4;
   return HPSI_OK;
+}
+
+// The fixed-point copy of a potential: at setup in a float64 context, in a mixed one on the first application of H in
+// float64 (the final quotients under HPSI_OPT_FINAL_FP64 = 1).
+int ensure_fixed_potential(Context& c, int slot, const FixedAxis ax[3]) {
+  if (c.vbufs[slot + 2]) return HPSI_OK;
+  const size_t nr = (size_t)ax[0].n * ax[1].n * ax[2].n;
+  if (cudaMalloc(&c.vbufs[slot + 2], sizeof(long long) * nr) != cudaSuccess ||
+      cudaMalloc(&c.vbufs[slot + 3], 16) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFree(c.vbufs[slot + 2]);
+    c.vbufs[slot + 2] = nullptr;
+    return fail(c, HPSI_ENOMEM, "device allocation of the fixed-point potential failed");
+  }
+  return fixed_potential(c, slot, ax, HPSI_K_DAVIDSON);
 }
 
 static int plan_for(Context& c, int n, FftPlan* out) {
@@ -207,17 +224,19 @@ static int plan_for(Context& c, int n, FftPlan* out) {
   if (rc) return rc;
   rc = upload(c, &tt.d32, tab32.data(), tab32.size());
   if (rc) return rc;
-  std::vector<double2> nat(n);
   std::vector<float2> nat32(n);
   for (int j = 0; j < n; ++j) {
     const double ang = -6.283185307179586476925286766559 * (double)j / (double)n;
-    nat[j] = make_double2(std::cos(ang), std::sin(ang));
-    nat32[j] = make_float2((float)nat[j].x, (float)nat[j].y);
+    nat32[j] = make_float2((float)std::cos(ang), (float)std::sin(ang));
   }
-  rc = upload(c, &tt.nat64, nat.data(), nat.size());
-  if (rc) return rc;
   rc = upload(c, &tt.nat32, nat32.data(), nat32.size());
   if (rc) return rc;
+  std::vector<int> fx;
+  const size_t slots = fixed_tables(n, fx, &tt.fixed);
+  rc = upload(c, &tt.fx, fx.data(), fx.size());
+  if (rc) return rc;
+  tt.fixed.tw = reinterpret_cast<const FxTw*>(tt.fx);
+  tt.fixed.slot = tt.fx ? tt.fx + slots : nullptr;
   tt.plan.tw64 = tt.d64;
   tt.plan.tw32 = tt.d32;
   c.tw.push_back(tt);
@@ -309,6 +328,10 @@ int set_potential(Context& c, int ik, const double* v64, double vmean) {
   cudaError_t e = cudaMemcpyAsync(d64, v64, sizeof(double) * nr, cudaMemcpyDeviceToDevice, c.stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "potential update");
   HPSI_LAUNCH(c, HPSI_K_SCF, (k_v_to_f32<<<(int)std::min<size_t>(4096, (nr + 255) / 256), 256, 0, c.stream>>>(nr, d64, d32)));
+  if (c.vbufs[p0.vslot + 2]) {
+    const int rc = fixed_potential(c, p0.vslot, p0.fixed.ax, HPSI_K_SCF);
+    if (rc) return rc;
+  }
   for (Problem& p : c.probs) {
     if (p.vslot != p0.vslot) continue;
     HPSI_LAUNCH(c, HPSI_K_SCF,
@@ -344,11 +367,12 @@ static int finish_problem(Context& c, Problem& p, const double* vr, int vslot_sh
     }
     if ((rc = upload(c, &p.d_ymap, ymap.data(), ymap.size()))) return rc;
     if ((rc = upload(c, &p.d_xmap, xmap.data(), xmap.size()))) return rc;
-    for (auto& t : c.tw)
-      if (t.n == p.n[0]) {
-        p.d_ftw64 = t.nat64;
-        p.d_ftw32 = t.nat32;
-      }
+    for (auto& t : c.tw) {
+      if (t.n == p.n[0]) p.d_ftw32 = t.nat32;
+      for (int a = 0; a < 3; ++a)
+        if (t.n == p.n[a]) p.fixed.ax[a] = t.fixed;
+    }
+    fixed_plan(p, c.smem_optin);
     for (int pr = 0; pr < 2; ++pr) p.fflags[pr] = local_fast_plan(p, pr, c.smem_optin);
   }
   if ((rc = upload(c, &p.d_planes, p.planes.data(), p.planes.size()))) return rc;
@@ -363,6 +387,7 @@ static int finish_problem(Context& c, Problem& p, const double* vr, int vslot_sh
   p.vslot = vslot_shared;
   p.d_v64 = reinterpret_cast<const double*>(c.vbufs[vslot_shared]);
   p.d_v32 = reinterpret_cast<const float*>(c.vbufs[vslot_shared + 1]);
+  if (p.fixed.ok && c.precision == HPSI_FP64 && (rc = ensure_fixed_potential(c, vslot_shared, p.fixed.ax))) return rc;
   // projectors and D (CSR of its nonzeros)
   const int P = p.nproj;
   std::vector<int> rowptr(P + 1, 0), col;
@@ -415,6 +440,9 @@ static int finish_problem(Context& c, Problem& p, const double* vr, int vslot_sh
     p.nbb[pr] = (int)std::max<size_t>(1, std::min<size_t>(4096, (size_t)(48u << 20) / std::max<size_t>(1, xper)));
     const size_t zper = 2 * cs * (size_t)p.n[2] * p.nst;
     p.nbbf[pr] = (int)std::max<size_t>(1, std::min<size_t>(4096, (size_t)(48u << 20) / std::max<size_t>(1, zper)));
+    // fixed point: at least eight waves of two plane CTAs per SM, since its time is arithmetic and a nearly empty
+    // last wave costs more than rows that leave the L2 (4% of a band's time at 144^3)
+    if (pr == HPSI_FP64 && p.fixed.ok) p.nbbf[pr] = std::max(p.nbbf[pr], (16 * c.sm_count + p.n[2] - 1) / p.n[2]);
   }
   if (c.precision == HPSI_MIXED && P > 0) {
     rc = mixed_prepare_beta(c, p);
@@ -452,8 +480,8 @@ static void free_context(Context& c) {
   for (auto& t : c.tw) {
     cudaFree(t.d64);
     cudaFree(t.d32);
-    cudaFree(t.nat64);
     cudaFree(t.nat32);
+    cudaFree(t.fx);
   }
   for (void* v : c.vbufs) cudaFree(v);
   cudaFree(c.d_err);
@@ -517,13 +545,14 @@ static int batch_apply_items(Context& c, int nitem, const int* prob, const int* 
   }
   std::stable_sort(fast.begin(), fast.end(),
                    [&](int x, int y) { return c.probs[prob[x]].n[0] < c.probs[prob[y]].n[0]; });
-  const size_t cs = cur_prec(c) == HPSI_FP64 ? sizeof(double2) : sizeof(float2);
   std::vector<size_t> off(fast.size());
+  auto rows = [&](size_t j) {
+    return (local_row_bytes(c.probs[prob[fast[j]]], cur_prec(c), nbnd[fast[j]]) + 255) & ~size_t(255);
+  };
   size_t total = 0;
   for (size_t j = 0; j < fast.size(); ++j) {
-    const Problem& p = c.probs[prob[fast[j]]];
     off[j] = total;
-    total += 2 * ((cs * (size_t)nbnd[fast[j]] * p.n[2] * p.nst + 255) & ~size_t(255));
+    total += 2 * rows(j);
   }
   if (!fast.empty()) {
     int rc = ensure_buffer(c, &c.ws.batch, &c.ws.batchbytes, total);
@@ -535,13 +564,12 @@ static int batch_apply_items(Context& c, int nitem, const int* prob, const int* 
     unsigned char* base = static_cast<unsigned char*>(c.ws.batch);
     for (size_t j = 0; j < fast.size(); ++j) {
       const int i = fast[j];
-      const Problem& p = c.probs[prob[i]];
       fp[j] = prob[i];
       fn[j] = nbnd[i];
       fi[j] = psi[i];
       fo[j] = hpsi[i];
       zt[j] = base + off[j];
-      yb[j] = base + off[j] + ((cs * (size_t)nbnd[i] * p.n[2] * p.nst + 255) & ~size_t(255));
+      yb[j] = base + off[j] + rows(j);
     }
     // one persistent launch per box edge (up to 32 items each), with the float64 nonlocal term of
     // its items; a group whose launch does not fit takes the launch-per-kernel path

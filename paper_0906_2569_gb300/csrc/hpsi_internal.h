@@ -42,6 +42,23 @@ struct PlaneDev {
   int g0;
 };
 
+// One axis of the fixed-point local path (local_fixed.cu): n = r1 r2 (0: the edge has no such factors), s2 = r1 for
+// coprime factors (no twiddles), 1 otherwise; device tables owned by the axis's TwiddleTable.
+struct FxTw;
+struct FixedAxis {
+  int n = 0, r1 = 0, r2 = 0, s2 = 0;
+  const FxTw* tw = nullptr;
+  const int* slot = nullptr;
+};
+// Tile sizes and growth bounds (bits) of a problem's fixed-point local term.
+struct FixedPlan {
+  bool ok = false;
+  FixedAxis ax[3];
+  int cw = 0, sc = 0, nch = 0;
+  int hz = 0, hy = 0, hx = 0, s3 = 0, hyf = 0, hzf = 0;
+  size_t smem_z = 0, smem_p = 0;
+};
+
 struct Problem {
   double cell[9];
   double recip[9];
@@ -77,8 +94,8 @@ struct Problem {
                                    // (0: not tuned yet)
   int* d_ymap = nullptr;           // [npl][n2]: stick of (plane, j2) or -1
   int* d_xmap = nullptr;           // [n1]: plane of ix or -1
-  const double2* d_ftw64 = nullptr;   // e^{-2 pi i j / n}, j < n (owned by the twiddle table)
-  const float2* d_ftw32 = nullptr;
+  const float2* d_ftw32 = nullptr;    // e^{-2 pi i j / n}, j < n (owned by the twiddle table)
+  FixedPlan fixed;                    // the local term in float64
   std::vector<double> vext;        // the potential given at setup, host, layout [n3][n2][n1]
   bool gamma_ok = false;           // the Gamma-point real form applies (gamma.cu)
   std::string gamma_why;           // why not, when it does not
@@ -97,8 +114,9 @@ struct TwiddleTable {
   FftPlan plan;   // with device pointers filled
   double2* d64 = nullptr;
   float2* d32 = nullptr;
-  double2* nat64 = nullptr;   // e^{-2 pi i j / n}, j < n
-  float2* nat32 = nullptr;
+  float2* nat32 = nullptr;    // e^{-2 pi i j / n}, j < n
+  FixedAxis fixed;
+  int* fx = nullptr;          // its twiddles and slots
 };
 
 struct Workspace {
@@ -135,7 +153,8 @@ struct Context {
   size_t smem_optin = 0;
   std::vector<Problem> probs;
   std::vector<TwiddleTable> tw;
-  std::vector<void*> vbufs;            // owned V buffers (64 and 32 bit)
+  std::vector<void*> vbufs;            // owned V buffers, four per slot: float64, float32, fixed point (or null)
+                                       // and the fixed-point one's scale
   Workspace ws;
   std::string err;
   double opt_tau = 0.1;                // Davidson: |<k+G|H|k+G> - eps| is kept >= tau (Ha)
@@ -259,6 +278,20 @@ int nonlocal_apply_mixed(Context& c, const Problem& p, const double2* psi, doubl
 int mixed_prepare_beta(Context& c, Problem& p);
 int wait_selftest(Context& c);
 size_t local_scratch_per_band(const Problem& p, int precision);
+// Bytes of one buffer of stick rows of nb bands (the fast paths keep two); the fixed-point path keeps its block
+// exponents behind the rows.
+size_t local_row_bytes(const Problem& p, int precision, int nb);
+void fixed_factors(int n, int* r1, int* r2);
+size_t fixed_tables(int n, std::vector<int>& table, FixedAxis* ax);
+void fixed_plan(Problem& p, size_t smem_optin);
+int ensure_fixed_potential(Context& c, int slot, const FixedAxis ax[3]);
+int fixed_potential(Context& c, int slot, const FixedAxis ax[3], int kernel_class);
+int local_fixed_apply(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd, void* Zt, void* Yb,
+                      int nbb);
+int local_fixed_apply_multi(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
+                            double2* const* hpsi, void* const* zt, void* const* yb);
+int local_fixed_persistent(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
+                           double2* const* hpsi, void* const* zt, void* const* yb, bool with_nl, bool* done);
 int local_fast_plan(const Problem& p, int precision, size_t smem_optin);
 std::vector<int> local_fast_candidates(const Problem& p, int precision, size_t smem_optin);
 int local_fast_apply(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd, void* Zt, void* Yb,

@@ -41,19 +41,12 @@ constexpr int kMaxItems = 32;
 // Every launch takes its items by value (the parameter block is 32 KB on sm_70 and later).
 struct FastBatch {
   int nitems, N;
-  const double2* tw64; // e^{-2 pi i j / N}, j < N
-  const float2* tw32;
+  const float2* tw32;  // e^{-2 pi i j / N}, j < N
   double inv_nr;
   FastItem item[kMaxItems];
 };
 
-template <typename V> __device__ __forceinline__ const V* twt(const FastBatch& a);
-template <> __device__ __forceinline__ const double2* twt<double2>(const FastBatch& a) { return a.tw64; }
-template <> __device__ __forceinline__ const float2* twt<float2>(const FastBatch& a) { return a.tw32; }
-
-template <typename V> __device__ __forceinline__ V d2v(double2 x);
-template <> __device__ __forceinline__ double2 d2v<double2>(double2 x) { return x; }
-template <> __device__ __forceinline__ float2 d2v<float2>(double2 x) { return make_float2((float)x.x, (float)x.y); }
+__device__ __forceinline__ float2 d2f(double2 x) { return make_float2((float)x.x, (float)x.y); }
 
 template <int R1, int R2> struct Geo {
   static constexpr int N = R1 * R2;
@@ -81,7 +74,7 @@ __device__ __forceinline__ void zinv_tile(const FastBatch& bt, int bx, int by, i
   const int grp = warp * Gm::LPW + lane / G, t = lane % G;
   const bool in_grp = lane < Gm::LPW * G;
   const int s0 = bx * SC, b = by;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = twt<V>(bt)[i];
+  for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = bt.tw32[i];
   __syncthreads();
   const int s = s0 + grp;
   const bool active = in_grp && s < a.nst;
@@ -93,7 +86,7 @@ __device__ __forceinline__ void zinv_tile(const FastBatch& bt, int bx, int by, i
     for (int n1 = 0; n1 < R1; ++n1) {
       int tt = R2 * n1 + t - st.z0;
       if (tt < 0) tt += N;
-      reg[n1] = tt < st.len ? d2v<V>(ps[tt]) : czero<V>();
+      reg[n1] = tt < st.len ? d2f(ps[tt]) : czero<V>();
     }
   }
   fft2_nat<R1, R2, +1>(reg, xbuf + (in_grp ? grp : 0) * Gm::XS, tw, t, active);
@@ -137,7 +130,7 @@ __device__ __forceinline__ void plane_tile(const FastBatch& bt, int bx, int by, 
   const int j3 = bx;
   const T* Vg = reinterpret_cast<const T*>(a.V) + (size_t)j3 * N * N;
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    tw[i] = twt<V>(bt)[i];
+    tw[i] = bt.tw32[i];
     xm[i] = a.xmap[i];
   }
   if (a.stage_v)
@@ -248,7 +241,7 @@ __device__ __forceinline__ void zfwd_tile(const FastBatch& bt, int bx, int by, i
   const int s0 = bx * SC, b = by;
   const int ns = min(SC, a.nst - s0);
   const V* Y = reinterpret_cast<const V*>(a.Yb) + (size_t)b * N * a.nst;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = twt<V>(bt)[i];
+  for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = bt.tw32[i];
   for (int i = threadIdx.x; i < N * SC; i += blockDim.x) {
     const int j3 = i / SC, sl = i - j3 * SC;
     ibuf[i] = sl < ns ? Y[(size_t)j3 * a.nst + s0 + sl] : czero<V>();
@@ -303,40 +296,6 @@ struct PersistCtl {
   int* err;
 };
 
-constexpr long long kPersistWait = 2000000000LL;   // clock cycles (about 1 s) per barrier wait
-
-__device__ bool persist_sync(unsigned* bar, unsigned target, int* err) {
-  __shared__ int ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-    int good = 1;
-    const long long t0 = clock64();
-    for (unsigned spins = 0;; ++spins) {
-      unsigned v;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-      if ((int)(v - target) >= 0) break;
-      if ((spins & 255u) == 255u && (*(volatile int*)err != 0 || clock64() - t0 > kPersistWait)) {
-        atomicCAS(err, 0, 3);
-        good = 0;
-        break;
-      }
-    }
-    ok = good;
-  }
-  __syncthreads();
-  return ok != 0;
-}
-
-// The CTA's next tile of a phase (all threads get the same index).
-__device__ __forceinline__ int persist_next(unsigned* ctr) {
-  __shared__ int tile;
-  __syncthreads();   // the previous tile is done with shared memory and with `tile`
-  if (threadIdx.x == 0) tile = (int)atomicAdd(ctr, 1u);
-  __syncthreads();
-  return tile;
-}
-
 template <typename T, int R1, int R2, bool NL>
 __global__ void __launch_bounds__(256) k_hpsi_batch(const __grid_constant__ FastBatch bt,
                                                     const __grid_constant__ NlBatch nl,
@@ -366,31 +325,7 @@ __global__ void __launch_bounds__(256) k_hpsi_batch(const __grid_constant__ Fast
     // the nonlocal term of every item, added to the local result; its tiles reuse the dynamic
     // shared memory of the FFT phases
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double2* sm = reinterpret_cast<double2*>(smem_raw);
-    if (!persist_sync(pc.bar, 3 * G, pc.err)) return;
-    const int nc = nl.off_cal[nl.nitems];
-    for (int t = persist_next(pc.bar + 4); t < nc; t = persist_next(pc.bar + 4)) {
-      const int i = find_item(nl.off_cal, nl.nitems, t);
-      const NlItem& a = nl.item[i];
-      const int l = t - nl.off_cal[i], r = l / a.tilesp;
-      calbec_tile(a.npw, a.nproj, a.nb, a.kchunk, a.beta, a.psi, a.part, l % a.tilesp, r % a.tilesb, r / a.tilesb,
-                  sm);
-    }
-    if (!persist_sync(pc.bar, 4 * G, pc.err)) return;
-    for (int t = blockIdx.x; t < nl.off_ds[nl.nitems]; t += G) {
-      const int i = find_item(nl.off_ds, nl.nitems, t);
-      const NlItem& a = nl.item[i];
-      dscale_one((t - nl.off_ds[i]) * blockDim.x + threadIdx.x, a.nproj, a.nb, a.nsplit, a.part, a.rowptr, a.col,
-                 a.dval, a.w);
-    }
-    if (!persist_sync(pc.bar, 5 * G, pc.err)) return;
-    const int na = nl.off_add[nl.nitems];
-    for (int t = persist_next(pc.bar + 5); t < na; t = persist_next(pc.bar + 5)) {
-      const int i = find_item(nl.off_add, nl.nitems, t);
-      const NlItem& a = nl.item[i];
-      const int l = t - nl.off_add[i];
-      addvus_tile(a.npw, a.nproj, a.nb, a.w, a.beta, a.hpsi, l % a.gtiles, l / a.gtiles, sm);
-    }
+    nonlocal_phases(nl, pc.bar, pc.err, G, 3, reinterpret_cast<double2*>(smem_raw));
   }
 }
 
@@ -531,6 +466,7 @@ bool dispatch_size(int n, F&& f) {
 // Shared-memory plan of the fast path for a problem (0 if the box has no fast kernels or the
 // plane does not fit): bit 0 stage V, bit 1 stage the stick row, bit 2 supported.
 int local_fast_plan(const Problem& p, int precision, size_t smem_optin) {
+  if (precision == HPSI_FP64) return p.fixed.ok ? 4 : 0;
   if (p.n[0] != p.n[1] || p.n[1] != p.n[2]) return 0;
   int flags = 0;
   auto pick = [&](auto k) {
@@ -543,8 +479,7 @@ int local_fast_plan(const Problem& p, int precision, size_t smem_optin) {
       }
     }
   };
-  if (precision == HPSI_FP64) dispatch_size<double>(p.n[0], pick);
-  else dispatch_size<float>(p.n[0], pick);
+  dispatch_size<float>(p.n[0], pick);
   return flags;
 }
 
@@ -555,7 +490,7 @@ static FastItem make_item(Context& c, const Problem& p, const double2* psi, doub
   it.npl = p.npl;
   it.nst = p.nst;
   it.bpc = 1;
-  const int fl = p.fflags[cur_prec(c)];
+  const int fl = p.fflags[HPSI_MIXED];
   it.stage_v = fl & 1;
   it.stage_row = (fl >> 1) & 1;
   it.sticks = p.d_sticks;
@@ -566,30 +501,27 @@ static FastItem make_item(Context& c, const Problem& p, const double2* psi, doub
   it.kin = p.d_kin;
   it.Zt = Zt;
   it.Yb = Yb;
-  it.V = cur_prec(c) == HPSI_FP64 ? (const void*)p.d_v64 : (const void*)p.d_v32;
+  it.V = p.d_v32;
   return it;
 }
 
 static size_t plane_smem(const Context& c, const Problem& p, int flags) {
   size_t r = 0;
   auto f = [&](auto k) { r = decltype(k)::smem_plane(p, flags & 1, (flags >> 1) & 1); };
-  if (cur_prec(c) == HPSI_FP64) dispatch_size<double>(p.n[0], f);
-  else dispatch_size<float>(p.n[0], f);
+  dispatch_size<float>(p.n[0], f);
   return r;
 }
 
 static int run_batch(Context& c, FastBatch& bt, size_t smem) {
   int rc = HPSI_EINVAL;
   auto go = [&](auto k) { rc = decltype(k)::run(c, bt, smem); };
-  if (cur_prec(c) == HPSI_FP64) dispatch_size<double>(bt.N, go);
-  else dispatch_size<float>(bt.N, go);
+  dispatch_size<float>(bt.N, go);
   return rc;
 }
 
 static void batch_header(FastBatch& bt, const Problem& p) {
   bt.nitems = 0;
   bt.N = p.n[0];
-  bt.tw64 = p.d_ftw64;
   bt.tw32 = p.d_ftw32;
   bt.inv_nr = 1.0 / ((double)p.n[0] * p.n[1] * p.n[2]);
 }
@@ -597,6 +529,7 @@ static void batch_header(FastBatch& bt, const Problem& p) {
 // Every plan (staging flags | 4) whose kernels fit the shared memory, for the autotuner.
 std::vector<int> local_fast_candidates(const Problem& p, int precision, size_t smem_optin) {
   std::vector<int> out;
+  if (precision == HPSI_FP64) return p.fixed.ok ? std::vector<int>{4} : out;
   if (p.n[0] != p.n[1] || p.n[1] != p.n[2]) return out;
   auto pick = [&](auto k) {
     using K = decltype(k);
@@ -604,15 +537,15 @@ std::vector<int> local_fast_candidates(const Problem& p, int precision, size_t s
       if (K::smem_z() <= smem_optin && K::smem_plane(p, cand & 1, (cand >> 1) & 1) <= smem_optin)
         out.push_back(4 | cand);
   };
-  if (precision == HPSI_FP64) dispatch_size<double>(p.n[0], pick);
-  else dispatch_size<float>(p.n[0], pick);
+  dispatch_size<float>(p.n[0], pick);
   return out;
 }
 
 int local_fast_apply(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd, void* Zt, void* Yb,
                      int nbb) {
+  if (cur_prec(c) == HPSI_FP64) return local_fixed_apply(c, p, psi, hpsi, nbnd, Zt, Yb, nbb);
   static FastBatch bt;   // host staging of the parameter block (calls are not thread-safe by contract)
-  const int fl = p.fflags[cur_prec(c)];
+  const int fl = p.fflags[HPSI_MIXED];
   batch_header(bt, p);
   const size_t smem = plane_smem(c, p, fl);
   for (int b0 = 0; b0 < nbnd; b0 += nbb) {
@@ -629,11 +562,11 @@ int local_fast_apply(Context& c, const Problem& p, const double2* psi, double2* 
 // scratch[i] holds item i's Zt and Y (each n3 * nst * nbnd complex values).
 int local_fast_apply_multi(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
                            double2* const* hpsi, void* const* zt, void* const* yb) {
+  if (cur_prec(c) == HPSI_FP64) return local_fixed_apply_multi(c, nitem, prob, nbnd, psi, hpsi, zt, yb);
   static FastBatch bt;
   int done = 0;
   while (done < nitem) {
     const Problem& p0 = c.probs[prob[done]];
-    const int pr = cur_prec(c);
     batch_header(bt, p0);
     size_t smem = 0;
     int n = 0;
@@ -641,7 +574,7 @@ int local_fast_apply_multi(Context& c, int nitem, const int* prob, const int* nb
       const Problem& p = c.probs[prob[done + n]];
       if (p.n[0] != p0.n[0]) break;
       bt.item[n] = make_item(c, p, psi[done + n], hpsi[done + n], nbnd[done + n], zt[done + n], yb[done + n]);
-      smem = std::max(smem, plane_smem(c, p, p.fflags[pr]));
+      smem = std::max(smem, plane_smem(c, p, p.fflags[HPSI_MIXED]));
       ++n;
     }
     bt.nitems = n;
@@ -666,6 +599,7 @@ int local_batch_persistent(Context& c, int nitem, const int* prob, const int* nb
     const Problem& p = c.probs[prob[i]];
     if (!(p.fflags[pr] & 4) || p.n[0] != p0.n[0] || nbnd[i] < 1) return HPSI_OK;
   }
+  if (pr == HPSI_FP64) return local_fixed_persistent(c, nitem, prob, nbnd, psi, hpsi, zt, yb, with_nl, done);
   static FastBatch bt;
   static NlBatch nl;
   batch_header(bt, p0);
@@ -678,57 +612,16 @@ int local_batch_persistent(Context& c, int nitem, const int* prob, const int* nb
   bt.nitems = nitem;
   const NlBatch* nlp = nullptr;
   if (with_nl) {
-    // partial sums and w of every item side by side in the workspace (as the launch-per-kernel form)
-    std::vector<size_t> off(nitem);
-    std::vector<int> ns(nitem), kc(nitem);
-    size_t total = 0;
-    for (int i = 0; i < nitem; ++i) {
-      size_t bytes = 0;
-      nonlocal_fp64_plan(c, c.probs[prob[i]], nbnd[i], &ns[i], &kc[i], &bytes);
-      off[i] = total;
-      total += (bytes + 255) & ~size_t(255);
-    }
-    int rc = ensure_buffer(c, &c.ws.part, &c.ws.partbytes, std::max<size_t>(total, 256));
+    const int rc = persistent_nl_batch(c, nitem, prob, nbnd, psi, hpsi, nl);
     if (rc) return rc;
-    unsigned char* base = static_cast<unsigned char*>(c.ws.part);
-    int n = 0;
-    nl.off_cal[0] = nl.off_ds[0] = nl.off_add[0] = 0;
-    for (int i = 0; i < nitem; ++i) {
-      const Problem& p = c.probs[prob[i]];
-      if (p.nproj == 0) continue;
-      NlItem& a = nl.item[n];
-      a.npw = p.npw;
-      a.nproj = p.nproj;
-      a.nb = nbnd[i];
-      a.kchunk = kc[i];
-      a.nsplit = ns[i];
-      a.tp = CB_TP;
-      a.tilesp = (p.nproj + CB_TP - 1) / CB_TP;
-      a.tilesb = (a.nb + CB_TB - 1) / CB_TB;
-      a.gtiles = (p.npw + AV_TG - 1) / AV_TG;
-      a.beta = p.d_beta;
-      a.psi = psi[i];
-      a.hpsi = hpsi[i];
-      a.part = reinterpret_cast<double2*>(base + off[i]);
-      a.w = a.part + (size_t)a.nsplit * a.nb * a.nproj;
-      a.rowptr = p.d_rowptr;
-      a.col = p.d_col;
-      a.dval = p.d_dval;
-      nl.off_cal[n + 1] = nl.off_cal[n] + a.tilesp * a.tilesb * a.nsplit;
-      nl.off_ds[n + 1] = nl.off_ds[n] + (a.nproj * a.nb + 255) / 256;
-      nl.off_add[n + 1] = nl.off_add[n] + a.gtiles * ((a.nb + AV_TB - 1) / AV_TB);
-      ++n;
-    }
-    nl.nitems = n;
-    if (n > 0) nlp = &nl;
+    if (nl.nitems > 0) nlp = &nl;
   }
   int rc = ensure_buffer(c, &c.ws.pbar, &c.ws.pbarbytes, 256);
   if (rc) return rc;
   unsigned* bar = static_cast<unsigned*>(c.ws.pbar);
   rc = HPSI_EINVAL;
   auto go = [&](auto k) { rc = decltype(k)::run_persistent(c, bt, smem, nlp, bar, done); };
-  if (pr == HPSI_FP64) dispatch_size<double>(bt.N, go);
-  else dispatch_size<float>(bt.N, go);
+  dispatch_size<float>(bt.N, go);
   return rc;
 }
 

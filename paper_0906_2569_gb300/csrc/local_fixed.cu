@@ -1,0 +1,892 @@
+// Local part of H|psi> in float64 contexts, in 64-bit fixed point (fixed_fft.cuh says why and how the line FFTs go).
+//
+// Three kernels per band block, the sphere-pruned order of the other local paths (App. A.1: V applied in real space
+// between the two transforms), for any box whose edges are products of two of 2, 3, 4, 5, 6, 8, 9, 10, 12, 15, 16:
+//   k_fx_zinv   per (chunk of sticks, band): psi(G) as integers with one exponent per chunk, inverse z-transform,
+//               Zt[b][j3][stick] and the chunk's exponent.
+//   k_fx_plane  per (z-plane, band): the plane [m1-plane][j2] in shared memory; inverse y, then in chunks of columns
+//               inverse x, x V, forward x, then forward y; Y[b][j3][stick] and the plane's exponent.
+//   k_fx_zfwd   per (chunk of sticks, band): forward z-transform, the sphere's values back to float64, 1/N_r,
+//               plus the kinetic term in float64.
+// Between the 1-D transforms a block is shifted so that its largest value (x: its largest column norm) and the
+// transform's growth bound just stay below 2^63.  The exponents travel beside the rows: rows from different
+// chunks or planes are aligned to the largest exponent of the block they meet in.  A non-finite psi makes its
+// chunk's exponent kFxNan, which spreads to every value that the transform would have reached (NaN out).
+//
+// Work distribution: a stage's items (one R-point DFT each) are dealt over all threads of the CTA, so warps are full
+// whatever R1 and R2 are, and the stages run in place in shared memory.  One kernel serves every box: the
+// radices are run-time switches over the same codelets, since a codelet is hundreds of instructions.
+//
+// What bounds it: instruction issue and the latency of the multiplications (an add is 2 instructions, a 64-bit
+// multiplication by a constant ~9).  Measured on the 90^3 box with 160 bands: plane kernel 19.35 -> 3.2 ms, z
+// kernels 1.07 + 1.17 -> 0.33 + 0.46 ms against float64 register codelets; 32 cells of 25^3 to 50^3: 9.6 -> 1.41 ms
+// (planes); 27 x 30 x 32: 428 -> 31 us against the float64 Stockham kernels.  Error of the local term against 128-bit
+// arithmetic: below the float64 kernels' at every edge tried (16 to 135), by 5 to 40%.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <vector>
+
+#include "fixed_fft.cuh"
+#include "hpsi_internal.h"
+
+namespace hpsi {
+
+namespace {
+
+constexpr int kFxNan = 1 << 28;      // exponent of a block that holds a non-finite value
+constexpr int kFxZero = -(1 << 20);  // exponent of a block of zeros
+constexpr int kFxMaxItems = 32;
+
+struct FxItem {
+  int nb, npw, npl, nst;
+  int n1, n2, n3;
+  FixedAxis ax[3];
+  int cw;                       // columns per x chunk
+  int sc;                       // sticks per z chunk
+  int nch;                      // z chunks
+  int hz, hy, hx, s3, hyf, hzf; // growth bounds of the transforms, in bits (FixedPlan)
+  const StickDev* sticks;
+  const int* ymap;
+  const int* xmap;
+  const double2* psi;
+  double2* hpsi;
+  const double* kin;
+  longlong2* Zt;                // [nb][n3][nst]
+  longlong2* Yb;                // [nb][n3][nst]
+  int* Ez;                      // [nb][nch]
+  int* Ey;                      // [nb][n3]
+  const long long* V;           // [n3][slot of j1][slot of j2], V 2^(62 - vexp)
+  const int* vexp;
+  double inv_nr;
+};
+
+struct FxBatch {
+  int nitems;
+  int off_z[kFxMaxItems + 1];   // first z tile of each item (nch x nb tiles)
+  int off_p[kFxMaxItems + 1];   // first plane tile (n3 x nb tiles)
+  FxItem item[kFxMaxItems];
+};
+
+// Resident threads per SM the plane kernel's registers allow (80 and 128 a thread): more warps hide more of the
+// multiplications' latency, but the 16-point codelet alone holds 64 registers of data.
+template <int MAXR> constexpr int kFxThreads = MAXR > 10 ? 512 : 768;
+
+template <int R> struct Rx {
+  static constexpr int value = R;
+};
+template <int MAXR, typename F>
+__device__ __forceinline__ void radix_switch(int r, F&& f) {
+  switch (r) {
+    case 2: f(Rx<2>()); break;
+    case 3: f(Rx<3>()); break;
+    case 4: f(Rx<4>()); break;
+    case 5: f(Rx<5>()); break;
+    case 6: f(Rx<6>()); break;
+    case 8: f(Rx<8>()); break;
+    case 9: f(Rx<9>()); break;
+    case 10: f(Rx<10>()); break;
+    default:
+      if constexpr (MAXR > 10) {
+        switch (r) {
+          case 12: f(Rx<12>()); break;
+          case 15: f(Rx<15>()); break;
+          default: f(Rx<16>()); break;
+        }
+      }
+  }
+}
+
+// it = a cnt + b with b < cnt, for the small non-negative numbers of a tile
+__device__ __forceinline__ void split_index(int it, int cnt, float inv, int& a, int& b) {
+  a = (int)(((float)it + 0.5f) * inv);
+  b = it - a * cnt;
+}
+
+__device__ __forceinline__ unsigned long long fx_mag(longlong2 v) {
+  return (unsigned long long)((v.x ^ (v.x >> 63)) | (v.y ^ (v.y >> 63)));
+}
+// q >> d with rounding, d >= 0 (any size)
+__device__ __forceinline__ longlong2 fx_align(longlong2 v, int d) {
+  longlong2 r;
+  if (d == 0) return v;
+  if (d > 62) {
+    r.x = r.y = 0;
+    return r;
+  }
+  r.x = (v.x + (1LL << (d - 1))) >> d;
+  r.y = (v.y + (1LL << (d - 1))) >> d;
+  return r;
+}
+
+// Shared scratch of a tile's CTA-wide reductions.
+struct FxShared {
+  unsigned long long mag;
+  int emax;
+  float norm;
+  int tile;
+};
+
+// One OR of every thread's bits (all threads call; sh->mag is cleared by the caller a barrier earlier).
+__device__ __forceinline__ void fx_or(FxShared* sh, unsigned long long m) {
+  const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)m);
+  const unsigned hi = __reduce_or_sync(0xffffffffu, (unsigned)(m >> 32));
+  if ((threadIdx.x & 31) == 0) {
+    unsigned* w = reinterpret_cast<unsigned*>(&sh->mag);
+    if (lo) atomicOr(w, lo);
+    if (hi) atomicOr(w + 1, hi);
+  }
+}
+// Shift that brings values below 2^bits(m) up to (or down to) 2^(63 - head)
+__device__ __forceinline__ int fx_headroom(unsigned long long m, int head) { return (int)__clzll((long long)m) - 1 - head; }
+
+// Stage 1 (or, REV, the last stage of the reversed sequence) of `cnt` lines of a tile: item (t, line), lines fastest
+// over the threads; ld(line, slot) and st(line, slot, value) reach the tile.
+template <int MAXR, bool REV, typename LD, typename ST>
+__device__ __forceinline__ void fx_stage1(const FixedAxis& ax, int cnt, const FxTw* tw, LD&& ld, ST&& st) {
+  radix_switch<MAXR>(ax.r1, [&](auto rc) {
+    constexpr int R = decltype(rc)::value;
+    const int items = cnt * ax.r2;
+    const float inv = 1.0f / (float)cnt;
+    for (int it = threadIdx.x; it < items; it += blockDim.x) {
+      int t, line;
+      split_index(it, cnt, inv, t, line);
+      longlong2 v[R];
+      int pos = t * ax.s2;
+#pragma unroll
+      for (int a = 0; a < R; ++a) {
+        v[a] = ld(line, pos);
+        pos += ax.r2;
+        if (pos >= ax.n) pos -= ax.n;
+      }
+      FxDft<R>::run(v);
+      if (!REV && ax.s2 == 1) {
+#pragma unroll
+        for (int a = 1; a < R; ++a) v[a] = fx_twiddle(v[a], tw[t * a]);
+      }
+      pos = t * ax.s2;
+#pragma unroll
+      for (int a = 0; a < R; ++a) {
+        st(line, pos, v[a]);
+        pos += ax.r2;
+        if (pos >= ax.n) pos -= ax.n;
+      }
+    }
+  });
+}
+
+// Stage 2 (or, REV, the first stage of the reversed sequence): item (k1, line)
+template <int MAXR, bool REV, typename LD, typename ST>
+__device__ __forceinline__ void fx_stage2(const FixedAxis& ax, int cnt, const FxTw* tw, LD&& ld, ST&& st) {
+  radix_switch<MAXR>(ax.r2, [&](auto rc) {
+    constexpr int R = decltype(rc)::value;
+    const int items = cnt * ax.r1;
+    const float inv = 1.0f / (float)cnt;
+    for (int it = threadIdx.x; it < items; it += blockDim.x) {
+      int k1, line;
+      split_index(it, cnt, inv, k1, line);
+      longlong2 v[R];
+      int pos = k1 * ax.r2;
+#pragma unroll
+      for (int b = 0; b < R; ++b) {
+        v[b] = ld(line, pos);
+        pos += ax.s2;
+        if (pos >= ax.n) pos -= ax.n;
+      }
+      FxDft<R>::run(v);
+      if (REV && ax.s2 == 1) {
+#pragma unroll
+        for (int b = 1; b < R; ++b) v[b] = fx_twiddle(v[b], tw[k1 * b]);
+      }
+      pos = k1 * ax.r2;
+#pragma unroll
+      for (int b = 0; b < R; ++b) {
+        st(line, pos, v[b]);
+        pos += ax.s2;
+        if (pos >= ax.n) pos -= ax.n;
+      }
+    }
+  });
+}
+
+__device__ __forceinline__ void load_table(FxTw* dst, const FixedAxis& ax) {
+  if (ax.s2 != 1) return;   // the prime-factor form has no twiddles
+  for (int i = threadIdx.x; i < ax.n; i += blockDim.x) dst[i] = ax.tw[i];
+}
+
+// Inverse z-transform of one chunk of sticks of one band.
+template <int MAXR>
+__device__ __forceinline__ void fx_zinv_tile(const FxItem& a, int ch, int b, unsigned char* smem, FxShared* sh) {
+  const int n = a.n3, ld = a.sc + 1;
+  FxTw* tw = reinterpret_cast<FxTw*>(smem);
+  longlong2* L = reinterpret_cast<longlong2*>(smem + sizeof(FxTw) * n);   // [slot][stick], rows of sc + 1
+  const int s0 = ch * a.sc, ns = min(a.sc, a.nst - s0);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  if (threadIdx.x == 0) sh->emax = 0;
+  load_table(tw, a.ax[2]);
+  __syncthreads();
+  // the largest exponent field of the chunk: its sticks are one contiguous range of G
+  const StickDev first = a.sticks[s0], last = a.sticks[s0 + ns - 1];
+  const int ng = last.g0 + last.len - first.g0;
+  const longlong2* ps = reinterpret_cast<const longlong2*>(a.psi + (size_t)b * a.npw);
+  unsigned hi = 0;
+  for (int i = threadIdx.x; i < ng; i += blockDim.x) {
+    const longlong2 v = ps[first.g0 + i];
+    hi = max(hi, max((unsigned)(v.x >> 32) & 0x7fffffffu, (unsigned)(v.y >> 32) & 0x7fffffffu));
+  }
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) atomicMax(&sh->emax, (int)(hi >> 20));
+  __syncthreads();
+  const int emax = sh->emax;
+  if (threadIdx.x == 0)
+    a.Ez[(size_t)b * a.nch + ch] = emax == 0x7ff ? kFxNan : emax == 0 ? kFxZero : emax - 1022 - 63 + a.hz;
+  if (emax == 0x7ff) return;   // (every thread) the plane kernel reads the exponent only
+  // |x| < 2^(emax - 1022), so q = x 2^(63 - hz - (emax - 1022)) stays below 2^(63 - hz)
+  const int e0 = emax - 10 + a.hz;
+  for (int s = warp; s < ns; s += nw) {
+    const StickDev st = a.sticks[s0 + s];
+    for (int pos = lane; pos < n; pos += 32) {
+      int tt = pos - st.z0;
+      if (tt < 0) tt += n;
+      longlong2 v = {0, 0};
+      if (tt < st.len) {
+        const longlong2 w = ps[st.g0 + tt];
+        v.x = fx_from_bits(w.x, e0);
+        v.y = fx_from_bits(w.y, e0);
+      }
+      L[pos * ld + s] = v;
+    }
+  }
+  __syncthreads();
+  auto get = [&](int line, int pos) { return L[pos * ld + line]; };
+  auto put = [&](int line, int pos, longlong2 v) { L[pos * ld + line] = v; };
+  fx_stage1<MAXR, false>(a.ax[2], ns, tw, get, put);
+  __syncthreads();
+  fx_stage2<MAXR, false>(a.ax[2], ns, tw, get, put);
+  __syncthreads();
+  longlong2* Z = a.Zt + (size_t)b * n * a.nst + s0;
+  const int per = blockDim.x / a.sc, r0 = threadIdx.x / a.sc, sl = threadIdx.x - r0 * a.sc;
+  if (sl < ns)
+    for (int j3 = r0; j3 < n; j3 += per) Z[(size_t)j3 * a.nst + sl] = L[a.ax[2].slot[j3] * ld + sl];
+}
+
+template <int MAXR>
+__device__ __forceinline__ void fx_plane_tile(const FxItem& a, int j3, int b, unsigned char* smem, FxShared* sh) {
+  const int n1 = a.n1, n2 = a.n2, npl = a.npl, PS = n2 | 1, cw = a.cw;
+  FxTw* twx = reinterpret_cast<FxTw*>(smem);
+  FxTw* twy = twx + (a.ax[0].s2 == 1 ? n1 : 0);
+  longlong2* P = reinterpret_cast<longlong2*>(twy + (a.ax[1].s2 == 1 ? n2 : 0));   // [plane][j2]
+  longlong2* X = P + (size_t)npl * PS;                                             // [slot of x][column of the chunk]
+  int* xm = reinterpret_cast<int*>(X + (size_t)n1 * cw);
+  float* cn = reinterpret_cast<float*>(X);                                         // column norms, before X is in use
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  if (threadIdx.x == 0) {
+    sh->mag = 0;
+    sh->emax = kFxZero;
+    sh->norm = 0.f;
+  }
+  load_table(twx, a.ax[0]);
+  load_table(twy, a.ax[1]);
+  for (int i = threadIdx.x; i < n1; i += blockDim.x) xm[i] = a.xmap[i];
+  __syncthreads();
+  const int* ez = a.Ez + (size_t)b * a.nch;
+  int em = kFxZero;
+  for (int i = threadIdx.x; i < a.nch; i += blockDim.x) em = max(em, ez[i]);
+  em = __reduce_max_sync(0xffffffffu, em);
+  if (lane == 0 && em > kFxZero) atomicMax(&sh->emax, em);
+  __syncthreads();
+  int e = sh->emax;
+  const int ve = *a.vexp;
+  if (e >= kFxNan / 2 || ve >= kFxNan / 2) {
+    if (threadIdx.x == 0) a.Ey[(size_t)b * a.n3 + j3] = kFxNan;
+    return;
+  }
+  // the plane's sticks, aligned to the largest exponent
+  const longlong2* zin = a.Zt + ((size_t)b * a.n3 + j3) * a.nst;
+  const int lsc = 31 - __clz(a.sc);   // sc is a power of two
+  unsigned long long m = 0;
+  for (int p = warp; p < npl; p += nw) {
+    const int* ym = a.ymap + (size_t)p * n2;
+    for (int j2 = lane; j2 < n2; j2 += 32) {
+      const int s = __ldg(ym + j2);
+      longlong2 v = {0, 0};
+      if (s >= 0) v = fx_align(zin[s], e - ez[s >> lsc]);
+      m |= fx_mag(v);
+      P[p * PS + j2] = v;
+    }
+  }
+  fx_or(sh, m);
+  __syncthreads();
+  m = sh->mag;
+  if (m == 0) {   // a plane of zeros: zeros out
+    longlong2* yo = a.Yb + ((size_t)b * a.n3 + j3) * a.nst;
+    const longlong2 z = {0, 0};
+    for (int i = threadIdx.x; i < a.nst; i += blockDim.x) yo[i] = z;
+    if (threadIdx.x == 0) a.Ey[(size_t)b * a.n3 + j3] = kFxZero;
+    return;
+  }
+  auto get = [&](int p, int pos) { return P[p * PS + pos]; };
+  auto put = [&](int p, int pos, longlong2 v) { P[p * PS + pos] = v; };
+  {
+    const int d = fx_headroom(m, a.hy);
+    e -= d;
+    const FxShift sh1(d);
+    fx_stage1<MAXR, false>(a.ax[1], npl, twy, [&](int p, int pos) { return sh1(P[p * PS + pos]); }, put);
+  }
+  __syncthreads();
+  fx_stage2<MAXR, false>(a.ax[1], npl, twy, get, put);
+  if (threadIdx.x == 0) sh->mag = 0;
+  __syncthreads();
+  // the largest column norm, in units of 2^32, rounded up (the +2 and the factor cover every rounding here)
+  for (int i = threadIdx.x; i < 4 * n2; i += blockDim.x) {
+    const int part = i / n2, c = i - part * n2;
+    float s = 0.f;
+    for (int p = part; p < npl; p += 4) {
+      const longlong2 v = P[p * PS + c];
+      const float x = (float)(abs((int)(v.x >> 32)) + 2), y = (float)(abs((int)(v.y >> 32)) + 2);
+      s = fmaf(x, x, fmaf(y, y, s));
+    }
+    cn[i] = s;
+  }
+  __syncthreads();
+  {
+    float s = 0.f;
+    for (int c = threadIdx.x; c < n2; c += blockDim.x) s = fmaxf(s, cn[c] + cn[n2 + c] + cn[2 * n2 + c] + cn[3 * n2 + c]);
+    const unsigned u = __reduce_max_sync(0xffffffffu, __float_as_uint(s));
+    if (lane == 0) atomicMax(reinterpret_cast<unsigned*>(&sh->norm), u);
+  }
+  __syncthreads();
+  // norm < 2^bits: bits from the exponent of its square
+  const float nrm = sh->norm * 1.001f;
+  const int sq = (int)((__float_as_uint(nrm) >> 23) & 0xff) - 126;   // square < 2^sq (in units of 2^64)
+  const int bits = 32 + ((sq + 1) >> 1);
+  const int dx = 63 - bits - a.hx;
+  const FxShift shx(dx);
+  e += ve + 2 + a.s3 - dx;
+  const long long* V = a.V + (size_t)j3 * n1 * n2;
+  unsigned long long my = 0;
+  for (int c0 = 0; c0 < n2; c0 += cw) {
+    const int nc = min(cw, n2 - c0);
+    fx_stage1<MAXR, false>(
+        a.ax[0], nc, twx,
+        [&](int c, int pos) {
+          const int pp = xm[pos];
+          longlong2 v = {0, 0};
+          if (pp >= 0) v = shx(P[pp * PS + c0 + c]);
+          return v;
+        },
+        [&](int c, int pos, longlong2 v) { X[pos * cw + c] = v; });
+    __syncthreads();
+    radix_switch<MAXR>(a.ax[0].r2, [&](auto rc) {
+      constexpr int R = decltype(rc)::value;
+      const FixedAxis& ax = a.ax[0];
+      const int items = nc * ax.r1;
+      const float inv = 1.0f / (float)nc;
+      for (int it = threadIdx.x; it < items; it += blockDim.x) {
+        int k1, c;
+        split_index(it, nc, inv, k1, c);
+        longlong2 v[R];
+        int pos = k1 * ax.r2;
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          v[i] = X[pos * cw + c];
+          pos += ax.s2;
+          if (pos >= n1) pos -= n1;
+        }
+        FxDft<R>::run(v);
+        pos = k1 * ax.r2;
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          const long long w = __ldg(V + (size_t)pos * n2 + c0 + c);
+          const int wh = fx_hi(w), wl = fx_lo(w);
+          const longlong2 u = {fx_mulr(v[i].y, wh, wl), fx_mulr(v[i].x, wh, wl)};   // swapped: the forward sign
+          v[i] = u;
+          pos += ax.s2;
+          if (pos >= n1) pos -= n1;
+        }
+        FxDft<R>::run(v);
+        const int s3 = a.s3;
+        const long long half = s3 ? 1LL << (s3 - 1) : 0;
+        pos = k1 * ax.r2;
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          longlong2 u = {(v[i].x + half) >> s3, (v[i].y + half) >> s3};
+          if (i > 0 && ax.s2 == 1) u = fx_twiddle(u, twx[k1 * i]);
+          X[pos * cw + c] = u;
+          pos += ax.s2;
+          if (pos >= n1) pos -= n1;
+        }
+      }
+    });
+    __syncthreads();
+    fx_stage1<MAXR, true>(
+        a.ax[0], nc, twx, [&](int c, int pos) { return X[pos * cw + c]; },
+        [&](int c, int pos, longlong2 v) {
+          const int pp = xm[pos];
+          if (pp >= 0) {
+            my |= fx_mag(v);
+            P[pp * PS + c0 + c] = v;   // still swapped
+          }
+        });
+    __syncthreads();
+  }
+  fx_or(sh, my);
+  __syncthreads();
+  my = sh->mag;
+  const int d = my ? fx_headroom(my, a.hyf) : 0;
+  e -= d;
+  const FxShift shy(d);
+  fx_stage2<MAXR, true>(a.ax[1], npl, twy, [&](int p, int pos) { return shy(P[p * PS + pos]); }, put);
+  __syncthreads();
+  fx_stage1<MAXR, true>(a.ax[1], npl, twy, get, put);
+  __syncthreads();
+  longlong2* yo = a.Yb + ((size_t)b * a.n3 + j3) * a.nst;
+  for (int p = warp; p < npl; p += nw) {
+    const int* ym = a.ymap + (size_t)p * n2;
+    for (int j2 = lane; j2 < n2; j2 += 32) {
+      const int s = __ldg(ym + j2);
+      if (s >= 0) yo[s] = P[p * PS + j2];   // still swapped: the z kernel goes on with the forward sign
+    }
+  }
+  if (threadIdx.x == 0) a.Ey[(size_t)b * a.n3 + j3] = my ? e : kFxZero;
+}
+
+template <int MAXR>
+__device__ __forceinline__ void fx_zfwd_tile(const FxItem& a, int ch, int b, unsigned char* smem, FxShared* sh) {
+  const int n = a.n3, ld = a.sc + 1;
+  FxTw* tw = reinterpret_cast<FxTw*>(smem);
+  longlong2* L = reinterpret_cast<longlong2*>(smem + sizeof(FxTw) * n);
+  const int s0 = ch * a.sc, ns = min(a.sc, a.nst - s0);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  if (threadIdx.x == 0) {
+    sh->emax = kFxZero;
+    sh->mag = 0;
+  }
+  load_table(tw, a.ax[2]);
+  __syncthreads();
+  const int* ey = a.Ey + (size_t)b * n;
+  int em = kFxZero;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) em = max(em, ey[i]);
+  em = __reduce_max_sync(0xffffffffu, em);
+  if (lane == 0 && em > kFxZero) atomicMax(&sh->emax, em);
+  __syncthreads();
+  int e = sh->emax;
+  const bool bad = e >= kFxNan / 2;
+  if (!bad) {
+    const longlong2* Y = a.Yb + (size_t)b * n * a.nst + s0;
+    const int per = blockDim.x / a.sc, r0 = threadIdx.x / a.sc, sl = threadIdx.x - r0 * a.sc;
+    unsigned long long m = 0;
+    if (sl < ns)
+      for (int j3 = r0; j3 < n; j3 += per) {
+        const longlong2 v = fx_align(Y[(size_t)j3 * a.nst + sl], e - ey[j3]);
+        m |= fx_mag(v);
+        L[a.ax[2].slot[j3] * ld + sl] = v;
+      }
+    fx_or(sh, m);
+    __syncthreads();
+    m = sh->mag;
+    const int d = m ? fx_headroom(m, a.hzf) : 0;
+    e -= d;
+    auto get = [&](int line, int pos) { return L[pos * ld + line]; };
+    auto put = [&](int line, int pos, longlong2 v) { L[pos * ld + line] = v; };
+    const FxShift shz(d);
+    fx_stage2<MAXR, true>(a.ax[2], ns, tw, [&](int line, int pos) { return shz(L[pos * ld + line]); }, put);
+    __syncthreads();
+    fx_stage1<MAXR, true>(a.ax[2], ns, tw, get, put);
+    __syncthreads();
+  }
+  // 2^e / N_r: by its exponent field where that stays a normal number
+  const int fe = (int)(__double_as_longlong(a.inv_nr) >> 52) + e;
+  const double f = bad                     ? __longlong_as_double(0x7ff8000000000000LL)
+                   : fe > 0 && fe < 0x7ff ? __longlong_as_double(__double_as_longlong(a.inv_nr) + ((long long)e << 52))
+                                          : ldexp(a.inv_nr, e);
+  for (int s = warp; s < ns; s += nw) {
+    const StickDev st = a.sticks[s0 + s];
+    const double2* ps = a.psi + (size_t)b * a.npw + st.g0;
+    double2* out = a.hpsi + (size_t)b * a.npw + st.g0;
+    const double* kin = a.kin + st.g0;
+    for (int tt = lane; tt < st.len; tt += 32) {
+      int pos = st.z0 + tt;
+      if (pos >= n) pos -= n;
+      const double2 x = ps[tt];
+      const double kg = kin[tt];
+      longlong2 v = {0, 0};
+      if (!bad) v = L[pos * ld + s];
+      out[tt] = make_double2(fma(kg, x.x, (double)v.y * f), fma(kg, x.y, (double)v.x * f));
+    }
+  }
+}
+
+__device__ __forceinline__ int fx_find(const int* off, int n, int t) {
+  int lo = 0, hi = n - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (off[mid] <= t) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+template <int MAXR>
+__global__ void __launch_bounds__(256, MAXR > 10 ? 2 : 3) k_fx_zinv(const __grid_constant__ FxBatch bt) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ FxShared sh;
+  const int i = fx_find(bt.off_z, bt.nitems, blockIdx.x), l = blockIdx.x - bt.off_z[i];
+  fx_zinv_tile<MAXR>(bt.item[i], l % bt.item[i].nch, l / bt.item[i].nch, smem_raw, &sh);
+}
+template <int MAXR>
+__global__ void __launch_bounds__(kFxThreads<MAXR>, 1) k_fx_plane(const __grid_constant__ FxBatch bt) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ FxShared sh;
+  const int i = fx_find(bt.off_p, bt.nitems, blockIdx.x), l = blockIdx.x - bt.off_p[i];
+  fx_plane_tile<MAXR>(bt.item[i], l % bt.item[i].n3, l / bt.item[i].n3, smem_raw, &sh);
+}
+template <int MAXR>
+__global__ void __launch_bounds__(256, MAXR > 10 ? 2 : 3) k_fx_zfwd(const __grid_constant__ FxBatch bt) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ FxShared sh;
+  const int i = fx_find(bt.off_z, bt.nitems, blockIdx.x), l = blockIdx.x - bt.off_z[i];
+  fx_zfwd_tile<MAXR>(bt.item[i], l % bt.item[i].nch, l / bt.item[i].nch, smem_raw, &sh);
+}
+
+#include "nonlocal_tiles.cuh"
+
+// The whole batch in one cooperative launch: the tiles of the three kernels above phase by phase, and, when
+// nl.nitems > 0, the float64 nonlocal term of the items, with a bounded grid barrier between the phases.  CTAs
+// take tiles from a phase's list one at a time through an atomic counter.
+struct FxPersist {
+  unsigned* bar;   // [0]: arrival counter; [1 + phase]: tile counters; zero at launch
+  int* err;
+};
+
+template <int MAXR>
+__global__ void __launch_bounds__(256, 2) k_fx_batch(const __grid_constant__ FxBatch bt,
+                                                     const __grid_constant__ NlBatch nl, const FxPersist pc) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ FxShared sh;
+  const unsigned G = gridDim.x;
+  const int nz = bt.off_z[bt.nitems], np = bt.off_p[bt.nitems];
+  for (int t = persist_next(pc.bar + 1); t < nz; t = persist_next(pc.bar + 1)) {
+    const int i = fx_find(bt.off_z, bt.nitems, t), l = t - bt.off_z[i];
+    fx_zinv_tile<MAXR>(bt.item[i], l % bt.item[i].nch, l / bt.item[i].nch, smem_raw, &sh);
+  }
+  if (!persist_sync(pc.bar, G, pc.err)) return;
+  for (int t = persist_next(pc.bar + 2); t < np; t = persist_next(pc.bar + 2)) {
+    const int i = fx_find(bt.off_p, bt.nitems, t), l = t - bt.off_p[i];
+    fx_plane_tile<MAXR>(bt.item[i], l % bt.item[i].n3, l / bt.item[i].n3, smem_raw, &sh);
+  }
+  if (!persist_sync(pc.bar, 2 * G, pc.err)) return;
+  for (int t = persist_next(pc.bar + 3); t < nz; t = persist_next(pc.bar + 3)) {
+    const int i = fx_find(bt.off_z, bt.nitems, t), l = t - bt.off_z[i];
+    fx_zfwd_tile<MAXR>(bt.item[i], l % bt.item[i].nch, l / bt.item[i].nch, smem_raw, &sh);
+  }
+  if (nl.nitems > 0) nonlocal_phases(nl, pc.bar, pc.err, G, 3, reinterpret_cast<double2*>(smem_raw));
+}
+
+// ---- setup ------------------------------------------------------------------------------------
+
+constexpr int kRadices[] = {2, 3, 4, 5, 6, 8, 9, 10, 12, 15, 16};
+
+int gcd(int a, int b) { return b ? gcd(b, a % b) : a; }
+int ceil_log2(double x) { return std::max(0, (int)std::ceil(std::log2(x))); }
+
+// The largest |V| bit pattern (NaN above infinity above every finite value)
+__global__ void k_fx_vmax(size_t n, const double* __restrict__ v, unsigned long long* __restrict__ out) {
+  unsigned long long m = 0;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+    m = max(m, (unsigned long long)__double_as_longlong(v[i]) & 0x7fffffffffffffffULL);
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+}
+// V[j3][j2][j1] -> [j3][slot of j1][slot of j2] as V 2^(62 - vexp), |V| < 2^vexp
+__global__ void k_fx_v(FixedAxis a1, FixedAxis a2, int n3, const double* __restrict__ v,
+                       const unsigned long long* __restrict__ vmax, long long* __restrict__ out, int* __restrict__ vexp) {
+  const int emax = (int)(*vmax >> 52);
+  const size_t n = (size_t)a1.n * a2.n * n3;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *vexp = emax == 0x7ff ? kFxNan : emax == 0 ? 0 : emax - 1022;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    const int j1 = (int)(i % a1.n), j2 = (int)(i / a1.n % a2.n);
+    const size_t j3 = i / ((size_t)a1.n * a2.n);
+    out[(j3 * a1.n + a1.slot[j1]) * a2.n + a2.slot[j2]] = fx_from_bits(__double_as_longlong(v[i]), emax - 9);
+  }
+}
+
+struct FxLaunch {
+  FxBatch bt;
+  size_t smem_z = 0, smem_p = 0;
+  int maxr = 0, items = 0;   // largest radix, largest stage of a plane
+  void add(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nb, void* zt, void* yb) {
+    const int i = bt.nitems++;
+    FxItem& it = bt.item[i];
+    const FixedPlan& f = p.fixed;
+    it.nb = nb;
+    it.npw = p.npw;
+    it.npl = p.npl;
+    it.nst = p.nst;
+    it.n1 = p.n[0];
+    it.n2 = p.n[1];
+    it.n3 = p.n[2];
+    for (int a = 0; a < 3; ++a) {
+      it.ax[a] = f.ax[a];
+      maxr = std::max(maxr, std::max(f.ax[a].r1, f.ax[a].r2));
+    }
+    items = std::max(items, std::max(it.npl * std::max(f.ax[1].r1, f.ax[1].r2), f.cw * std::max(f.ax[0].r1, f.ax[0].r2)) + 31);
+    it.cw = f.cw;
+    it.sc = f.sc;
+    it.nch = f.nch;
+    it.hz = f.hz;
+    it.hy = f.hy;
+    it.hx = f.hx;
+    it.s3 = f.s3;
+    it.hyf = f.hyf;
+    it.hzf = f.hzf;
+    it.sticks = p.d_sticks;
+    it.ymap = p.d_ymap;
+    it.xmap = p.d_xmap;
+    it.psi = psi;
+    it.hpsi = hpsi;
+    it.kin = p.d_kin;
+    const size_t rows = (size_t)nb * p.n[2] * p.nst;
+    it.Zt = static_cast<longlong2*>(zt);
+    it.Yb = static_cast<longlong2*>(yb);
+    it.Ez = reinterpret_cast<int*>(it.Zt + rows);   // beside the rows (local_row_bytes)
+    it.Ey = reinterpret_cast<int*>(it.Yb + rows);
+    it.V = static_cast<const long long*>(c.vbufs[p.vslot + 2]);
+    it.vexp = static_cast<const int*>(c.vbufs[p.vslot + 3]) + 2;
+    it.inv_nr = 1.0 / ((double)p.n[0] * p.n[1] * p.n[2]);
+    bt.off_z[i + 1] = bt.off_z[i] + f.nch * nb;
+    bt.off_p[i + 1] = bt.off_p[i] + p.n[2] * nb;
+    smem_z = std::max(smem_z, f.smem_z);
+    smem_p = std::max(smem_p, f.smem_p);
+  }
+  void reset() {
+    bt.nitems = 0;
+    bt.off_z[0] = bt.off_p[0] = 0;
+    smem_z = smem_p = 0;
+    maxr = items = 0;
+  }
+  template <int MAXR> int run_t(Context& c) {
+    static bool attr = false;
+    if (!attr) {
+      const int mx = (int)c.smem_optin - 64;
+      cudaFuncSetAttribute(k_fx_zinv<MAXR>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+      cudaFuncSetAttribute(k_fx_plane<MAXR>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+      cudaFuncSetAttribute(k_fx_zfwd<MAXR>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+      attr = true;
+    }
+    const int nz = bt.off_z[bt.nitems], np = bt.off_p[bt.nitems];
+    // the plane kernel's block: the resident threads over the CTAs that fit an SM (or that there are), no more than a
+    // stage has items
+    const int fit = std::max<int>(1, std::min<size_t>(16, c.smem_optin / (smem_p + 1100)));
+    const int ctas = std::max(1, std::min(fit, (np + c.sm_count - 1) / c.sm_count));
+    const int block = std::max(64, std::min(kFxThreads<MAXR> / ctas, items) / 32 * 32);
+    HPSI_LAUNCH(c, HPSI_K_INV_ZY, (k_fx_zinv<MAXR><<<nz, 256, smem_z, c.stream>>>(bt)));
+    HPSI_LAUNCH(c, HPSI_K_XVX_Y, (k_fx_plane<MAXR><<<np, block, smem_p, c.stream>>>(bt)));
+    HPSI_LAUNCH(c, HPSI_K_FWD_Z, (k_fx_zfwd<MAXR><<<nz, 256, smem_z, c.stream>>>(bt)));
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(c, e, "fixed-point local kernels launch");
+    return HPSI_OK;
+  }
+  int run(Context& c) { return maxr > 10 ? run_t<16>(c) : run_t<10>(c); }
+  static constexpr size_t kFxTwoCtas = 112 * 1024;   // dynamic shared memory that still allows two CTAs per SM
+
+  template <int MAXR> int persistent_t(Context& c, const NlBatch& nl, unsigned* bar, bool* done) {
+    const void* kern = (const void*)k_fx_batch<MAXR>;
+    size_t dyn = std::max(smem_z, smem_p);
+    if (nl.nitems > 0) dyn = std::max(dyn, sizeof(double2) * (size_t)std::max(CB_SMEM, AV_SMEM));
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || fa.sharedSizeBytes + dyn > c.smem_optin ||
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) {
+      cudaGetLastError();
+      return HPSI_OK;
+    }
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 256, dyn) != cudaSuccess || occ < 1) {
+      cudaGetLastError();
+      return HPSI_OK;
+    }
+    cudaError_t e = cudaMemsetAsync(bar, 0, 8 * sizeof(unsigned), c.stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "persistent batch barrier reset");
+    FxPersist pc{bar, c.d_err};
+    void* args[] = {(void*)&bt, (void*)&nl, (void*)&pc};
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(occ * c.sm_count);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = dyn;
+    cfg.stream = c.stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    HPSI_LAUNCH(c, HPSI_K_BATCH, (e = cudaLaunchKernelExC(&cfg, kern, args)));
+    if (e != cudaSuccess) return cuda_fail(c, e, "persistent batched H|psi> launch");
+    *done = true;
+    return HPSI_OK;
+  }
+  int persistent(Context& c, const NlBatch& nl, unsigned* bar, bool* done) {
+    return maxr > 10 ? persistent_t<16>(c, nl, bar, done) : persistent_t<10>(c, nl, bar, done);
+  }
+};
+
+}  // namespace
+
+// Factors of an edge (0 if it has none): coprime ones first (no twiddles), then the smaller larger factor; r1 >= r2,
+// which gives the x stage between the transforms more items and a tighter bound.
+void fixed_factors(int n, int* r1, int* r2) {
+  *r1 = *r2 = 0;
+  bool best_cop = false;
+  for (int a : kRadices)
+    for (int b : kRadices) {
+      if (a * b != n || a < b) continue;
+      const bool cop = gcd(a, b) == 1;
+      if (*r1 == 0 || (cop && !best_cop) || (cop == best_cop && a < *r1)) {
+        *r1 = a;
+        *r2 = b;
+        best_cop = cop;
+      }
+    }
+}
+
+// The table of an edge (empty if it has no factors): in the Cooley-Tukey form the twiddles e^{2 pi i j / n}, then the
+// slot of every index after the inverse transform; returns where the slots begin.
+size_t fixed_tables(int n, std::vector<int>& tw, FixedAxis* ax) {
+  int r1, r2;
+  fixed_factors(n, &r1, &r2);
+  ax->n = n;
+  ax->r1 = r1;
+  ax->r2 = r2;
+  tw.clear();
+  if (!r1) return 0;
+  const bool pfa = gcd(r1, r2) == 1;
+  ax->s2 = pfa ? r1 : 1;
+  for (int j = 0; j < (pfa ? 0 : n); ++j) {
+    // reduced to the first octant, so that long double keeps 62 bits
+    const int o = 8 * j / n, r = 8 * j % n;
+    const long double pi4 = 0.785398163397448309615660845819875721L;
+    const long double th = pi4 * (long double)((o & 1) ? n - r : r) / (long double)n;
+    const long double c0 = std::cos(th), s0 = std::sin(th);
+    long double c = 0, s = 0;
+    switch (o) {
+      case 0: c = c0; s = s0; break;
+      case 1: c = s0; s = c0; break;
+      case 2: c = -s0; s = c0; break;
+      case 3: c = -c0; s = s0; break;
+      case 4: c = -c0; s = -s0; break;
+      case 5: c = -s0; s = -c0; break;
+      case 6: c = s0; s = -c0; break;
+      default: c = c0; s = -s0; break;
+    }
+    for (const long double x : {c, s}) {
+      const long long q = std::llround(x * 4611686018427387904.0L);
+      tw.push_back(fx_hi(q));
+      tw.push_back(fx_lo(q));
+    }
+  }
+  const size_t slots = tw.size();
+  for (int k = 0; k < n; ++k) tw.push_back((r2 * (k % r1) + ax->s2 * (pfa ? k % r2 : k / r1)) % n);
+  return slots;
+}
+
+// The plan of a problem whose axes are filled in (ok = false: no factors, or a plane does not fit).
+void fixed_plan(Problem& p, size_t smem_optin) {
+  FixedPlan& f = p.fixed;
+  f.ok = false;
+  for (int a = 0; a < 3; ++a)
+    if (!f.ax[a].r1) return;
+  const int n1 = p.n[0], n2 = p.n[1], n3 = p.n[2];
+  auto tws = [&](int a) { return f.ax[a].s2 == 1 ? sizeof(FxTw) * (size_t)p.n[a] : 0; };
+  // z chunks: 32 sticks fill a stage's items and the store's rows; 16 where that would take over half an SM's memory
+  f.sc = n3 <= 100 ? 32 : 16;
+  f.nch = (p.nst + f.sc - 1) / f.sc;
+  f.smem_z = sizeof(FxTw) * (size_t)n3 + sizeof(longlong2) * (size_t)n3 * (f.sc + 1);
+  // x columns per chunk: two CTAs per SM where the plane leaves at least 12 columns for that, else one
+  const size_t base = tws(0) + tws(1) + sizeof(longlong2) * (size_t)p.npl * (n2 | 1) + sizeof(int) * n1;
+  const size_t col = sizeof(longlong2) * (size_t)n1;
+  auto width = [&](size_t room) { return room > base ? (int)std::min<size_t>((room - base) / col, 48) : 0; };
+  int cw = width(FxLaunch::kFxTwoCtas);
+  if (cw < std::min(12, n2)) cw = width(smem_optin - 1024);
+  cw = std::min(cw, n2);
+  if (cw < 4 && cw < n2) return;
+  const int chunks = (n2 + cw - 1) / cw;
+  f.cw = (n2 + chunks - 1) / chunks;
+  f.smem_p = base + col * f.cw;
+  if (col * f.cw < sizeof(float) * 4 * (size_t)n2 || f.smem_z > smem_optin - 1024) return;
+  int zl = 1;
+  for (const StickDev& s : p.sticks) zl = std::max(zl, s.len);
+  // growth bounds: sum |x_n| <= L sqrt2 max for the stages scaled by their largest component ...
+  const double r2 = std::sqrt(2.0);
+  f.hz = ceil_log2(kFixGain * r2 * zl);
+  f.hy = ceil_log2(kFixGain * r2 * p.ns_max);
+  f.hyf = ceil_log2(kFixGain * r2 * n2);
+  f.hzf = ceil_log2(kFixGain * r2 * n3);
+  // ... and for the x stages, scaled by the largest column 2-norm B: sqrt(npl) B before V; behind V (scaled to 1/4)
+  // sqrt(n1) B / 4 is the line's 2-norm, so sqrt(R2 n1) B / 4 after the first codelet and n1 B / 4 at the end, with
+  // s3 further bits given up in between
+  f.hx = ceil_log2(kFixGain * std::max(std::sqrt((double)p.npl), std::sqrt((double)f.ax[0].r2 * n1) / 4.0));
+  f.s3 = std::max(0, ceil_log2(kFixGain * n1 / 4.0) - f.hx);
+  f.ok = true;
+}
+
+// Fixed-point copy of V (vbufs[slot + 2], its exponent in vbufs[slot + 3]) from the float64 one.
+int fixed_potential(Context& c, int slot, const FixedAxis ax[3], int kernel_class) {
+  unsigned long long* vm = static_cast<unsigned long long*>(c.vbufs[slot + 3]);
+  const size_t nr = (size_t)ax[0].n * ax[1].n * ax[2].n;
+  const double* v = static_cast<const double*>(c.vbufs[slot]);
+  const int grid = (int)std::min<size_t>(4 * c.sm_count, (nr + 255) / 256);
+  cudaError_t e = cudaMemsetAsync(vm, 0, 16, c.stream);
+  if (e != cudaSuccess) return cuda_fail(c, e, "fixed-point potential");
+  HPSI_LAUNCH(c, kernel_class, (k_fx_vmax<<<grid, 256, 0, c.stream>>>(nr, v, vm)));
+  HPSI_LAUNCH(c, kernel_class, (k_fx_v<<<grid, 256, 0, c.stream>>>(ax[0], ax[1], ax[2].n, v, vm,
+                                                                   static_cast<long long*>(c.vbufs[slot + 2]),
+                                                                   reinterpret_cast<int*>(vm) + 2)));
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(c, e, "fixed-point potential");
+  return HPSI_OK;
+}
+
+int local_fixed_apply(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd, void* Zt, void* Yb,
+                      int nbb) {
+  static FxLaunch fl;   // host staging of the parameter block (calls are not thread-safe by contract)
+  const int rv = ensure_fixed_potential(c, p.vslot, p.fixed.ax);
+  if (rv) return rv;
+  for (int b0 = 0; b0 < nbnd; b0 += nbb) {
+    fl.reset();
+    fl.add(c, p, psi + (size_t)b0 * p.npw, hpsi + (size_t)b0 * p.npw, std::min(nbb, nbnd - b0), Zt, Yb);
+    const int rc = fl.run(c);
+    if (rc) return rc;
+  }
+  return HPSI_OK;
+}
+
+int local_fixed_apply_multi(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
+                            double2* const* hpsi, void* const* zt, void* const* yb) {
+  static FxLaunch fl;
+  for (int i0 = 0; i0 < nitem; i0 += kFxMaxItems) {
+    fl.reset();
+    for (int i = i0; i < std::min(nitem, i0 + kFxMaxItems); ++i)
+      fl.add(c, c.probs[prob[i]], psi[i], hpsi[i], nbnd[i], zt[i], yb[i]);
+    const int rc = fl.run(c);
+    if (rc) return rc;
+  }
+  return HPSI_OK;
+}
+
+int local_fixed_persistent(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
+                           double2* const* hpsi, void* const* zt, void* const* yb, bool with_nl, bool* done) {
+  static FxLaunch fl;
+  static NlBatch nl;
+  fl.reset();
+  for (int i = 0; i < nitem; ++i) fl.add(c, c.probs[prob[i]], psi[i], hpsi[i], nbnd[i], zt[i], yb[i]);
+  nl.nitems = 0;
+  if (with_nl) {
+    const int rc = persistent_nl_batch(c, nitem, prob, nbnd, psi, hpsi, nl);
+    if (rc) return rc;
+  }
+  int rc = ensure_buffer(c, &c.ws.pbar, &c.ws.pbarbytes, 256);
+  if (rc) return rc;
+  return fl.persistent(c, nl, static_cast<unsigned*>(c.ws.pbar), done);
+}
+
+}  // namespace hpsi

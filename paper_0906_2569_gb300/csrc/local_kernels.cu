@@ -232,10 +232,16 @@ size_t local_smem_bytes(const Problem& p, int precision, int which) {
   return cs * (size_t)p.ns_max * p.n[2];
 }
 
+size_t local_row_bytes(const Problem& p, int precision, int nb) {
+  const size_t cs = precision == HPSI_FP64 ? sizeof(double2) : sizeof(float2);
+  const size_t rows = cs * (size_t)nb * p.n[2] * p.nst;
+  return precision == HPSI_FP64 && p.fixed.ok ? rows + sizeof(int) * (size_t)nb * std::max(p.fixed.nch, p.n[2]) : rows;
+}
+
 // Autotuner of the fast path: time every plan that fits the shared memory (which of the V plane
 // and the stick row the plane kernel stages) against band blocks of half, one and two times the
 // default, on this call's own bands, and keep the fastest.  Neither choice changes the arithmetic.
-static int tune_fast(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd, size_t cs) {
+static int tune_fast(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd) {
   const int pr = cur_prec(c);
   const std::vector<int> plans = local_fast_candidates(p, pr, c.smem_optin);
   const int nb0 = p.nbbf[pr];
@@ -256,7 +262,7 @@ static int tune_fast(Context& c, const Problem& p, const double2* psi, double2* 
   int rc = HPSI_OK;
   for (int plan : plans)
     for (int nb : blocks) {
-      const size_t need = cs * (size_t)nb * p.n[2] * p.nst;
+      const size_t need = local_row_bytes(p, pr, nb);
       rc = ensure_buffer(c, &c.ws.X, &c.ws.xbytes, need);
       if (!rc) rc = ensure_buffer(c, &c.ws.Y, &c.ws.ybytes, need);
       if (rc) break;
@@ -289,12 +295,15 @@ static int local_apply_t(Context& c, const Problem& p, const double2* psi, doubl
   if ((p.fflags[cur_prec(c)] & 4) && !c.force_generic) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(c.stream, &cap);
-    if (c.autotune && !p.tuned[cur_prec(c)] && nbnd >= 4 && cap == cudaStreamCaptureStatusNone) {
-      int rc = tune_fast(c, p, psi, hpsi, nbnd, cs);
+    // (the fixed-point float64 form has one plan, and its time hardly depends on the block)
+    if (c.autotune && cur_prec(c) == HPSI_MIXED && !p.tuned[HPSI_MIXED] && nbnd >= 4 &&
+        cap == cudaStreamCaptureStatusNone) {
+      int rc = tune_fast(c, p, psi, hpsi, nbnd);
       if (rc) return rc;
     }
-    const int nbf = std::max(1, std::min(p.nbbf[cur_prec(c)], nbnd));
-    const size_t zneed = cs * (size_t)nbf * p.n[2] * p.nst;
+    int nbf = std::max(1, std::min(p.nbbf[cur_prec(c)], nbnd));
+    if (cur_prec(c) == HPSI_FP64) nbf = (nbnd + (nbnd + nbf - 1) / nbf - 1) / ((nbnd + nbf - 1) / nbf);   // even blocks
+    const size_t zneed = local_row_bytes(p, cur_prec(c), nbf);
     int rc = ensure_buffer(c, &c.ws.X, &c.ws.xbytes, zneed);
     if (rc) return rc;
     rc = ensure_buffer(c, &c.ws.Y, &c.ws.ybytes, zneed);

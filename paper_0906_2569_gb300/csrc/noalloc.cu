@@ -91,9 +91,11 @@ extern "C" int hpsi_apply_noalloc(hpsi_ctx* ctx, int ik, const void* psi_in, voi
   const bool fast = (p.fflags[prec] & 4) && !c.force_generic;
   const size_t cs = prec == HPSI_FP64 ? sizeof(double2) : sizeof(float2);
   auto xbytes = [&](int nb) {
-    return align256(cs * (size_t)nb * p.n[2] * (fast ? (size_t)p.nst : (size_t)p.npl * p.n[1]));
+    return align256(fast ? hpsi::local_row_bytes(p, prec, nb) : cs * (size_t)nb * p.n[2] * p.npl * p.n[1]);
   };
-  auto ybytes = [&](int nb) { return align256(cs * (size_t)nb * p.n[2] * p.nst); };
+  auto ybytes = [&](int nb) {
+    return align256(fast ? hpsi::local_row_bytes(p, prec, nb) : cs * (size_t)nb * p.n[2] * p.nst);
+  };
   const size_t per_band = xbytes(1) + ybytes(1);
   int chunk = 0;
   for (int nb = std::min(nbnd, 4096); nb >= 1; nb = nb > 64 ? nb - 32 : nb - 1) {

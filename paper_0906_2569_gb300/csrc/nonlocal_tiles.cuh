@@ -4,6 +4,8 @@
 // tiles.  Included inside an anonymous namespace of namespace hpsi, once per translation unit.
 #pragma once
 
+#include "persist.cuh"
+
 // acc += conj(x) y and acc += x y, four float64 FMAs each
 __device__ __forceinline__ void cmac_conj(double2& acc, double2 x, double2 y) {
   acc.x = fma(x.x, y.x, acc.x);
@@ -203,3 +205,78 @@ __device__ __forceinline__ int find_item(const int* off, int nitems, int blk) {
   return i;
 }
 
+// The nonlocal phases of a persistent launch: calbec, D-scale and add_vuspsi tiles of every item, each after a grid
+// barrier; `before` barriers have been passed, and phase counters bar[2 + before] on are unused so far.
+__device__ __forceinline__ void nonlocal_phases(const NlBatch& nl, unsigned* bar, int* err, unsigned G, int before,
+                                                double2* sm) {
+  if (!persist_sync(bar, before * G, err)) return;
+  const int nc = nl.off_cal[nl.nitems];
+  for (int t = persist_next(bar + before + 1); t < nc; t = persist_next(bar + before + 1)) {
+    const int i = find_item(nl.off_cal, nl.nitems, t);
+    const NlItem& a = nl.item[i];
+    const int l = t - nl.off_cal[i], r = l / a.tilesp;
+    calbec_tile(a.npw, a.nproj, a.nb, a.kchunk, a.beta, a.psi, a.part, l % a.tilesp, r % a.tilesb, r / a.tilesb, sm);
+  }
+  if (!persist_sync(bar, (before + 1) * G, err)) return;
+  for (int t = blockIdx.x; t < nl.off_ds[nl.nitems]; t += G) {
+    const int i = find_item(nl.off_ds, nl.nitems, t);
+    const NlItem& a = nl.item[i];
+    dscale_one((t - nl.off_ds[i]) * blockDim.x + threadIdx.x, a.nproj, a.nb, a.nsplit, a.part, a.rowptr, a.col, a.dval,
+               a.w);
+  }
+  if (!persist_sync(bar, (before + 2) * G, err)) return;
+  const int na = nl.off_add[nl.nitems];
+  for (int t = persist_next(bar + before + 2); t < na; t = persist_next(bar + before + 2)) {
+    const int i = find_item(nl.off_add, nl.nitems, t);
+    const NlItem& a = nl.item[i];
+    const int l = t - nl.off_add[i];
+    addvus_tile(a.npw, a.nproj, a.nb, a.w, a.beta, a.hpsi, l % a.gtiles, l / a.gtiles, sm);
+  }
+}
+
+// The items' nonlocal geometry for a persistent launch; partial sums and w side by side in the workspace.
+inline int persistent_nl_batch(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
+                               double2* const* hpsi, NlBatch& nl) {
+  std::vector<size_t> off(nitem);
+  std::vector<int> ns(nitem), kc(nitem);
+  size_t total = 0;
+  for (int i = 0; i < nitem; ++i) {
+    size_t bytes = 0;
+    nonlocal_fp64_plan(c, c.probs[prob[i]], nbnd[i], &ns[i], &kc[i], &bytes);
+    off[i] = total;
+    total += (bytes + 255) & ~size_t(255);
+  }
+  int rc = ensure_buffer(c, &c.ws.part, &c.ws.partbytes, std::max<size_t>(total, 256));
+  if (rc) return rc;
+  unsigned char* base = static_cast<unsigned char*>(c.ws.part);
+  int n = 0;
+  nl.off_cal[0] = nl.off_ds[0] = nl.off_add[0] = 0;
+  for (int i = 0; i < nitem; ++i) {
+    const Problem& p = c.probs[prob[i]];
+    if (p.nproj == 0) continue;
+    NlItem& a = nl.item[n];
+    a.npw = p.npw;
+    a.nproj = p.nproj;
+    a.nb = nbnd[i];
+    a.kchunk = kc[i];
+    a.nsplit = ns[i];
+    a.tp = CB_TP;
+    a.tilesp = (p.nproj + CB_TP - 1) / CB_TP;
+    a.tilesb = (a.nb + CB_TB - 1) / CB_TB;
+    a.gtiles = (p.npw + AV_TG - 1) / AV_TG;
+    a.beta = p.d_beta;
+    a.psi = psi[i];
+    a.hpsi = hpsi[i];
+    a.part = reinterpret_cast<double2*>(base + off[i]);
+    a.w = a.part + (size_t)a.nsplit * a.nb * a.nproj;
+    a.rowptr = p.d_rowptr;
+    a.col = p.d_col;
+    a.dval = p.d_dval;
+    nl.off_cal[n + 1] = nl.off_cal[n] + a.tilesp * a.tilesb * a.nsplit;
+    nl.off_ds[n + 1] = nl.off_ds[n] + (a.nproj * a.nb + 255) / 256;
+    nl.off_add[n + 1] = nl.off_add[n] + a.gtiles * ((a.nb + AV_TB - 1) / AV_TB);
+    ++n;
+  }
+  nl.nitems = n;
+  return HPSI_OK;
+}
