@@ -469,6 +469,7 @@ static void free_problem(Problem& p) {
   cudaFree(p.d_dvalr);
   cudaFree(p.d_betar_bf);
   cudaFree(p.d_betar_df);
+  for (SlicePlanes& s : p.slices) cudaFree(s.digits);
 }
 
 static void free_context(Context& c) {
@@ -574,7 +575,9 @@ static int batch_apply_items(Context& c, int nitem, const int* prob, const int* 
     // one persistent launch per box edge (up to 32 items each), with the float64 nonlocal term of
     // its items; a group whose launch does not fit takes the launch-per-kernel path
     if (c.persistent && slow.empty()) {
-      const bool with_nl = nl_prec(c) == HPSI_FP64;
+      // (items large enough for the tensor-core contractions take those, as in the separate launches)
+      bool with_nl = nl_prec(c) == HPSI_FP64;
+      for (size_t j = 0; with_nl && j < fast.size(); ++j) with_nl = !nonlocal_slices_use(c.probs[fp[j]], fn[j]);
       const int nf = (int)fast.size();
       for (int g0 = 0; g0 < nf;) {
         const Problem& q = c.probs[fp[g0]];

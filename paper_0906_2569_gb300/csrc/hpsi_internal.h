@@ -59,6 +59,14 @@ struct FixedPlan {
   size_t smem_z = 0, smem_p = 0;
 };
 
+// Digit planes of a problem's projectors for the float64 contractions on the tensor cores (nonlocal_slices.cu).
+struct SlicePlanes {
+  void* digits = nullptr;
+  int* exps = nullptr;
+  int kpad = 0;
+  bool no_room = false;   // the device had no memory for them
+};
+
 struct Problem {
   double cell[9];
   double recip[9];
@@ -106,6 +114,7 @@ struct Problem {
   double* d_betar = nullptr;
   double* d_dvalr = nullptr;
   uint16_t* d_betar_bf = nullptr;
+  mutable SlicePlanes slices[4];
   float2* d_betar_df = nullptr;    // (mixed contexts) betar as double-float pairs
 };
 
@@ -318,6 +327,18 @@ int nonlocal_fp64_into(Context& c, const Problem& p, const double2* psi, double2
 // The float64 nonlocal term of several problems' band blocks, one launch per kernel class
 int nonlocal_batch_fp64(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
                         double2* const* hpsi);
+
+// The float64 contractions as exact integer products on the tensor cores (nonlocal_slices.cu); *ok = false: no room for
+// the projectors' digits, the caller takes the CUDA-core kernels.
+bool nonlocal_slices_use(const Problem& p, int nbnd);
+int slices_w(Context& c, const Problem& p, const double2* psi, int nbnd, double2* w, bool* ok);
+int slices_add(Context& c, const Problem& p, const double2* w, double2* hpsi, int nbnd, bool* ok);
+bool gamma_slices_use(const Problem& p, int nbnd);
+int gamma_slices_w(Context& c, const Problem& p, const void* x, bool x32, int nbnd, bool scaled, double* w, bool* ok);
+int gamma_slices_add(Context& c, const Problem& p, const double* w, double* out, int nbnd, bool* ok);
+// w = D (sum of the splits' partial <beta|psi>), complex and Gamma form
+int dscale_fp64(Context& c, const Problem& p, int nb, int nsplit, const double2* part, double2* w);
+int gamma_dscale_fp64(Context& c, const Problem& p, int nb, int nsplit, const double* part, double* w);
 
 // ---- context helpers (api.cpp) ----
 int ensure_buffer(Context& c, void** ptr, size_t* have, size_t need);

@@ -2,8 +2,9 @@
 //   becp[b][p] = <beta_p|psi_b> = sum_G conj(beta_p(G)) psi_b(G)            (calbec)
 //   w[b][p]    = sum_q D_pq becp[b][q]                                          (D-scale, CSR of D)
 //   hpsi_b(G) += sum_p beta_p(G) w[b][p]                                        (add_vuspsi)
-// On GB300 float64 runs at ~1.2 TFLOP/s on the CUDA cores (the FP64 MMA path is not faster), so
-// these are plain shared-memory-tiled complex GEMMs whose inner loop is DFMA-bound; calbec
+// On GB300 float64 runs at ~1.2 TFLOP/s on the CUDA cores (the FP64 MMA path is not faster).  Large blocks go to
+// the tensor cores as exact integer products (nonlocal_slices.cu); here are the small ones:
+// plain shared-memory-tiled complex GEMMs whose inner loop is DFMA-bound; calbec
 // (P x nb outputs, K = npw) splits K across CTAs and reduces the partials deterministically in
 // the D-scale kernel.
 #include <cuda_runtime.h>
@@ -307,10 +308,38 @@ int gamma_w_df(Context& c, const Problem& p, const void* x, bool x32, int nb, bo
   return HPSI_OK;
 }
 
+int dscale_fp64(Context& c, const Problem& p, int nb, int nsplit, const double2* part, double2* w) {
+  const int n = p.nproj * nb;
+  HPSI_LAUNCH(c, HPSI_K_DSCALE,
+              (k_dscale64<<<(n + 255) / 256, 256, 0, c.stream>>>(p.nproj, nb, nsplit, part, p.d_rowptr, p.d_col,
+                                                                 p.d_dval, w)));
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(c, e, "float64 projection kernels launch");
+  return HPSI_OK;
+}
+
+int gamma_dscale_fp64(Context& c, const Problem& p, int nb, int nsplit, const double* part, double* w) {
+  const int n = p.nproj * nb;
+  HPSI_LAUNCH(c, HPSI_K_DSCALE,
+              (k_dscale64r<<<(n + 255) / 256, 256, 0, c.stream>>>(p.nproj, nb, nsplit, part, p.d_rowptr, p.d_col,
+                                                                  p.d_dvalr, w)));
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(c, e, "Gamma-form float64 projection kernels launch");
+  return HPSI_OK;
+}
+
 // w = D' <betar|x> of the real form in float64 (calbec and D-scale); *w points into the workspace.
 int gamma_w_fp64(Context& c, const Problem& p, const void* x, bool x32, int nb, bool scaled, double** wout) {
   if (!p.d_betar) return fail(c, HPSI_EINVAL, "Gamma-form projectors are not prepared");
   const int nr = 2 * ((p.npw + 1) / 2);
+  if (gamma_slices_use(p, nb)) {
+    int rc = ensure_buffer(c, &c.ws.w, &c.ws.wbytes, sizeof(double) * (size_t)nb * p.nproj);
+    if (rc) return rc;
+    *wout = static_cast<double*>(c.ws.w);
+    bool ok = false;
+    rc = gamma_slices_w(c, p, x, x32, nb, scaled, *wout, &ok);
+    if (rc || ok) return rc;
+  }
   const int tilesp = (p.nproj + RB_TP - 1) / RB_TP, tilesb = (nb + RB_TB - 1) / RB_TB;
   int nsplit = std::max(1, (3 * c.sm_count) / std::max(1, tilesp * tilesb));
   int kchunk = (nr + nsplit - 1) / nsplit;
@@ -331,14 +360,8 @@ int gamma_w_fp64(Context& c, const Problem& p, const void* x, bool x32, int nb, 
     HPSI_LAUNCH(c, HPSI_K_CALBEC, (k_calbec64r<double><<<gc, 256, 0, c.stream>>>(
                                       nr, p.nproj, nb, kchunk, scaled ? 1 : 0, p.d_betar,
                                       static_cast<const double*>(x), part)));
-  const int n = p.nproj * nb;
-  HPSI_LAUNCH(c, HPSI_K_DSCALE,
-              (k_dscale64r<<<(n + 255) / 256, 256, 0, c.stream>>>(p.nproj, nb, nsplit, part, p.d_rowptr, p.d_col,
-                                                                  p.d_dvalr, w)));
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(c, e, "Gamma-form float64 projection kernels launch");
   *wout = w;
-  return HPSI_OK;
+  return gamma_dscale_fp64(c, p, nb, nsplit, part, w);
 }
 
 int gamma_nonlocal_fp64(Context& c, const Problem& p, const void* x, bool x32, int nb, bool scaled, double* out) {
@@ -347,6 +370,11 @@ int gamma_nonlocal_fp64(Context& c, const Problem& p, const void* x, bool x32, i
   double* w = nullptr;
   int rc = gamma_w_fp64(c, p, x, x32, nb, scaled, &w);
   if (rc) return rc;
+  if (gamma_slices_use(p, nb)) {
+    bool ok = false;
+    rc = gamma_slices_add(c, p, w, out, nb, &ok);
+    if (rc || ok) return rc;
+  }
   HPSI_LAUNCH(c, HPSI_K_ADDVUS,
               (k_addvus64r<<<dim3((nr + RA_TR - 1) / RA_TR, (nb + RA_TB - 1) / RA_TB), 256, 0, c.stream>>>(
                   nr, p.nproj, nb, w, p.d_betar, out)));
@@ -357,6 +385,14 @@ int gamma_nonlocal_fp64(Context& c, const Problem& p, const void* x, bool x32, i
 
 // w = D <beta|psi> of the complex form in float64 (calbec and D-scale); *w points into the workspace.
 int nonlocal_w_fp64(Context& c, const Problem& p, const double2* psi, int nbnd, double2** wout) {
+  if (nonlocal_slices_use(p, nbnd)) {
+    int rc = ensure_buffer(c, &c.ws.w, &c.ws.wbytes, sizeof(double2) * (size_t)nbnd * p.nproj);
+    if (rc) return rc;
+    *wout = static_cast<double2*>(c.ws.w);
+    bool ok = false;
+    rc = slices_w(c, p, psi, nbnd, *wout, &ok);
+    if (rc || ok) return rc;
+  }
   const int tilesp = (p.nproj + CB_TP - 1) / CB_TP, tilesb = (nbnd + CB_TB - 1) / CB_TB;
   int nsplit = 0, kchunk = 0;
   size_t bytes = 0;
@@ -370,14 +406,8 @@ int nonlocal_w_fp64(Context& c, const Problem& p, const double2* psi, int nbnd, 
   HPSI_LAUNCH(c, HPSI_K_CALBEC,
               (k_calbec64<<<dim3(tilesp, tilesb, nsplit), 256, 0, c.stream>>>(p.npw, p.nproj, nbnd, kchunk,
                                                                               p.d_beta, psi, part)));
-  const int n = p.nproj * nbnd;
-  HPSI_LAUNCH(c, HPSI_K_DSCALE,
-              (k_dscale64<<<(n + 255) / 256, 256, 0, c.stream>>>(p.nproj, nbnd, nsplit, part, p.d_rowptr, p.d_col,
-                                                                 p.d_dval, w)));
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(c, e, "float64 projection kernels launch");
   *wout = w;
-  return HPSI_OK;
+  return dscale_fp64(c, p, nbnd, nsplit, part, w);
 }
 
 int nonlocal_apply_fp64(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd) {
@@ -385,6 +415,11 @@ int nonlocal_apply_fp64(Context& c, const Problem& p, const double2* psi, double
   double2* w = nullptr;
   int rc = nonlocal_w_fp64(c, p, psi, nbnd, &w);
   if (rc) return rc;
+  if (nonlocal_slices_use(p, nbnd)) {
+    bool ok = false;
+    rc = slices_add(c, p, w, hpsi, nbnd, &ok);
+    if (rc || ok) return rc;
+  }
   HPSI_LAUNCH(c, HPSI_K_ADDVUS,
               (k_addvus64<<<dim3((p.npw + AV_TG - 1) / AV_TG, (nbnd + AV_TB - 1) / AV_TB), 256, 0, c.stream>>>(
                   p.npw, p.nproj, nbnd, w, p.d_beta, hpsi)));
@@ -445,7 +480,14 @@ int nonlocal_batch_fp64(Context& c, int nitem, const int* prob, const int* nbnd,
                         double2* const* hpsi) {
   std::vector<int> items;
   for (int i = 0; i < nitem; ++i)
-    if (nbnd[i] > 0 && c.probs[prob[i]].nproj > 0) items.push_back(i);
+    if (nbnd[i] > 0 && c.probs[prob[i]].nproj > 0) {
+      if (nonlocal_slices_use(c.probs[prob[i]], nbnd[i])) {   // large items one by one on the tensor cores
+        const int rc = nonlocal_apply_fp64(c, c.probs[prob[i]], psi[i], hpsi[i], nbnd[i]);
+        if (rc) return rc;
+      } else {
+        items.push_back(i);
+      }
+    }
   // partial sums and w of every item side by side in one workspace
   std::vector<size_t> off(items.size());
   std::vector<int> ns(items.size()), kc(items.size());

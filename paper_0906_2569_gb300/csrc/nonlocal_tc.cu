@@ -28,8 +28,24 @@
 #include <mutex>
 
 #include "hpsi_internal.h"
+#include "tcgen05.cuh"
 
 namespace hpsi {
+
+int tma_encoder(Context& c, PFN_cuTensorMapEncodeTiled_v12000* fn) {
+  static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f);
+  });
+  if (!encode) return fail(c, HPSI_ECUDA, "cuTensorMapEncodeTiled is not available");
+  *fn = encode;
+  return HPSI_OK;
+}
 
 namespace {
 
@@ -37,7 +53,6 @@ constexpr int TBM = 128;             // rows of A per tile (TMEM lanes)
 constexpr int TBN = 128;             // rows of B per tile (accumulator columns)
 constexpr int TBK = 64;              // bf16 per 128-byte swizzled row
 constexpr int kTileBytes = TBM * TBK * 2;   // 16 KB, A and B tiles alike
-constexpr long long kWaitCycles = 4000000000LL;   // ~2 s at 2 GHz
 constexpr int kInnerKsteps = 8;      // subspace inner products: K steps per float32 accumulation
 constexpr int kCalbecKsteps = 16;    // calbec: at most this many K steps per float32 accumulation by default;
                                      // the error of a float32 accumulation grows with its length, and
@@ -63,36 +78,6 @@ struct TcArgs {
   int* err;
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// Bounded wait: false if the clock limit expired or another thread of the CTA aborted.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                          long long limit = kWaitCycles) {
-  const long long t0 = clock64();
-  for (unsigned it = 0;; ++it) {
-    if (mbar_try(bar, parity)) return true;
-    if ((it & 255u) == 255u) {
-      if (*abort_flag) return false;
-      if (clock64() - t0 > limit) {
-        *abort_flag = 1;
-        return false;
-      }
-    }
-  }
-}
-
 // Self-test of the failure path: one thread waits, with a short limit, on an mbarrier that no
 // thread and no copy ever arrives at; the expiry raises the error word exactly as in k_tc_gemm.
 __global__ void k_wait_selftest(int* err, long long limit) {
@@ -106,25 +91,6 @@ __global__ void k_wait_selftest(int* err, long long limit) {
   }
 }
 
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n" ::"r"(
-          dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
-
-// K-major operand, 128-byte swizzle: 8-row groups of 128-byte rows, 1024 bytes apart.
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;              // leading byte offset (not used by swizzled K-major)
-  d |= (uint64_t)(1024 >> 4) << 32;    // stride byte offset
-  d |= (uint64_t)1 << 46;              // descriptor version
-  d |= (uint64_t)2 << 61;              // 128-byte swizzle
-  return d;
-}
-
 // kind::f16 instruction descriptor: D f32, A and B bf16, both K-major, M = 128, N = 128.
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TBN >> 3) << 17) |
                             ((uint32_t)(TBM >> 4) << 24);
@@ -135,11 +101,6 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b
       " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
       "l"(a), "l"(b), "r"(kIdesc), "r"(accumulate)
       : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
-               : "memory");
 }
 
 template <int NT>
@@ -582,21 +543,6 @@ __global__ void k_split_rows64(int rows, int kin, int kpad, const double* __rest
 
 // ---- host side ------------------------------------------------------------------------------
 
-PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
-std::once_flag g_encode_once;
-
-int get_encoder(Context& c) {
-  std::call_once(g_encode_once, [] {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-  });
-  if (!g_encode) return fail(c, HPSI_ECUDA, "cuTensorMapEncodeTiled is not available");
-  return HPSI_OK;
-}
-
 // Map over a K-major bf16 matrix [rows][kpad], tiles of 128 rows x 64 columns, 128-byte swizzle.
 int make_map(Context& c, CUtensorMap* m, const void* base, int rows, int kpad) {
   if ((reinterpret_cast<uintptr_t>(base) & 15) || (kpad % TBK)) return fail(c, HPSI_EINVAL, "tensor map alignment");
@@ -604,7 +550,10 @@ int make_map(Context& c, CUtensorMap* m, const void* base, int rows, int kpad) {
   cuuint64_t strides[1] = {(cuuint64_t)kpad * 2};
   cuuint32_t box[2] = {(cuuint32_t)TBK, (cuuint32_t)TBM};
   cuuint32_t es[2] = {1, 1};
-  CUresult r = g_encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, es,
+  PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
+  int rc = tma_encoder(c, &encode);
+  if (rc) return rc;
+  CUresult r = encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, es,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(c, HPSI_ECUDA, "cuTensorMapEncodeTiled failed with code " + std::to_string((int)r));
@@ -931,7 +880,8 @@ int gamma_add_tc(Context& c, const Problem& p, const double* w, int nb, const fl
 
 int gamma_prepare_tc(Context& c, Problem& p) {
   if (p.nproj == 0 || p.d_betar_bf) return HPSI_OK;
-  int rc = get_encoder(c);
+  PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
+  int rc = tma_encoder(c, &encode);
   if (rc) return rc;
   return c.nl_terms == 3 ? gamma_prepare_t<3>(c, p) : gamma_prepare_t<2>(c, p);
 }
@@ -959,7 +909,8 @@ int wait_selftest(Context& c) {
 }
 
 int mixed_prepare_beta(Context& c, Problem& p) {
-  int rc = get_encoder(c);
+  PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
+  int rc = tma_encoder(c, &encode);
   if (rc) return rc;
   return c.nl_terms == 3 ? prepare_t<3>(c, p) : prepare_t<2>(c, p);
 }
@@ -988,7 +939,8 @@ int tc_inner32(Context& c, TcInner& t, bool cache_a, int rows_cap, const float2*
                int npw, double2* out64, float2* out32, int ldo) {
   constexpr int NT = 3;
   if (M <= 0 || nb <= 0) return HPSI_OK;
-  int rc = get_encoder(c);
+  PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
+  int rc = tma_encoder(c, &encode);
   if (rc) return rc;
   const int kc = round_up(2 * npw, TBK), nks = kc / TBK;
   const int tiles = ((2 * nb + TBN - 1) / TBN) * ((M + TBM - 1) / TBM);
