@@ -337,7 +337,7 @@ bool gamma_slices_use(const Problem& p, int nbnd);
 int gamma_slices_w(Context& c, const Problem& p, const void* x, bool x32, int nbnd, bool scaled, double* w, bool* ok);
 int gamma_slices_add(Context& c, const Problem& p, const double* w, double* out, int nbnd, bool* ok);
 // w = D (sum of the splits' partial <beta|psi>), complex and Gamma form
-int dscale_fp64(Context& c, const Problem& p, int nb, int nsplit, const double2* part, double2* w);
+int dscale_fp64(Context& c, const Problem& p, int nb, int nsplit, double2* part, double2* w);
 int gamma_dscale_fp64(Context& c, const Problem& p, int nb, int nsplit, const double* part, double* w);
 
 // ---- context helpers (api.cpp) ----

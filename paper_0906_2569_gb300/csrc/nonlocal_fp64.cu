@@ -20,11 +20,25 @@ namespace {
 
 #include "nonlocal_tiles.cuh"
 
+template <int TP>
 __global__ void __launch_bounds__(256) k_calbec64(int npw, int nproj, int nb, int kchunk,
                                                   const double2* __restrict__ beta,
                                                   const double2* __restrict__ psi, double2* __restrict__ part) {
   __shared__ double2 sm[CB_SMEM];
-  calbec_tile(npw, nproj, nb, kchunk, beta, psi, part, blockIdx.x, blockIdx.y, blockIdx.z, sm);
+  calbec_tile_t<TP>(npw, nproj, nb, kchunk, beta, psi, part, blockIdx.x, blockIdx.y, blockIdx.z, sm);
+}
+
+// part[0][i] = sum of the splits in order: the sums that a D with several nonzeros a row would repeat for each
+__global__ void k_sum_part64(int n, int nsplit, double2* __restrict__ part) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  double2 s = make_double2(0.0, 0.0);
+  for (int k = 0; k < nsplit; ++k) {
+    const double2 t = part[(size_t)k * n + i];
+    s.x += t.x;
+    s.y += t.y;
+  }
+  part[i] = s;
 }
 
 __global__ void k_dscale64(int nproj, int nb, int nsplit, const double2* __restrict__ part,
@@ -33,10 +47,11 @@ __global__ void k_dscale64(int nproj, int nb, int nsplit, const double2* __restr
   dscale_one(blockIdx.x * blockDim.x + threadIdx.x, nproj, nb, nsplit, part, rowptr, col, val, w);
 }
 
+template <int TB>
 __global__ void __launch_bounds__(256) k_addvus64(int npw, int nproj, int nb, const double2* __restrict__ w,
                                                   const double2* __restrict__ beta, double2* __restrict__ hpsi) {
   __shared__ double2 sm[AV_SMEM];
-  addvus_tile(npw, nproj, nb, w, beta, hpsi, blockIdx.x, blockIdx.y, sm);
+  addvus_tile<TB>(npw, nproj, nb, w, beta, hpsi, blockIdx.x, blockIdx.y, sm);
 }
 
 __global__ void __launch_bounds__(256) k_calbec64_batch(const __grid_constant__ NlBatch bt) {
@@ -308,8 +323,36 @@ int gamma_w_df(Context& c, const Problem& p, const void* x, bool x32, int nb, bo
   return HPSI_OK;
 }
 
-int dscale_fp64(Context& c, const Problem& p, int nb, int nsplit, const double2* part, double2* w) {
+// calbec of one problem: tiles of as many projectors as it has (up to 32), so that few rows are padding
+static void launch_calbec64(Context& c, const Problem& p, int nb, int nsplit, int kchunk, const double2* psi,
+                            double2* part) {
+  const int tp = calbec_tp(p.nproj);
+  const dim3 grid((p.nproj + tp - 1) / tp, (nb + CB_TB - 1) / CB_TB, nsplit);
+  auto go = [&](auto k) {
+    HPSI_LAUNCH(c, HPSI_K_CALBEC, (k<<<grid, 256, 0, c.stream>>>(p.npw, p.nproj, nb, kchunk, p.d_beta, psi, part)));
+  };
+  if (tp == 8) go(k_calbec64<8>);
+  else if (tp == 16) go(k_calbec64<16>);
+  else go(k_calbec64<CB_TP>);
+}
+
+// add_vuspsi of one problem: 8 bands per CTA where tiles of 32 would leave SMs without work
+static void launch_addvus64(Context& c, const Problem& p, int nb, const double2* w, double2* hpsi) {
+  const int gt = (p.npw + AV_TG - 1) / AV_TG;
+  auto go = [&](auto k, int tb) {
+    HPSI_LAUNCH(c, HPSI_K_ADDVUS, (k<<<dim3(gt, (nb + tb - 1) / tb), 256, 0, c.stream>>>(p.npw, p.nproj, nb, w, p.d_beta,
+                                                                                       hpsi)));
+  };
+  if (gt * ((nb + AV_TB - 1) / AV_TB) < 2 * c.sm_count) go(k_addvus64<8>, 8);
+  else go(k_addvus64<AV_TB>, AV_TB);
+}
+
+int dscale_fp64(Context& c, const Problem& p, int nb, int nsplit, double2* part, double2* w) {
   const int n = p.nproj * nb;
+  if (nsplit > 1 && p.nnz > p.nproj) {
+    HPSI_LAUNCH(c, HPSI_K_DSCALE, (k_sum_part64<<<(n + 127) / 128, 128, 0, c.stream>>>(n, nsplit, part)));
+    nsplit = 1;
+  }
   HPSI_LAUNCH(c, HPSI_K_DSCALE,
               (k_dscale64<<<(n + 255) / 256, 256, 0, c.stream>>>(p.nproj, nb, nsplit, part, p.d_rowptr, p.d_col,
                                                                  p.d_dval, w)));
@@ -393,7 +436,6 @@ int nonlocal_w_fp64(Context& c, const Problem& p, const double2* psi, int nbnd, 
     rc = slices_w(c, p, psi, nbnd, *wout, &ok);
     if (rc || ok) return rc;
   }
-  const int tilesp = (p.nproj + CB_TP - 1) / CB_TP, tilesb = (nbnd + CB_TB - 1) / CB_TB;
   int nsplit = 0, kchunk = 0;
   size_t bytes = 0;
   nonlocal_fp64_plan(c, p, nbnd, &nsplit, &kchunk, &bytes);
@@ -403,9 +445,7 @@ int nonlocal_w_fp64(Context& c, const Problem& p, const double2* psi, int nbnd, 
   if (rc) return rc;
   double2* part = reinterpret_cast<double2*>(c.ws.part);
   double2* w = reinterpret_cast<double2*>(c.ws.w);
-  HPSI_LAUNCH(c, HPSI_K_CALBEC,
-              (k_calbec64<<<dim3(tilesp, tilesb, nsplit), 256, 0, c.stream>>>(p.npw, p.nproj, nbnd, kchunk,
-                                                                              p.d_beta, psi, part)));
+  launch_calbec64(c, p, nbnd, nsplit, kchunk, psi, part);
   *wout = w;
   return dscale_fp64(c, p, nbnd, nsplit, part, w);
 }
@@ -420,9 +460,7 @@ int nonlocal_apply_fp64(Context& c, const Problem& p, const double2* psi, double
     rc = slices_add(c, p, w, hpsi, nbnd, &ok);
     if (rc || ok) return rc;
   }
-  HPSI_LAUNCH(c, HPSI_K_ADDVUS,
-              (k_addvus64<<<dim3((p.npw + AV_TG - 1) / AV_TG, (nbnd + AV_TB - 1) / AV_TB), 256, 0, c.stream>>>(
-                  p.npw, p.nproj, nbnd, w, p.d_beta, hpsi)));
+  launch_addvus64(c, p, nbnd, w, hpsi);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "nonlocal float64 kernels launch");
   return HPSI_OK;
@@ -441,7 +479,9 @@ void nonlocal_fp64_plan(const Context& c, const Problem& p, int nbnd, int* nspli
     ns = std::min<size_t>(ns, cap > 1 ? cap - 1 : 1);
   }
   int kc = (p.npw + ns - 1) / ns;
-  kc = std::max(CB_TK * 4, ((kc + CB_TK - 1) / CB_TK) * CB_TK);
+  // at least two shared-memory tiles of G: a thread's chain of float64 FMAs runs at 76 cycles each and scheduler, so
+  // a short chunk is what makes a small problem fast (1503 plane waves, 8 projectors, 16 bands: 133 -> 12 us, with tiles of 8)
+  kc = std::max(CB_TK * 2, ((kc + CB_TK - 1) / CB_TK) * CB_TK);
   ns = (p.npw + kc - 1) / kc;   // never above the ns that kc was derived from
   *nsplit = ns;
   *kchunk = kc;
@@ -457,19 +497,12 @@ int nonlocal_fp64_into(Context& c, const Problem& p, const double2* psi, double2
   size_t bytes = 0;
   nonlocal_fp64_plan(c, p, nbnd, &nsplit, &kchunk, &bytes, capacity);
   if (bytes > capacity) return fail(c, HPSI_EINVAL, "nonlocal float64 kernels: partial sums do not fit the scratch");
-  const int tilesp = (p.nproj + CB_TP - 1) / CB_TP, tilesb = (nbnd + CB_TB - 1) / CB_TB;
   double2* part = reinterpret_cast<double2*>(scratch);
   double2* w = part + (size_t)nsplit * nbnd * p.nproj;
-  HPSI_LAUNCH(c, HPSI_K_CALBEC,
-              (k_calbec64<<<dim3(tilesp, tilesb, nsplit), 256, 0, c.stream>>>(p.npw, p.nproj, nbnd, kchunk,
-                                                                              p.d_beta, psi, part)));
-  const int n = p.nproj * nbnd;
-  HPSI_LAUNCH(c, HPSI_K_DSCALE,
-              (k_dscale64<<<(n + 255) / 256, 256, 0, c.stream>>>(p.nproj, nbnd, nsplit, part, p.d_rowptr, p.d_col,
-                                                                 p.d_dval, w)));
-  HPSI_LAUNCH(c, HPSI_K_ADDVUS,
-              (k_addvus64<<<dim3((p.npw + AV_TG - 1) / AV_TG, (nbnd + AV_TB - 1) / AV_TB), 256, 0, c.stream>>>(
-                  p.npw, p.nproj, nbnd, w, p.d_beta, hpsi)));
+  launch_calbec64(c, p, nbnd, nsplit, kchunk, psi, part);
+  const int rc = dscale_fp64(c, p, nbnd, nsplit, part, w);
+  if (rc) return rc;
+  launch_addvus64(c, p, nbnd, w, hpsi);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "nonlocal float64 kernels launch");
   return HPSI_OK;

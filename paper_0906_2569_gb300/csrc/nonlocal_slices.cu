@@ -532,7 +532,7 @@ int slices_w(Context& c, const Problem& p, const double2* psi, int nbnd, double2
     rc = slice_gemm(c, static_cast<const __nv_bfloat16*>(s.digits), s.exps, P, d, e, 2 * nb, s.kpad, ns, per, true, false,
                     static_cast<double*>(c.ws.part), 2 * (size_t)nb * P, P, HPSI_K_CALBEC);
     if (!rc) rc = sum_splits(c, 2 * (size_t)nb * P, ns);
-    if (!rc) rc = dscale_fp64(c, p, nb, 1, static_cast<const double2*>(c.ws.part), w + (size_t)b0 * P);
+    if (!rc) rc = dscale_fp64(c, p, nb, 1, static_cast<double2*>(c.ws.part), w + (size_t)b0 * P);
     if (rc) return rc;
   }
   return HPSI_OK;
