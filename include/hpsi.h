@@ -60,9 +60,9 @@ enum hpsi_option {
   HPSI_OPT_KERNEL_TIMING = 3, /* 1: bracket every launch of the library's kernels with CUDA events */
   HPSI_OPT_NL_TERMS = 4,      /* mixed path: bf16 terms per nonlocal operand, 3 (six products,
                                  default) or 2 (three products); re-splits the projectors */
-  HPSI_OPT_LOCAL_PATH = 5,    /* 0 (default): where the box allows them, register-codelet kernels (float32)
-                                 or 64-bit fixed-point kernels (float64);
-                                 1: always the generic radix-2/3/4/5 kernels */
+  HPSI_OPT_LOCAL_PATH = 5,    /* 0 (default): where the box allows them (every edge the product of two of 2, 3,
+                                 4, 5, 6, 8, 9, 10, 12, 15, 16), the two-codelet kernels, in float32 or, for
+                                 float64, in 64-bit fixed point; 1: always the generic radix-2/3/4/5 kernels */
   HPSI_OPT_TC_KSPLIT = 6,     /* mixed path: at most this many 64-wide K steps accumulate in one
                                  tensor-memory accumulator of <beta|psi> before the partial sums
                                  are added in float64 (0, default: at most 16, fewer where the
@@ -78,13 +78,10 @@ enum hpsi_option {
                                  vectors (2: the basic 2N form, 3 or 4) before a restart; 0
                                  (default): 3 in a mixed context, 4 in a float64 one */
   HPSI_OPT_AUTOTUNE = 9,      /* 1 (default): the first hpsi_apply of a problem with >= 4 bands at
-                                 HPSI_MIXED times every shared-memory plan of the register-codelet
-                                 kernels and three band-block sizes on its own bands and keeps the
-                                 fastest (results do not depend on the choice); it
-                                 also times caps of 4, 8 and 16 K-steps per float32 accumulation of
-                                 the tensor-core calbec (unless HPSI_OPT_TC_KSPLIT is set; results
-                                 differ at float32 rounding level).  That call synchronizes.
-                                 0: fixed defaults */
+                                 HPSI_MIXED times caps of 4, 8 and 16 K-steps per float32 accumulation of
+                                 the tensor-core calbec on its own bands and keeps the fastest (unless
+                                 HPSI_OPT_TC_KSPLIT is set; results differ at float32 rounding level).
+                                 That call synchronizes.  0: fixed defaults */
   HPSI_OPT_EIGENSOLVER = 10,  /* reduced eigenproblems of davidson_solve and hpsi_eigh_lowest:
                                  1 (default): the library's own kernels (Householder reduction,
                                  Sturm multisection, inverse iteration, back-transformation) for
@@ -145,7 +142,7 @@ enum hpsi_option {
                                  hpsi_eigh_lowest_sym and the float64 davidson_solve_gamma (float64
                                  eigenvector GEMMs) */
   HPSI_OPT_PERSISTENT = 24,   /* hpsi_apply_batch: 1: one persistent cooperative launch per box edge
-                                 (<= 32 items each) when every item has the register-codelet
+                                 (<= 32 items each) when every item has the two-codelet
                                  kernels; 0 (default): one launch per kernel class and box edge.
                                  The results are identical; the separate launches, replayed from a
                                  CUDA graph, are faster since each kernel runs at its own occupancy */
@@ -321,8 +318,8 @@ HPSI_API int davidson_solve_gamma(hpsi_ctx* ctx, int ik, int nbnd, double tol, i
 /*
  * hpsi_apply_batch -- H psi for several problems (k-points or cells) in one launch sequence:
  * for i < nitem: hpsi_out[i] = H(prob[i]) psi_in[i] with nbnd[i] bands.  Device pointers only.
- * Items whose cubic box has register-codelet kernels share one launch of each local-potential
- * kernel per box edge (blockIdx.z runs over the items), and the nonlocal term follows: one launch
+ * Items whose box has the two-codelet kernels share one launch of each local-potential
+ * kernel (32 items each, whatever their boxes), and the nonlocal term follows: one launch
  * per kernel class over all items in float64, which a mixed context also takes when every item has
  * at most 64 projectors (HPSI_OPT_BATCH_NL), else the tensor-core form per item.  With
  * HPSI_OPT_PERSISTENT = 1, and every item on those kernels, each box edge (<= 32 items) is instead

@@ -187,25 +187,31 @@ static int upload_potential(Context& c, const int n[3], const double* vr, int* s
   rc = upload(c, &d32, t32.data(), nr);
   if (rc) return rc;
   c.vbufs.push_back(d32);
-  c.vbufs.push_back(nullptr);   // made by the first problem whose local term can run in fixed point
-  c.vbufs.push_back(nullptr);
+  for (int i = 0; i < 2; ++i) c.vbufs.push_back(nullptr);   // made by the first problem that can use them
   *slot = (int)c.vbufs.size() - 4;
   return HPSI_OK;
 }
 
 // The fixed-point copy of a potential: at setup in a float64 context, in a mixed one on the first application of H in
 // float64 (the final quotients under HPSI_OPT_FINAL_FP64 = 1).
-int ensure_fixed_potential(Context& c, int slot, const FixedAxis ax[3]) {
+int ensure_fixed_potential(Context& c, int slot, const LineAxis ax[3]) {
   if (c.vbufs[slot + 2]) return HPSI_OK;
   const size_t nr = (size_t)ax[0].n * ax[1].n * ax[2].n;
-  if (cudaMalloc(&c.vbufs[slot + 2], sizeof(long long) * nr) != cudaSuccess ||
-      cudaMalloc(&c.vbufs[slot + 3], 16) != cudaSuccess) {
+  if (cudaMalloc(&c.vbufs[slot + 2], sizeof(long long) * nr + kFixedScaleBytes) != cudaSuccess) {
     cudaGetLastError();
-    cudaFree(c.vbufs[slot + 2]);
     c.vbufs[slot + 2] = nullptr;
     return fail(c, HPSI_ENOMEM, "device allocation of the fixed-point potential failed");
   }
   return fixed_potential(c, slot, ax, HPSI_K_DAVIDSON);
+}
+
+static int ensure_float_potential(Context& c, int slot, const LineAxis ax[3]) {
+  if (c.vbufs[slot + 3]) return HPSI_OK;
+  if (cudaMalloc(&c.vbufs[slot + 3], sizeof(float) * (size_t)ax[0].n * ax[1].n * ax[2].n) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(c, HPSI_ENOMEM, "device allocation failed during setup");
+  }
+  return float_potential(c, slot, ax, HPSI_K_DAVIDSON);
 }
 
 static int plan_for(Context& c, int n, FftPlan* out) {
@@ -224,19 +230,28 @@ static int plan_for(Context& c, int n, FftPlan* out) {
   if (rc) return rc;
   rc = upload(c, &tt.d32, tab32.data(), tab32.size());
   if (rc) return rc;
-  std::vector<float2> nat32(n);
-  for (int j = 0; j < n; ++j) {
-    const double ang = -6.283185307179586476925286766559 * (double)j / (double)n;
-    nat32[j] = make_float2((float)std::cos(ang), (float)std::sin(ang));
+  // the fast paths' tables: fixed point (every context can apply H in float64) and, in a mixed one, float32
+  std::vector<int> all;
+  size_t at[2] = {0, 0}, ftw[2] = {0, 0}, cells[2] = {0, 0};
+  const int npr = c.precision == HPSI_MIXED ? 2 : 1;
+  for (int pr = 0; pr < npr; ++pr) {
+    std::vector<int> lines;
+    line_tables(n, pr, lines, &ftw[pr], &cells[pr], &tt.axis[pr]);
+    at[pr] = all.size();
+    all.insert(all.end(), lines.begin(), lines.end());
+    while (all.size() % 4) all.push_back(0);   // the fixed-point twiddles are read as int4
+    if (!lines.empty()) tt.cells[pr].assign(lines.begin() + cells[pr], lines.begin() + cells[pr] + n);
   }
-  rc = upload(c, &tt.nat32, nat32.data(), nat32.size());
+  rc = upload(c, &tt.tables, all.data(), all.size());
   if (rc) return rc;
-  std::vector<int> fx;
-  const size_t slots = fixed_tables(n, fx, &tt.fixed);
-  rc = upload(c, &tt.fx, fx.data(), fx.size());
-  if (rc) return rc;
-  tt.fixed.tw = reinterpret_cast<const FxTw*>(tt.fx);
-  tt.fixed.slot = tt.fx ? tt.fx + slots : nullptr;
+  for (int pr = 0; pr < npr; ++pr) {
+    LineAxis& ax = tt.axis[pr];
+    if (tt.cells[pr].empty()) continue;
+    ax.fxtw = reinterpret_cast<const FxTw*>(tt.tables + at[pr]);
+    ax.ftw = reinterpret_cast<const float2*>(tt.tables + at[pr] + ftw[pr]);
+    ax.cell = tt.tables + at[pr] + cells[pr];
+    ax.slot = ax.cell + n;
+  }
   tt.plan.tw64 = tt.d64;
   tt.plan.tw32 = tt.d32;
   c.tw.push_back(tt);
@@ -328,10 +343,10 @@ int set_potential(Context& c, int ik, const double* v64, double vmean) {
   cudaError_t e = cudaMemcpyAsync(d64, v64, sizeof(double) * nr, cudaMemcpyDeviceToDevice, c.stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "potential update");
   HPSI_LAUNCH(c, HPSI_K_SCF, (k_v_to_f32<<<(int)std::min<size_t>(4096, (nr + 255) / 256), 256, 0, c.stream>>>(nr, d64, d32)));
-  if (c.vbufs[p0.vslot + 2]) {
-    const int rc = fixed_potential(c, p0.vslot, p0.fixed.ax, HPSI_K_SCF);
-    if (rc) return rc;
-  }
+  int rc = HPSI_OK;
+  if (c.vbufs[p0.vslot + 2]) rc = fixed_potential(c, p0.vslot, p0.fixed.ax, HPSI_K_SCF);
+  if (!rc && c.vbufs[p0.vslot + 3]) rc = float_potential(c, p0.vslot, p0.fast.ax, HPSI_K_SCF);
+  if (rc) return rc;
   for (Problem& p : c.probs) {
     if (p.vslot != p0.vslot) continue;
     HPSI_LAUNCH(c, HPSI_K_SCF,
@@ -358,22 +373,51 @@ static int finish_problem(Context& c, Problem& p, const double* vr, int vslot_sh
   }
   if ((rc = upload(c, &p.d_sticks, p.sticks.data(), p.sticks.size()))) return rc;
   {
-    // lookup maps of the fast path: stick of (plane, j2) and plane of ix
-    std::vector<int> ymap((size_t)p.npl * p.n[1], -1), xmap(p.n[0], -1);
-    for (int q = 0; q < p.npl; ++q) {
-      xmap[p.planes[q].ix] = q;
-      for (int s = p.planes[q].s0; s < p.planes[q].s0 + p.planes[q].ns; ++s)
-        ymap[(size_t)q * p.n[1] + p.sticks[s].iy] = s;
+    // lookup tables of the fast paths
+    std::vector<int> xmap(p.n[0], -1);
+    for (int q = 0; q < p.npl; ++q) xmap[p.planes[q].ix] = q;
+    std::vector<int> all(xmap);   // one upload: the tables side by side
+    size_t at[2] = {0, 0};
+    bool have[2] = {false, false};
+    for (int pr = 0; pr < (c.precision == HPSI_MIXED ? 2 : 1); ++pr) {
+      const std::vector<int>*ycell = nullptr, *zcell = nullptr;
+      for (auto& t : c.tw) {
+        if (t.n == p.n[1]) ycell = &t.cells[pr];
+        if (t.n == p.n[2]) zcell = &t.cells[pr];
+      }
+      if (ycell->empty() || zcell->empty()) continue;
+      have[pr] = true;
+      at[pr] = all.size();
+      all.resize(all.size() + p.nst + p.npw);
+      int *so = all.data() + at[pr], *zo = so + p.nst;
+      std::vector<int> zbeg;
+      for (int q = 0; q < p.npl; ++q)
+        for (int s = p.planes[q].s0; s < p.planes[q].s0 + p.planes[q].ns; ++s)
+          so[s] = q * (p.n[1] | 1) + (*ycell)[p.sticks[s].iy];
+      for (int s = 0; s < p.nst; ++s) {
+        const StickDev& st = p.sticks[s];
+        if (s % kStickChunk == 0) zbeg.push_back(st.g0);
+        for (int t = 0; t < st.len; ++t)
+          zo[st.g0 + t] = (*zcell)[(st.z0 + t) % p.n[2]] * (kStickChunk + 1) + s % kStickChunk;
+      }
+      zbeg.push_back(p.npw);
+      all.insert(all.end(), zbeg.begin(), zbeg.end());
     }
-    if ((rc = upload(c, &p.d_ymap, ymap.data(), ymap.size()))) return rc;
-    if ((rc = upload(c, &p.d_xmap, xmap.data(), xmap.size()))) return rc;
-    for (auto& t : c.tw) {
-      if (t.n == p.n[0]) p.d_ftw32 = t.nat32;
+    if ((rc = upload(c, &p.d_xmap, all.data(), all.size()))) return rc;
+    for (int pr = 0; pr < 2; ++pr) {
+      if (!have[pr]) continue;
+      p.tab[pr].soff = p.d_xmap + at[pr];
+      p.tab[pr].zoff = p.tab[pr].soff + p.nst;
+      p.tab[pr].zbeg = p.tab[pr].zoff + p.npw;
+    }
+    for (auto& t : c.tw)
       for (int a = 0; a < 3; ++a)
-        if (t.n == p.n[a]) p.fixed.ax[a] = t.fixed;
-    }
+        if (t.n == p.n[a]) {
+          p.fixed.ax[a] = t.axis[HPSI_FP64];
+          p.fast.ax[a] = t.axis[HPSI_MIXED];
+        }
     fixed_plan(p, c.smem_optin);
-    for (int pr = 0; pr < 2; ++pr) p.fflags[pr] = local_fast_plan(p, pr, c.smem_optin);
+    float_plan(p, c.smem_optin);
   }
   if ((rc = upload(c, &p.d_planes, p.planes.data(), p.planes.size()))) return rc;
   if ((rc = upload(c, &p.d_kin, p.kin.data(), p.kin.size()))) return rc;
@@ -388,6 +432,7 @@ static int finish_problem(Context& c, Problem& p, const double* vr, int vslot_sh
   p.d_v64 = reinterpret_cast<const double*>(c.vbufs[vslot_shared]);
   p.d_v32 = reinterpret_cast<const float*>(c.vbufs[vslot_shared + 1]);
   if (p.fixed.ok && c.precision == HPSI_FP64 && (rc = ensure_fixed_potential(c, vslot_shared, p.fixed.ax))) return rc;
+  if (p.fast.ok && c.precision == HPSI_MIXED && (rc = ensure_float_potential(c, vslot_shared, p.fast.ax))) return rc;
   // projectors and D (CSR of its nonzeros)
   const int P = p.nproj;
   std::vector<int> rowptr(P + 1, 0), col;
@@ -440,9 +485,10 @@ static int finish_problem(Context& c, Problem& p, const double* vr, int vslot_sh
     p.nbb[pr] = (int)std::max<size_t>(1, std::min<size_t>(4096, (size_t)(48u << 20) / std::max<size_t>(1, xper)));
     const size_t zper = 2 * cs * (size_t)p.n[2] * p.nst;
     p.nbbf[pr] = (int)std::max<size_t>(1, std::min<size_t>(4096, (size_t)(48u << 20) / std::max<size_t>(1, zper)));
-    // fixed point: at least eight waves of two plane CTAs per SM, since its time is arithmetic and a nearly empty
-    // last wave costs more than rows that leave the L2 (4% of a band's time at 144^3)
-    if (pr == HPSI_FP64 && p.fixed.ok) p.nbbf[pr] = std::max(p.nbbf[pr], (16 * c.sm_count + p.n[2] - 1) / p.n[2]);
+    // at least eight waves of two plane CTAs per SM (float32: four), since the planes' time is arithmetic and a nearly
+    // empty last wave costs more than rows that leave the L2 (fixed point: 4% of a band's time at 144^3)
+    const int waves = pr == HPSI_FP64 ? 8 : 4;
+    p.nbbf[pr] = std::max(p.nbbf[pr], (2 * waves * c.sm_count + p.n[2] - 1) / p.n[2]);
   }
   if (c.precision == HPSI_MIXED && P > 0) {
     rc = mixed_prepare_beta(c, p);
@@ -456,7 +502,6 @@ static int finish_problem(Context& c, Problem& p, const double* vr, int vslot_sh
 static void free_problem(Problem& p) {
   cudaFree(p.d_sticks);
   cudaFree(p.d_planes);
-  cudaFree(p.d_ymap);
   cudaFree(p.d_xmap);
   cudaFree(p.d_kin);
   cudaFree(p.d_hdiag);
@@ -481,8 +526,7 @@ static void free_context(Context& c) {
   for (auto& t : c.tw) {
     cudaFree(t.d64);
     cudaFree(t.d32);
-    cudaFree(t.nat32);
-    cudaFree(t.fx);
+    cudaFree(t.tables);
   }
   for (void* v : c.vbufs) cudaFree(v);
   cudaFree(c.d_err);
@@ -498,6 +542,7 @@ static void free_context(Context& c) {
   cudaFree(c.ws.gout);
   cudaFree(c.ws.gnl);
   cudaFree(c.ws.gdf);
+  cudaFree(c.ws.pbar);
   if (c.graph.exec) cudaGraphExecDestroy(c.graph.exec);
   if (c.cap_stream) cudaStreamDestroy(c.cap_stream);
   davidson_release(c);
@@ -541,7 +586,7 @@ static int batch_apply_items(Context& c, int nitem, const int* prob, const int* 
   for (int i = 0; i < nitem; ++i) {
     if (nbnd[i] == 0) continue;
     const Problem& p = c.probs[prob[i]];
-    if ((p.fflags[cur_prec(c)] & 4) && !c.force_generic) fast.push_back(i);
+    if (local_fast_ok(p, cur_prec(c)) && !c.force_generic) fast.push_back(i);
     else slow.push_back(i);
   }
   std::stable_sort(fast.begin(), fast.end(),

@@ -12,13 +12,13 @@
 // kGain sum |x_n|; the largest coefficient is sin 72 + sin 36 = 1.539 of the 5-point kernel.
 //
 // The transforms have the sign e^{+2 pi i}; the opposite sign is the same code with real and imaginary parts
-// swapped on the way in and out.  A line of n = R1 R2 values is transformed in place in two stages:
-//   stage 1, item t < R2:   R1-point DFT over the slots  t s2 + R2 a  (mod n), a < R1
-//   stage 2, item k1 < R1:  R2-point DFT over the slots  k1 R2 + s2 b (mod n), b < R2
-// With coprime R1, R2 (s2 = R1) this is the prime-factor form, which needs no twiddles between the stages; otherwise
-// (s2 = 1) stage 1 multiplies its output k1 by e^{2 pi i t k1 / n} (the Cooley-Tukey form).  Values start in natural
-// order and end with X[k] in slot (R2 (k mod R1) + s2 b(k)) mod n, b = k mod R2 or k div R1.  The reversed
-// sequence (stage 2, the twiddles, stage 1) takes values in those slots to natural order.
+// swapped on the way in and out.  A line of n = R1 R2 values lies in n cells and is transformed in place in two stages:
+//   stage 1, item t < R2:   R1-point DFT over the cells  a R2 + t, a < R1
+//   stage 2, item k1 < R1:  R2-point DFT over the cells  k1 R2 + b, b < R2
+// Coprime R1, R2 use the prime-factor form: value n starts in cell a R2 + t with n = R2 a + R1 t (mod n), X[k] ends in cell
+// (k mod R1) R2 + (k mod R2), and there are no twiddles.  Otherwise (Cooley-Tukey) values start in natural order, stage
+// 1 multiplies its output k1 by e^{2 pi i t k1 / n}, and X[k] ends in cell (k mod R1) R2 + (k div R1).  The reversed
+// sequence (stage 2, the twiddles, stage 1) goes from the last order to the first.
 #pragma once
 
 #include <cuda_runtime.h>

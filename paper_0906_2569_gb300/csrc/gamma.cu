@@ -27,6 +27,7 @@
 #include <string>
 #include <vector>
 
+#include "convert.cuh"
 #include "hpsi_internal.h"
 
 namespace hpsi {
@@ -90,6 +91,113 @@ __global__ void k_gamma_pack(int npw, int nb, const S* __restrict__ x, int scale
         cb.y = -cb.y;
       }
       fq[i] = make_double2(ca.x - cb.y, ca.y + cb.x);
+    }
+  }
+}
+
+// Pack in float32 for the raw local term (mixed contexts): f(G) = c_a(G) + i c_b(G), f(-G) = conj c_a + i conj c_b, the
+// sums of float64 coefficients rounded once (each coefficient as two floats; a cast or a float64 add runs at the
+// float64 rate).  One thread per G of the half sphere writes both members of the pair.
+__device__ __forceinline__ float sum_rounded(float2 a, float2 b) {
+  const float s = __fadd_rn(a.x, b.x), z = __fsub_rn(s, a.x);
+  const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, z)), __fsub_rn(b.x, z));
+  return __fadd_rn(s, __fadd_rn(e, __fadd_rn(a.y, b.y)));
+}
+template <typename S>
+__global__ void __launch_bounds__(256) k_gamma_pack_raw(int npw, int nb, const S* __restrict__ x, int scaled,
+                                                        float2* __restrict__ f) {
+  const int nh = (npw + 1) / 2, i0 = nh - 1;
+  const int q = blockIdx.y, a = 2 * q, b = 2 * q + 1;
+  const S* xa = x + (size_t)a * nh;
+  const S* xb = x + (size_t)b * nh;
+  float2* fq = f + (size_t)q * npw;
+  for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < nh; h += gridDim.x * blockDim.x) {
+    float2 p, m;   // f(G), f(-G)
+    if constexpr (sizeof(S) == sizeof(float2)) {
+      float2 ca = xa[h], cb = b < nb ? xb[h] : make_float2(0.f, 0.f);
+      if (scaled && h > 0) {
+        ca.x *= (float)kInvSqrt2; ca.y *= (float)kInvSqrt2;
+        cb.x *= (float)kInvSqrt2; cb.y *= (float)kInvSqrt2;
+      }
+      if (h == 0) ca.y = cb.y = 0.f;   // a real orbital has a real G = 0 component
+      p = make_float2(ca.x - cb.y, ca.y + cb.x);
+      m = make_float2(ca.x + cb.y, cb.x - ca.y);
+    } else {
+      double2 da = ld2(xa + h), db = b < nb ? ld2(xb + h) : make_double2(0.0, 0.0);
+      if (scaled && h > 0) {
+        da.x *= kInvSqrt2; da.y *= kInvSqrt2;
+        db.x *= kInvSqrt2; db.y *= kInvSqrt2;
+      }
+      const float2 z = make_float2(0.f, 0.f);
+      const float2 ax = f64_split(da.x), ay = h ? f64_split(da.y) : z, bx = f64_split(db.x), by = h ? f64_split(db.y) : z;
+      const float2 nay = make_float2(-ay.x, -ay.y), nby = make_float2(-by.x, -by.y);
+      p = make_float2(sum_rounded(ax, nby), sum_rounded(ay, bx));
+      m = make_float2(sum_rounded(ax, by), sum_rounded(bx, nay));
+    }
+    fq[i0 + h] = p;
+    if (h) fq[i0 - h] = m;
+  }
+}
+
+// Unpack the raw local term L f of a pair and add the kinetic term (float64 results: in float64, one FMA a component)
+// and the nonlocal term's float32 partial sums nl32 [ns32][nb][nr] in real-basis coordinates (null: none).
+template <typename S>
+__global__ void __launch_bounds__(256) k_gamma_unpack_raw(int npw, int nb, const float2* __restrict__ F, int scaled,
+                                                          const double* __restrict__ kin, const S* __restrict__ x,
+                                                          const float* __restrict__ nl32, int ns32, S* __restrict__ y) {
+  const int nh = (npw + 1) / 2, i0 = nh - 1;
+  const size_t nr = 2 * (size_t)nh, plane = (size_t)nb * nr;
+  const int q = blockIdx.y, a = 2 * q, b = 2 * q + 1;
+  const float2* Fq = F + (size_t)q * npw;
+  for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < nh; h += gridDim.x * blockDim.x) {
+    const float2 fp = Fq[i0 + h], fm = Fq[i0 - h];
+    // conj(F(-G)) = (fm.x, -fm.y)
+    float2 ya = make_float2(0.5f * (fp.x + fm.x), 0.5f * (fp.y - fm.y));
+    float2 yb = make_float2(0.5f * (fp.y + fm.y), -0.5f * (fp.x - fm.x));
+    if (scaled && h > 0) {
+      ya.x *= (float)kSqrt2; ya.y *= (float)kSqrt2;
+      yb.x *= (float)kSqrt2; yb.y *= (float)kSqrt2;
+    }
+    if (nl32) {
+      const float sn = (!scaled && h > 0) ? (float)kInvSqrt2 : 1.f;
+      float2 na = make_float2(0.f, 0.f), nc = na;
+      const size_t ia = (size_t)a * nr + 2 * h, ib = (size_t)b * nr + 2 * h;
+      for (int sp = 0; sp < ns32; ++sp) {
+        const float2 va = *reinterpret_cast<const float2*>(nl32 + sp * plane + ia);
+        na.x += va.x;
+        na.y += va.y;
+        if (b < nb) {
+          const float2 vb = *reinterpret_cast<const float2*>(nl32 + sp * plane + ib);
+          nc.x += vb.x;
+          nc.y += vb.y;
+        }
+      }
+      ya.x = fmaf(sn, na.x, ya.x);
+      ya.y = fmaf(sn, na.y, ya.y);
+      yb.x = fmaf(sn, nc.x, yb.x);
+      yb.y = fmaf(sn, nc.y, yb.y);
+    }
+    const double kg = kin[i0 + h];
+    if constexpr (sizeof(S) == sizeof(float2)) {
+      // kin as two floats: the product and the sum round once
+      const float2 k2 = f64_split(kg);
+      const float2 xa = x[(size_t)a * nh + h];
+      y[(size_t)a * nh + h] = make_float2(fmaf(k2.x, xa.x, fmaf(k2.y, xa.x, ya.x)),
+                                          h ? fmaf(k2.x, xa.y, fmaf(k2.y, xa.y, ya.y)) : ya.y);
+      if (b < nb) {
+        const float2 xb = x[(size_t)b * nh + h];
+        y[(size_t)b * nh + h] = make_float2(fmaf(k2.x, xb.x, fmaf(k2.y, xb.x, yb.x)),
+                                            h ? fmaf(k2.x, xb.y, fmaf(k2.y, xb.y, yb.y)) : yb.y);
+      }
+    } else {
+      const double2 xa = ld2(x + (size_t)a * nh + h);
+      st2(y + (size_t)a * nh + h, make_double2(fma(kg, xa.x, f32_to_f64(ya.x)),
+                                               h ? fma(kg, xa.y, f32_to_f64(ya.y)) : f32_to_f64(ya.y)));
+      if (b < nb) {
+        const double2 xb = ld2(x + (size_t)b * nh + h);
+        st2(y + (size_t)b * nh + h, make_double2(fma(kg, xb.x, f32_to_f64(yb.x)),
+                                                 h ? fma(kg, xb.y, f32_to_f64(yb.y)) : f32_to_f64(yb.y)));
+      }
     }
   }
 }
@@ -305,16 +413,25 @@ static int gamma_apply_t(Context& c, int ik, const S* x, S* y, int nb, bool scal
   int rc = gamma_nl_prepare(c, p);
   if (rc) return rc;
   const int npairs = (nb + 1) / 2;
-  const size_t bytes = sizeof(double2) * (size_t)npairs * p.npw;
+  // the local term at mixed precision: the pairs stay in float32 from the pack to the unpack, which adds the kinetic
+  // term (half the bytes, no float64 conversions); else complex128 pairs through H without its nonlocal term
+  const bool raw = cur_prec(c) == HPSI_MIXED && p.fast.ok && !c.force_generic && nl_prec(c) != HPSI_FP64;
+  const size_t bytes = (raw ? sizeof(float2) : sizeof(double2)) * (size_t)npairs * p.npw;
   rc = ensure_buffer(c, &c.ws.gin, &c.ws.ginbytes, bytes);
   if (rc) return rc;
   rc = ensure_buffer(c, &c.ws.gout, &c.ws.goutbytes, bytes);
   if (rc) return rc;
   double2* f = static_cast<double2*>(c.ws.gin);
   double2* F = static_cast<double2*>(c.ws.gout);
-  HPSI_LAUNCH(c, HPSI_K_GAMMA, (k_gamma_pack<S><<<dim3(grid_x(p.npw), npairs), 256, 0, c.stream>>>(
-                                   p.npw, nb, x, scaled ? 1 : 0, f)));
-  rc = local_apply(c, p, f, F, npairs);
+  if (raw) {
+    HPSI_LAUNCH(c, HPSI_K_GAMMA, (k_gamma_pack_raw<S><<<dim3(grid_x((p.npw + 1) / 2), npairs), 256, 0, c.stream>>>(
+                                     p.npw, nb, x, scaled ? 1 : 0, static_cast<float2*>(c.ws.gin))));
+    rc = local_raw_apply(c, p, static_cast<const float2*>(c.ws.gin), static_cast<float2*>(c.ws.gout), npairs);
+  } else {
+    HPSI_LAUNCH(c, HPSI_K_GAMMA, (k_gamma_pack<S><<<dim3(grid_x(p.npw), npairs), 256, 0, c.stream>>>(
+                                     p.npw, nb, x, scaled ? 1 : 0, f)));
+    rc = local_apply(c, p, f, F, npairs);
+  }
   if (rc) return rc;
   const double* nl64 = nullptr;
   const float* nl32 = nullptr;
@@ -341,8 +458,14 @@ static int gamma_apply_t(Context& c, int ik, const S* x, S* y, int nb, bool scal
     if (rc) return rc;
   }
   c.band_apps += nb;
-  HPSI_LAUNCH(c, HPSI_K_GAMMA, (k_gamma_unpack<S><<<dim3(grid_x((p.npw + 1) / 2), npairs), 256, 0, c.stream>>>(
-                                   p.npw, nb, F, scaled ? 1 : 0, nl64, nl32, ns32, y)));
+  const dim3 gu(grid_x((p.npw + 1) / 2), npairs);
+  if (raw)
+    HPSI_LAUNCH(c, HPSI_K_GAMMA, (k_gamma_unpack_raw<S><<<gu, 256, 0, c.stream>>>(
+                                     p.npw, nb, static_cast<const float2*>(c.ws.gout), scaled ? 1 : 0, p.d_kin, x, nl32,
+                                     ns32, y)));
+  else
+    HPSI_LAUNCH(c, HPSI_K_GAMMA, (k_gamma_unpack<S><<<gu, 256, 0, c.stream>>>(p.npw, nb, F, scaled ? 1 : 0, nl64, nl32,
+                                                                              ns32, y)));
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "gamma pack / unpack kernels");
   return HPSI_OK;

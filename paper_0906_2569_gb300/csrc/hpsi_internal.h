@@ -45,16 +45,19 @@ struct PlaneDev {
 // One axis of the fixed-point local path (local_fixed.cu): n = r1 r2 (0: the edge has no such factors), s2 = r1 for
 // coprime factors (no twiddles), 1 otherwise; device tables owned by the axis's TwiddleTable.
 struct FxTw;
-struct FixedAxis {
+struct LineAxis {
   int n = 0, r1 = 0, r2 = 0, s2 = 0;
-  const FxTw* tw = nullptr;
-  const int* slot = nullptr;
+  int twiddled = 0;
+  const FxTw* fxtw = nullptr;     // e^{2 pi i j / n} in fixed point and in float32 (Cooley-Tukey form only)
+  const float2* ftw = nullptr;
+  const int* cell = nullptr;      // cell of every index before the inverse transform, and
+  const int* slot = nullptr;      // after it
 };
 // Tile sizes and growth bounds (bits) of a problem's fixed-point local term.
 struct FixedPlan {
   bool ok = false;
-  FixedAxis ax[3];
-  int cw = 0, sc = 0, nch = 0;
+  LineAxis ax[3];
+  int cw = 0, nch = 0, block = 0;
   int hz = 0, hy = 0, hx = 0, s3 = 0, hyf = 0, hzf = 0;
   size_t smem_z = 0, smem_p = 0;
 };
@@ -66,6 +69,23 @@ struct SlicePlanes {
   int kpad = 0;
   bool no_room = false;   // the device had no memory for them
 };
+
+// Tile sizes of a problem's float32 local term (local_fast.cu).
+struct FloatPlan {
+  bool ok = false;
+  LineAxis ax[3];
+  int cw = 0, nch = 0, block = 0;
+  size_t smem_z = 0, smem_p = 0;
+};
+// Lookup tables of a problem's fast path at a precision (its axes' cells differ between the two).
+struct LocalTables {
+  const int* soff = nullptr;   // [nst]: stick's place in the plane array, plane (n2 | 1) + cell of j2
+  const int* zoff = nullptr;   // [npw]: G's place in its z tile, cell (kStickChunk + 1) + stick within the chunk
+  const int* zbeg = nullptr;   // [chunks + 1]: first G of each z tile
+};
+
+constexpr size_t kFixedScaleBytes = 16;   // behind a fixed-point potential: the largest |V|'s bits, then its exponent
+constexpr int kStickChunk = 32;   // sticks of a z tile: they fill a stage's items and the rows of its stores
 
 struct Problem {
   double cell[9];
@@ -95,15 +115,13 @@ struct Problem {
   FftPlan plan[3];
   // per precision (index HPSI_FP64 / HPSI_MIXED): band blocks and the fast-path plan
   int nbb[2] = {1, 1};             // band block of the generic local kernels
-  mutable int fflags[2] = {0, 0};  // fast path: bit 2 enabled, bit 0 stage V, bit 1 stage the stick row
-  mutable int nbbf[2] = {1, 1};    // band block of the fast local kernels
-  mutable bool tuned[2] = {false, false};   // autotuner has chosen fflags / nbbf
+  int nbbf[2] = {1, 1};            // band block of the fast local kernels
   mutable int nl_kmax = 0;         // mixed calbec: K-steps per float32 accumulation the autotuner chose
                                    // (0: not tuned yet)
-  int* d_ymap = nullptr;           // [npl][n2]: stick of (plane, j2) or -1
+  LocalTables tab[2];              // per precision (local_fixed.cu, local_fast.cu)
   int* d_xmap = nullptr;           // [n1]: plane of ix or -1
-  const float2* d_ftw32 = nullptr;    // e^{-2 pi i j / n}, j < n (owned by the twiddle table)
-  FixedPlan fixed;                    // the local term in float64
+  FixedPlan fixed;                 // the local term in float64
+  FloatPlan fast;                  // the local term in float32
   std::vector<double> vext;        // the potential given at setup, host, layout [n3][n2][n1]
   bool gamma_ok = false;           // the Gamma-point real form applies (gamma.cu)
   std::string gamma_why;           // why not, when it does not
@@ -123,9 +141,9 @@ struct TwiddleTable {
   FftPlan plan;   // with device pointers filled
   double2* d64 = nullptr;
   float2* d32 = nullptr;
-  float2* nat32 = nullptr;    // e^{-2 pi i j / n}, j < n
-  FixedAxis fixed;
-  int* fx = nullptr;          // its twiddles and slots
+  LineAxis axis[2];           // per precision
+  int* tables = nullptr;      // their twiddles, cells and slots
+  std::vector<int> cells[2];
 };
 
 struct Workspace {
@@ -162,8 +180,8 @@ struct Context {
   size_t smem_optin = 0;
   std::vector<Problem> probs;
   std::vector<TwiddleTable> tw;
-  std::vector<void*> vbufs;            // owned V buffers, four per slot: float64, float32, fixed point (or null)
-                                       // and the fixed-point one's scale
+  std::vector<void*> vbufs;            // owned V buffers, four per slot: float64, float32, fixed point (then its
+                                       // scale), float32 / N_r in slot order (the last two may be null)
   Workspace ws;
   std::string err;
   double opt_tau = 0.1;                // Davidson: |<k+G|H|k+G> - eps| is kept >= tau (Ha)
@@ -290,21 +308,30 @@ size_t local_scratch_per_band(const Problem& p, int precision);
 // Bytes of one buffer of stick rows of nb bands (the fast paths keep two); the fixed-point path keeps its block
 // exponents behind the rows.
 size_t local_row_bytes(const Problem& p, int precision, int nb);
-void fixed_factors(int n, int* r1, int* r2);
-size_t fixed_tables(int n, std::vector<int>& table, FixedAxis* ax);
+void line_tables(int n, int precision, std::vector<int>& table, size_t* ftw, size_t* cells, LineAxis* ax);
+// Columns per x chunk and threads per CTA of a plane kernel (line_tiles.cpp): `base` + cw `col` bytes of shared memory a CTA,
+// `threads` resident threads an SM at most; *cw = 0 if nothing fits.
+void plane_shape(const LineAxis& x, const LineAxis& y, int npl, size_t base, size_t col, size_t smem_optin, int threads,
+                 int* cw, int* block);
+void float_plan(Problem& p, size_t smem_optin);
+int float_potential(Context& c, int slot, const LineAxis ax[3], int kernel_class);
+inline bool local_fast_ok(const Problem& p, int precision) {
+  return precision == HPSI_FP64 ? p.fixed.ok : p.fast.ok;
+}
 void fixed_plan(Problem& p, size_t smem_optin);
-int ensure_fixed_potential(Context& c, int slot, const FixedAxis ax[3]);
-int fixed_potential(Context& c, int slot, const FixedAxis ax[3], int kernel_class);
+int ensure_fixed_potential(Context& c, int slot, const LineAxis ax[3]);
+int fixed_potential(Context& c, int slot, const LineAxis ax[3], int kernel_class);
 int local_fixed_apply(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd, void* Zt, void* Yb,
                       int nbb);
 int local_fixed_apply_multi(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
                             double2* const* hpsi, void* const* zt, void* const* yb);
 int local_fixed_persistent(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
                            double2* const* hpsi, void* const* zt, void* const* yb, bool with_nl, bool* done);
-int local_fast_plan(const Problem& p, int precision, size_t smem_optin);
-std::vector<int> local_fast_candidates(const Problem& p, int precision, size_t smem_optin);
 int local_fast_apply(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd, void* Zt, void* Yb,
                      int nbb);
+// The local term alone (no kinetic part) of float32 bands in float32; needs local_fast_ok in float32.
+int local_raw_apply(Context& c, const Problem& p, const float2* f, float2* F, int nbnd);
+int local_fast_apply_raw(Context& c, const Problem& p, const float2* f, float2* F, int nbnd, void* Zt, void* Yb, int nbb);
 int local_fast_apply_multi(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
                            double2* const* hpsi, void* const* zt, void* const* yb);
 // The whole batch (and with_nl its float64 nonlocal term) in one persistent cooperative launch;

@@ -1,375 +1,360 @@
-// Fast local part of H|psi> for cubic boxes whose edge N = R1 * R2 has register codelets.
+// Local part of H|psi> in float32 (mixed contexts), for any box whose edges are products of two of 2, 3, 4, 5, 6, 8, 9, 10,
+// 12, 15, 16 (App. A.1: V applied in real space between the two transforms).  Three kernels per band block:
+//   k_zinv   per (chunk of sticks, band): psi(G) to float32 into the z-sticks (zeros elsewhere), inverse z-transform,
+//            Zt[b][j3][stick].
+//   k_plane  per (z-plane, band): the plane [m1-plane][j2] in shared memory; inverse y, then in chunks of columns
+//            inverse x, x V, forward x keeping the m1-planes, then forward y keeping the sticks -> Y[b][j3][stick].
+//   k_zfwd   per (chunk of sticks, band): forward z-transform, keep the sphere, add the kinetic term |k+G|^2/2 psi(G)
+//            in float64 (1/N_r is in the float32 copy of V).
+// The transforms are the in-place two-stage form of line_stages.cuh: a stage's items are dealt over all threads of the CTA,
+// coprime factors need no twiddles, and one kernel (run-time radix switch) serves every box, cubic or not.
+// psi is read, and H psi written, by integer conversions (convert.cuh), since a cast costs as much as a float64 FMA.
 //
-// Three kernels per band block (App. A.1: V applied in real space between the two transforms):
-//   k_zinv   per (band, chunk of sticks): scatter psi(G) into each z-stick (zero elsewhere), inverse
-//            z-transform, stage the chunk in shared memory and write Zt[b][j3][stick] coalesced.
-//   k_plane  per (z-plane j3, group of bands): per m1-plane an inverse y-transform of its sticks,
-//            per j2 an inverse x-transform over the m1-planes, x V(r), forward x-transform keeping
-//            the m1-planes, per m1-plane a forward y-transform keeping the sticks -> Y[b][j3][stick].
-//            The plane [m1-plane][j2] lives in shared memory; nothing but the stick rows touches HBM.
-//   k_zfwd   per (band, chunk of sticks): forward z-transform, keep the sphere, 1/N_r, add the
-//            kinetic term |k+G|^2/2 psi(G) in float64.
-// Each line transform is fft2_nat / fft2_rev (fft_codelets.cuh) on a group of max(R1, R2) threads.
+// What bounds it: instruction issue (a codelet's ~10 float32 instructions a value and stage, a load, a store and their
+// addresses) and the barriers between stages.  Measured with 160 bands on 90^3: planes 729 -> 594 us, z kernels 295 ->
+// 240 us against register codelets with a fixed line group per warp (24 to 30 of 32 lanes busy, cubic boxes of
+// 20 edges only); 81^3, which had only the generic kernels, H|psi> 8.2 -> 1.0 ms.
+//
+// The raw form takes float32 psi and gives the local term alone in float32, [nb][npw] both: the Gamma form packs two
+// real bands into one complex one in float32 and adds the kinetic term itself (gamma.cu).
 #include <cuda_runtime.h>
 
 #include <algorithm>
 
-#include "fft_codelets.cuh"
+#include "convert.cuh"
+#include "float_fft.cuh"
 #include "hpsi_internal.h"
 
 namespace hpsi {
 
 namespace {
 
-// One problem's share of a launch (a k-point or a cell with its band block).
-struct FastItem {
-  int nb, npw, npl, nst, bpc;  // bpc: bands per k_plane CTA
-  int stage_v, stage_row;      // the item's plan: V plane and stick row staged in shared memory
-  const StickDev* sticks;
-  const int* ymap;     // [npl][N]: stick of (plane, j2) or -1
-  const int* xmap;     // [N]: plane of ix or -1
-  const double2* psi;  // [nb][npw]
-  double2* hpsi;
-  const double* kin;
-  void* Zt;            // [nb][N][nst]
-  void* Yb;            // [nb][N][nst]
-  const void* V;       // [N][N][N] as [j3][j2][j1]
+#include "line_stages.cuh"
+
+struct FloatArith {
+  using V = float2;
+  using Tw = float2;
+  template <int R> using Dft = FfDft<R>;
+  static __device__ __forceinline__ float2 twiddle(float2 v, float2 w) { return ff_mul(v, w.x, w.y); }
 };
 
-constexpr int kMaxItems = 32;
+struct FastItem {
+  int nb, npw, npl, nst;
+  int n1, n2, n3;
+  LineAxis ax[3];
+  int cw, nch;                 // columns per x chunk, z chunks
+  int raw;
+  const int *soff, *zoff, *zbeg;   // Problem's lookup tables
+  const int* xmap;             // [n1]: plane of ix or -1
+  const void* psi;             // double2 (raw: float2) [nb][npw]
+  void* hpsi;
+  const double* kin;
+  float2* Zt;                  // [nb][n3][nst]
+  float2* Yb;
+  const float* V;              // [n3][slot of j1][slot of j2], V / N_r
+};
 
 // Every launch takes its items by value (the parameter block is 32 KB on sm_70 and later).
 struct FastBatch {
-  int nitems, N;
-  const float2* tw32;  // e^{-2 pi i j / N}, j < N
-  double inv_nr;
-  FastItem item[kMaxItems];
+  int nitems;
+  int off_z[kMaxLocalItems + 1];
+  int off_p[kMaxLocalItems + 1];
+  FastItem item[kMaxLocalItems];
 };
 
-__device__ __forceinline__ float2 d2f(double2 x) { return make_float2((float)x.x, (float)x.y); }
-
-template <int R1, int R2> struct Geo {
-  static constexpr int N = R1 * R2;
-  static constexpr int G = R1 > R2 ? R1 : R2;
-  static constexpr int LPW = 32 / G;          // line groups per warp
-  static constexpr int GROUPS = 8 * LPW;      // per 256-thread CTA
-  static constexpr int XS = Xch<R1, R2>::size; // exchange-buffer entries per group
-  static constexpr int PS = N + 1;            // row stride of the plane array (one pad entry)
+struct Placed {   // a value and its place in the tile
+  float2 v;
+  int at;
 };
 
-// Each kernel's work is a tile function of its block coordinates (bx, by, bz), so that the
-// persistent batched kernel below runs exactly the same code on the same tiles.
-template <typename T, int R1, int R2>
-__device__ __forceinline__ void zinv_tile(const FastBatch& bt, int bx, int by, int bz) {
-  using V = typename Cx<T>::type;
-  using Gm = Geo<R1, R2>;
-  constexpr int N = Gm::N, G = Gm::G, SC = Gm::GROUPS;
-  const FastItem& a = bt.item[bz];
-  if (bx * SC >= a.nst || by >= a.nb) return;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* tw = reinterpret_cast<V*>(smem_raw);
-  V* xbuf = tw + N;                       // [SC][XS]
-  V* obuf = xbuf + SC * Gm::XS;           // [N][SC]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int grp = warp * Gm::LPW + lane / G, t = lane % G;
-  const bool in_grp = lane < Gm::LPW * G;
-  const int s0 = bx * SC, b = by;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = bt.tw32[i];
+template <int MAXR>
+__device__ __forceinline__ void zinv_tile(const FastItem& a, int ch, int b, unsigned char* smem) {
+  constexpr int SC = kStickChunk, ld = SC + 1;
+  const int n = a.n3;
+  float2* tw = reinterpret_cast<float2*>(smem);
+  float2* L = tw + n;                                   // [cell][stick], rows of SC + 1
+  const int s0 = ch * SC, ns = min(SC, a.nst - s0);
+  const int g0 = a.zbeg[ch], ng = a.zbeg[ch + 1] - g0;
+  load_table(tw, a.ax[2].ftw, a.ax[2]);
+  for (int i = threadIdx.x; i < n * ld; i += blockDim.x) L[i] = make_float2(0.f, 0.f);
   __syncthreads();
-  const int s = s0 + grp;
-  const bool active = in_grp && s < a.nst;
-  V reg[G];
-  if (active && t < R2) {
-    const StickDev st = a.sticks[s];
-    const double2* ps = a.psi + (size_t)b * a.npw + st.g0;
-#pragma unroll
-    for (int n1 = 0; n1 < R1; ++n1) {
-      int tt = R2 * n1 + t - st.z0;
-      if (tt < 0) tt += N;
-      reg[n1] = tt < st.len ? d2f(ps[tt]) : czero<V>();
-    }
-  }
-  fft2_nat<R1, R2, +1>(reg, xbuf + (in_grp ? grp : 0) * Gm::XS, tw, t, active);
-  if (active && t < R1) {
-#pragma unroll
-    for (int k2 = 0; k2 < R2; ++k2) obuf[(t + R1 * k2) * SC + grp] = reg[k2];
+  const size_t row = (size_t)b * a.npw + g0;
+  auto place = [&](int, Placed q) { L[q.at] = q.v; };
+  if (a.raw) {
+    const float2* ps = static_cast<const float2*>(a.psi) + row;
+    staged_loop(ng, [&](int i) { return Placed{ps[i], a.zoff[g0 + i]}; }, place);
+  } else {
+    const double2* ps = static_cast<const double2*>(a.psi) + row;
+    staged_loop(ng, [&](int i) { return Placed{f64_to_f32(ps[i]), a.zoff[g0 + i]}; }, place);
   }
   __syncthreads();
-  V* Z = reinterpret_cast<V*>(a.Zt) + (size_t)b * N * a.nst;
-  const int ns = min(SC, a.nst - s0);
-  for (int i = threadIdx.x; i < N * SC; i += blockDim.x) {
-    const int j3 = i / SC, sl = i - j3 * SC;
-    if (sl < ns) Z[(size_t)j3 * a.nst + s0 + sl] = obuf[i];
-  }
-}
-
-template <typename T, int R1, int R2>
-__global__ void __launch_bounds__(256) k_zinv(const __grid_constant__ FastBatch bt) {
-  zinv_tile<T, R1, R2>(bt, blockIdx.x, blockIdx.y, blockIdx.z);
-}
-
-template <typename T, int R1, int R2>
-__device__ __forceinline__ void plane_tile(const FastBatch& bt, int bx, int by, int bz) {
-  using V = typename Cx<T>::type;
-  using Gm = Geo<R1, R2>;
-  constexpr int N = Gm::N, G = Gm::G, NG = Gm::GROUPS;
-  const FastItem& a = bt.item[bz];
-  if (by * a.bpc >= a.nb) return;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* tw = reinterpret_cast<V*>(smem_raw);
-  constexpr int PS = Gm::PS;
-  V* xbuf = tw + N;                              // [NG][XS]
-  V* P = xbuf + NG * Gm::XS;                     // [npl][PS]
-  V* row = P + (size_t)a.npl * PS;               // [nst] if stage_row
-  T* vpl = reinterpret_cast<T*>(row + (a.stage_row ? a.nst : 0));   // [N][N] if stage_v
-  int* xm = reinterpret_cast<int*>(vpl + (a.stage_v ? N * N : 0));  // [N]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int grp = warp * Gm::LPW + lane / G, t = lane % G;
-  const bool in_grp = lane < Gm::LPW * G;
-  V* xb = xbuf + (in_grp ? grp : 0) * Gm::XS;
-  const int j3 = bx;
-  const T* Vg = reinterpret_cast<const T*>(a.V) + (size_t)j3 * N * N;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    tw[i] = bt.tw32[i];
-    xm[i] = a.xmap[i];
-  }
-  if (a.stage_v)
-    for (int i = threadIdx.x; i < N * N; i += blockDim.x) vpl[i] = Vg[i];
-  const T* Vp = a.stage_v ? vpl : Vg;
-  for (int bi = 0; bi < a.bpc; ++bi) {
-    const int b = by * a.bpc + bi;
-    if (b >= a.nb) break;
-    const V* zin = reinterpret_cast<const V*>(a.Zt) + ((size_t)b * N + j3) * a.nst;
-    V* yout = reinterpret_cast<V*>(a.Yb) + ((size_t)b * N + j3) * a.nst;
-    __syncthreads();
-    if (a.stage_row)
-      for (int i = threadIdx.x; i < a.nst; i += blockDim.x) row[i] = zin[i];
-    __syncthreads();
-    const V* src = a.stage_row ? row : zin;
-    V reg[G];
-    // inverse y per m1-plane: inputs at the plane's sticks
-    for (int p0 = 0; p0 < a.npl; p0 += NG) {
-      const int p = p0 + grp;
-      const bool act = in_grp && p < a.npl;
-      if (act && t < R2) {
-        const int* ym = a.ymap + (size_t)p * N;
-#pragma unroll
-        for (int n1 = 0; n1 < R1; ++n1) {
-          const int s = __ldg(ym + R2 * n1 + t);
-          reg[n1] = s >= 0 ? src[s] : czero<V>();
-        }
-      }
-      fft2_nat<R1, R2, +1>(reg, xb, tw, t, act);
-      if (act && t < R1) {
-#pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) P[(size_t)p * PS + t + R1 * k2] = reg[k2];
-      }
-    }
-    __syncthreads();
-    // x lines: inverse over the m1-planes, x V, forward keeping the m1-planes
-    for (int q0 = 0; q0 < N; q0 += NG) {
-      const int j2 = q0 + grp;
-      const bool act = in_grp && j2 < N;
-      if (act && t < R2) {
-#pragma unroll
-        for (int n1 = 0; n1 < R1; ++n1) {
-          const int pp = xm[R2 * n1 + t];
-          reg[n1] = pp >= 0 ? P[(size_t)pp * PS + j2] : czero<V>();
-        }
-      }
-      fft2_nat<R1, R2, +1>(reg, xb, tw, t, act);
-      if (act && t < R1) {
-        const T* vr = Vp + (size_t)j2 * N;
-#pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) reg[k2] = cscale(reg[k2], vr[t + R1 * k2]);
-      }
-      fft2_rev<R1, R2, -1>(reg, xb, tw, t, act);
-      if (act && t < R2) {
-#pragma unroll
-        for (int m1 = 0; m1 < R1; ++m1) {
-          const int pp = xm[t + R2 * m1];
-          if (pp >= 0) P[(size_t)pp * PS + j2] = reg[m1];
-        }
-      }
-    }
-    __syncthreads();
-    // forward y per m1-plane, keep the sticks
-    V* dst = a.stage_row ? row : yout;
-    for (int p0 = 0; p0 < a.npl; p0 += NG) {
-      const int p = p0 + grp;
-      const bool act = in_grp && p < a.npl;
-      if (act && t < R2) {
-#pragma unroll
-        for (int n1 = 0; n1 < R1; ++n1) reg[n1] = P[(size_t)p * PS + R2 * n1 + t];
-      }
-      fft2_nat<R1, R2, -1>(reg, xb, tw, t, act);
-      if (act && t < R1) {
-        const int* ym = a.ymap + (size_t)p * N;
-#pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) {
-          const int s = __ldg(ym + t + R1 * k2);
-          if (s >= 0) dst[s] = reg[k2];
-        }
-      }
-    }
-    if (a.stage_row) {
-      __syncthreads();
-      for (int i = threadIdx.x; i < a.nst; i += blockDim.x) yout[i] = row[i];
-    }
-  }
-}
-
-template <typename T, int R1, int R2>
-__global__ void __launch_bounds__(256) k_plane(const __grid_constant__ FastBatch bt) {
-  plane_tile<T, R1, R2>(bt, blockIdx.x, blockIdx.y, blockIdx.z);
-}
-
-template <typename T, int R1, int R2>
-__device__ __forceinline__ void zfwd_tile(const FastBatch& bt, int bx, int by, int bz) {
-  using V = typename Cx<T>::type;
-  using Gm = Geo<R1, R2>;
-  constexpr int N = Gm::N, G = Gm::G, SC = Gm::GROUPS;
-  const FastItem& a = bt.item[bz];
-  if (bx * SC >= a.nst || by >= a.nb) return;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* tw = reinterpret_cast<V*>(smem_raw);
-  V* xbuf = tw + N;                       // [SC][XS]
-  V* ibuf = xbuf + SC * Gm::XS;           // [N][SC]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int grp = warp * Gm::LPW + lane / G, t = lane % G;
-  const bool in_grp = lane < Gm::LPW * G;
-  const int s0 = bx * SC, b = by;
-  const int ns = min(SC, a.nst - s0);
-  const V* Y = reinterpret_cast<const V*>(a.Yb) + (size_t)b * N * a.nst;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = bt.tw32[i];
-  for (int i = threadIdx.x; i < N * SC; i += blockDim.x) {
-    const int j3 = i / SC, sl = i - j3 * SC;
-    ibuf[i] = sl < ns ? Y[(size_t)j3 * a.nst + s0 + sl] : czero<V>();
-  }
+  const LineView<float2> lines{L, 1, ld};
+  line_stage1<FloatArith, MAXR, false>(a.ax[2], ns, tw, lines);
   __syncthreads();
-  const int s = s0 + grp;
-  const bool active = in_grp && s < a.nst;
-  V reg[G];
-  if (active && t < R2) {
+  line_stage2<FloatArith, MAXR, false>(a.ax[2], ns, tw, lines);
+  __syncthreads();
+  float2* Z = a.Zt + (size_t)b * n * a.nst + s0;
+  const int per = blockDim.x / SC, r0 = threadIdx.x / SC, sl = threadIdx.x % SC;
+  if (sl < ns)
+    for (int j3 = r0; j3 < n; j3 += per) Z[(size_t)j3 * a.nst + sl] = L[a.ax[2].slot[j3] * ld + sl];
+}
+
+template <int MAXR>
+__device__ __forceinline__ void plane_tile(const FastItem& a, int j3, int b, unsigned char* smem) {
+  const int n1 = a.n1, n2 = a.n2, npl = a.npl, PS = n2 | 1, cw = a.cw;
+  float2* twx = reinterpret_cast<float2*>(smem);
+  float2* twy = twx + (a.ax[0].twiddled ? n1 : 0);
+  float2* P = twy + (a.ax[1].twiddled ? n2 : 0);        // [plane][cell of j2], a row of zeros
+  float2* X = P + (npl + 1) * PS;                       // [cell of x][column of the chunk]
+  int* xo = reinterpret_cast<int*>(X + n1 * cw);
+  xo += (4 - ((reinterpret_cast<uintptr_t>(xo) >> 2) & 3)) & 3;   // read as int4
+  load_table(twx, a.ax[0].ftw, a.ax[0]);
+  load_table(twy, a.ax[1].ftw, a.ax[1]);
+  build_row_table(xo, a.ax[0], a.xmap, PS, npl * PS);
+  for (int i = threadIdx.x; i < (npl + 1) * PS; i += blockDim.x) P[i] = make_float2(0.f, 0.f);
+  __syncthreads();
+  const float2* zin = a.Zt + ((size_t)b * a.n3 + j3) * a.nst;
+  staged_loop(a.nst, [&](int i) { return Placed{zin[i], a.soff[i]}; }, [&](int, Placed q) { P[q.at] = q.v; });
+  __syncthreads();
+  const LineView<float2> rows{P, PS, 1}, cols{X, 1, cw};
+  line_stage1<FloatArith, MAXR, false>(a.ax[1], npl, twy, rows);
+  __syncthreads();
+  line_stage2<FloatArith, MAXR, false>(a.ax[1], npl, twy, rows);
+  __syncthreads();
+  const float* V = a.V + (size_t)j3 * n1 * n2;
+  for (int c0 = 0; c0 < n2; c0 += cw) {
+    const int nc = min(cw, n2 - c0);
+    x_stage1<FloatArith, MAXR>(a.ax[0], nc, twx, xo, P + c0, cols);
+    __syncthreads();
+    // the last inverse stage, x V, and the first forward one on the same registers; from here on real and imaginary
+    // parts are swapped, which turns the codelets' sign into the forward one
+    radix_switch<MAXR>(a.ax[0].r2, [&](auto rc) {
+      constexpr int R = decltype(rc)::value;
+      const LineAxis& ax = a.ax[0];
+      const int items = nc * ax.r1;
+      const float inv = 1.0f / (float)nc;
+      for (int it = threadIdx.x; it < items; it += blockDim.x) {
+        int k1, c;
+        split_index(it, nc, inv, k1, c);
+        float2* q = X + k1 * R * cw + c;
+        const float* vp = V + k1 * R * n2 + c0 + c;
+        float2 v[R];
+        float w[R];
 #pragma unroll
-    for (int n1 = 0; n1 < R1; ++n1) reg[n1] = ibuf[(R2 * n1 + t) * SC + grp];
-  }
-  fft2_nat<R1, R2, -1>(reg, xbuf + (in_grp ? grp : 0) * Gm::XS, tw, t, active);
-  if (active && t < R1) {
-    const StickDev st = a.sticks[s];
-    const double2* ps = a.psi + (size_t)b * a.npw + st.g0;
-    double2* out = a.hpsi + (size_t)b * a.npw + st.g0;
-    const double* kin = a.kin + st.g0;
+        for (int i = 0; i < R; ++i) {
+          v[i] = q[i * cw];
+          w[i] = __ldg(vp + i * n2);
+        }
+        FfDft<R>::run(v);
 #pragma unroll
-    for (int k2 = 0; k2 < R2; ++k2) {
-      int tt = t + R1 * k2 - st.z0;
-      if (tt < 0) tt += N;
-      if (tt < st.len) {
-        const double2 x = ps[tt];
-        const double kg = kin[tt];
-        const V v = reg[k2];
-        out[tt] = make_double2(kg * x.x + (double)v.x * bt.inv_nr, kg * x.y + (double)v.y * bt.inv_nr);
+        for (int i = 0; i < R; ++i) v[i] = make_float2(v[i].y * w[i], v[i].x * w[i]);
+        FfDft<R>::run(v);
+        if (ax.twiddled) {
+#pragma unroll
+          for (int i = 1; i < R; ++i) v[i] = FloatArith::twiddle(v[i], twx[k1 * i]);
+        }
+#pragma unroll
+        for (int i = 0; i < R; ++i) q[i * cw] = v[i];
       }
-    }
+    });
+    __syncthreads();
+    x_stage1_rev<FloatArith, MAXR>(a.ax[0], nc, xo, npl * PS, cols, P + c0, [](float2) {});
+    __syncthreads();
+  }
+  line_stage2<FloatArith, MAXR, true>(a.ax[1], npl, twy, rows);
+  __syncthreads();
+  line_stage1<FloatArith, MAXR, true>(a.ax[1], npl, twy, rows);
+  __syncthreads();
+  float2* yo = a.Yb + ((size_t)b * a.n3 + j3) * a.nst;
+  staged_loop(a.nst, [&](int i) { return a.soff[i]; }, [&](int i, int at) { yo[i] = P[at]; });
+}
+
+template <int MAXR>
+__device__ __forceinline__ void zfwd_tile(const FastItem& a, int ch, int b, unsigned char* smem) {
+  constexpr int SC = kStickChunk, ld = SC + 1;
+  const int n = a.n3;
+  float2* tw = reinterpret_cast<float2*>(smem);
+  float2* L = tw + n;
+  const int s0 = ch * SC, ns = min(SC, a.nst - s0);
+  const int g0 = a.zbeg[ch], ng = a.zbeg[ch + 1] - g0;
+  load_table(tw, a.ax[2].ftw, a.ax[2]);
+  const float2* Y = a.Yb + (size_t)b * n * a.nst + s0;
+  // (sticks past the last one are transformed with the others, from whatever the tile holds, and not read)
+  staged_loop(
+      n * SC, [&](int i) { return i % SC < ns ? Y[(size_t)(i / SC) * a.nst + i % SC] : make_float2(0.f, 0.f); },
+      [&](int i, float2 v) { L[a.ax[2].slot[i / SC] * ld + i % SC] = v; });
+  __syncthreads();
+  const LineView<float2> lines{L, 1, ld};
+  line_stage2<FloatArith, MAXR, true>(a.ax[2], ns, tw, lines);
+  __syncthreads();
+  line_stage1<FloatArith, MAXR, true>(a.ax[2], ns, tw, lines);
+  __syncthreads();
+  const size_t row = (size_t)b * a.npw + g0;
+  if (a.raw) {
+    float2* out = static_cast<float2*>(a.hpsi) + row;
+    staged_loop(ng, [&](int i) { return a.zoff[g0 + i]; },
+                [&](int i, int at) {
+                  const float2 v = L[at];   // swapped
+                  out[i] = make_float2(v.y, v.x);
+                });
+  } else {
+    struct In {
+      double2 x;
+      double kg;
+      int at;
+    };
+    const double2* ps = static_cast<const double2*>(a.psi) + row;
+    double2* out = static_cast<double2*>(a.hpsi) + row;
+    staged_loop(ng, [&](int i) { return In{ps[i], a.kin[g0 + i], a.zoff[g0 + i]}; },
+                [&](int i, In q) {
+                  const float2 v = L[q.at];   // swapped
+                  out[i] = make_double2(fma(q.kg, q.x.x, f32_to_f64(v.y)), fma(q.kg, q.x.y, f32_to_f64(v.x)));
+                });
   }
 }
 
-template <typename T, int R1, int R2>
-__global__ void __launch_bounds__(256) k_zfwd(const __grid_constant__ FastBatch bt) {
-  zfwd_tile<T, R1, R2>(bt, blockIdx.x, blockIdx.y, blockIdx.z);
+// Threads per SM that the kernels' registers allow
+template <int MAXR> constexpr int kPlaneThreads = MAXR > 12 ? 768 : 1024;
+inline int plane_threads(int rmax) { return rmax > 12 ? kPlaneThreads<16> : kPlaneThreads<10>; }
+
+template <int MAXR>
+__global__ void __launch_bounds__(512, MAXR > 12 ? 1 : 2) k_zinv(const __grid_constant__ FastBatch bt) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int i = tile_item(bt.off_z, bt.nitems, blockIdx.x), l = blockIdx.x - bt.off_z[i];
+  zinv_tile<MAXR>(bt.item[i], l % bt.item[i].nch, l / bt.item[i].nch, smem_raw);
+}
+template <int MAXR>
+__global__ void __launch_bounds__(kPlaneThreads<MAXR>, 1) k_plane(const __grid_constant__ FastBatch bt) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int i = tile_item(bt.off_p, bt.nitems, blockIdx.x), l = blockIdx.x - bt.off_p[i];
+  plane_tile<MAXR>(bt.item[i], l % bt.item[i].n3, l / bt.item[i].n3, smem_raw);
+}
+template <int MAXR>
+__global__ void __launch_bounds__(512, MAXR > 12 ? 1 : 2) k_zfwd(const __grid_constant__ FastBatch bt) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int i = tile_item(bt.off_z, bt.nitems, blockIdx.x), l = blockIdx.x - bt.off_z[i];
+  zfwd_tile<MAXR>(bt.item[i], l % bt.item[i].nch, l / bt.item[i].nch, smem_raw);
 }
 
 #include "nonlocal_tiles.cuh"
 
-// ---- persistent batched H|psi> (hpsi_apply_batch): one cooperative launch over every item ----
-// The grid works through the tile list of each phase in turn (the same tile functions as the
-// separate kernels: zinv, plane, zfwd, and in float64 the nonlocal calbec, D-scale and add_vuspsi of
-// all items), with a grid barrier between phases.  A phase's list holds each item's own tiles only
-// (items with fewer bands have fewer), and CTAs take tiles from it one at a time through an atomic
-// counter, so that uneven items balance as they do under the hardware block scheduler.  Every wait
-// is bounded: on expiry the CTA raises the context's error word and leaves.
-struct PersistCtl {
-  int nitems;
-  int off_z[kMaxItems + 1];   // first zinv / zfwd tile of each item (zch_i x nb_i tiles)
-  int off_p[kMaxItems + 1];   // first plane tile of each item (N x ceil(nb_i / bpc) tiles)
-  unsigned* bar;              // [0]: arrival counter; [1 + phase]: tile counters; zero at launch
+// The whole batch in one cooperative launch: the tiles of the three kernels above phase by phase, and, when
+// nl.nitems > 0, the float64 nonlocal term of the items, with a bounded grid barrier between the phases.
+struct FastPersist {
+  unsigned* bar;   // [0]: arrival counter; [1 + phase]: tile counters; zero at launch
   int* err;
 };
-
-template <typename T, int R1, int R2, bool NL>
+template <int MAXR>
 __global__ void __launch_bounds__(256) k_hpsi_batch(const __grid_constant__ FastBatch bt,
-                                                    const __grid_constant__ NlBatch nl,
-                                                    const __grid_constant__ PersistCtl pc) {
-  using Gm = Geo<R1, R2>;
-  constexpr int N = Gm::N;
+                                                    const __grid_constant__ NlBatch nl, const FastPersist pc) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   const unsigned G = gridDim.x;
-  const int nz = pc.off_z[pc.nitems], np = pc.off_p[pc.nitems];
+  const int nz = bt.off_z[bt.nitems], np = bt.off_p[bt.nitems];
   for (int t = persist_next(pc.bar + 1); t < nz; t = persist_next(pc.bar + 1)) {
-    const int i = find_item(pc.off_z, pc.nitems, t);
-    const int l = t - pc.off_z[i], zch = (bt.item[i].nst + Gm::GROUPS - 1) / Gm::GROUPS;
-    zinv_tile<T, R1, R2>(bt, l % zch, l / zch, i);
+    const int i = tile_item(bt.off_z, bt.nitems, t), l = t - bt.off_z[i];
+    zinv_tile<MAXR>(bt.item[i], l % bt.item[i].nch, l / bt.item[i].nch, smem_raw);
   }
   if (!persist_sync(pc.bar, G, pc.err)) return;
   for (int t = persist_next(pc.bar + 2); t < np; t = persist_next(pc.bar + 2)) {
-    const int i = find_item(pc.off_p, pc.nitems, t);
-    const int l = t - pc.off_p[i];
-    plane_tile<T, R1, R2>(bt, l % N, l / N, i);
+    const int i = tile_item(bt.off_p, bt.nitems, t), l = t - bt.off_p[i];
+    plane_tile<MAXR>(bt.item[i], l % bt.item[i].n3, l / bt.item[i].n3, smem_raw);
   }
   if (!persist_sync(pc.bar, 2 * G, pc.err)) return;
   for (int t = persist_next(pc.bar + 3); t < nz; t = persist_next(pc.bar + 3)) {
-    const int i = find_item(pc.off_z, pc.nitems, t);
-    const int l = t - pc.off_z[i], zch = (bt.item[i].nst + Gm::GROUPS - 1) / Gm::GROUPS;
-    zfwd_tile<T, R1, R2>(bt, l % zch, l / zch, i);
+    const int i = tile_item(bt.off_z, bt.nitems, t), l = t - bt.off_z[i];
+    zfwd_tile<MAXR>(bt.item[i], l % bt.item[i].nch, l / bt.item[i].nch, smem_raw);
   }
-  if constexpr (NL) {
-    // the nonlocal term of every item, added to the local result; its tiles reuse the dynamic
-    // shared memory of the FFT phases
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    nonlocal_phases(nl, pc.bar, pc.err, G, 3, reinterpret_cast<double2*>(smem_raw));
+  if (nl.nitems > 0) nonlocal_phases(nl, pc.bar, pc.err, G, 3, reinterpret_cast<double2*>(smem_raw));
+}
+
+// V[j3][j2][j1] -> [j3][slot of j1][slot of j2] in float32, times 1/N_r
+__global__ void k_fast_v(LineAxis a1, LineAxis a2, int n3, double inv_nr, const double* __restrict__ v,
+                         float* __restrict__ out) {
+  const size_t n = (size_t)a1.n * a2.n * n3;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    const int j1 = (int)(i % a1.n), j2 = (int)(i / a1.n % a2.n);
+    const size_t j3 = i / ((size_t)a1.n * a2.n);
+    out[(j3 * a1.n + a1.slot[j1]) * a2.n + a2.slot[j2]] = (float)(v[i] * inv_nr);
   }
 }
 
-template <typename T, int R1, int R2>
-struct FastKernels {
-  using V = typename Cx<T>::type;
-  using Gm = Geo<R1, R2>;
-  static size_t smem_z() { return sizeof(V) * (size_t)(Gm::N + Gm::GROUPS * Gm::XS + Gm::GROUPS * Gm::N); }
-  static size_t smem_plane(const Problem& p, int sv, int sr) {
-    return sizeof(V) * (size_t)(Gm::N + Gm::GROUPS * Gm::XS + (size_t)p.npl * Gm::PS + (sr ? p.nst : 0)) +
-           (sv ? sizeof(T) * (size_t)Gm::N * Gm::N : 0) + sizeof(int) * Gm::N;
+struct FastLaunch {
+  FastBatch bt;
+  size_t smem_z = 0, smem_p = 0;
+  int maxr = 0, items_z = 0, items_p = 0;   // largest radix, largest stages
+  int block = 0;                            // plane block of the item with the largest planes
+  void reset() {
+    bt.nitems = 0;
+    bt.off_z[0] = bt.off_p[0] = 0;
+    smem_z = smem_p = 0;
+    maxr = items_z = items_p = 0;
   }
-  // Tile grid of the three kernels over the batch; sets each item's bands per k_plane CTA.
-  static void geometry(const Context& c, FastBatch& bt, size_t max_plane_smem, int* zch, int* nbmax, int* pyb) {
-    int total_rows = 0;
-    for (int i = 0; i < bt.nitems; ++i) {
-      const FastItem& it = bt.item[i];
-      *zch = std::max(*zch, (it.nst + Gm::GROUPS - 1) / Gm::GROUPS);
-      *nbmax = std::max(*nbmax, it.nb);
-      total_rows += it.nb;
+  void add(Context& c, const Problem& p, const void* psi, void* hpsi, int nb, void* zt, void* yb, bool raw = false) {
+    const int i = bt.nitems++;
+    FastItem& it = bt.item[i];
+    const FloatPlan& f = p.fast;
+    it.nb = nb;
+    it.npw = p.npw;
+    it.npl = p.npl;
+    it.nst = p.nst;
+    it.n1 = p.n[0];
+    it.n2 = p.n[1];
+    it.n3 = p.n[2];
+    for (int a = 0; a < 3; ++a) {
+      it.ax[a] = p.fast.ax[a];
+      maxr = std::max(maxr, std::max(it.ax[a].r1, it.ax[a].r2));
     }
-    // bands per k_plane CTA: amortise the staged V plane while keeping >= 2 waves over the batch
-    const int occ = max_plane_smem <= c.smem_optin / 2 ? 2 : 1;
-    int bpc = std::max(1, (Gm::N * total_rows) / (2 * c.sm_count * occ));
-    bpc = std::min(bpc, 8);
-    for (int i = 0; i < bt.nitems; ++i) {
-      bt.item[i].bpc = bpc;
-      *pyb = std::max(*pyb, (bt.item[i].nb + bpc - 1) / bpc);
-    }
+    it.cw = f.cw;
+    it.nch = f.nch;
+    it.raw = raw;
+    it.soff = p.tab[HPSI_MIXED].soff;
+    it.zoff = p.tab[HPSI_MIXED].zoff;
+    it.zbeg = p.tab[HPSI_MIXED].zbeg;
+    it.xmap = p.d_xmap;
+    it.psi = psi;
+    it.hpsi = hpsi;
+    it.kin = p.d_kin;
+    it.Zt = static_cast<float2*>(zt);
+    it.Yb = static_cast<float2*>(yb);
+    it.V = static_cast<const float*>(c.vbufs[p.vslot + 3]);
+    items_z = std::max(items_z, kStickChunk * std::max(it.ax[2].r1, it.ax[2].r2));
+    items_p = std::max(items_p, std::max(it.npl * std::max(it.ax[1].r1, it.ax[1].r2),
+                                         f.cw * std::max(it.ax[0].r1, it.ax[0].r2)));
+    bt.off_z[i + 1] = bt.off_z[i] + f.nch * nb;
+    bt.off_p[i + 1] = bt.off_p[i] + p.n[2] * nb;
+    smem_z = std::max(smem_z, f.smem_z);
+    if (f.smem_p > smem_p) block = f.block;
+    smem_p = std::max(smem_p, f.smem_p);
   }
-  // The whole batch in one cooperative launch of k_hpsi_batch (with the float64 nonlocal term when
-  // nl is given); *done = false, and nothing launched, when the kernel does not fit.
-  static int run_persistent(Context& c, FastBatch& bt, size_t max_plane_smem, const NlBatch* nl, unsigned* bar,
-                            bool* done) {
-    *done = false;
-    const void* kern = nl ? (const void*)k_hpsi_batch<T, R1, R2, true> : (const void*)k_hpsi_batch<T, R1, R2, false>;
-    size_t dyn = std::max(smem_z(), max_plane_smem);
-    if (nl) dyn = std::max(dyn, sizeof(double2) * (size_t)std::max(CB_SMEM, AV_SMEM));
+  template <int MAXR> int run_t(Context& c) {
+    static bool attr = false;
+    if (!attr) {
+      const int mx = (int)c.smem_optin - 64;
+      cudaFuncSetAttribute(k_zinv<MAXR>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+      cudaFuncSetAttribute(k_plane<MAXR>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+      cudaFuncSetAttribute(k_zfwd<MAXR>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+      attr = true;
+    }
+    const int nz = bt.off_z[bt.nitems], np = bt.off_p[bt.nitems];
+    auto warps = [](int items) { return (items + 31) / 32 * 32; };
+    // z: one round of a stage's items; planes: plane_shape's block, or one round where there is a CTA per SM at most
+    const int bz = std::max(128, std::min(512, warps(items_z)));
+    const int bp = np <= c.sm_count ? std::max(block, std::min(kPlaneThreads<MAXR>, warps(items_p))) : block;
+    HPSI_LAUNCH(c, HPSI_K_INV_ZY, (k_zinv<MAXR><<<nz, bz, smem_z, c.stream>>>(bt)));
+    HPSI_LAUNCH(c, HPSI_K_XVX_Y, (k_plane<MAXR><<<np, bp, smem_p, c.stream>>>(bt)));
+    HPSI_LAUNCH(c, HPSI_K_FWD_Z, (k_zfwd<MAXR><<<nz, bz, smem_z, c.stream>>>(bt)));
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(c, e, "fast local kernels launch");
+    return HPSI_OK;
+  }
+  int run(Context& c) { return maxr > 12 ? run_t<16>(c) : maxr > 10 ? run_t<12>(c) : run_t<10>(c); }
+  template <int MAXR> int persistent_t(Context& c, const NlBatch& nl, unsigned* bar, bool* done) {
+    const void* kern = (const void*)k_hpsi_batch<MAXR>;
+    size_t dyn = std::max(smem_z, smem_p);
+    if (nl.nitems > 0) dyn = std::max(dyn, sizeof(double2) * (size_t)std::max(CB_SMEM, AV_SMEM));
     cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || fa.sharedSizeBytes + dyn > c.smem_optin) {
-      cudaGetLastError();
-      return HPSI_OK;
-    }
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) {
+    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || fa.sharedSizeBytes + dyn > c.smem_optin ||
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) {
       cudaGetLastError();
       return HPSI_OK;
     }
@@ -378,23 +363,10 @@ struct FastKernels {
       cudaGetLastError();
       return HPSI_OK;
     }
-    static PersistCtl pc;
-    int zch = 1, nbmax = 1, pyb = 1;
-    geometry(c, bt, max_plane_smem, &zch, &nbmax, &pyb);   // sets each item's bands per plane tile
-    pc.nitems = bt.nitems;
-    pc.off_z[0] = pc.off_p[0] = 0;
-    for (int i = 0; i < bt.nitems; ++i) {
-      const FastItem& it = bt.item[i];
-      pc.off_z[i + 1] = pc.off_z[i] + ((it.nst + Gm::GROUPS - 1) / Gm::GROUPS) * it.nb;
-      pc.off_p[i + 1] = pc.off_p[i] + Gm::N * ((it.nb + it.bpc - 1) / it.bpc);
-    }
-    pc.bar = bar;
-    pc.err = c.d_err;
-    static NlBatch empty;   // nitems = 0 (zero-initialised); the float32 form takes no nonlocal phases
-    const NlBatch& nb = nl ? *nl : empty;
     cudaError_t e = cudaMemsetAsync(bar, 0, 8 * sizeof(unsigned), c.stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "persistent batch barrier reset");
-    void* args[] = {(void*)&bt, (void*)&nb, (void*)&pc};
+    FastPersist pc{bar, c.d_err};
+    void* args[] = {(void*)&bt, (void*)&nl, (void*)&pc};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(occ * c.sm_count);
     cfg.blockDim = dim3(256);
@@ -410,219 +382,110 @@ struct FastKernels {
     *done = true;
     return HPSI_OK;
   }
-  // One launch of each kernel over every item of the batch (all share the edge N).
-  static int run(Context& c, FastBatch& bt, size_t max_plane_smem) {
-    static bool attr = false;
-    if (!attr) {
-      const int mx = (int)c.smem_optin;
-      cudaFuncSetAttribute(k_zinv<T, R1, R2>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-      cudaFuncSetAttribute(k_plane<T, R1, R2>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-      cudaFuncSetAttribute(k_zfwd<T, R1, R2>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-      attr = true;
-    }
-    const size_t sz = smem_z();
-    int zch = 1, nbmax = 1, pyb = 1;
-    geometry(c, bt, max_plane_smem, &zch, &nbmax, &pyb);
-    HPSI_LAUNCH(c, HPSI_K_INV_ZY, (k_zinv<T, R1, R2><<<dim3(zch, nbmax, bt.nitems), 256, sz, c.stream>>>(bt)));
-    HPSI_LAUNCH(c, HPSI_K_XVX_Y,
-                (k_plane<T, R1, R2><<<dim3(Gm::N, pyb, bt.nitems), 256, max_plane_smem, c.stream>>>(bt)));
-    HPSI_LAUNCH(c, HPSI_K_FWD_Z, (k_zfwd<T, R1, R2><<<dim3(zch, nbmax, bt.nitems), 256, sz, c.stream>>>(bt)));
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(c, e, "fast local kernels launch");
-    return HPSI_OK;
+  int persistent(Context& c, const NlBatch& nl, unsigned* bar, bool* done) {
+    return maxr > 10 ? persistent_t<16>(c, nl, bar, done) : persistent_t<10>(c, nl, bar, done);
   }
 };
 
-// Factorisations N = R1 * R2 of the supported cubic edges.
-template <typename T, typename F>
-bool dispatch_size(int n, F&& f) {
-  switch (n) {
-    case 24: f(FastKernels<T, 4, 6>()); return true;
-    case 25: f(FastKernels<T, 5, 5>()); return true;
-    case 27: f(FastKernels<T, 3, 9>()); return true;
-    case 30: f(FastKernels<T, 5, 6>()); return true;
-    case 32: f(FastKernels<T, 4, 8>()); return true;
-    case 36: f(FastKernels<T, 6, 6>()); return true;
-    case 40: f(FastKernels<T, 5, 8>()); return true;
-    case 45: f(FastKernels<T, 5, 9>()); return true;
-    case 48: f(FastKernels<T, 6, 8>()); return true;
-    case 50: f(FastKernels<T, 5, 10>()); return true;
-    case 60: f(FastKernels<T, 6, 10>()); return true;
-    case 64: f(FastKernels<T, 8, 8>()); return true;
-    case 72: f(FastKernels<T, 8, 9>()); return true;
-    case 80: f(FastKernels<T, 8, 10>()); return true;
-    case 90: f(FastKernels<T, 9, 10>()); return true;
-    case 96: f(FastKernels<T, 8, 12>()); return true;
-    case 100: f(FastKernels<T, 10, 10>()); return true;
-    case 120: f(FastKernels<T, 10, 12>()); return true;
-    case 128: f(FastKernels<T, 8, 16>()); return true;
-    case 144: f(FastKernels<T, 12, 12>()); return true;
-    default: return false;
-  }
-}
-
 }  // namespace
 
-// Shared-memory plan of the fast path for a problem (0 if the box has no fast kernels or the
-// plane does not fit): bit 0 stage V, bit 1 stage the stick row, bit 2 supported.
-int local_fast_plan(const Problem& p, int precision, size_t smem_optin) {
-  if (precision == HPSI_FP64) return p.fixed.ok ? 4 : 0;
-  if (p.n[0] != p.n[1] || p.n[1] != p.n[2]) return 0;
-  int flags = 0;
-  auto pick = [&](auto k) {
-    using K = decltype(k);
-    for (int cand : {3, 2, 0}) {
-      const int sv = cand & 1, sr = (cand >> 1) & 1;
-      if (K::smem_z() <= smem_optin && K::smem_plane(p, sv, sr) <= smem_optin) {
-        flags = 4 | sv | (sr << 1);
-        return;
-      }
-    }
-  };
-  dispatch_size<float>(p.n[0], pick);
-  return flags;
+// Tile sizes of a problem's float32 local term (ok = false: an edge without factors, or a plane that does not fit).
+void float_plan(Problem& p, size_t smem_optin) {
+  FloatPlan& f = p.fast;
+  f.ok = false;
+  for (int a = 0; a < 3; ++a)
+    if (!p.fast.ax[a].r1) return;
+  const int n1 = p.n[0], n2 = p.n[1], n3 = p.n[2];
+  auto tws = [&](int a) { return p.fast.ax[a].twiddled ? sizeof(float2) * (size_t)p.n[a] : 0; };
+  f.nch = (p.nst + kStickChunk - 1) / kStickChunk;
+  f.smem_z = sizeof(float2) * (size_t)n3 * (kStickChunk + 2);
+  const size_t base = tws(0) + tws(1) + sizeof(float2) * (size_t)(p.npl + 1) * (n2 | 1) +
+                      sizeof(int) * (p.fast.ax[0].r2 * (size_t)((p.fast.ax[0].r1 + 3) & ~3) + 4);
+  const size_t col = sizeof(float2) * (size_t)n1;
+  int rmax = 0;
+  for (int a = 0; a < 3; ++a) rmax = std::max(rmax, p.fast.ax[a].r1);
+  plane_shape(p.fast.ax[0], p.fast.ax[1], p.npl, base, col, smem_optin, plane_threads(rmax),
+              &f.cw, &f.block);
+  if (f.cw == 0) return;
+  f.smem_p = base + col * f.cw;
+  f.ok = f.smem_z <= smem_optin - 1024;
 }
 
-static FastItem make_item(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nb, void* Zt, void* Yb) {
-  FastItem it;
-  it.nb = nb;
-  it.npw = p.npw;
-  it.npl = p.npl;
-  it.nst = p.nst;
-  it.bpc = 1;
-  const int fl = p.fflags[HPSI_MIXED];
-  it.stage_v = fl & 1;
-  it.stage_row = (fl >> 1) & 1;
-  it.sticks = p.d_sticks;
-  it.ymap = p.d_ymap;
-  it.xmap = p.d_xmap;
-  it.psi = psi;
-  it.hpsi = hpsi;
-  it.kin = p.d_kin;
-  it.Zt = Zt;
-  it.Yb = Yb;
-  it.V = p.d_v32;
-  return it;
-}
-
-static size_t plane_smem(const Context& c, const Problem& p, int flags) {
-  size_t r = 0;
-  auto f = [&](auto k) { r = decltype(k)::smem_plane(p, flags & 1, (flags >> 1) & 1); };
-  dispatch_size<float>(p.n[0], f);
-  return r;
-}
-
-static int run_batch(Context& c, FastBatch& bt, size_t smem) {
-  int rc = HPSI_EINVAL;
-  auto go = [&](auto k) { rc = decltype(k)::run(c, bt, smem); };
-  dispatch_size<float>(bt.N, go);
-  return rc;
-}
-
-static void batch_header(FastBatch& bt, const Problem& p) {
-  bt.nitems = 0;
-  bt.N = p.n[0];
-  bt.tw32 = p.d_ftw32;
-  bt.inv_nr = 1.0 / ((double)p.n[0] * p.n[1] * p.n[2]);
-}
-
-// Every plan (staging flags | 4) whose kernels fit the shared memory, for the autotuner.
-std::vector<int> local_fast_candidates(const Problem& p, int precision, size_t smem_optin) {
-  std::vector<int> out;
-  if (precision == HPSI_FP64) return p.fixed.ok ? std::vector<int>{4} : out;
-  if (p.n[0] != p.n[1] || p.n[1] != p.n[2]) return out;
-  auto pick = [&](auto k) {
-    using K = decltype(k);
-    for (int cand : {3, 2, 1, 0})
-      if (K::smem_z() <= smem_optin && K::smem_plane(p, cand & 1, (cand >> 1) & 1) <= smem_optin)
-        out.push_back(4 | cand);
-  };
-  dispatch_size<float>(p.n[0], pick);
-  return out;
+// V / N_r in float32 in slot order (vbufs[slot + 3]) from the float64 V.
+int float_potential(Context& c, int slot, const LineAxis ax[3], int kernel_class) {
+  const size_t nr = (size_t)ax[0].n * ax[1].n * ax[2].n;
+  HPSI_LAUNCH(c, kernel_class, (k_fast_v<<<(int)std::min<size_t>(4 * c.sm_count, (nr + 255) / 256), 256, 0, c.stream>>>(
+                                   ax[0], ax[1], ax[2].n, 1.0 / (double)nr, static_cast<const double*>(c.vbufs[slot]),
+                                   static_cast<float*>(c.vbufs[slot + 3]))));
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(c, e, "float32 potential");
+  return HPSI_OK;
 }
 
 int local_fast_apply(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd, void* Zt, void* Yb,
                      int nbb) {
   if (cur_prec(c) == HPSI_FP64) return local_fixed_apply(c, p, psi, hpsi, nbnd, Zt, Yb, nbb);
-  static FastBatch bt;   // host staging of the parameter block (calls are not thread-safe by contract)
-  const int fl = p.fflags[HPSI_MIXED];
-  batch_header(bt, p);
-  const size_t smem = plane_smem(c, p, fl);
+  static FastLaunch fl;   // host staging of the parameter block (calls are not thread-safe by contract)
   for (int b0 = 0; b0 < nbnd; b0 += nbb) {
-    const int nb = std::min(nbb, nbnd - b0);
-    bt.nitems = 1;
-    bt.item[0] = make_item(c, p, psi + (size_t)b0 * p.npw, hpsi + (size_t)b0 * p.npw, nb, Zt, Yb);
-    int rc = run_batch(c, bt, smem);
+    fl.reset();
+    fl.add(c, p, psi + (size_t)b0 * p.npw, hpsi + (size_t)b0 * p.npw, std::min(nbb, nbnd - b0), Zt, Yb);
+    const int rc = fl.run(c);
     if (rc) return rc;
   }
   return HPSI_OK;
 }
 
-// Several problems with the same cubic edge in one launch per kernel, each item with its own plan;
-// scratch[i] holds item i's Zt and Y (each n3 * nst * nbnd complex values).
+int local_fast_apply_raw(Context& c, const Problem& p, const float2* f, float2* F, int nbnd, void* Zt, void* Yb, int nbb) {
+  static FastLaunch fl;
+  for (int b0 = 0; b0 < nbnd; b0 += nbb) {
+    fl.reset();
+    fl.add(c, p, f + (size_t)b0 * p.npw, F + (size_t)b0 * p.npw, std::min(nbb, nbnd - b0), Zt, Yb, true);
+    const int rc = fl.run(c);
+    if (rc) return rc;
+  }
+  return HPSI_OK;
+}
+
+// Several problems in one launch per kernel; zt[i], yb[i] hold item i's stick rows (local_row_bytes).
 int local_fast_apply_multi(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
                            double2* const* hpsi, void* const* zt, void* const* yb) {
   if (cur_prec(c) == HPSI_FP64) return local_fixed_apply_multi(c, nitem, prob, nbnd, psi, hpsi, zt, yb);
-  static FastBatch bt;
-  int done = 0;
-  while (done < nitem) {
-    const Problem& p0 = c.probs[prob[done]];
-    batch_header(bt, p0);
-    size_t smem = 0;
-    int n = 0;
-    while (done + n < nitem && n < kMaxItems) {
-      const Problem& p = c.probs[prob[done + n]];
-      if (p.n[0] != p0.n[0]) break;
-      bt.item[n] = make_item(c, p, psi[done + n], hpsi[done + n], nbnd[done + n], zt[done + n], yb[done + n]);
-      smem = std::max(smem, plane_smem(c, p, p.fflags[HPSI_MIXED]));
-      ++n;
-    }
-    bt.nitems = n;
-    int rc = run_batch(c, bt, smem);
+  static FastLaunch fl;
+  for (int i0 = 0; i0 < nitem; i0 += kMaxLocalItems) {
+    fl.reset();
+    for (int i = i0; i < std::min(nitem, i0 + kMaxLocalItems); ++i)
+      fl.add(c, c.probs[prob[i]], psi[i], hpsi[i], nbnd[i], zt[i], yb[i]);
+    const int rc = fl.run(c);
     if (rc) return rc;
-    done += n;
   }
   return HPSI_OK;
 }
 
-// The whole hpsi_apply_batch in one persistent launch: every item on the fast path with one box
-// edge, at most kMaxItems of them (and kNlBatch with a nonlocal term in float64).  with_nl:
-// the float64 nonlocal term of the items joins the launch.  *done = false: nothing was launched
-// and the caller takes the launch-per-kernel path.
+// The whole hpsi_apply_batch in one persistent launch: every item on the fast path with one box edge, at most
+// kMaxLocalItems of them (and kNlBatch with a nonlocal term in float64).  with_nl: the float64 nonlocal term of the
+// items joins the launch.  *done = false: nothing was launched and the caller takes the launch-per-kernel path.
 int local_batch_persistent(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
                            double2* const* hpsi, void* const* zt, void* const* yb, bool with_nl, bool* done) {
   *done = false;
-  if (nitem < 1 || nitem > kMaxItems || nitem > kNlBatch || c.force_generic) return HPSI_OK;
+  if (nitem < 1 || nitem > kMaxLocalItems || nitem > kNlBatch || c.force_generic) return HPSI_OK;
   const int pr = cur_prec(c);
-  const Problem& p0 = c.probs[prob[0]];
   for (int i = 0; i < nitem; ++i) {
     const Problem& p = c.probs[prob[i]];
-    if (!(p.fflags[pr] & 4) || p.n[0] != p0.n[0] || nbnd[i] < 1) return HPSI_OK;
+    if (!local_fast_ok(p, pr) || p.n[0] != c.probs[prob[0]].n[0] || nbnd[i] < 1) return HPSI_OK;
   }
   if (pr == HPSI_FP64) return local_fixed_persistent(c, nitem, prob, nbnd, psi, hpsi, zt, yb, with_nl, done);
-  static FastBatch bt;
+  static FastLaunch fl;
   static NlBatch nl;
-  batch_header(bt, p0);
-  size_t smem = 0;
-  for (int i = 0; i < nitem; ++i) {
-    const Problem& p = c.probs[prob[i]];
-    bt.item[i] = make_item(c, p, psi[i], hpsi[i], nbnd[i], zt[i], yb[i]);
-    smem = std::max(smem, plane_smem(c, p, p.fflags[pr]));
-  }
-  bt.nitems = nitem;
-  const NlBatch* nlp = nullptr;
+  fl.reset();
+  for (int i = 0; i < nitem; ++i) fl.add(c, c.probs[prob[i]], psi[i], hpsi[i], nbnd[i], zt[i], yb[i]);
+  nl.nitems = 0;
   if (with_nl) {
     const int rc = persistent_nl_batch(c, nitem, prob, nbnd, psi, hpsi, nl);
     if (rc) return rc;
-    if (nl.nitems > 0) nlp = &nl;
   }
-  int rc = ensure_buffer(c, &c.ws.pbar, &c.ws.pbarbytes, 256);
+  const int rc = ensure_buffer(c, &c.ws.pbar, &c.ws.pbarbytes, 256);
   if (rc) return rc;
-  unsigned* bar = static_cast<unsigned*>(c.ws.pbar);
-  rc = HPSI_EINVAL;
-  auto go = [&](auto k) { rc = decltype(k)::run_persistent(c, bt, smem, nlp, bar, done); };
-  dispatch_size<float>(bt.N, go);
-  return rc;
+  return fl.persistent(c, nl, static_cast<unsigned*>(c.ws.pbar), done);
 }
 
 }  // namespace hpsi

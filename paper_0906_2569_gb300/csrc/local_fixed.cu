@@ -26,6 +26,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "fixed_fft.cuh"
@@ -35,20 +36,27 @@ namespace hpsi {
 
 namespace {
 
+#include "line_stages.cuh"
+
+// Fixed-point arithmetic for the line stages
+struct FixArith {
+  using V = longlong2;
+  using Tw = FxTw;
+  template <int R> using Dft = FxDft<R>;
+  static __device__ __forceinline__ longlong2 twiddle(longlong2 v, FxTw w) { return fx_twiddle(v, w); }
+};
+
 constexpr int kFxNan = 1 << 28;      // exponent of a block that holds a non-finite value
 constexpr int kFxZero = -(1 << 20);  // exponent of a block of zeros
-constexpr int kFxMaxItems = 32;
 
 struct FxItem {
   int nb, npw, npl, nst;
   int n1, n2, n3;
-  FixedAxis ax[3];
+  LineAxis ax[3];
   int cw;                       // columns per x chunk
-  int sc;                       // sticks per z chunk
   int nch;                      // z chunks
   int hz, hy, hx, s3, hyf, hzf; // growth bounds of the transforms, in bits (FixedPlan)
-  const StickDev* sticks;
-  const int* ymap;
+  const int *soff, *zoff, *zbeg;   // Problem's lookup tables
   const int* xmap;
   const double2* psi;
   double2* hpsi;
@@ -64,45 +72,14 @@ struct FxItem {
 
 struct FxBatch {
   int nitems;
-  int off_z[kFxMaxItems + 1];   // first z tile of each item (nch x nb tiles)
-  int off_p[kFxMaxItems + 1];   // first plane tile (n3 x nb tiles)
-  FxItem item[kFxMaxItems];
+  int off_z[kMaxLocalItems + 1];   // first z tile of each item (nch x nb tiles)
+  int off_p[kMaxLocalItems + 1];   // first plane tile (n3 x nb tiles)
+  FxItem item[kMaxLocalItems];
 };
 
 // Resident threads per SM the plane kernel's registers allow (80 and 128 a thread): more warps hide more of the
 // multiplications' latency, but the 16-point codelet alone holds 64 registers of data.
 template <int MAXR> constexpr int kFxThreads = MAXR > 10 ? 512 : 768;
-
-template <int R> struct Rx {
-  static constexpr int value = R;
-};
-template <int MAXR, typename F>
-__device__ __forceinline__ void radix_switch(int r, F&& f) {
-  switch (r) {
-    case 2: f(Rx<2>()); break;
-    case 3: f(Rx<3>()); break;
-    case 4: f(Rx<4>()); break;
-    case 5: f(Rx<5>()); break;
-    case 6: f(Rx<6>()); break;
-    case 8: f(Rx<8>()); break;
-    case 9: f(Rx<9>()); break;
-    case 10: f(Rx<10>()); break;
-    default:
-      if constexpr (MAXR > 10) {
-        switch (r) {
-          case 12: f(Rx<12>()); break;
-          case 15: f(Rx<15>()); break;
-          default: f(Rx<16>()); break;
-        }
-      }
-  }
-}
-
-// it = a cnt + b with b < cnt, for the small non-negative numbers of a tile
-__device__ __forceinline__ void split_index(int it, int cnt, float inv, int& a, int& b) {
-  a = (int)(((float)it + 0.5f) * inv);
-  b = it - a * cnt;
-}
 
 __device__ __forceinline__ unsigned long long fx_mag(longlong2 v) {
   return (unsigned long long)((v.x ^ (v.x >> 63)) | (v.y ^ (v.y >> 63)));
@@ -141,100 +118,34 @@ __device__ __forceinline__ void fx_or(FxShared* sh, unsigned long long m) {
 // Shift that brings values below 2^bits(m) up to (or down to) 2^(63 - head)
 __device__ __forceinline__ int fx_headroom(unsigned long long m, int head) { return (int)__clzll((long long)m) - 1 - head; }
 
-// Stage 1 (or, REV, the last stage of the reversed sequence) of `cnt` lines of a tile: item (t, line), lines fastest
-// over the threads; ld(line, slot) and st(line, slot, value) reach the tile.
-template <int MAXR, bool REV, typename LD, typename ST>
-__device__ __forceinline__ void fx_stage1(const FixedAxis& ax, int cnt, const FxTw* tw, LD&& ld, ST&& st) {
-  radix_switch<MAXR>(ax.r1, [&](auto rc) {
-    constexpr int R = decltype(rc)::value;
-    const int items = cnt * ax.r2;
-    const float inv = 1.0f / (float)cnt;
-    for (int it = threadIdx.x; it < items; it += blockDim.x) {
-      int t, line;
-      split_index(it, cnt, inv, t, line);
-      longlong2 v[R];
-      int pos = t * ax.s2;
-#pragma unroll
-      for (int a = 0; a < R; ++a) {
-        v[a] = ld(line, pos);
-        pos += ax.r2;
-        if (pos >= ax.n) pos -= ax.n;
-      }
-      FxDft<R>::run(v);
-      if (!REV && ax.s2 == 1) {
-#pragma unroll
-        for (int a = 1; a < R; ++a) v[a] = fx_twiddle(v[a], tw[t * a]);
-      }
-      pos = t * ax.s2;
-#pragma unroll
-      for (int a = 0; a < R; ++a) {
-        st(line, pos, v[a]);
-        pos += ax.r2;
-        if (pos >= ax.n) pos -= ax.n;
-      }
-    }
-  });
-}
-
-// Stage 2 (or, REV, the first stage of the reversed sequence): item (k1, line)
-template <int MAXR, bool REV, typename LD, typename ST>
-__device__ __forceinline__ void fx_stage2(const FixedAxis& ax, int cnt, const FxTw* tw, LD&& ld, ST&& st) {
-  radix_switch<MAXR>(ax.r2, [&](auto rc) {
-    constexpr int R = decltype(rc)::value;
-    const int items = cnt * ax.r1;
-    const float inv = 1.0f / (float)cnt;
-    for (int it = threadIdx.x; it < items; it += blockDim.x) {
-      int k1, line;
-      split_index(it, cnt, inv, k1, line);
-      longlong2 v[R];
-      int pos = k1 * ax.r2;
-#pragma unroll
-      for (int b = 0; b < R; ++b) {
-        v[b] = ld(line, pos);
-        pos += ax.s2;
-        if (pos >= ax.n) pos -= ax.n;
-      }
-      FxDft<R>::run(v);
-      if (REV && ax.s2 == 1) {
-#pragma unroll
-        for (int b = 1; b < R; ++b) v[b] = fx_twiddle(v[b], tw[k1 * b]);
-      }
-      pos = k1 * ax.r2;
-#pragma unroll
-      for (int b = 0; b < R; ++b) {
-        st(line, pos, v[b]);
-        pos += ax.s2;
-        if (pos >= ax.n) pos -= ax.n;
-      }
-    }
-  });
-}
-
-__device__ __forceinline__ void load_table(FxTw* dst, const FixedAxis& ax) {
-  if (ax.s2 != 1) return;   // the prime-factor form has no twiddles
-  for (int i = threadIdx.x; i < ax.n; i += blockDim.x) dst[i] = ax.tw[i];
-}
+struct FxPlaced {   // a value and its place in the tile
+  longlong2 v;
+  int at;
+};
 
 // Inverse z-transform of one chunk of sticks of one band.
 template <int MAXR>
 __device__ __forceinline__ void fx_zinv_tile(const FxItem& a, int ch, int b, unsigned char* smem, FxShared* sh) {
-  const int n = a.n3, ld = a.sc + 1;
+  constexpr int SC = kStickChunk, ld = SC + 1;
+  const int n = a.n3;
   FxTw* tw = reinterpret_cast<FxTw*>(smem);
-  longlong2* L = reinterpret_cast<longlong2*>(smem + sizeof(FxTw) * n);   // [slot][stick], rows of sc + 1
-  const int s0 = ch * a.sc, ns = min(a.sc, a.nst - s0);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  longlong2* L = reinterpret_cast<longlong2*>(smem + sizeof(FxTw) * n);   // [cell][stick], rows of SC + 1
+  const int s0 = ch * SC, ns = min(SC, a.nst - s0);
+  const int lane = threadIdx.x & 31;
+  // the chunk's sticks are one contiguous range of G
+  const int g0 = a.zbeg[ch], ng = a.zbeg[ch + 1] - g0;
+  const longlong2* ps = reinterpret_cast<const longlong2*>(a.psi + (size_t)b * a.npw + g0);
   if (threadIdx.x == 0) sh->emax = 0;
-  load_table(tw, a.ax[2]);
+  load_table(tw, a.ax[2].fxtw, a.ax[2]);
+  for (int i = threadIdx.x; i < n * ld; i += blockDim.x) L[i] = {0, 0};
   __syncthreads();
-  // the largest exponent field of the chunk: its sticks are one contiguous range of G
-  const StickDev first = a.sticks[s0], last = a.sticks[s0 + ns - 1];
-  const int ng = last.g0 + last.len - first.g0;
-  const longlong2* ps = reinterpret_cast<const longlong2*>(a.psi + (size_t)b * a.npw);
+  // float64 bits into their places, and the largest exponent field
   unsigned hi = 0;
-  for (int i = threadIdx.x; i < ng; i += blockDim.x) {
-    const longlong2 v = ps[first.g0 + i];
-    hi = max(hi, max((unsigned)(v.x >> 32) & 0x7fffffffu, (unsigned)(v.y >> 32) & 0x7fffffffu));
-  }
+  staged_loop(ng, [&](int i) { return FxPlaced{ps[i], a.zoff[g0 + i]}; },
+              [&](int, FxPlaced q) {
+                hi = max(hi, max((unsigned)(q.v.x >> 32) & 0x7fffffffu, (unsigned)(q.v.y >> 32) & 0x7fffffffu));
+                L[q.at] = q.v;
+              });
   hi = __reduce_max_sync(0xffffffffu, hi);
   if (lane == 0) atomicMax(&sh->emax, (int)(hi >> 20));
   __syncthreads();
@@ -242,31 +153,22 @@ __device__ __forceinline__ void fx_zinv_tile(const FxItem& a, int ch, int b, uns
   if (threadIdx.x == 0)
     a.Ez[(size_t)b * a.nch + ch] = emax == 0x7ff ? kFxNan : emax == 0 ? kFxZero : emax - 1022 - 63 + a.hz;
   if (emax == 0x7ff) return;   // (every thread) the plane kernel reads the exponent only
-  // |x| < 2^(emax - 1022), so q = x 2^(63 - hz - (emax - 1022)) stays below 2^(63 - hz)
+  // |x| < 2^(emax - 1022), so q = x 2^(63 - hz - (emax - 1022)) stays below 2^(63 - hz).  The bits become integers as the
+  // first stage reads them (a cell without a G holds the bits of zero).
   const int e0 = emax - 10 + a.hz;
-  for (int s = warp; s < ns; s += nw) {
-    const StickDev st = a.sticks[s0 + s];
-    for (int pos = lane; pos < n; pos += 32) {
-      int tt = pos - st.z0;
-      if (tt < 0) tt += n;
-      longlong2 v = {0, 0};
-      if (tt < st.len) {
-        const longlong2 w = ps[st.g0 + tt];
-        v.x = fx_from_bits(w.x, e0);
-        v.y = fx_from_bits(w.y, e0);
-      }
-      L[pos * ld + s] = v;
-    }
-  }
+  auto to_fixed = [&](longlong2 w) {
+    longlong2 v;
+    v.x = fx_from_bits(w.x, e0);
+    v.y = fx_from_bits(w.y, e0);
+    return v;
+  };
+  const LineView<longlong2> lines{L, 1, ld};
+  line_stage1<FixArith, MAXR, false>(a.ax[2], ns, tw, lines, to_fixed);
   __syncthreads();
-  auto get = [&](int line, int pos) { return L[pos * ld + line]; };
-  auto put = [&](int line, int pos, longlong2 v) { L[pos * ld + line] = v; };
-  fx_stage1<MAXR, false>(a.ax[2], ns, tw, get, put);
-  __syncthreads();
-  fx_stage2<MAXR, false>(a.ax[2], ns, tw, get, put);
+  line_stage2<FixArith, MAXR, false>(a.ax[2], ns, tw, lines);
   __syncthreads();
   longlong2* Z = a.Zt + (size_t)b * n * a.nst + s0;
-  const int per = blockDim.x / a.sc, r0 = threadIdx.x / a.sc, sl = threadIdx.x - r0 * a.sc;
+  const int per = blockDim.x / SC, r0 = threadIdx.x / SC, sl = threadIdx.x % SC;
   if (sl < ns)
     for (int j3 = r0; j3 < n; j3 += per) Z[(size_t)j3 * a.nst + sl] = L[a.ax[2].slot[j3] * ld + sl];
 }
@@ -275,20 +177,21 @@ template <int MAXR>
 __device__ __forceinline__ void fx_plane_tile(const FxItem& a, int j3, int b, unsigned char* smem, FxShared* sh) {
   const int n1 = a.n1, n2 = a.n2, npl = a.npl, PS = n2 | 1, cw = a.cw;
   FxTw* twx = reinterpret_cast<FxTw*>(smem);
-  FxTw* twy = twx + (a.ax[0].s2 == 1 ? n1 : 0);
-  longlong2* P = reinterpret_cast<longlong2*>(twy + (a.ax[1].s2 == 1 ? n2 : 0));   // [plane][j2]
-  longlong2* X = P + (size_t)npl * PS;                                             // [slot of x][column of the chunk]
-  int* xm = reinterpret_cast<int*>(X + (size_t)n1 * cw);
+  FxTw* twy = twx + (a.ax[0].twiddled ? n1 : 0);
+  longlong2* P = reinterpret_cast<longlong2*>(twy + (a.ax[1].twiddled ? n2 : 0));  // [plane][cell of j2], a row of zeros
+  longlong2* X = P + (size_t)(npl + 1) * PS;                                       // [cell of x][column of the chunk]
+  int* xo = reinterpret_cast<int*>(X + (size_t)n1 * cw);
   float* cn = reinterpret_cast<float*>(X);                                         // column norms, before X is in use
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     sh->mag = 0;
     sh->emax = kFxZero;
     sh->norm = 0.f;
   }
-  load_table(twx, a.ax[0]);
-  load_table(twy, a.ax[1]);
-  for (int i = threadIdx.x; i < n1; i += blockDim.x) xm[i] = a.xmap[i];
+  load_table(twx, a.ax[0].fxtw, a.ax[0]);
+  load_table(twy, a.ax[1].fxtw, a.ax[1]);
+  build_row_table(xo, a.ax[0], a.xmap, PS, npl * PS);
+  for (int i = threadIdx.x; i < (npl + 1) * PS; i += blockDim.x) P[i] = {0, 0};
   __syncthreads();
   const int* ez = a.Ez + (size_t)b * a.nch;
   int em = kFxZero;
@@ -304,18 +207,17 @@ __device__ __forceinline__ void fx_plane_tile(const FxItem& a, int j3, int b, un
   }
   // the plane's sticks, aligned to the largest exponent
   const longlong2* zin = a.Zt + ((size_t)b * a.n3 + j3) * a.nst;
-  const int lsc = 31 - __clz(a.sc);   // sc is a power of two
+  struct In {
+    longlong2 v;
+    int at, e;
+  };
   unsigned long long m = 0;
-  for (int p = warp; p < npl; p += nw) {
-    const int* ym = a.ymap + (size_t)p * n2;
-    for (int j2 = lane; j2 < n2; j2 += 32) {
-      const int s = __ldg(ym + j2);
-      longlong2 v = {0, 0};
-      if (s >= 0) v = fx_align(zin[s], e - ez[s >> lsc]);
-      m |= fx_mag(v);
-      P[p * PS + j2] = v;
-    }
-  }
+  staged_loop(a.nst, [&](int i) { return In{zin[i], a.soff[i], ez[i / kStickChunk]}; },
+              [&](int, In q) {
+                const longlong2 v = fx_align(q.v, e - q.e);
+                m |= fx_mag(v);
+                P[q.at] = v;
+              });
   fx_or(sh, m);
   __syncthreads();
   m = sh->mag;
@@ -326,16 +228,14 @@ __device__ __forceinline__ void fx_plane_tile(const FxItem& a, int j3, int b, un
     if (threadIdx.x == 0) a.Ey[(size_t)b * a.n3 + j3] = kFxZero;
     return;
   }
-  auto get = [&](int p, int pos) { return P[p * PS + pos]; };
-  auto put = [&](int p, int pos, longlong2 v) { P[p * PS + pos] = v; };
+  const LineView<longlong2> rows{P, PS, 1};
   {
     const int d = fx_headroom(m, a.hy);
     e -= d;
-    const FxShift sh1(d);
-    fx_stage1<MAXR, false>(a.ax[1], npl, twy, [&](int p, int pos) { return sh1(P[p * PS + pos]); }, put);
+    line_stage1<FixArith, MAXR, false>(a.ax[1], npl, twy, rows, FxShift(d));
   }
   __syncthreads();
-  fx_stage2<MAXR, false>(a.ax[1], npl, twy, get, put);
+  line_stage2<FixArith, MAXR, false>(a.ax[1], npl, twy, rows);
   if (threadIdx.x == 0) sh->mag = 0;
   __syncthreads();
   // the largest column norm, in units of 2^32, rounded up (the +2 and the factor cover every rounding here)
@@ -366,69 +266,45 @@ __device__ __forceinline__ void fx_plane_tile(const FxItem& a, int j3, int b, un
   e += ve + 2 + a.s3 - dx;
   const long long* V = a.V + (size_t)j3 * n1 * n2;
   unsigned long long my = 0;
+  const LineView<longlong2> cols{X, 1, cw};
   for (int c0 = 0; c0 < n2; c0 += cw) {
     const int nc = min(cw, n2 - c0);
-    fx_stage1<MAXR, false>(
-        a.ax[0], nc, twx,
-        [&](int c, int pos) {
-          const int pp = xm[pos];
-          longlong2 v = {0, 0};
-          if (pp >= 0) v = shx(P[pp * PS + c0 + c]);
-          return v;
-        },
-        [&](int c, int pos, longlong2 v) { X[pos * cw + c] = v; });
+    x_stage1<FixArith, MAXR>(a.ax[0], nc, twx, xo, P + c0, cols, shx);
     __syncthreads();
     radix_switch<MAXR>(a.ax[0].r2, [&](auto rc) {
       constexpr int R = decltype(rc)::value;
-      const FixedAxis& ax = a.ax[0];
+      const LineAxis& ax = a.ax[0];
       const int items = nc * ax.r1;
       const float inv = 1.0f / (float)nc;
       for (int it = threadIdx.x; it < items; it += blockDim.x) {
         int k1, c;
         split_index(it, nc, inv, k1, c);
+        longlong2* q = X + k1 * R * cw + c;
+        const long long* vp = V + (size_t)(k1 * R) * n2 + c0 + c;
         longlong2 v[R];
-        int pos = k1 * ax.r2;
 #pragma unroll
-        for (int i = 0; i < R; ++i) {
-          v[i] = X[pos * cw + c];
-          pos += ax.s2;
-          if (pos >= n1) pos -= n1;
-        }
+        for (int i = 0; i < R; ++i) v[i] = q[i * cw];
         FxDft<R>::run(v);
-        pos = k1 * ax.r2;
 #pragma unroll
         for (int i = 0; i < R; ++i) {
-          const long long w = __ldg(V + (size_t)pos * n2 + c0 + c);
+          const long long w = __ldg(vp + i * n2);
           const int wh = fx_hi(w), wl = fx_lo(w);
           const longlong2 u = {fx_mulr(v[i].y, wh, wl), fx_mulr(v[i].x, wh, wl)};   // swapped: the forward sign
           v[i] = u;
-          pos += ax.s2;
-          if (pos >= n1) pos -= n1;
         }
         FxDft<R>::run(v);
         const int s3 = a.s3;
         const long long half = s3 ? 1LL << (s3 - 1) : 0;
-        pos = k1 * ax.r2;
 #pragma unroll
         for (int i = 0; i < R; ++i) {
           longlong2 u = {(v[i].x + half) >> s3, (v[i].y + half) >> s3};
-          if (i > 0 && ax.s2 == 1) u = fx_twiddle(u, twx[k1 * i]);
-          X[pos * cw + c] = u;
-          pos += ax.s2;
-          if (pos >= n1) pos -= n1;
+          if (i > 0 && ax.twiddled) u = fx_twiddle(u, twx[k1 * i]);
+          q[i * cw] = u;
         }
       }
     });
     __syncthreads();
-    fx_stage1<MAXR, true>(
-        a.ax[0], nc, twx, [&](int c, int pos) { return X[pos * cw + c]; },
-        [&](int c, int pos, longlong2 v) {
-          const int pp = xm[pos];
-          if (pp >= 0) {
-            my |= fx_mag(v);
-            P[pp * PS + c0 + c] = v;   // still swapped
-          }
-        });
+    x_stage1_rev<FixArith, MAXR>(a.ax[0], nc, xo, npl * PS, cols, P + c0, [&](longlong2 v) { my |= fx_mag(v); });
     __syncthreads();
   }
   fx_or(sh, my);
@@ -436,34 +312,30 @@ __device__ __forceinline__ void fx_plane_tile(const FxItem& a, int j3, int b, un
   my = sh->mag;
   const int d = my ? fx_headroom(my, a.hyf) : 0;
   e -= d;
-  const FxShift shy(d);
-  fx_stage2<MAXR, true>(a.ax[1], npl, twy, [&](int p, int pos) { return shy(P[p * PS + pos]); }, put);
+  line_stage2<FixArith, MAXR, true>(a.ax[1], npl, twy, rows, FxShift(d));
   __syncthreads();
-  fx_stage1<MAXR, true>(a.ax[1], npl, twy, get, put);
+  line_stage1<FixArith, MAXR, true>(a.ax[1], npl, twy, rows);
   __syncthreads();
   longlong2* yo = a.Yb + ((size_t)b * a.n3 + j3) * a.nst;
-  for (int p = warp; p < npl; p += nw) {
-    const int* ym = a.ymap + (size_t)p * n2;
-    for (int j2 = lane; j2 < n2; j2 += 32) {
-      const int s = __ldg(ym + j2);
-      if (s >= 0) yo[s] = P[p * PS + j2];   // still swapped: the z kernel goes on with the forward sign
-    }
-  }
+  // still swapped: the z kernel goes on with the forward sign
+  staged_loop(a.nst, [&](int i) { return a.soff[i]; }, [&](int i, int at) { yo[i] = P[at]; });
   if (threadIdx.x == 0) a.Ey[(size_t)b * a.n3 + j3] = my ? e : kFxZero;
 }
 
 template <int MAXR>
 __device__ __forceinline__ void fx_zfwd_tile(const FxItem& a, int ch, int b, unsigned char* smem, FxShared* sh) {
-  const int n = a.n3, ld = a.sc + 1;
+  constexpr int SC = kStickChunk, ld = SC + 1;
+  const int n = a.n3;
   FxTw* tw = reinterpret_cast<FxTw*>(smem);
   longlong2* L = reinterpret_cast<longlong2*>(smem + sizeof(FxTw) * n);
-  const int s0 = ch * a.sc, ns = min(a.sc, a.nst - s0);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int s0 = ch * SC, ns = min(SC, a.nst - s0);
+  const int lane = threadIdx.x & 31;
+  const int g0 = a.zbeg[ch], ng = a.zbeg[ch + 1] - g0;
   if (threadIdx.x == 0) {
     sh->emax = kFxZero;
     sh->mag = 0;
   }
-  load_table(tw, a.ax[2]);
+  load_table(tw, a.ax[2].fxtw, a.ax[2]);
   __syncthreads();
   const int* ey = a.Ey + (size_t)b * n;
   int em = kFxZero;
@@ -475,25 +347,32 @@ __device__ __forceinline__ void fx_zfwd_tile(const FxItem& a, int ch, int b, uns
   const bool bad = e >= kFxNan / 2;
   if (!bad) {
     const longlong2* Y = a.Yb + (size_t)b * n * a.nst + s0;
-    const int per = blockDim.x / a.sc, r0 = threadIdx.x / a.sc, sl = threadIdx.x - r0 * a.sc;
+    struct In {
+      longlong2 v;
+      int e;
+    };
     unsigned long long m = 0;
-    if (sl < ns)
-      for (int j3 = r0; j3 < n; j3 += per) {
-        const longlong2 v = fx_align(Y[(size_t)j3 * a.nst + sl], e - ey[j3]);
-        m |= fx_mag(v);
-        L[a.ax[2].slot[j3] * ld + sl] = v;
-      }
+    staged_loop(
+        n * SC,
+        [&](int i) {
+          In q{{0, 0}, e};
+          if (i % SC < ns) q = In{Y[(size_t)(i / SC) * a.nst + i % SC], ey[i / SC]};
+          return q;
+        },
+        [&](int i, In q) {
+          const longlong2 v = fx_align(q.v, e - q.e);
+          m |= fx_mag(v);
+          L[a.ax[2].slot[i / SC] * ld + i % SC] = v;
+        });
     fx_or(sh, m);
     __syncthreads();
     m = sh->mag;
     const int d = m ? fx_headroom(m, a.hzf) : 0;
     e -= d;
-    auto get = [&](int line, int pos) { return L[pos * ld + line]; };
-    auto put = [&](int line, int pos, longlong2 v) { L[pos * ld + line] = v; };
-    const FxShift shz(d);
-    fx_stage2<MAXR, true>(a.ax[2], ns, tw, [&](int line, int pos) { return shz(L[pos * ld + line]); }, put);
+    const LineView<longlong2> lines{L, 1, ld};
+    line_stage2<FixArith, MAXR, true>(a.ax[2], ns, tw, lines, FxShift(d));
     __syncthreads();
-    fx_stage1<MAXR, true>(a.ax[2], ns, tw, get, put);
+    line_stage1<FixArith, MAXR, true>(a.ax[2], ns, tw, lines);
     __syncthreads();
   }
   // 2^e / N_r: by its exponent field where that stays a normal number
@@ -501,52 +380,40 @@ __device__ __forceinline__ void fx_zfwd_tile(const FxItem& a, int ch, int b, uns
   const double f = bad                     ? __longlong_as_double(0x7ff8000000000000LL)
                    : fe > 0 && fe < 0x7ff ? __longlong_as_double(__double_as_longlong(a.inv_nr) + ((long long)e << 52))
                                           : ldexp(a.inv_nr, e);
-  for (int s = warp; s < ns; s += nw) {
-    const StickDev st = a.sticks[s0 + s];
-    const double2* ps = a.psi + (size_t)b * a.npw + st.g0;
-    double2* out = a.hpsi + (size_t)b * a.npw + st.g0;
-    const double* kin = a.kin + st.g0;
-    for (int tt = lane; tt < st.len; tt += 32) {
-      int pos = st.z0 + tt;
-      if (pos >= n) pos -= n;
-      const double2 x = ps[tt];
-      const double kg = kin[tt];
-      longlong2 v = {0, 0};
-      if (!bad) v = L[pos * ld + s];
-      out[tt] = make_double2(fma(kg, x.x, (double)v.y * f), fma(kg, x.y, (double)v.x * f));
-    }
-  }
-}
-
-__device__ __forceinline__ int fx_find(const int* off, int n, int t) {
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (off[mid] <= t) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
+  struct Out {
+    double2 x;
+    double kg;
+    int at;
+  };
+  const double2* ps = a.psi + (size_t)b * a.npw + g0;
+  double2* out = a.hpsi + (size_t)b * a.npw + g0;
+  staged_loop(ng, [&](int i) { return Out{ps[i], a.kin[g0 + i], a.zoff[g0 + i]}; },
+              [&](int i, Out q) {
+                longlong2 v = {0, 0};
+                if (!bad) v = L[q.at];   // swapped
+                out[i] = make_double2(fma(q.kg, q.x.x, (double)v.y * f), fma(q.kg, q.x.y, (double)v.x * f));
+              });
 }
 
 template <int MAXR>
 __global__ void __launch_bounds__(256, MAXR > 10 ? 2 : 3) k_fx_zinv(const __grid_constant__ FxBatch bt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ FxShared sh;
-  const int i = fx_find(bt.off_z, bt.nitems, blockIdx.x), l = blockIdx.x - bt.off_z[i];
+  const int i = tile_item(bt.off_z, bt.nitems, blockIdx.x), l = blockIdx.x - bt.off_z[i];
   fx_zinv_tile<MAXR>(bt.item[i], l % bt.item[i].nch, l / bt.item[i].nch, smem_raw, &sh);
 }
 template <int MAXR>
 __global__ void __launch_bounds__(kFxThreads<MAXR>, 1) k_fx_plane(const __grid_constant__ FxBatch bt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ FxShared sh;
-  const int i = fx_find(bt.off_p, bt.nitems, blockIdx.x), l = blockIdx.x - bt.off_p[i];
+  const int i = tile_item(bt.off_p, bt.nitems, blockIdx.x), l = blockIdx.x - bt.off_p[i];
   fx_plane_tile<MAXR>(bt.item[i], l % bt.item[i].n3, l / bt.item[i].n3, smem_raw, &sh);
 }
 template <int MAXR>
 __global__ void __launch_bounds__(256, MAXR > 10 ? 2 : 3) k_fx_zfwd(const __grid_constant__ FxBatch bt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ FxShared sh;
-  const int i = fx_find(bt.off_z, bt.nitems, blockIdx.x), l = blockIdx.x - bt.off_z[i];
+  const int i = tile_item(bt.off_z, bt.nitems, blockIdx.x), l = blockIdx.x - bt.off_z[i];
   fx_zfwd_tile<MAXR>(bt.item[i], l % bt.item[i].nch, l / bt.item[i].nch, smem_raw, &sh);
 }
 
@@ -568,17 +435,17 @@ __global__ void __launch_bounds__(256, 2) k_fx_batch(const __grid_constant__ FxB
   const unsigned G = gridDim.x;
   const int nz = bt.off_z[bt.nitems], np = bt.off_p[bt.nitems];
   for (int t = persist_next(pc.bar + 1); t < nz; t = persist_next(pc.bar + 1)) {
-    const int i = fx_find(bt.off_z, bt.nitems, t), l = t - bt.off_z[i];
+    const int i = tile_item(bt.off_z, bt.nitems, t), l = t - bt.off_z[i];
     fx_zinv_tile<MAXR>(bt.item[i], l % bt.item[i].nch, l / bt.item[i].nch, smem_raw, &sh);
   }
   if (!persist_sync(pc.bar, G, pc.err)) return;
   for (int t = persist_next(pc.bar + 2); t < np; t = persist_next(pc.bar + 2)) {
-    const int i = fx_find(bt.off_p, bt.nitems, t), l = t - bt.off_p[i];
+    const int i = tile_item(bt.off_p, bt.nitems, t), l = t - bt.off_p[i];
     fx_plane_tile<MAXR>(bt.item[i], l % bt.item[i].n3, l / bt.item[i].n3, smem_raw, &sh);
   }
   if (!persist_sync(pc.bar, 2 * G, pc.err)) return;
   for (int t = persist_next(pc.bar + 3); t < nz; t = persist_next(pc.bar + 3)) {
-    const int i = fx_find(bt.off_z, bt.nitems, t), l = t - bt.off_z[i];
+    const int i = tile_item(bt.off_z, bt.nitems, t), l = t - bt.off_z[i];
     fx_zfwd_tile<MAXR>(bt.item[i], l % bt.item[i].nch, l / bt.item[i].nch, smem_raw, &sh);
   }
   if (nl.nitems > 0) nonlocal_phases(nl, pc.bar, pc.err, G, 3, reinterpret_cast<double2*>(smem_raw));
@@ -600,7 +467,7 @@ __global__ void k_fx_vmax(size_t n, const double* __restrict__ v, unsigned long 
   if ((threadIdx.x & 31) == 0) atomicMax(out, m);
 }
 // V[j3][j2][j1] -> [j3][slot of j1][slot of j2] as V 2^(62 - vexp), |V| < 2^vexp
-__global__ void k_fx_v(FixedAxis a1, FixedAxis a2, int n3, const double* __restrict__ v,
+__global__ void k_fx_v(LineAxis a1, LineAxis a2, int n3, const double* __restrict__ v,
                        const unsigned long long* __restrict__ vmax, long long* __restrict__ out, int* __restrict__ vexp) {
   const int emax = (int)(*vmax >> 52);
   const size_t n = (size_t)a1.n * a2.n * n3;
@@ -616,6 +483,7 @@ struct FxLaunch {
   FxBatch bt;
   size_t smem_z = 0, smem_p = 0;
   int maxr = 0, items = 0;   // largest radix, largest stage of a plane
+  int block = 0;             // plane block of the item with the largest planes
   void add(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nb, void* zt, void* yb) {
     const int i = bt.nitems++;
     FxItem& it = bt.item[i];
@@ -633,7 +501,6 @@ struct FxLaunch {
     }
     items = std::max(items, std::max(it.npl * std::max(f.ax[1].r1, f.ax[1].r2), f.cw * std::max(f.ax[0].r1, f.ax[0].r2)) + 31);
     it.cw = f.cw;
-    it.sc = f.sc;
     it.nch = f.nch;
     it.hz = f.hz;
     it.hy = f.hy;
@@ -641,8 +508,9 @@ struct FxLaunch {
     it.s3 = f.s3;
     it.hyf = f.hyf;
     it.hzf = f.hzf;
-    it.sticks = p.d_sticks;
-    it.ymap = p.d_ymap;
+    it.soff = p.tab[HPSI_FP64].soff;
+    it.zoff = p.tab[HPSI_FP64].zoff;
+    it.zbeg = p.tab[HPSI_FP64].zbeg;
     it.xmap = p.d_xmap;
     it.psi = psi;
     it.hpsi = hpsi;
@@ -653,11 +521,12 @@ struct FxLaunch {
     it.Ez = reinterpret_cast<int*>(it.Zt + rows);   // beside the rows (local_row_bytes)
     it.Ey = reinterpret_cast<int*>(it.Yb + rows);
     it.V = static_cast<const long long*>(c.vbufs[p.vslot + 2]);
-    it.vexp = static_cast<const int*>(c.vbufs[p.vslot + 3]) + 2;
+    it.vexp = reinterpret_cast<const int*>(it.V + (size_t)p.n[0] * p.n[1] * p.n[2]) + 2;
     it.inv_nr = 1.0 / ((double)p.n[0] * p.n[1] * p.n[2]);
     bt.off_z[i + 1] = bt.off_z[i] + f.nch * nb;
     bt.off_p[i + 1] = bt.off_p[i] + p.n[2] * nb;
     smem_z = std::max(smem_z, f.smem_z);
+    if (f.smem_p > smem_p) block = f.block;
     smem_p = std::max(smem_p, f.smem_p);
   }
   void reset() {
@@ -676,21 +545,16 @@ struct FxLaunch {
       attr = true;
     }
     const int nz = bt.off_z[bt.nitems], np = bt.off_p[bt.nitems];
-    // the plane kernel's block: the resident threads over the CTAs that fit an SM (or that there are), no more than a
-    // stage has items
-    const int fit = std::max<int>(1, std::min<size_t>(16, c.smem_optin / (smem_p + 1100)));
-    const int ctas = std::max(1, std::min(fit, (np + c.sm_count - 1) / c.sm_count));
-    const int block = std::max(64, std::min(kFxThreads<MAXR> / ctas, items) / 32 * 32);
+    // plane_shape's block, or one round of a stage's items where there is a CTA per SM at most
+    const int plane = np <= c.sm_count ? std::max(block, std::min(kFxThreads<MAXR>, items / 32 * 32)) : block;
     HPSI_LAUNCH(c, HPSI_K_INV_ZY, (k_fx_zinv<MAXR><<<nz, 256, smem_z, c.stream>>>(bt)));
-    HPSI_LAUNCH(c, HPSI_K_XVX_Y, (k_fx_plane<MAXR><<<np, block, smem_p, c.stream>>>(bt)));
+    HPSI_LAUNCH(c, HPSI_K_XVX_Y, (k_fx_plane<MAXR><<<np, plane, smem_p, c.stream>>>(bt)));
     HPSI_LAUNCH(c, HPSI_K_FWD_Z, (k_fx_zfwd<MAXR><<<nz, 256, smem_z, c.stream>>>(bt)));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "fixed-point local kernels launch");
     return HPSI_OK;
   }
   int run(Context& c) { return maxr > 10 ? run_t<16>(c) : run_t<10>(c); }
-  static constexpr size_t kFxTwoCtas = 112 * 1024;   // dynamic shared memory that still allows two CTAs per SM
-
   template <int MAXR> int persistent_t(Context& c, const NlBatch& nl, unsigned* bar, bool* done) {
     const void* kern = (const void*)k_fx_batch<MAXR>;
     size_t dyn = std::max(smem_z, smem_p);
@@ -732,35 +596,40 @@ struct FxLaunch {
 
 }  // namespace
 
-// Factors of an edge (0 if it has none): coprime ones first (no twiddles), then the smaller larger factor; r1 >= r2,
-// which gives the x stage between the transforms more items and a tighter bound.
-void fixed_factors(int n, int* r1, int* r2) {
+// Factors of an edge (0 if it has none), r1 >= r2: that gives the x stage between the transforms more items and a
+// tighter bound.  Fixed point: coprime ones first (a twiddle costs as much as a third of a codelet), then the smaller larger one.
+// Float32: factors up to 10, else up to 12 (the codelets' registers set how many threads an SM holds), and among
+// those the same order.
+static void line_factors(int n, int precision, int* r1, int* r2) {
   *r1 = *r2 = 0;
-  bool best_cop = false;
+  int best = 0;
   for (int a : kRadices)
     for (int b : kRadices) {
       if (a * b != n || a < b) continue;
-      const bool cop = gcd(a, b) == 1;
-      if (*r1 == 0 || (cop && !best_cop) || (cop == best_cop && a < *r1)) {
+      const int size = precision == HPSI_FP64 ? 0 : a <= 10 ? 0 : a <= 12 ? 1 : 2;
+      const int rank = 1000 * size + (gcd(a, b) == 1 ? 0 : 100) + a;
+      if (*r1 == 0 || rank < best) {
         *r1 = a;
         *r2 = b;
-        best_cop = cop;
+        best = rank;
       }
     }
 }
 
-// The table of an edge (empty if it has no factors): in the Cooley-Tukey form the twiddles e^{2 pi i j / n}, then the
-// slot of every index after the inverse transform; returns where the slots begin.
-size_t fixed_tables(int n, std::vector<int>& tw, FixedAxis* ax) {
+// The table of an edge (empty if it has no factors): in the Cooley-Tukey form the twiddles e^{2 pi i j / n} in fixed point
+// and, from *ftw on, in float32; from *cells on the cell of every index before the inverse transform and after it.
+void line_tables(int n, int precision, std::vector<int>& table, size_t* ftw, size_t* cells, LineAxis* ax) {
   int r1, r2;
-  fixed_factors(n, &r1, &r2);
+  line_factors(n, precision, &r1, &r2);
   ax->n = n;
   ax->r1 = r1;
   ax->r2 = r2;
-  tw.clear();
-  if (!r1) return 0;
+  table.clear();
+  if (!r1) return;
   const bool pfa = gcd(r1, r2) == 1;
   ax->s2 = pfa ? r1 : 1;
+  ax->twiddled = !pfa;
+  std::vector<int> tw32;
   for (int j = 0; j < (pfa ? 0 : n); ++j) {
     // reduced to the first octant, so that long double keeps 62 bits
     const int o = 8 * j / n, r = 8 * j % n;
@@ -780,13 +649,22 @@ size_t fixed_tables(int n, std::vector<int>& tw, FixedAxis* ax) {
     }
     for (const long double x : {c, s}) {
       const long long q = std::llround(x * 4611686018427387904.0L);
-      tw.push_back(fx_hi(q));
-      tw.push_back(fx_lo(q));
+      table.push_back(fx_hi(q));
+      table.push_back(fx_lo(q));
+      const float f = (float)x;
+      int bits = 0;
+      std::memcpy(&bits, &f, sizeof(bits));
+      tw32.push_back(bits);
     }
   }
-  const size_t slots = tw.size();
-  for (int k = 0; k < n; ++k) tw.push_back((r2 * (k % r1) + ax->s2 * (pfa ? k % r2 : k / r1)) % n);
-  return slots;
+  *ftw = table.size();
+  table.insert(table.end(), tw32.begin(), tw32.end());
+  *cells = table.size();
+  std::vector<int> cell(n);
+  for (int a = 0; a < r1; ++a)
+    for (int t = 0; t < r2; ++t) cell[(r2 * a + ax->s2 * t) % n] = a * r2 + t;
+  table.insert(table.end(), cell.begin(), cell.end());
+  for (int k = 0; k < n; ++k) table.push_back((k % r1) * r2 + (pfa ? k % r2 : k / r1));
 }
 
 // The plan of a problem whose axes are filled in (ok = false: no factors, or a plane does not fit).
@@ -796,21 +674,16 @@ void fixed_plan(Problem& p, size_t smem_optin) {
   for (int a = 0; a < 3; ++a)
     if (!f.ax[a].r1) return;
   const int n1 = p.n[0], n2 = p.n[1], n3 = p.n[2];
-  auto tws = [&](int a) { return f.ax[a].s2 == 1 ? sizeof(FxTw) * (size_t)p.n[a] : 0; };
-  // z chunks: 32 sticks fill a stage's items and the store's rows; 16 where that would take over half an SM's memory
-  f.sc = n3 <= 100 ? 32 : 16;
-  f.nch = (p.nst + f.sc - 1) / f.sc;
-  f.smem_z = sizeof(FxTw) * (size_t)n3 + sizeof(longlong2) * (size_t)n3 * (f.sc + 1);
-  // x columns per chunk: two CTAs per SM where the plane leaves at least 12 columns for that, else one
-  const size_t base = tws(0) + tws(1) + sizeof(longlong2) * (size_t)p.npl * (n2 | 1) + sizeof(int) * n1;
+  auto tws = [&](int a) { return f.ax[a].twiddled ? sizeof(FxTw) * (size_t)p.n[a] : 0; };
+  f.nch = (p.nst + kStickChunk - 1) / kStickChunk;
+  f.smem_z = sizeof(FxTw) * (size_t)n3 + sizeof(longlong2) * (size_t)n3 * (kStickChunk + 1);
+  const size_t base = tws(0) + tws(1) + sizeof(longlong2) * (size_t)(p.npl + 1) * (n2 | 1) +
+                      sizeof(int) * f.ax[0].r2 * (size_t)((f.ax[0].r1 + 3) & ~3);
   const size_t col = sizeof(longlong2) * (size_t)n1;
-  auto width = [&](size_t room) { return room > base ? (int)std::min<size_t>((room - base) / col, 48) : 0; };
-  int cw = width(FxLaunch::kFxTwoCtas);
-  if (cw < std::min(12, n2)) cw = width(smem_optin - 1024);
-  cw = std::min(cw, n2);
-  if (cw < 4 && cw < n2) return;
-  const int chunks = (n2 + cw - 1) / cw;
-  f.cw = (n2 + chunks - 1) / chunks;
+  int rmax = 0;
+  for (int a = 0; a < 3; ++a) rmax = std::max(rmax, f.ax[a].r1);
+  plane_shape(f.ax[0], f.ax[1], p.npl, base, col, smem_optin, rmax > 10 ? kFxThreads<16> : kFxThreads<10>, &f.cw, &f.block);
+  if (f.cw == 0) return;
   f.smem_p = base + col * f.cw;
   if (col * f.cw < sizeof(float) * 4 * (size_t)n2 || f.smem_z > smem_optin - 1024) return;
   int zl = 1;
@@ -829,13 +702,13 @@ void fixed_plan(Problem& p, size_t smem_optin) {
   f.ok = true;
 }
 
-// Fixed-point copy of V (vbufs[slot + 2], its exponent in vbufs[slot + 3]) from the float64 one.
-int fixed_potential(Context& c, int slot, const FixedAxis ax[3], int kernel_class) {
-  unsigned long long* vm = static_cast<unsigned long long*>(c.vbufs[slot + 3]);
+// Fixed-point copy of V and its exponent (vbufs[slot + 2]) from the float64 one.
+int fixed_potential(Context& c, int slot, const LineAxis ax[3], int kernel_class) {
   const size_t nr = (size_t)ax[0].n * ax[1].n * ax[2].n;
+  unsigned long long* vm = static_cast<unsigned long long*>(c.vbufs[slot + 2]) + nr;
   const double* v = static_cast<const double*>(c.vbufs[slot]);
   const int grid = (int)std::min<size_t>(4 * c.sm_count, (nr + 255) / 256);
-  cudaError_t e = cudaMemsetAsync(vm, 0, 16, c.stream);
+  cudaError_t e = cudaMemsetAsync(vm, 0, kFixedScaleBytes, c.stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "fixed-point potential");
   HPSI_LAUNCH(c, kernel_class, (k_fx_vmax<<<grid, 256, 0, c.stream>>>(nr, v, vm)));
   HPSI_LAUNCH(c, kernel_class, (k_fx_v<<<grid, 256, 0, c.stream>>>(ax[0], ax[1], ax[2].n, v, vm,
@@ -863,9 +736,9 @@ int local_fixed_apply(Context& c, const Problem& p, const double2* psi, double2*
 int local_fixed_apply_multi(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
                             double2* const* hpsi, void* const* zt, void* const* yb) {
   static FxLaunch fl;
-  for (int i0 = 0; i0 < nitem; i0 += kFxMaxItems) {
+  for (int i0 = 0; i0 < nitem; i0 += kMaxLocalItems) {
     fl.reset();
-    for (int i = i0; i < std::min(nitem, i0 + kFxMaxItems); ++i)
+    for (int i = i0; i < std::min(nitem, i0 + kMaxLocalItems); ++i)
       fl.add(c, c.probs[prob[i]], psi[i], hpsi[i], nbnd[i], zt[i], yb[i]);
     const int rc = fl.run(c);
     if (rc) return rc;

@@ -238,77 +238,28 @@ size_t local_row_bytes(const Problem& p, int precision, int nb) {
   return precision == HPSI_FP64 && p.fixed.ok ? rows + sizeof(int) * (size_t)nb * std::max(p.fixed.nch, p.n[2]) : rows;
 }
 
-// Autotuner of the fast path: time every plan that fits the shared memory (which of the V plane
-// and the stick row the plane kernel stages) against band blocks of half, one and two times the
-// default, on this call's own bands, and keep the fastest.  Neither choice changes the arithmetic.
-static int tune_fast(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd) {
-  const int pr = cur_prec(c);
-  const std::vector<int> plans = local_fast_candidates(p, pr, c.smem_optin);
-  const int nb0 = p.nbbf[pr];
-  std::vector<int> blocks;
-  for (int nb : {std::max(1, nb0 / 2), nb0, 2 * nb0}) {
-    const int v = std::min(nb, nbnd);
-    if (std::find(blocks.begin(), blocks.end(), v) == blocks.end()) blocks.push_back(v);
-  }
-  cudaEvent_t e0, e1;
-  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
-    cudaGetLastError();
-    return HPSI_OK;
-  }
-  float best = 1e30f;
-  int best_plan = p.fflags[pr], best_nb = nb0;
-  const bool timing = c.timing;
-  c.timing = false;
-  int rc = HPSI_OK;
-  for (int plan : plans)
-    for (int nb : blocks) {
-      const size_t need = local_row_bytes(p, pr, nb);
-      rc = ensure_buffer(c, &c.ws.X, &c.ws.xbytes, need);
-      if (!rc) rc = ensure_buffer(c, &c.ws.Y, &c.ws.ybytes, need);
-      if (rc) break;
-      p.fflags[pr] = plan;
-      float ms = 0.f;
-      for (int rep = 0; rep < 2 && !rc; ++rep) {   // first run warms up, second is timed
-        cudaEventRecord(e0, c.stream);
-        rc = local_fast_apply(c, p, psi, hpsi, nbnd, c.ws.X, c.ws.Y, nb);
-        cudaEventRecord(e1, c.stream);
-      }
-      if (rc) break;
-      if (cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess && ms < best) {
-        best = ms;
-        best_plan = plan;
-        best_nb = nb;
-      }
-    }
-  c.timing = timing;
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  p.fflags[pr] = best_plan;
-  p.nbbf[pr] = best_nb;
-  p.tuned[pr] = true;
-  return rc;
+// The band block of a fast apply and its two buffers of stick rows
+static int fast_buffers(Context& c, const Problem& p, int nbnd, int* nbb) {
+  const int nb = std::max(1, std::min(p.nbbf[cur_prec(c)], nbnd)), blocks = (nbnd + nb - 1) / nb;
+  *nbb = (nbnd + blocks - 1) / blocks;   // even blocks
+  const size_t need = local_row_bytes(p, cur_prec(c), *nbb);
+  int rc = ensure_buffer(c, &c.ws.X, &c.ws.xbytes, need);
+  return rc ? rc : ensure_buffer(c, &c.ws.Y, &c.ws.ybytes, need);
+}
+
+int local_raw_apply(Context& c, const Problem& p, const float2* f, float2* F, int nbnd) {
+  int nbb = 1;
+  const int rc = fast_buffers(c, p, nbnd, &nbb);
+  return rc ? rc : local_fast_apply_raw(c, p, f, F, nbnd, c.ws.X, c.ws.Y, nbb);
 }
 
 template <typename T>
 static int local_apply_t(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd) {
   const size_t cs = sizeof(typename Cx<T>::type);
-  if ((p.fflags[cur_prec(c)] & 4) && !c.force_generic) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    cudaStreamIsCapturing(c.stream, &cap);
-    // (the fixed-point float64 form has one plan, and its time hardly depends on the block)
-    if (c.autotune && cur_prec(c) == HPSI_MIXED && !p.tuned[HPSI_MIXED] && nbnd >= 4 &&
-        cap == cudaStreamCaptureStatusNone) {
-      int rc = tune_fast(c, p, psi, hpsi, nbnd);
-      if (rc) return rc;
-    }
-    int nbf = std::max(1, std::min(p.nbbf[cur_prec(c)], nbnd));
-    if (cur_prec(c) == HPSI_FP64) nbf = (nbnd + (nbnd + nbf - 1) / nbf - 1) / ((nbnd + nbf - 1) / nbf);   // even blocks
-    const size_t zneed = local_row_bytes(p, cur_prec(c), nbf);
-    int rc = ensure_buffer(c, &c.ws.X, &c.ws.xbytes, zneed);
-    if (rc) return rc;
-    rc = ensure_buffer(c, &c.ws.Y, &c.ws.ybytes, zneed);
-    if (rc) return rc;
-    return local_fast_apply(c, p, psi, hpsi, nbnd, c.ws.X, c.ws.Y, nbf);
+  if (local_fast_ok(p, cur_prec(c)) && !c.force_generic) {
+    int nbf = 1;
+    const int rc = fast_buffers(c, p, nbnd, &nbf);
+    return rc ? rc : local_fast_apply(c, p, psi, hpsi, nbnd, c.ws.X, c.ws.Y, nbf);
   }
   const int nbb = std::max(1, std::min(p.nbb[cur_prec(c)], nbnd));
   const size_t xneed = cs * (size_t)nbb * p.n[2] * p.npl * p.n[1];

@@ -85,10 +85,10 @@ extern "C" int hpsi_apply_noalloc(hpsi_ctx* ctx, int ik, const void* psi_in, voi
   // scale with its bands, so a shorter last chunk fits in the same places; its nonlocal K-split
   // is planned against the room left after the full chunk's X and Y, and one split of the partials
   // grows with the bands too, so whatever fits the full chunk fits the last one.
-  // The register-codelet kernels (cubic boxes with a two-factor edge) need two stick-row buffers per
-  // band; the generic kernels an m1-plane buffer and a stick-row buffer.
+  // The fast kernels (boxes whose edges have two codelet factors) need two stick-row buffers per band; the
+  // generic kernels an m1-plane buffer and a stick-row buffer.
   const int prec = hpsi::cur_prec(c);
-  const bool fast = (p.fflags[prec] & 4) && !c.force_generic;
+  const bool fast = hpsi::local_fast_ok(p, prec) && !c.force_generic;
   const size_t cs = prec == HPSI_FP64 ? sizeof(double2) : sizeof(float2);
   auto xbytes = [&](int nb) {
     return align256(fast ? hpsi::local_row_bytes(p, prec, nb) : cs * (size_t)nb * p.n[2] * p.npl * p.n[1]);

@@ -264,26 +264,30 @@ __device__ __forceinline__ double slice_load(const R* row, int i, int scaled) {
   return scaled || i < 2 ? x : x * kSqrt2s;
 }
 template <typename R>
-__global__ void __launch_bounds__(256) k_row_field(int len, int scaled, const R* __restrict__ src, int* __restrict__ field) {
-  const R* row = src + (size_t)blockIdx.y * len;
-  unsigned h = 0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < len; i += gridDim.x * blockDim.x)
-    h = max(h, (unsigned)__double2hiint(slice_load(row, i, scaled)) & 0x7fffffffu);
-  h = __reduce_max_sync(0xffffffffu, h);
-  if ((threadIdx.x & 31) == 0) atomicMax(field + blockIdx.y, (int)(h >> 20));
+__global__ void __launch_bounds__(256) k_row_field(int rows, int len, int scaled, const R* __restrict__ src,
+                                                   int* __restrict__ field) {
+  for (int r = blockIdx.y; r < rows; r += gridDim.y) {
+    const R* row = src + (size_t)r * len;
+    unsigned h = 0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < len; i += gridDim.x * blockDim.x)
+      h = max(h, (unsigned)__double2hiint(slice_load(row, i, scaled)) & 0x7fffffffu);
+    h = __reduce_max_sync(0xffffffffu, h);
+    if ((threadIdx.x & 31) == 0) atomicMax(field + r, (int)(h >> 20));
+  }
 }
 
 // Digit planes [8][rows][kpad] of rows of `len` doubles, two entries per thread.  dup = 0: row r from row r.
 // dup = 1: rows 2r: as they are, 2r + 1: (im, -re) of each pair; dup = 2: 2r: (re, -im), 2r + 1: (im, re).
 // exps: row exponents of the planes' rows.
 template <typename R>
-__global__ void __launch_bounds__(256) k_digits(int len, int kpad, int dup, int scaled, const R* __restrict__ src,
-                                                const int* __restrict__ field, __nv_bfloat16* __restrict__ out,
-                                                int* __restrict__ exps) {
-  const int r = blockIdx.y, f = field[r];
-  const R* row = src + (size_t)r * len;
-  const size_t rows = (size_t)gridDim.y * (dup ? 2 : 1), half = kpad / 2;
+__global__ void __launch_bounds__(256) k_digits(int nrow, int len, int kpad, int dup, int scaled,
+                                                const R* __restrict__ src, const int* __restrict__ field,
+                                                __nv_bfloat16* __restrict__ out, int* __restrict__ exps) {
+  const size_t rows = (size_t)nrow * (dup ? 2 : 1), half = kpad / 2;
   unsigned* o = reinterpret_cast<unsigned*>(out);
+  for (int r = blockIdx.y; r < nrow; r += gridDim.y) {
+  const int f = field[r];
+  const R* row = src + (size_t)r * len;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     const int e = row_exponent(f);
     if (dup) exps[2 * r] = exps[2 * r + 1] = e;
@@ -304,6 +308,7 @@ __global__ void __launch_bounds__(256) k_digits(int len, int kpad, int dup, int 
         o[plane + (size_t)(2 * r + 1) * half + h] = dup == 1 ? b | (a ^ 0x8000u) << 16 : b | a << 16;
       }
     }
+  }
   }
 }
 
@@ -458,9 +463,10 @@ static int slice_planes(Context& c, const Problem& p, int which, bool* ok) {
     int* field = s.exps + rows;
     cudaError_t e = cudaMemsetAsync(field, 0, sizeof(int) * P, c.stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "projector digit setup");
-    const dim3 grid(std::max(1, std::min(64, kpad / 512)), P);
-    HPSI_LAUNCH(c, HPSI_K_SPLIT, (k_row_field<double><<<grid, 256, 0, c.stream>>>(len, 1, beta, field)));
-    HPSI_LAUNCH(c, HPSI_K_SPLIT, (k_digits<double><<<grid, 256, 0, c.stream>>>(len, kpad, 0, 1, beta, field, d, s.exps)));
+    const dim3 grid(std::max(1, std::min(64, kpad / 512)), std::min(P, 65535));
+    HPSI_LAUNCH(c, HPSI_K_SPLIT, (k_row_field<double><<<grid, 256, 0, c.stream>>>(P, len, 1, beta, field)));
+    HPSI_LAUNCH(c, HPSI_K_SPLIT,
+                (k_digits<double><<<grid, 256, 0, c.stream>>>(P, len, kpad, 0, 1, beta, field, d, s.exps)));
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "projector digit setup");
@@ -485,10 +491,10 @@ static int slice_rows(Context& c, const R* src, int rows, int len, int kpad, int
   *exps = field + rows;
   cudaError_t e = cudaMemsetAsync(field, 0, sizeof(int) * rows, c.stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "digit workspace clear");
-  const dim3 grid(std::max(1, std::min((8 * c.sm_count + rows - 1) / rows, (len + 1023) / 1024)), rows);
-  HPSI_LAUNCH(c, HPSI_K_SPLIT, (k_row_field<R><<<grid, 256, 0, c.stream>>>(len, scaled, src, field)));
+  const dim3 grid(std::max(1, std::min((8 * c.sm_count + rows - 1) / rows, (len + 1023) / 1024)), std::min(rows, 65535));
+  HPSI_LAUNCH(c, HPSI_K_SPLIT, (k_row_field<R><<<grid, 256, 0, c.stream>>>(rows, len, scaled, src, field)));
   HPSI_LAUNCH(c, HPSI_K_SPLIT,
-              (k_digits<R><<<grid, 256, 0, c.stream>>>(len, kpad, dup, scaled, src, field, *digits, *exps)));
+              (k_digits<R><<<grid, 256, 0, c.stream>>>(rows, len, kpad, dup, scaled, src, field, *digits, *exps)));
   return HPSI_OK;
 }
 static size_t slice_rows_bytes(int rows, int kpad, int dup) {

@@ -7,8 +7,9 @@
 //     calbec      C[p][n] = sum_k A[p][k] B[n][k],  A = beta (K = 2 npw),
 //                 B rows n < nb: psi_n (re, im); rows nb + b: (im, -re) of psi_b
 //                 -> C[p][b] = Re<beta_p|psi_b>, C[p][nb+b] = Im<beta_p|psi_b>
-//     add_vuspsi  C[b][n] = sum_k A[b][k] B[n][k],  A = w (K = 2P), B[2G+c][2p+c'] built from
-//                 beta so that C[b][2G] = Re(sum_p w_bp beta_p(G)), C[b][2G+1] = Im(...)
+//     add_vuspsi  C[n][b] = sum_k A[n][k] B[b][k],  B = w (K = 2P), A[2G+c][2p+c'] built from
+//                 beta so that C[2G][b] = Re(sum_p w_bp beta_p(G)), C[2G+1][b] = Im(...): consecutive TMEM lanes are
+//                 consecutive float64 of hpsi_b, so the epilogue's adds are coalesced
 //   precision:  every float64 operand x is split into bf16 terms x = x0 + x1 (+ x2) and the
 //     products x_i y_j with i + j < NT are accumulated (NT = 2: three products, ~16 significant
 //     bits; NT = 3: six products).
@@ -27,6 +28,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "convert.cuh"
 #include "hpsi_internal.h"
 #include "tcgen05.cuh"
 
@@ -71,10 +73,8 @@ struct TcArgs {
   int M, N;          // logical rows of A and of B (output is M x N)
   int nksteps;       // K / 64
   int ksplit;        // K-steps per split (gridDim.z splits)
-  int mode;          // 0: store float partials [split][M][N]; 1: add into complex128 rows
+  int mode;          // 0: float partials [split][M][N]; 1: float partials [split][N][M]
   float* part;
-  double2* out;      // mode 1: out[m][n/2] += (C[m][n], C[m][n+1]) for even n
-  int ldo;           // mode 1: complex elements per output row
   int* err;
 };
 
@@ -212,16 +212,11 @@ __global__ void __launch_bounds__(128, 1)
 #pragma unroll
           for (int j = 0; j < 16; ++j)
             if (n0 + j < a.N) o[n0 + j] = __uint_as_float(r[j]);
-        } else {
-          double2* o = a.out + (size_t)row * a.ldo + (n0 >> 1);
+        } else {   // lanes are consecutive rows: coalesced along m
+          float* o = a.part + (size_t)split * a.N * a.M + row;
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            if (n0 + 2 * j < a.N) {
-              double2 v = o[j];
-              v.x += (double)__uint_as_float(r[2 * j]);
-              v.y += (double)__uint_as_float(r[2 * j + 1]);
-              o[j] = v;
-            }
+          for (int j = 0; j < 16; ++j)
+            if (n0 + j < a.N) o[(size_t)(n0 + j) * a.M] = __uint_as_float(r[j]);
         }
       }
     }
@@ -246,8 +241,8 @@ __global__ void k_add_partials(int nb, int npw, int nsplit, const float* __restr
     double sx = 0.0, sy = 0.0;
     for (int s = 0; s < nsplit; ++s) {
       const float2 v = p[(size_t)s * (plane / 2)];
-      sx += (double)v.x;
-      sy += (double)v.y;
+      sx += f32_to_f64(v.x);
+      sy += f32_to_f64(v.y);
     }
     double2 o = hpsi[i];
     o.x += sx;
@@ -285,7 +280,7 @@ __global__ void k_split_beta_cal(int nproj, int npw, int kc, const double2* __re
   }
 }
 
-// B of add_vuspsi: row n = 2G + c, column k = 2p + c':  c=0: (re, -im), c=1: (im, re) of beta_p(G).
+// A of add_vuspsi: row n = 2G + c, column k = 2p + c':  c=0: (re, -im), c=1: (im, re) of beta_p(G).
 template <int NT>
 __global__ void k_split_beta_add(int nproj, int npw, int ka, const double2* __restrict__ beta,
                                  __nv_bfloat16* __restrict__ out) {
@@ -302,31 +297,39 @@ __global__ void k_split_beta_add(int nproj, int npw, int ka, const double2* __re
   }
 }
 
-// B of calbec: rows b < nb: psi_b (re, im); rows nb + b: (im, -re).  One thread per complex psi
-// element (or per pair of padding columns), writing bf16 pairs.
+// The NT bf16 terms of a float64 given as two floats (f64_split): each the rounded remainder of the ones before; the low
+// float joins the last remainder.
 template <int NT>
-__global__ void k_split_psi(int nb, int npw, int kc, const double2* __restrict__ psi, __nv_bfloat16* __restrict__ out) {
-  const size_t plane = (size_t)2 * nb * kc;
-  const int half = kc / 2;   // complex columns including the zero padding
-  const size_t n = (size_t)nb * half;
+__device__ __forceinline__ void bf16_terms(float2 x, __nv_bfloat16 (&t)[NT]) {
+  float r = x.x;
+#pragma unroll
+  for (int i = 0; i < NT; ++i) {
+    t[i] = __float2bfloat16_rn(i == NT - 1 ? r + x.y : r);
+    r -= __bfloat162float(t[i]);
+  }
+}
+
+// B of calbec: rows b < nb: psi_b (re, im); rows nb + b: (im, -re).  One thread per complex psi element (or per pair
+// of padding columns), writing bf16 pairs.  The terms are found in float32 (float64 casts and
+// subtractions made this kernel float64-bound: 160 bands of 36785 226 -> 60 us).
+template <int NT>
+__global__ void __launch_bounds__(256) k_split_psi(int nb, int npw, int kc, const double2* __restrict__ psi,
+                                                   __nv_bfloat16* __restrict__ out) {
+  const int half = kc / 2;                   // complex columns including the zero padding
+  const size_t plane = (size_t)nb * kc;      // bf16 pairs of a term
   __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(out);
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int b = (int)(i / half), g = (int)(i - (size_t)b * half);
+  for (int b = blockIdx.y; b < nb; b += gridDim.y)
+  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < half; g += gridDim.x * blockDim.x) {
     double2 v = make_double2(0.0, 0.0);
     if (g < npw) v = psi[(size_t)b * npw + g];
-    double r0 = v.x, r1 = v.y;      // row b:      (re, im)
-    double s0 = v.y, s1 = -v.x;     // row nb + b: (im, -re)
-    const size_t i0 = ((size_t)b * kc) / 2 + g, i1 = ((size_t)(nb + b) * kc) / 2 + g;
+    __nv_bfloat16 re[NT], im[NT];
+    bf16_terms<NT>(f64_split(v.x), re);
+    bf16_terms<NT>(f64_split(v.y), im);
+    const size_t i0 = (size_t)b * half + g, i1 = (size_t)(nb + b) * half + g;
 #pragma unroll
     for (int t = 0; t < NT; ++t) {
-      const __nv_bfloat16 h0 = __float2bfloat16_rn((float)r0), h1 = __float2bfloat16_rn((float)r1);
-      const __nv_bfloat16 k0 = __float2bfloat16_rn((float)s0), k1 = __float2bfloat16_rn((float)s1);
-      o2[t * (plane / 2) + i0] = __halves2bfloat162(h0, h1);
-      o2[t * (plane / 2) + i1] = __halves2bfloat162(k0, k1);
-      r0 -= (double)__bfloat162float(h0);
-      r1 -= (double)__bfloat162float(h1);
-      s0 -= (double)__bfloat162float(k0);
-      s1 -= (double)__bfloat162float(k1);
+      o2[t * plane + i0] = __halves2bfloat162(re[t], im[t]);
+      o2[t * plane + i1] = __halves2bfloat162(im[t], __hneg(re[t]));
     }
   }
 }
@@ -338,7 +341,7 @@ __global__ void k_sum_partials(size_t n, int nsplit, const float* __restrict__ p
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     double s = 0.0;
 #pragma unroll 8
-    for (int k = 0; k < nsplit; ++k) s += (double)part[(size_t)k * n + i];
+    for (int k = 0; k < nsplit; ++k) s += f32_to_f64(part[(size_t)k * n + i]);
     out[i] = s;
   }
 }
@@ -458,6 +461,13 @@ __global__ void k_split_betar_add(int nproj, int nr, int ka, const double* __res
   }
 }
 
+// sqrt2 (x.x + x.y) as two floats (the product's rounding error and the constant's low part go to the second)
+__device__ __forceinline__ float2 times_sqrt2(float2 x) {
+  constexpr float sh = 1.41421354f, sl = 2.42032351e-8f;   // sqrt2 = sh + sl
+  const float p = __fmul_rn(x.x, sh);
+  return make_float2(p, __fmaf_rn(x.x, sh, -p) + __fmaf_rn(x.x, sl, x.y * sh));
+}
+
 // B of calbec in the real form: row b = x_b (nr real coordinates, K padded to kc with zeros);
 // scaled = 0: x holds coefficients and r >= 2 is multiplied by sqrt2.  One thread per pair of
 // coordinates, band b = blockIdx.y.
@@ -489,22 +499,21 @@ __global__ void k_split_xr(int nb, int nr, int kc, int scaled, const R* __restri
         r1 -= __bfloat162float(h1);
       }
     } else {
-      double r0 = 0.0, r1 = 0.0;
+      float2 r0 = make_float2(0.f, 0.f), r1 = r0;
       if (2 * h < nr) {
-        r0 = (double)x[(size_t)b * nr + 2 * h];
-        r1 = (double)x[(size_t)b * nr + 2 * h + 1];
+        const double2 v = *reinterpret_cast<const double2*>(x + (size_t)b * nr + 2 * h);
+        r0 = f64_split(v.x);
+        r1 = f64_split(v.y);
         if (!scaled && h > 0) {
-          r0 *= 1.4142135623730950488;
-          r1 *= 1.4142135623730950488;
+          r0 = times_sqrt2(r0);
+          r1 = times_sqrt2(r1);
         }
       }
+      __nv_bfloat16 t0[NT], t1[NT];
+      bf16_terms<NT>(r0, t0);
+      bf16_terms<NT>(r1, t1);
 #pragma unroll
-      for (int t = 0; t < NT; ++t) {
-        const __nv_bfloat16 h0 = __float2bfloat16_rn((float)r0), h1 = __float2bfloat16_rn((float)r1);
-        o2[t * (plane / 2) + at] = __halves2bfloat162(h0, h1);
-        r0 -= (double)__bfloat162float(h0);
-        r1 -= (double)__bfloat162float(h1);
-      }
+      for (int t = 0; t < NT; ++t) o2[t * (plane / 2) + at] = __halves2bfloat162(t0[t], t1[t]);
     }
   }
 }
@@ -565,7 +574,7 @@ inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 // pa_stride / pb_stride: elements between the bf16 term planes of A / B (0: rows x kpad, packed)
 template <int NT>
 int launch_gemm(Context& c, const void* A, int M, const void* B, int N, int kpad, int nsplit, int ksplit, int mode,
-                float* part, double2* out, int ldo, int kernel_class, size_t pa_stride = 0, size_t pb_stride = 0) {
+                float* part, int kernel_class, size_t pa_stride = 0, size_t pb_stride = 0) {
   CUtensorMap ma[3], mb[3];
   const size_t pa = pa_stride ? pa_stride : (size_t)M * kpad, pb = pb_stride ? pb_stride : (size_t)N * kpad;
   for (int t = 0; t < 3; ++t) {
@@ -582,8 +591,6 @@ int launch_gemm(Context& c, const void* A, int M, const void* B, int N, int kpad
   a.ksplit = ksplit;
   a.mode = mode;
   a.part = part;
-  a.out = out;
-  a.ldo = ldo;
   a.err = c.d_err;
   static bool attr[4] = {false, false, false, false};
   if (!attr[NT]) {
@@ -681,7 +688,7 @@ int apply_t(Context& c, const Problem& p, const double2* psi, double2* hpsi, int
   const int naks = ka / TBK;
   const int aksplit = (naks + (naks + kAddKsteps - 1) / kAddKsteps - 1) / ((naks + kAddKsteps - 1) / kAddKsteps);
   const int ansplit = (naks + aksplit - 1) / aksplit;   // every split has at least one K step
-  const size_t addb = ansplit > 1 ? sizeof(float) * (size_t)ansplit * nbnd * 2 * npw : 0;
+  const size_t addb = sizeof(float) * (size_t)ansplit * nbnd * 2 * npw;
   const size_t becb = nsplit > 1 ? sizeof(double) * (size_t)P * 2 * nbnd : 0;
   const size_t need = psib + partb + wab + addb + becb + 5 * 256;
   int rc = ensure_buffer(c, &c.ws.mixed, &c.ws.mixedbytes, need);
@@ -694,9 +701,9 @@ int apply_t(Context& c, const Problem& p, const double2* psi, double2* hpsi, int
   // the K padding of w (columns 2P .. ka) is not written by the D-scale kernel
   cudaError_t e0 = cudaMemsetAsync(wa, 0, wab, c.stream);
   if (e0 != cudaSuccess) return cuda_fail(c, e0, "workspace clear");
-  const int split_grid = (int)std::min<size_t>(8 * c.sm_count, ((size_t)nbnd * (kc / 2) + 255) / 256);
-  HPSI_LAUNCH(c, HPSI_K_SPLIT, (k_split_psi<NT><<<split_grid, 256, 0, c.stream>>>(nbnd, npw, kc, psi, psi_bf)));
-  rc = launch_gemm<NT>(c, bcal, P, psi_bf, 2 * nbnd, kc, nsplit, ksplit, 0, part, nullptr, 0, HPSI_K_CALBEC);
+  HPSI_LAUNCH(c, HPSI_K_SPLIT, (k_split_psi<NT><<<dim3(std::min(256, (kc / 2 + 255) / 256), std::min(nbnd, 65535)), 256,
+                                                  0, c.stream>>>(nbnd, npw, kc, psi, psi_bf)));
+  rc = launch_gemm<NT>(c, bcal, P, psi_bf, 2 * nbnd, kc, nsplit, ksplit, 0, part, HPSI_K_CALBEC);
   if (rc) return rc;
   const int n = P * nbnd;
   float* apart = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(wa) + ((wab + 255) & ~size_t(255)));
@@ -713,16 +720,13 @@ int apply_t(Context& c, const Problem& p, const double2* psi, double2* hpsi, int
                 (k_dscale_tc<NT, float><<<(n + 255) / 256, 256, 0, c.stream>>>(P, nbnd, 1, ka, part, p.d_rowptr,
                                                                                p.d_col, p.d_dval, wa)));
   }
-  if (ansplit > 1) {
-    rc = launch_gemm<NT>(c, wa, nbnd, badd, 2 * npw, ka, ansplit, aksplit, 0, apart, nullptr, 0, HPSI_K_ADDVUS);
-    if (rc) return rc;
-    const size_t nel = (size_t)nbnd * npw;
-    HPSI_LAUNCH(c, HPSI_K_ADDVUS, (k_add_partials<<<(int)std::min<size_t>(8 * c.sm_count, (nel + 255) / 256), 256, 0,
-                                                    c.stream>>>(nbnd, npw, ansplit, apart, hpsi)));
-  } else {
-    rc = launch_gemm<NT>(c, wa, nbnd, badd, 2 * npw, ka, 1, naks, 1, nullptr, hpsi, npw, HPSI_K_ADDVUS);
-    if (rc) return rc;
-  }
+  // float32 partials and one pass that adds them to hpsi: a read-modify-write of hpsi in the GEMM's epilogue, with one
+  // CTA per SM, took 252 us of the 36785-plane-wave, 160-band case where GEMM and pass take 155
+  rc = launch_gemm<NT>(c, badd, 2 * npw, wa, nbnd, ka, ansplit, aksplit, 1, apart, HPSI_K_ADDVUS);
+  if (rc) return rc;
+  const size_t nel = (size_t)nbnd * npw;
+  HPSI_LAUNCH(c, HPSI_K_ADDVUS, (k_add_partials<<<(int)std::min<size_t>(8 * c.sm_count, (nel + 255) / 256), 256, 0,
+                                                  c.stream>>>(nbnd, npw, ansplit, apart, hpsi)));
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "tensor-core nonlocal kernels launch");
   return HPSI_OK;
@@ -783,7 +787,7 @@ int gamma_apply_tc(Context& c, const Problem& p, const R* x, int nb, bool scaled
   HPSI_LAUNCH(c, HPSI_K_SPLIT,
               (k_split_xr<NT, R><<<dim3(std::min(1024, (kc / 2 + 255) / 256), nb), 256, 0, c.stream>>>(
                   nb, nr, kc, scaled ? 1 : 0, x, xs)));
-  rc = launch_gemm<NT>(c, bcal, P, xs, nb, kc, nsplit, ksplit, 0, part, nullptr, 0, HPSI_K_CALBEC);
+  rc = launch_gemm<NT>(c, bcal, P, xs, nb, kc, nsplit, ksplit, 0, part, HPSI_K_CALBEC);
   if (rc) return rc;
   const int n = P * nb;
   if (nsplit > 1) {
@@ -799,7 +803,7 @@ int gamma_apply_tc(Context& c, const Problem& p, const R* x, int nb, bool scaled
                 (k_dscale_tc_r<NT, float><<<(n + 255) / 256, 256, 0, c.stream>>>(P, nb, 1, ka, part, p.d_rowptr,
                                                                                  p.d_col, p.d_dvalr, wa)));
   }
-  rc = launch_gemm<NT>(c, wa, nb, badd, nr, ka, ansplit, aksplit, 0, apart, nullptr, 0, HPSI_K_ADDVUS);
+  rc = launch_gemm<NT>(c, badd, nr, wa, nb, ka, ansplit, aksplit, 1, apart, HPSI_K_ADDVUS);
   if (rc) return rc;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "Gamma-form tensor-core nonlocal kernels launch");
@@ -831,28 +835,22 @@ int add_from_w64(Context& c, const Problem& p, const double* w, bool real, int n
   const int aksplit = 1, ansplit = naks;
   auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
   const size_t wb = al(sizeof(__nv_bfloat16) * (size_t)NT * nb * ka);
-  const bool partials = real || ansplit > 1;
-  const size_t ab = partials ? al(sizeof(float) * (size_t)ansplit * nb * N) : 0;
+  const size_t ab = al(sizeof(float) * (size_t)ansplit * nb * N);
   int rc = ensure_buffer(c, &c.ws.mixed, &c.ws.mixedbytes, wb + ab);
   if (rc) return rc;
   unsigned char* w0 = static_cast<unsigned char*>(c.ws.mixed);
   __nv_bfloat16* wa = reinterpret_cast<__nv_bfloat16*>(w0);
   float* apart = reinterpret_cast<float*>(w0 + wb);
   HPSI_LAUNCH(c, HPSI_K_SPLIT, (k_split_rows64<NT><<<4 * c.sm_count, 256, 0, c.stream>>>(nb, kin, ka, w, wa)));
-  if (partials) {
-    rc = launch_gemm<NT>(c, wa, nb, badd, N, ka, ansplit, aksplit, 0, apart, nullptr, 0, HPSI_K_ADDVUS);
-    if (rc) return rc;
-    if (real) {
-      *out = apart;
-      *nout = ansplit;
-    } else {
-      const size_t nel = (size_t)nb * p.npw;
-      HPSI_LAUNCH(c, HPSI_K_ADDVUS, (k_add_partials<<<(int)std::min<size_t>(8 * c.sm_count, (nel + 255) / 256), 256,
-                                                      0, c.stream>>>(nb, p.npw, ansplit, apart, hpsi)));
-    }
+  rc = launch_gemm<NT>(c, badd, N, wa, nb, ka, ansplit, aksplit, 1, apart, HPSI_K_ADDVUS);
+  if (rc) return rc;
+  if (real) {
+    *out = apart;
+    *nout = ansplit;
   } else {
-    rc = launch_gemm<NT>(c, wa, nb, badd, N, ka, 1, naks, 1, nullptr, hpsi, p.npw, HPSI_K_ADDVUS);
-    if (rc) return rc;
+    const size_t nel = (size_t)nb * p.npw;
+    HPSI_LAUNCH(c, HPSI_K_ADDVUS, (k_add_partials<<<(int)std::min<size_t>(8 * c.sm_count, (nel + 255) / 256), 256, 0,
+                                                    c.stream>>>(nb, p.npw, ansplit, apart, hpsi)));
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "tensor-core add_vuspsi launch");
@@ -1001,7 +999,7 @@ int tc_inner32(Context& c, TcInner& t, bool cache_a, int rows_cap, const float2*
     asplit = as;
   }
   HPSI_LAUNCH(c, HPSI_K_SPLIT, (k_split_inner_b<NT><<<4 * c.sm_count, 256, 0, c.stream>>>(nb, npw, kc, B, bsplit)));
-  rc = launch_gemm<NT>(c, asplit, M, bsplit, 2 * nb, kc, nsplit, ksplit, 0, part, nullptr, 0, HPSI_K_DAVIDSON, pa);
+  rc = launch_gemm<NT>(c, asplit, M, bsplit, 2 * nb, kc, nsplit, ksplit, 0, part, HPSI_K_DAVIDSON, pa);
   if (rc) return rc;
   const size_t n = (size_t)M * nb;
   HPSI_LAUNCH(c, HPSI_K_DAVIDSON,
