@@ -24,7 +24,7 @@
 //
 // The eps in D is eps_i per band by default (D approximates (H - eps_i S)^-1); option
 // HPSI_OPT_PRECOND_SHIFT = 1 takes one eps for all bands, the highest Ritz value of the block
-// (the "estimate of the highest occupied eigenvalue" of the diagonal form of D).  Subspace products are cuBLAS ZGEMMs (library GEMMs);
+// (the "estimate of the highest occupied eigenvalue" of the diagonal form of D).  Subspace products are the kernels of subspace_fp64.cu;
 // residuals, norms and the preconditioner are the kernels below.  Only the residual norms and
 // eigenvalues cross to the host each iteration.
 #include <cublas_v2.h>
@@ -197,8 +197,6 @@ __global__ void k_copy_matrix(int rows, int cols, const double2* __restrict__ sr
 }
 
 const cuDoubleComplex kOne = {1.0, 0.0};
-const cuDoubleComplex kZero = {0.0, 0.0};
-const cuDoubleComplex kMinusOne = {-1.0, 0.0};
 
 inline cuDoubleComplex* Z(double2* p) { return reinterpret_cast<cuDoubleComplex*>(p); }
 inline const cuDoubleComplex* Z(const double2* p) { return reinterpret_cast<const cuDoubleComplex*>(p); }
@@ -404,10 +402,10 @@ static int canonical_orth(Context& c, DavHandles& h, const double2* x, int n, do
   DavWork& w = h.wk;
   const int npw = w.npw;
   // Cholesky QR when the block is well conditioned: x <- x U^-1 with S = U^H U
-  BCK(cublasZgemm(h.blas, CUBLAS_OP_C, CUBLAS_OP_N, n, n, npw, &kOne, Z(x), npw, Z(x), npw, &kZero, Z(w.ovl), n),
-      "zgemm overlap");
+  int rc0 = fp64_inner(c, x, n, x, n, npw, w.ovl, n);
+  if (rc0) return rc0;
   bool chol_ok = false;
-  int rc0 = chol_overlap(c, h, n, relative ? 1e-10 : 1e-6, relative, &chol_ok);
+  rc0 = chol_overlap(c, h, n, relative ? 1e-10 : 1e-6, relative, &chol_ok);
   if (rc0) return rc0;
   if (chol_ok) {
     DCK(cudaMemcpyAsync(out, x, sizeof(double2) * (size_t)n * npw, cudaMemcpyDeviceToDevice, c.stream), "copy");
@@ -417,10 +415,10 @@ static int canonical_orth(Context& c, DavHandles& h, const double2* x, int n, do
     *nkeep = n;
     return HPSI_OK;
   }
-  BCK(cublasZgemm(h.blas, CUBLAS_OP_C, CUBLAS_OP_N, n, n, npw, &kOne, Z(x), npw, Z(x), npw, &kZero, Z(w.ovl), n),
-      "zgemm overlap");
+  int rc = fp64_inner(c, x, n, x, n, npw, w.ovl, n);
+  if (rc) return rc;
   // evec / w receive the decomposition of the overlap (the Ritz vectors were formed already)
-  int rc = small_eigh(c, h, w.ovl, n, n);
+  rc = small_eigh(c, h, w.ovl, n, n);
   if (rc) return rc;
   std::vector<double> lam(n);
   DCK(cudaMemcpyAsync(lam.data(), w.w, sizeof(double) * n, cudaMemcpyDeviceToHost, c.stream), "overlap eigenvalues");
@@ -432,9 +430,7 @@ static int canonical_orth(Context& c, DavHandles& h, const double2* x, int n, do
   *nkeep = nk;
   if (nk == 0) return HPSI_OK;
   HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k_canon_scale<<<(n * nk + 255) / 256, 256, 0, c.stream>>>(n, n, first, nk, w.evec, w.w, w.small)));
-  BCK(cublasZgemm(h.blas, CUBLAS_OP_N, CUBLAS_OP_N, npw, nk, n, &kOne, Z(x), npw, Z(w.small), n, &kZero, Z(out), npw),
-      "zgemm orthonormalise");
-  return HPSI_OK;
+  return fp64_outer(c, x, n, w.small, n, nk, npw, 1.0, false, out);
 }
 
 // ---- mixed path: float32 basis, float64 small problems, norms and Rayleigh quotients ----------
@@ -901,17 +897,10 @@ struct Fp64Ops {
   int apply(const V* x, V* hx, int nb) { return apply_device(c, ik, x, hx, nb); }
   // H_sub[0:rows, col0:col0+ncol] = phi[0:rows]^H hphi[col0:col0+ncol]
   int hsub(int rows, int col0, int ncol) {
-    BCK(cublasZgemm(h.blas, CUBLAS_OP_C, CUBLAS_OP_N, rows, ncol, npw, &kOne, Z(w.phi), npw,
-                    Z(w.hphi + (size_t)col0 * npw), npw, &kZero, Z(w.hsub + (size_t)col0 * w.mmax), w.mmax),
-        "zgemm H_sub columns");
-    return HPSI_OK;
+    return fp64_inner(c, w.phi, rows, w.hphi + (size_t)col0 * npw, ncol, npw, w.hsub + (size_t)col0 * w.mmax, w.mmax);
   }
   // out = src[0:m] times the leading n columns of the reduced eigenvectors (ld m)
-  int rotate(const V* src, int m, int n, V* out) {
-    BCK(cublasZgemm(h.blas, CUBLAS_OP_N, CUBLAS_OP_N, npw, n, m, &kOne, Z(src), npw, Z(w.evec), m, &kZero, Z(out), npw),
-        "zgemm Ritz vectors");
-    return HPSI_OK;
-  }
+  int rotate(const V* src, int m, int n, V* out) { return fp64_outer(c, src, m, w.evec, m, n, npw, 1.0, false, out); }
   // Ritz vectors psi = phi C[:, 0:NA], hpsi = hphi C[:, 0:NA]; residuals into t, norms into rnorm
   int ritz_residuals(int m, int NA) {
     int rc = rotate(w.phi, m, NA, w.psi);
@@ -950,13 +939,8 @@ struct Fp64Ops {
   }
   // tnew[0:nc] -= phi[0:m] (phi[0:m]^H tnew)
   int project(int m, int /*locked*/, int nc, V* tnew) {
-    BCK(cublasZgemm(h.blas, CUBLAS_OP_C, CUBLAS_OP_N, m, nc, npw, &kOne, Z(w.phi), npw, Z(tnew), npw, &kZero,
-                    Z(w.small), m),
-        "zgemm projection");
-    BCK(cublasZgemm(h.blas, CUBLAS_OP_N, CUBLAS_OP_N, npw, nc, m, &kMinusOne, Z(w.phi), npw, Z(w.small), m, &kOne,
-                    Z(tnew), npw),
-        "zgemm projection update");
-    return HPSI_OK;
+    const int rc = fp64_inner(c, w.phi, m, tnew, nc, npw, w.small, m);
+    return rc ? rc : fp64_outer(c, w.phi, m, w.small, m, nc, npw, -1.0, true, tnew);
   }
   int norm2(int nc, const V* tnew) {
     HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k_norm2<<<nc, 256, 0, c.stream>>>(npw, tnew, w.cn2)));

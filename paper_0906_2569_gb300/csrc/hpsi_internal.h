@@ -363,6 +363,17 @@ int slices_add(Context& c, const Problem& p, const double2* w, double2* hpsi, in
 bool gamma_slices_use(const Problem& p, int nbnd);
 int gamma_slices_w(Context& c, const Problem& p, const void* x, bool x32, int nbnd, bool scaled, double* w, bool* ok);
 int gamma_slices_add(Context& c, const Problem& p, const double* w, double* out, int nbnd, bool* ok);
+// Subspace products of float64 blocks of rows [.][npw] (subspace_fp64.cu): out[i + j ldo] = <a_i|b_j>, and
+// out_j = (accumulate ? out_j : 0) + sign sum_i coef[i + j ldc] a_i (out may be none of the a_i).  Work in ws.part and ws.mixed.
+int fp64_inner(Context& c, const double2* a, int m, const double2* b, int n, int npw, double2* out, int ldo);
+int fp64_outer(Context& c, const double2* a, int k, const double2* coef, int ldc, int n, int npw, double sign,
+               bool accumulate, double2* out);
+// Their form on the tensor cores, for complex or real rows of len entries; *ok = false: no room for the digit planes
+int slices_inner(Context& c, const double* a, int m, const double* b, int n, int len, bool real, double* out, int ldo,
+                 bool* ok);
+int slices_outer(Context& c, const double* a, int k, const double* coef, int ldc, int n, int len, bool real, double sign,
+                 bool accumulate, double* out, bool* ok);
+constexpr double kDigitMacs = 2.0e7;   // complex multiply-adds from which that form is taken (real: four times as many)
 // w = D (sum of the splits' partial <beta|psi>), complex and Gamma form
 int dscale_fp64(Context& c, const Problem& p, int nb, int nsplit, double2* part, double2* w);
 int gamma_dscale_fp64(Context& c, const Problem& p, int nb, int nsplit, const double* part, double* w);

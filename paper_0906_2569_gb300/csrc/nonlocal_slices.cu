@@ -30,6 +30,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "fixed_fft.cuh"
 #include "hpsi_internal.h"
@@ -614,6 +615,122 @@ int gamma_slices_add(Context& c, const Problem& p, const double* w, double* out,
   return slice_gemm(c, static_cast<const __nv_bfloat16*>(s.digits), s.exps, nr, d, e, nbnd, s.kpad, 1,
                     (s.kpad / SK + kChunkSteps - 1) / kChunkSteps * kChunkSteps, false, false, out, 0, nr,
                     HPSI_K_ADDVUS);
+}
+
+
+// ---- subspace products (subspace_fp64.cu) -------------------------------------------------------
+
+// out[i + j ldo] = src[j][i], rows of m
+template <typename V>
+static __global__ void __launch_bounds__(256) k_copy_cols(int m, int n, const V* __restrict__ src, V* __restrict__ out,
+                                                          int ldo) {
+  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < (size_t)m * n; t += (size_t)gridDim.x * blockDim.x)
+    out[t / m * ldo + t % m] = src[t];
+}
+// dst[j][i] = sign coef[i + j ldc], rows of k entries of CW doubles
+template <int CW>
+static __global__ void __launch_bounds__(256) k_pack_coef(int k, int n, double sign, const double* __restrict__ coef, int ldc,
+                                                          double* __restrict__ dst) {
+  const int kw = CW * k;
+  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < (size_t)kw * n; t += (size_t)gridDim.x * blockDim.x)
+    dst[t] = sign * coef[t / kw * ldc * CW + t % kw];
+}
+static int few_ctas(const Context& c, size_t n) { return (int)std::min<size_t>(8 * c.sm_count, (n + 255) / 256); }
+
+// out[i + j ldo] = <a_i|b_j> for complex (CW = 2) or real (1) rows of len entries; *ok = false: no room for the digit planes
+// (nothing was done)
+template <int CW>
+static int slices_inner_t(Context& c, const double* a, int m, const double* b, int n, int len, double* out, int ldo,
+                          bool* ok) {
+  using V = typename std::conditional<CW == 2, double2, double>::type;
+  constexpr int dup = CW == 2 ? 1 : 0;
+  *ok = false;
+  const int kpad = pad32(CW * len);
+  const int nbk = slice_band_block(n, slice_rows_bytes(1, kpad, dup)), mbk = slice_band_block(m, slice_rows_bytes(1, kpad, 0));
+  const size_t bb = slice_rows_bytes(nbk, kpad, dup), ab = slice_rows_bytes(mbk, kpad, 0);
+  int rc = ensure_buffer(c, &c.ws.mixed, &c.ws.mixedbytes, ab + bb);
+  if (rc == HPSI_ENOMEM) return HPSI_OK;
+  if (rc) return rc;
+  unsigned char* w0 = static_cast<unsigned char*>(c.ws.mixed);
+  for (int j0 = 0; j0 < n; j0 += nbk) {
+    const int nj = std::min(nbk, n - j0);
+    __nv_bfloat16 *db = nullptr, *da = nullptr;
+    int *eb = nullptr, *ea = nullptr;
+    rc = slice_rows(c, b + (size_t)j0 * len * CW, nj, CW * len, kpad, dup, 1, w0, &db, &eb);
+    if (rc) return rc;
+    for (int i0 = 0; i0 < m; i0 += mbk) {
+      const int mi = std::min(mbk, m - i0);
+      rc = slice_rows(c, a + (size_t)i0 * len * CW, mi, CW * len, kpad, 0, 1, w0 + bb, &da, &ea);
+      if (rc) return rc;
+      int per = 0;
+      const int ns = slice_splits(c, mi, CW * nj, kpad / SK, &per);
+      rc = ensure_buffer(c, &c.ws.part, &c.ws.partbytes, sizeof(V) * (size_t)ns * mi * nj);
+      if (rc) return rc;
+      double* part = static_cast<double*>(c.ws.part);
+      rc = slice_gemm(c, da, ea, mi, db, eb, CW * nj, kpad, ns, per, CW == 2, false, part, CW * (size_t)mi * nj, mi,
+                      HPSI_K_DAVIDSON);
+      if (!rc) rc = sum_splits(c, CW * (size_t)mi * nj, ns);
+      if (rc) return rc;
+      HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k_copy_cols<V><<<few_ctas(c, (size_t)mi * nj), 256, 0, c.stream>>>(
+                                          mi, nj, reinterpret_cast<const V*>(part),
+                                          reinterpret_cast<V*>(out) + (size_t)j0 * ldo + i0, ldo)));
+    }
+  }
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(c, e, "subspace inner products");
+  *ok = true;
+  return HPSI_OK;
+}
+
+// out_j = (accumulate ? out_j : 0) + sign sum_i coef[i + j ldc] a_i
+template <int CW>
+static int slices_outer_t(Context& c, const double* a, int k, const double* coef, int ldc, int n, int len, double sign,
+                          bool accumulate, double* out, bool* ok) {
+  constexpr int dup = CW == 2 ? 2 : 0;
+  *ok = false;
+  // the rows' digits [len][CW k] in blocks of k that stay near 2 GB
+  const size_t per_k = sizeof(__nv_bfloat16) * kDigits * CW * (size_t)len;
+  const int blocks = (int)std::max<size_t>(1, (per_k * k + (2ull << 30) - 1) / (2ull << 30));
+  const int kbk = ((k + blocks - 1) / blocks + 15) / 16 * 16;
+  const int kpad0 = pad32(CW * std::min(k, kbk));
+  const size_t eb_ = al256(sizeof(int) * (size_t)len);
+  const size_t ab = al256(sizeof(__nv_bfloat16) * kDigits * (size_t)len * kpad0) + eb_;
+  const size_t bb = slice_rows_bytes(n, kpad0, dup), cb = al256(sizeof(double) * CW * (size_t)n * kbk);
+  int rc = ensure_buffer(c, &c.ws.mixed, &c.ws.mixedbytes, ab + bb + cb);
+  if (rc == HPSI_ENOMEM) return HPSI_OK;
+  if (rc) return rc;
+  unsigned char* w0 = static_cast<unsigned char*>(c.ws.mixed);
+  __nv_bfloat16* da = reinterpret_cast<__nv_bfloat16*>(w0);
+  int* ea = reinterpret_cast<int*>(w0 + ab - eb_);
+  double* pack = reinterpret_cast<double*>(w0 + ab + bb);
+  for (int k0 = 0; k0 < k; k0 += kbk) {
+    const int nk = std::min(kbk, k - k0), kpad = pad32(CW * nk);
+    HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k_pack_coef<CW><<<few_ctas(c, CW * (size_t)nk * n), 256, 0, c.stream>>>(
+                                        nk, n, sign, coef + (size_t)k0 * CW, ldc, pack)));
+    HPSI_LAUNCH(c, HPSI_K_SPLIT, (k_digits_transposed<CW><<<(len + 31) / 32, 256, 0, c.stream>>>(
+                                     nk, len, kpad, a + (size_t)k0 * len * CW, da, ea)));
+    __nv_bfloat16* db = nullptr;
+    int* eb = nullptr;
+    rc = slice_rows(c, static_cast<const double*>(pack), n, CW * nk, kpad, dup, 1, w0 + ab, &db, &eb);
+    if (rc) return rc;
+    rc = slice_gemm(c, da, ea, len, db, eb, CW * n, kpad, 1, (kpad / SK + kChunkSteps - 1) / kChunkSteps * kChunkSteps,
+                    CW == 2, accumulate || k0 > 0, out, 0, len, HPSI_K_DAVIDSON);
+    if (rc) return rc;
+  }
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(c, e, "subspace combinations");
+  *ok = true;
+  return HPSI_OK;
+}
+
+int slices_inner(Context& c, const double* a, int m, const double* b, int n, int len, bool real, double* out, int ldo,
+                 bool* ok) {
+  return real ? slices_inner_t<1>(c, a, m, b, n, len, out, ldo, ok) : slices_inner_t<2>(c, a, m, b, n, len, out, ldo, ok);
+}
+int slices_outer(Context& c, const double* a, int k, const double* coef, int ldc, int n, int len, bool real, double sign,
+                 bool accumulate, double* out, bool* ok) {
+  return real ? slices_outer_t<1>(c, a, k, coef, ldc, n, len, sign, accumulate, out, ok)
+              : slices_outer_t<2>(c, a, k, coef, ldc, n, len, sign, accumulate, out, ok);
 }
 
 }  // namespace hpsi

@@ -311,7 +311,7 @@ __device__ __forceinline__ void bf16_terms(float2 x, __nv_bfloat16 (&t)[NT]) {
 
 // B of calbec: rows b < nb: psi_b (re, im); rows nb + b: (im, -re).  One thread per complex psi element (or per pair
 // of padding columns), writing bf16 pairs.  The terms are found in float32 (float64 casts and
-// subtractions made this kernel float64-bound: 160 bands of 36785 226 -> 60 us).
+// subtractions made this kernel float64-bound: 160 bands of 36785 226 -> 38 us).
 template <int NT>
 __global__ void __launch_bounds__(256) k_split_psi(int nb, int npw, int kc, const double2* __restrict__ psi,
                                                    __nv_bfloat16* __restrict__ out) {

@@ -74,7 +74,8 @@ __device__ __forceinline__ void calbec_tile_t(int npw, int nproj, int nb, int kc
 #pragma unroll
       for (int i = 0; i < PI; ++i)
 #pragma unroll
-        for (int j = 0; j < BJ; ++j) cmac_conj(acc[i][j], x[i], y[j]);
+        for (int j = 0; j < BJ; ++j)
+          if (j == 0 || b0 + (int)(threadIdx.x & ~31u) / TX + TY * j < nb) cmac_conj(acc[i][j], x[i], y[j]);
     }
     }
     __syncthreads();
