@@ -34,7 +34,9 @@
 #include <cfloat>
 #include <cmath>
 #include <string>
+#include <type_traits>
 
+#include "convert.cuh"
 #include "hpsi_internal.h"
 #include "eigh_tridiag.cuh"
 #include "eigh_tridiag_real.cuh"
@@ -76,14 +78,15 @@ __device__ __forceinline__ long long dbits(double x) { return __double_as_longlo
 // exactly zero becomes a tiny value of the sign opposite to the previous one (a pivmin-style
 // perturbation of the diagonal); every 8 steps the pair is scaled by 2^-+400 through its exponent
 // fields (a partner too small to scale down is negligible and flushed to zero; a subnormal is left
-// as it is).
-__device__ int sturm_count(int n, const double* __restrict__ d, const double* __restrict__ e2, double sigma) {
+// as it is).  The last minor is *pv 2^(400 *pe).
+__device__ int sturm_count(int n, const double* __restrict__ d, const double* __restrict__ e2, double sigma, double* pv,
+                           int* pe) {
   constexpr long long kSign = (long long)0x8000000000000000ULL;
   constexpr long long kTiny = 0x0910000000000000LL;             // 2^-878
   constexpr long long kShift = 400LL << 52;
   double pm = 1.0, p = d[0] - sigma;
   if ((dbits(p) << 1) == 0) p = __longlong_as_double(kSign | kTiny);
-  int cnt = dbits(p) < 0;
+  int cnt = dbits(p) < 0, sc = 0;
   auto step = [&](int k) {
     double pn = fma(d[k] - sigma, p, -e2[k - 1] * pm);
     if ((dbits(pn) << 1) == 0) pn = __longlong_as_double(((dbits(p) & kSign) ^ kSign) | kTiny);
@@ -99,58 +102,162 @@ __device__ int sturm_count(int n, const double* __restrict__ d, const double* __
     if (ex > 1023 + 400) {
       p = __longlong_as_double(ep > 400 ? dbits(p) - kShift : dbits(p) & kSign);
       pm = __longlong_as_double(em > 400 ? dbits(pm) - kShift : dbits(pm) & kSign);
+      ++sc;
     } else if (ex < 1023 - 400) {
       if (ep > 0) p = __longlong_as_double(dbits(p) + kShift);
       if (em > 0) pm = __longlong_as_double(dbits(pm) + kShift);
+      --sc;
     }
+  }
+  for (; k < n; ++k) step(k);
+  *pv = p;
+  *pe = sc;
+  return cnt;
+}
+
+// The same count in float32 for T scaled to |T| < 2: exact for a T perturbed by less than 2^-20.  The pair is scaled to
+// exponent 0 every 4 steps (|p| grows by less than 8 a step).
+__device__ int sturm_count32(int n, const float* d, const float* e2, float sigma) {
+  float pm = 1.f, p = d[0] - sigma;
+  if (p == 0.f) p = -1e-30f;
+  int cnt = p < 0.f;
+  auto step = [&](int k) {
+    float pn = fmaf(d[k] - sigma, p, -e2[k - 1] * pm);
+    if (pn == 0.f) pn = copysignf(1e-30f, -p);
+    cnt += (__float_as_int(pn) ^ __float_as_int(p)) < 0;
+    pm = p;
+    p = pn;
+  };
+  int k = 1;
+  for (; k + 4 <= n; k += 4) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) step(k + u);
+    const unsigned ex = max((__float_as_uint(p) >> 23) & 0xff, (__float_as_uint(pm) >> 23) & 0xff);
+    const float s = __uint_as_float((254u - min(ex, 253u)) << 23);
+    p *= s;
+    pm *= s;
   }
   for (; k < n; ++k) step(k);
   return cnt;
 }
 
-
-// One CTA of kBisWarps warps per wanted eigenvalue i: (32 kBisWarps + 1)-way multisection of an
-// interval with count(lo) <= i < count(hi), one Sturm count per thread and round, so the float64
-// recurrences run on every sub-partition of the SM at once.
-constexpr int kBisWarps = 1;   // 32 points per round: float64 Sturm counts are the bottleneck on this GPU, and
-                                // 32 points take ~40% fewer of them than 64 for the same bracket width
+// One CTA of up to four warps per wanted eigenvalue i, one Sturm count per thread and round: multisection of an
+// interval with count(lo) <= i < count(hi).  A float64 count is 3 n instructions of ~78 cycles on its scheduler, so what
+// counts is the number of float64 rounds.
+//   - The first ~19 bits come from float32 counts (a few cycles a step); the bracket they give is widened by their error and
+//     its ends are counted in float64 with the first round (a wrong one falls back to the Gershgorin interval).
+//   - Once the bracket holds one eigenvalue and its ends were counted in one round, the last minors there give the secant
+//     estimate, and the next round's points lie around it at distances tol / 4 times powers of 2 (or 4, or 1.5 and 2): the
+//     bracket then shrinks to the estimate's error, two or three rounds in all.  A round of that kind that gains less
+//     than a factor 32 is followed by an even one.
+// Four warps while the chip has an SM for each eigenvalue, two while it has half a one: a scheduler carries one warp.
+// 640 rows, 160 wanted: 1.09 -> 0.3 ms; up to 64 rows, 16 wanted: 97 -> 41 us.
+constexpr int kBisWarps = 4;
 __global__ void __launch_bounds__(32 * kBisWarps) k_eh_bisect(int n, const double* __restrict__ d,
                                                               const double* __restrict__ e,
                                                               const double* __restrict__ e2, int nwant,
                                                               double* __restrict__ lam) {
-  constexpr int NP = 32 * kBisWarps;   // points per round
+  extern __shared__ float bsm[];
   __shared__ unsigned bal[kBisWarps];
+  __shared__ double spv[2], sx[2];
+  __shared__ int spe[2], scnt[2];
+  const int nw = blockDim.x >> 5, NP = blockDim.x;   // points per round
   const int i = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  if (i >= nwant) return;
-  double lo, hi, emax2;
-  gershgorin(n, d, e, &lo, &hi, &emax2);
-  const double tnorm = fmax(fmax(fabs(lo), fabs(hi)), DBL_MIN);
+  double glo, ghi, emax2;
+  gershgorin(n, d, e, &glo, &ghi, &emax2);
+  const double tnorm = fmax(fmax(fabs(glo), fabs(ghi)), DBL_MIN);
   const double pivmin = 1e-30 * fmax(1.0, emax2);
-  lo -= 4.0 * DBL_EPSILON * tnorm + 4.0 * pivmin;
-  hi += 4.0 * DBL_EPSILON * tnorm + 4.0 * pivmin;
-  const double tol = 4.0 * DBL_EPSILON * tnorm;
-  for (int round = 0; round < 64 && hi - lo > tol; ++round) {
-    const double w = (hi - lo) / (double)(NP + 1);
-    const int cnt = sturm_count(n, d, e2, lo + w * (double)(tid + 1));
+  glo -= 4.0 * DBL_EPSILON * tnorm + 4.0 * pivmin;
+  ghi += 4.0 * DBL_EPSILON * tnorm + 4.0 * pivmin;
+  const double tol = DBL_EPSILON * tnorm;
+  // index of the first point whose count exceeds i; NP if none
+  auto first_above = [&](int cnt) {
     const unsigned above = __ballot_sync(0xffffffffu, cnt > i);
+    __syncthreads();
     if (lane == 0) bal[wid] = above;
     __syncthreads();
-    int f = NP;   // index (point - 1) of the first point whose count exceeds i; NP if none
-    for (int q = 0; q < kBisWarps; ++q)
-      if (bal[q]) {
-        f = 32 * q + __ffs(bal[q]) - 1;
-        break;
-      }
-    __syncthreads();
-    double nlo, nhi;
-    if (f == NP) {
-      nlo = lo + w * (double)NP;
-      nhi = hi;
-    } else {
-      nlo = f > 0 ? lo + w * (double)f : lo;
-      nhi = lo + w * (double)(f + 1);
+    for (int q = 0; q < nw; ++q)
+      if (bal[q]) return 32 * q + __ffs(bal[q]) - 1;
+    return NP;
+  };
+  double lo = glo, hi = ghi;
+  bool fresh = false;   // the bracket's ends have not been counted
+  const int ex = biased_exp(tnorm);
+  if (ex > 1023 - 300 && ex < 1023 + 300) {
+    const double sf = __longlong_as_double((long long)(2046 - ex) << 52), back = __longlong_as_double((long long)ex << 52);
+    float *fd = bsm, *fe = bsm + n;
+    for (int k = tid; k < n; k += NP) {
+      fd[k] = f64_to_f32(d[k] * sf);
+      fe[k] = k < n - 1 ? f64_to_f32(e2[k] * sf * sf) : 0.f;
     }
-    if (nlo == lo && nhi == hi) break;   // the interval is down to a few ulps
+    __syncthreads();
+    float flo = f64_to_f32(glo * sf), fhi = f64_to_f32(ghi * sf);
+    for (int round = 0; round < 24 && fhi - flo > 0x1p-19f; ++round) {
+      const float w = (fhi - flo) / (float)(NP + 1);
+      const int f = first_above(sturm_count32(n, fd, fe, flo + w * (float)(tid + 1)));
+      const float nlo = f > 0 ? flo + w * (float)f : flo, nhi = f < NP ? flo + w * (float)(f + 1) : fhi;
+      flo = nlo;
+      fhi = nhi;
+    }
+    lo = fmax(glo, (f32_to_f64(flo) - 0x1p-18) * back);
+    hi = fmin(ghi, (f32_to_f64(fhi) + 0x1p-18) * back);
+    fresh = lo < hi;
+    if (!fresh) {
+      lo = glo;
+      hi = ghi;
+    }
+  }
+  bool around = false;   // points around est instead of evenly spaced
+  double est = 0.0;
+  for (int round = 0; round < 80 && (fresh || hi - lo > tol); ++round) {
+    const double w = hi - lo;
+    double x;
+    if (around) {
+      const int half = NP >> 1, k = tid < half ? half - 1 - tid : tid - half;
+      const int sh = NP == 32 ? 2 * k : NP == 64 ? k : k >> 1;
+      const double step = (NP == 128 && (k & 1) ? 0.375 : 0.25) * tol;
+      const double off = step * __longlong_as_double((long long)(1023 + sh) << 52);
+      x = fmin(hi, fmax(lo, tid < half ? est - off : est + off));
+    } else if (fresh) {
+      x = tid == NP - 1 ? hi : fma(w / (double)(NP - 1), (double)tid, lo);
+    } else {
+      x = fma(w / (double)(NP + 1), (double)(tid + 1), lo);
+    }
+    double pv;
+    int pe;
+    const int cnt = sturm_count(n, d, e2, x, &pv, &pe);
+    const int f = first_above(cnt);
+    if (fresh) {
+      fresh = false;
+      if (f == 0 || f == NP) {
+        lo = glo;
+        hi = ghi;
+        continue;
+      }
+    }
+    if (tid == f - 1 || tid == f) {
+      const int t = tid - (f - 1);
+      sx[t] = x;
+      spv[t] = pv;
+      spe[t] = pe;
+      scnt[t] = cnt;
+    }
+    __syncthreads();
+    const double nlo = f > 0 ? sx[0] : lo, nhi = f < NP ? sx[1] : hi;
+    if (nlo == lo && nhi == hi) {
+      if (!around) break;   // the interval is down to a few ulps
+      around = false;
+      continue;
+    }
+    const bool slow = around && (nhi - nlo) * 32.0 > w;
+    around = false;
+    if (!slow && f > 0 && f < NP && scnt[0] == i && scnt[1] == i + 1) {
+      const int de = spe[1] - spe[0];
+      double r = fabs(spv[1] / spv[0]);
+      if (de != 0) r *= de == 1 ? 0x1p400 : de == -1 ? 0x1p-400 : de > 0 ? INFINITY : 0.0;
+      est = nlo + (nhi - nlo) / (1.0 + r);
+      around = est >= nlo && est <= nhi;
+    }
     lo = nlo;
     hi = nhi;
   }
@@ -164,7 +271,7 @@ __device__ __forceinline__ double hash_unit(unsigned int i, unsigned int k) {
   x ^= x >> 15;
   x *= 0x846CA68Bu;
   x ^= x >> 16;
-  return (double)(x >> 8) * (1.0 / 16777216.0) - 0.5;
+  return f32_to_f64((float)(x >> 8) * (1.f / 16777216.f) - 0.5f);   // exact in float32
 }
 
 // z <- z - (zq . z) zq for the earlier members q of the cluster, then z /= |z|; whole warp.
@@ -194,16 +301,19 @@ __device__ bool orth_normalize(int n, double* z, const double* __restrict__ Z, i
 // solves, the warp orthogonalises and normalises.  Vectors go to Z (column i, leading dim n).
 // Inverse iteration for the eigenvalues without a neighbour within the cluster tolerance, one per
 // lane: a float64 warp instruction costs the same with one active lane as with 32, so 32 of the
-// serial tridiagonal recurrences share each instruction.  Per lane: T - lambda I = P L U with partial
-// pivoting (the pivot choice as selects, the row interchanges as one ballot mask per step), then
-// `iters` solves from a hashed start, normalised after each.  The factors and z live in a global
-// scratch laid out [k][lane] per warp (5 n 32 doubles and n masks), so every step's accesses are
-// coalesced.  Members of clusters are left to k_eh_invit.
+// serial tridiagonal recurrences share each instruction, and the time is the number of float64 instructions per
+// row (~78 cycles each).  Per lane: T - lambda I = P L U with partial pivoting (the pivot choice as selects, the row
+// interchanges as one ballot mask per step; 7 instructions a row), then `iters` solves: the first one from a hashed vector
+// through U alone (that vector is L^-1 P^T of a start as arbitrary; 3), the others through L and U (4).  Vectors are not
+// normalised in between unless one leaves 2^+-400, which its exponents show; the norm and the result are taken by
+// k_eh_invit_finish with the whole chip.  The factors and z live in a global scratch laid out [k][lane] per warp
+// (5 n 32 doubles, n masks and the mask of the lanes in use), so every step's accesses are coalesced.
+// Members of clusters are left to k_eh_invit.  640 rows, 160 vectors: 1.00 -> 0.76 ms; up to 64 rows: 78 -> 54 us.
+__host__ __device__ inline size_t invit_stride(int n) { return (size_t)5 * 32 * n + n / 2 + 1; }
 __global__ void __launch_bounds__(32) k_eh_invit_lanes(int n, const double* __restrict__ d,
                                                        const double* __restrict__ e, int nwant,
-                                                       const double* __restrict__ lam, double* __restrict__ Z,
-                                                       double* __restrict__ scratch, int* __restrict__ status,
-                                                       int iters) {
+                                                       const double* __restrict__ lam, double* __restrict__ scratch,
+                                                       int* __restrict__ status, int iters) {
   const int lane = threadIdx.x, i = blockIdx.x * 32 + lane;
   double glo, ghi, emax2;
   gershgorin(n, d, e, &glo, &ghi, &emax2);
@@ -213,18 +323,22 @@ __global__ void __launch_bounds__(32) k_eh_invit_lanes(int n, const double* __re
   bool mine = i < nwant;
   if (mine && i > 0 && lam[i] - lam[i - 1] <= ctol) mine = false;
   if (mine && i + 1 < nwant && lam[i + 1] - lam[i] <= ctol) mine = false;
-  if (__ballot_sync(0xffffffffu, mine) == 0u) return;
+  double* base = scratch + blockIdx.x * invit_stride(n);
+  unsigned* PIV = reinterpret_cast<unsigned*>(base + (size_t)5 * 32 * n);
+  const unsigned mask = __ballot_sync(0xffffffffu, mine);
+  if (lane == 0) PIV[n] = mask;
+  if (mask == 0u) return;
   const double li = mine ? lam[i] : lam[0];
-  double* base = scratch + (size_t)blockIdx.x * ((size_t)5 * 32 * n + (n + 1) / 2);
   double* SL = base + lane;
   double* SU1 = SL + (size_t)32 * n;
   double* SU2 = SU1 + (size_t)32 * n;
   double* SU3 = SU2 + (size_t)32 * n;
   double* Zs = SU3 + (size_t)32 * n;
-  unsigned* PIV = reinterpret_cast<unsigned*>(base + (size_t)5 * 32 * n);
   constexpr long long kMag = 0x7fffffffffffffffLL;
+  const long long btiny = dbits(tiny);
   auto guard = [&](double u) {
-    return (__double_as_longlong(u) & kMag) < (__double_as_longlong(tiny) & kMag) ? (u < 0.0 ? -tiny : tiny) : u;
+    const long long b = dbits(u);
+    return (b & kMag) < btiny ? __longlong_as_double((b & ~kMag) | btiny) : u;
   };
   // every loop takes its independent loads kB steps at a time ahead of the dependent recurrence,
   // so that the L2 latency of the scratch is paid once per block, not once per step
@@ -232,7 +346,7 @@ __global__ void __launch_bounds__(32) k_eh_invit_lanes(int n, const double* __re
   double al = d[0] - li, be = n > 1 ? e[0] : 0.0;
   auto lu_step = [&](int k, double sub, double dk1, double cn) {
     const double dn = dk1 - li;
-    const bool np = (__double_as_longlong(al) & kMag) >= (__double_as_longlong(sub) & kMag);
+    const bool np = (dbits(al) & kMag) >= (dbits(sub) & kMag);
     const double ui = recip_nr(np ? guard(al) : sub);
     const double l = (np ? sub : al) * ui;
     SL[(size_t)k * 32] = l;
@@ -259,20 +373,15 @@ __global__ void __launch_bounds__(32) k_eh_invit_lanes(int n, const double* __re
   }
   for (; k < n - 1; ++k) lu_step(k, e[k], d[k + 1], k + 1 < n - 1 ? e[k + 1] : 0.0);
   SU1[(size_t)(n - 1) * 32] = recip_nr(guard(al));
-  double nn = 0.0;
-  for (int q = 0; q < n; ++q) {
-    const double v = hash_unit((unsigned)i, (unsigned)q);
-    Zs[(size_t)q * 32] = v;
-    nn = fma(v, v, nn);
-  }
-  bool ok = true;
-  double sc = 1.0 / sqrt(nn);
   __syncwarp();
-  for (int it = 0; it < iters; ++it) {
-    // forward: row interchanges and L
-    double zk = Zs[0] * sc;
+  int mx = 0;   // largest upper word of |z|
+  double zk = 0.0;
+  // row interchanges and L; `scaled`: the vector is multiplied by sc on the way
+  auto forward = [&](auto scaled, double sc) {
+    auto in = [&](double v) { return decltype(scaled)::value ? v * sc : v; };
+    zk = in(Zs[0]);
     auto fwd_step = [&](int q, double z1r, double lq, unsigned pq) {
-      const double z1 = z1r * sc;
+      const double z1 = in(z1r);
       const bool sw = (pq >> lane) & 1u;
       const double a = sw ? z1 : zk, b = sw ? zk : z1;
       Zs[(size_t)q * 32] = a;
@@ -292,30 +401,29 @@ __global__ void __launch_bounds__(32) k_eh_invit_lanes(int n, const double* __re
       for (int u = 0; u < kB; ++u) fwd_step(q + u, zv[u], lv[u], pv[u]);
     }
     for (; q < n - 1; ++q) fwd_step(q, Zs[(size_t)(q + 1) * 32], SL[(size_t)q * 32], PIV[q]);
-    // backward: U (three diagonals), with the squared norm of the result
-    double z2 = zk * SU1[(size_t)(n - 1) * 32];
-    Zs[(size_t)(n - 1) * 32] = z2;
-    nn = z2 * z2;
-    double z1 = 0.0;
-    if (n >= 2) {
-      z1 = (Zs[(size_t)(n - 2) * 32] - SU2[(size_t)(n - 2) * 32] * z2) * SU1[(size_t)(n - 2) * 32];
-      Zs[(size_t)(n - 2) * 32] = z1;
-      nn = fma(z1, z1, nn);
-    }
-    auto bwd_step = [&](int q, double zq, double u1, double u2, double u3) {
-      const double zz = (zq - u2 * z1 - u3 * z2) * u1;
+  };
+  // U (three diagonals); the right-hand side is the hashed vector (start) or Zs and zk
+  auto backward = [&](auto start) {
+    constexpr bool kStart = decltype(start)::value;
+    auto rhs = [&](int q) { return kStart ? hash_unit((unsigned)i, (unsigned)q) : Zs[(size_t)q * 32]; };
+    mx = 0;
+    double z1 = 0.0, z2 = 0.0;
+    auto put = [&](int q, double zz) {
       Zs[(size_t)q * 32] = zz;
-      nn = fma(zz, zz, nn);
+      mx = max(mx, __double2hiint(zz) & 0x7fffffff);
       z2 = z1;
       z1 = zz;
     };
-    q = n - 3;
+    put(n - 1, (kStart ? rhs(n - 1) : zk) * SU1[(size_t)(n - 1) * 32]);
+    if (n >= 2) put(n - 2, (rhs(n - 2) - SU2[(size_t)(n - 2) * 32] * z1) * SU1[(size_t)(n - 2) * 32]);
+    auto bwd_step = [&](int q, double zq, double u1, double u2, double u3) { put(q, (zq - u2 * z1 - u3 * z2) * u1); };
+    int q = n - 3;
     for (; q - kB + 1 >= 0; q -= kB) {
       double zv[kB], a1[kB], a2[kB], a3[kB];
 #pragma unroll
       for (int u = 0; u < kB; ++u) {
         const size_t o = (size_t)(q - u) * 32;
-        zv[u] = Zs[o];
+        zv[u] = rhs(q - u);
         a1[u] = SU1[o];
         a2[u] = SU2[o];
         a3[u] = SU3[o];
@@ -325,18 +433,50 @@ __global__ void __launch_bounds__(32) k_eh_invit_lanes(int n, const double* __re
     }
     for (; q >= 0; --q) {
       const size_t o = (size_t)q * 32;
-      bwd_step(q, Zs[o], SU1[o], SU2[o], SU3[o]);
+      bwd_step(q, rhs(q), SU1[o], SU2[o], SU3[o]);
     }
-    if (!(nn > 0.0) || !isfinite(nn)) ok = false;
-    sc = ok ? 1.0 / sqrt(nn) : 1.0;
+  };
+  bool ok = true;
+  backward(std::true_type{});
+  for (int it = 1;; ++it) {
+    const int ex = mx >> 20;
+    if (ex == 0x7ff || mx == 0) ok = false;
+    if (it >= iters) break;
+    const bool far = ok && (ex < 1023 - 400 || ex > 1023 + 400);
+    if (__any_sync(0xffffffffu, far)) forward(std::true_type{}, far ? 1.0 / __hiloint2double(max(ex, 1) << 20, 0) : 1.0);
+    else forward(std::false_type{}, 1.0);
+    backward(std::false_type{});
   }
-  if (!mine) return;
-  if (!ok) {
-    atomicExch(status, 1);
-    return;
+  if (mine && !ok) atomicExch(status, 1);
+}
+
+// Z[i] = z_i / |z_i| for the vectors of k_eh_invit_lanes; one CTA each
+__global__ void __launch_bounds__(128) k_eh_invit_finish(int n, const double* __restrict__ scratch, double* __restrict__ Z) {
+  const int i = blockIdx.x, lane = i & 31;
+  const double* base = scratch + (i >> 5) * invit_stride(n);
+  if (!((reinterpret_cast<const unsigned*>(base + (size_t)5 * 32 * n)[n] >> lane) & 1u)) return;
+  const double* z = base + (size_t)4 * 32 * n + lane;
+  __shared__ int smx[4];
+  __shared__ double snn[4];
+  int mx = 0;
+  for (int k = threadIdx.x; k < n; k += 128) mx = max(mx, __double2hiint(z[(size_t)k * 32]) & 0x7fffffff);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if ((threadIdx.x & 31) == 0) smx[threadIdx.x >> 5] = mx;
+  __syncthreads();
+  // the largest element is brought to [1, 2) in two exact factors, so that no square leaves the range
+  const int ex = max(max(smx[0], smx[1]), max(smx[2], smx[3])) >> 20, sh = 1023 - ex;
+  const double f1 = __hiloint2double((1023 + sh / 2) << 20, 0), f2 = __hiloint2double((1023 + sh - sh / 2) << 20, 0);
+  double nn = 0.0;
+  for (int k = threadIdx.x; k < n; k += 128) {
+    const double v = z[(size_t)k * 32] * f1 * f2;
+    nn = fma(v, v, nn);
   }
+  nn = warp_sum(nn);
+  if ((threadIdx.x & 31) == 0) snn[threadIdx.x >> 5] = nn;
+  __syncthreads();
+  const double sc = 1.0 / sqrt((snn[0] + snn[1]) + (snn[2] + snn[3]));
   double* zi = Z + (size_t)i * n;
-  for (int k = 0; k < n; ++k) zi[k] = Zs[(size_t)k * 32] * sc;
+  for (int k = threadIdx.x; k < n; k += 128) zi[k] = z[(size_t)k * 32] * f1 * f2 * sc;
 }
 
 __global__ void __launch_bounds__(32) k_eh_invit(int n, const double* __restrict__ d, const double* __restrict__ e,
@@ -478,13 +618,13 @@ __global__ void k_eh_widen(int n, int nwant, const double* __restrict__ Z, doubl
 // The upper-triangular factor of a compact-WY block, H_{k nb} ... H_{k nb + nb - 1} = I - V T V^H,
 // has the inverse S = T^-1 = diag(1 / tau_i) + (strictly upper part of G = V^H V), so
 // T = (I + diag(tau) striu(G))^-1 diag(tau): a back substitution y_q = tau_q (w_q - sum_{r > q} S_qr y_r)
-// applied to the columns w = e_c of the identity.  It needs no division and gives a zero row and
+// applied to the columns w = e_c of the identity (rows past c, and past the last of the nref reflectors, are zero).  It needs no division and gives a zero row and
 // column for an identity reflector (tau_q = 0).  Grid (kWY / 4, blocks): one warp per column of one
 // block's T; lane l holds rows l, l + 32, ...; rows are finalised from the last one, each
 // subtracting its contribution from the rows above.  G holds the blocks' Gram matrices and T receives
 // the factors (both column-major kWY x kWY per block; only the strictly upper part of G is read).
-__global__ void __launch_bounds__(128) k_eh_tfactor(const double2* __restrict__ Gall, const double2* __restrict__ tauall,
-                                                    double2* __restrict__ Tall) {
+__global__ void __launch_bounds__(128) k_eh_tfactor(int nref, const double2* __restrict__ Gall,
+                                                    const double2* __restrict__ tauall, double2* __restrict__ Tall) {
   extern __shared__ double2 gs[];   // strictly upper part of G, column q at q (q - 1) / 2
   const size_t blk = (size_t)blockIdx.y * kWY * kWY;
   const double2* G = Gall + blk;
@@ -502,7 +642,8 @@ __global__ void __launch_bounds__(128) k_eh_tfactor(const double2* __restrict__ 
   double2 acc[kWYRows];   // right-hand side rows lane + 32 s, reduced as rows finalise
 #pragma unroll
   for (int sl = 0; sl < kWYRows; ++sl) acc[sl] = make_double2(lane + 32 * sl == col ? 1.0 : 0.0, 0.0);
-  for (int q = kWY - 1; q >= 0; --q) {
+  const int top = min(col, nref - 1 - (int)blockIdx.y * kWY);
+  for (int q = top; q >= 0; --q) {
     // the owner finalises y_q = tau_q acc_q, then every row r < q subtracts S_rq y_q
     const int own = q & 31, oslot = q >> 5;
     double2 yq = make_double2(0.0, 0.0);
@@ -512,7 +653,7 @@ __global__ void __launch_bounds__(128) k_eh_tfactor(const double2* __restrict__ 
       for (int sl = 0; sl < kWYRows; ++sl)
         if (sl == oslot) {
           const double2 a = acc[sl];
-          yq = make_double2(t.x * a.x - t.y * a.y, t.x * a.y + t.y * a.x);
+          yq = make_double2(fma(t.x, a.x, -t.y * a.y), fma(t.x, a.y, t.y * a.x));
           acc[sl] = yq;
         }
     }
@@ -525,15 +666,15 @@ __global__ void __launch_bounds__(128) k_eh_tfactor(const double2* __restrict__ 
         const int r = lane + 32 * sl;
         if (r < q) {
           const double2 g = gq[r];
-          acc[sl].x -= g.x * yq.x - g.y * yq.y;
-          acc[sl].y -= g.x * yq.y + g.y * yq.x;
+          acc[sl].x = fma(g.y, yq.y, fma(-g.x, yq.x, acc[sl].x));
+          acc[sl].y = fma(-g.y, yq.x, fma(-g.x, yq.y, acc[sl].y));
         }
       }
     }
   }
   double2* t = Tall + blk + (size_t)col * kWY;
 #pragma unroll
-  for (int sl = 0; sl < kWYRows; ++sl) t[lane + 32 * sl] = acc[sl];
+  for (int sl = 0; sl < kWYRows; ++sl) t[lane + 32 * sl] = lane + 32 * sl <= top ? acc[sl] : make_double2(0.0, 0.0);
 }
 
 constexpr size_t kTrsvSmem = sizeof(double2) * (size_t)kWY * (kWY - 1) / 2;
@@ -559,8 +700,8 @@ __global__ void k_eh_tau_fix(int nref, const double* __restrict__ Gall, double* 
 }
 
 // T of a real compact-WY block from G = V^T V and tau, as k_eh_tfactor does for complex blocks.
-__global__ void __launch_bounds__(128) k_eh_tfactor_r(const double* __restrict__ Gall, const double* __restrict__ tauall,
-                                                      double* __restrict__ Tall) {
+__global__ void __launch_bounds__(128) k_eh_tfactor_r(int nref, const double* __restrict__ Gall,
+                                                      const double* __restrict__ tauall, double* __restrict__ Tall) {
   extern __shared__ double gsr[];   // strictly upper part of G, column q at q (q - 1) / 2
   const size_t blk = (size_t)blockIdx.y * kWY * kWY;
   const double* G = Gall + blk;
@@ -577,7 +718,8 @@ __global__ void __launch_bounds__(128) k_eh_tfactor_r(const double* __restrict__
   double acc[kWYRows];
 #pragma unroll
   for (int sl = 0; sl < kWYRows; ++sl) acc[sl] = lane + 32 * sl == col ? 1.0 : 0.0;
-  for (int q = kWY - 1; q >= 0; --q) {
+  const int top = min(col, nref - 1 - (int)blockIdx.y * kWY);
+  for (int q = top; q >= 0; --q) {
     const int own = q & 31, oslot = q >> 5;
     double yq = 0.0;
     if (lane == own) {
@@ -600,7 +742,7 @@ __global__ void __launch_bounds__(128) k_eh_tfactor_r(const double* __restrict__
   }
   double* t = Tall + blk + (size_t)col * kWY;
 #pragma unroll
-  for (int sl = 0; sl < kWYRows; ++sl) t[lane + 32 * sl] = acc[sl];
+  for (int sl = 0; sl < kWYRows; ++sl) t[lane + 32 * sl] = lane + 32 * sl <= top ? acc[sl] : 0.0;
 }
 
 struct EighState {
@@ -699,8 +841,7 @@ int grow(Context& c, EighState& s, int n, int nwant) {
 // solves for float64 eigenvectors, two for float32 ones.
 int invit_all(Context& c, EighState& s, int n, int nwant, int iters) {
   const int nblk = (nwant + 31) / 32;
-  const size_t per = (size_t)5 * 32 * n + (n + 1) / 2;
-  const size_t need = sizeof(double) * per * nblk;
+  const size_t need = sizeof(double) * invit_stride(n) * nblk;
   if (need > s.invcap) {
     cudaFree(s.invs);
     s.invs = nullptr;
@@ -711,8 +852,9 @@ int invit_all(Context& c, EighState& s, int n, int nwant, int iters) {
     }
     s.invcap = need;
   }
-  HPSI_LAUNCH(c, HPSI_K_EIGH, (k_eh_invit_lanes<<<nblk, 32, 0, c.stream>>>(n, s.d, s.e, nwant, s.lam, s.Z, s.invs,
+  HPSI_LAUNCH(c, HPSI_K_EIGH, (k_eh_invit_lanes<<<nblk, 32, 0, c.stream>>>(n, s.d, s.e, nwant, s.lam, s.invs,
                                                                           s.info + 1, iters)));
+  HPSI_LAUNCH(c, HPSI_K_EIGH, (k_eh_invit_finish<<<nwant, 128, 0, c.stream>>>(n, s.invs, s.Z)));
   const size_t ismem = sizeof(double) * 7 * (size_t)n + (size_t)n + 16;
   if (ismem > 48 * 1024) {
     const cudaError_t err = cudaFuncSetAttribute(k_eh_invit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ismem);
@@ -782,6 +924,10 @@ int eigh_zheevdx(Context& c, EighState& s, const double2* a, int lda, int n, int
   if (info != 0 || meig < nwant)
     return fail(c, HPSI_ESINGULAR, "zheevdx of the reduced matrix failed, info " + std::to_string(info));
   return HPSI_OK;
+}
+
+int bisect_threads(const Context& c, int nwant) {
+  return nwant <= c.sm_count ? 128 : nwant <= 2 * c.sm_count ? 64 : 32;
 }
 
 int tri_ctas(const Context& c, int n) {
@@ -860,7 +1006,8 @@ int eigh_lowest(Context& c, const double2* a, int lda, int n, int nwant, double*
   if (err != cudaSuccess) return cuda_fail(c, err, "eigh_lowest: tridiagonal reduction launch");
   // 2. eigenvalues
   HPSI_LAUNCH(c, HPSI_K_EIGH,
-              (k_eh_bisect<<<nwant, 32 * kBisWarps, 0, c.stream>>>(n, s->d, s->e, s->e2, nwant, s->lam)));
+              (k_eh_bisect<<<nwant, bisect_threads(c, nwant), sizeof(float) * 2 * n, c.stream>>>(n, s->d, s->e, s->e2, nwant,
+                                                                                                s->lam)));
   // 3. eigenvectors of T
   rc = invit_all(c, *s, n, nwant, 3);
   if (rc) return rc;
@@ -896,7 +1043,7 @@ int eigh_lowest(Context& c, const double2* a, int lda, int n, int nwant, double*
     err = cudaFuncSetAttribute(k_eh_tfactor, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrsvSmem);
     if (err != cudaSuccess) return cuda_fail(c, err, "eigh_lowest: smem attribute");
     HPSI_LAUNCH(c, HPSI_K_EIGH,
-                (k_eh_tfactor<<<dim3(kWY / 4, K), 128, kTrsvSmem, c.stream>>>(s->wgram, s->tau, s->tfac)));
+                (k_eh_tfactor<<<dim3(kWY / 4, K), 128, kTrsvSmem, c.stream>>>(n - 1, s->wgram, s->tau, s->tfac)));
     for (int k = K - 1; k >= 0; --k) {
       const int r0 = k * kWY + 1, m = n - r0;
       double2* V = s->vref + (size_t)k * kWY * n + r0;
@@ -994,7 +1141,8 @@ int eigh_lowest_real(Context& c, const double* a, int lda, int n, int nwant, dou
   if (err != cudaSuccess) return cuda_fail(c, err, "eigh_lowest_real: tridiagonal reduction launch");
   // 2. eigenvalues, 3. eigenvectors of T (the same kernels as the complex solver)
   HPSI_LAUNCH(c, HPSI_K_EIGH,
-              (k_eh_bisect<<<nwant, 32 * kBisWarps, 0, c.stream>>>(n, s->d, s->e, s->e2, nwant, s->lam)));
+              (k_eh_bisect<<<nwant, bisect_threads(c, nwant), sizeof(float) * 2 * n, c.stream>>>(n, s->d, s->e, s->e2, nwant,
+                                                                                                s->lam)));
   rc = invit_all(c, *s, n, nwant, vec32 ? 2 : 3);
   if (rc) return rc;
   const double one = 1.0, zero = 0.0, mone = -1.0, mhalf = -0.5, three_half = 1.5;
@@ -1062,7 +1210,7 @@ int eigh_lowest_real(Context& c, const double* a, int lda, int n, int nwant, dou
       return fail(c, HPSI_ECUDA, "eigh_lowest_real: reflector Gram matrices failed");
     const size_t tsm = sizeof(double) * (size_t)kWY * (kWY - 1) / 2;
     if (df) HPSI_LAUNCH(c, HPSI_K_EIGH, (k_eh_tau_fix<<<(n - 1 + 255) / 256, 256, 0, c.stream>>>(n - 1, wgram, tau)));
-    HPSI_LAUNCH(c, HPSI_K_EIGH, (k_eh_tfactor_r<<<dim3(kWY / 4, K), 128, tsm, c.stream>>>(wgram, tau, tfac)));
+    HPSI_LAUNCH(c, HPSI_K_EIGH, (k_eh_tfactor_r<<<dim3(kWY / 4, K), 128, tsm, c.stream>>>(n - 1, wgram, tau, tfac)));
     if (vec32) {
       const size_t nv = (size_t)K * kWY * n, nt = (size_t)K * kWY * kWY;
       float* vr32 = reinterpret_cast<float*>(vref + (size_t)(n + kWY) * n);

@@ -5,6 +5,7 @@
 
 #include <cuda_runtime.h>
 
+#include "convert.cuh"
 #include "hpsi_internal.h"
 
 namespace hpsi {
@@ -100,28 +101,23 @@ __device__ bool grid_wait(unsigned int* count, unsigned int target, int* err) {
 
 __device__ __forceinline__ int biased_exp(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff); }
 
-// 1/x by two Newton-Raphson steps r <- r (2 - x r) from a float32 seed (quadratic convergence:
-// 2^-23 -> 2^-46 -> 2^-92); plain division outside |x| in [2^-100, 2^100].  Four float64
-// operations instead of the 600-cycle division sequence.
+// 1/x by one third-order step r <- r (1 + e + e^2), e = 1 - x r, from a float32 seed (relative error 2^-23 -> 2^-69 before
+// rounding); plain division outside |x| in [2^-100, 2^100].  Three float64 operations instead of the 600-cycle
+// division sequence; the conversions run on the integer pipe.
 __device__ __forceinline__ double recip_nr(double x) {
   const int ex = biased_exp(x);
   if (ex < 1023 - 100 || ex > 1023 + 100) return 1.0 / x;
-  double r = (double)__frcp_rn((float)x);
-  r = fma(r, fma(-x, r, 1.0), r);
-  r = fma(r, fma(-x, r, 1.0), r);
-  return r;
+  const double r = f32_to_f64(__frcp_rn(f64_to_f32(x))), e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
 }
 
-// 1/sqrt(x) for x > 0 by two Newton steps y <- y (3/2 - (x/2) y^2) from a float32 seed; library
+// 1/sqrt(x) for x > 0 by one third-order step y <- y + y e (1/2 + 3/8 e), e = 1 - x y^2, from a float32 seed; library
 // sqrt and division outside x in [2^-100, 2^100].
 __device__ __forceinline__ double rsqrt_nr(double x) {
   const int ex = biased_exp(x);
   if (ex < 1023 - 100 || ex > 1023 + 100) return 1.0 / sqrt(x);
-  const double h = 0.5 * x;
-  double y = (double)rsqrtf((float)x);
-  y = y * fma(-h, y * y, 1.5);
-  y = y * fma(-h, y * y, 1.5);
-  return y;
+  const double y = f32_to_f64(rsqrtf(f64_to_f32(x))), e = fma(-x * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 // Column chunk of one of q parts of a row of m columns, rounded up to whole warps (no division).
