@@ -937,7 +937,7 @@ int tri_ctas(const Context& c, int n) {
 
 size_t tri_smem(int n, int G) {
   const int R = (n + G - 1) / G;
-  return sizeof(double2) * ((size_t)(3 + R) * n + 8 * (size_t)R);
+  return sizeof(double2) * ((size_t)(3 + R) * n + 9 * (size_t)R);
 }
 
 size_t tri_smem_r(int n, int G) {

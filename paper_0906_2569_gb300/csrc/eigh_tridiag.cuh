@@ -37,6 +37,39 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// warp_sum on the integer pipes: the lanes' values as multiples of 2^-57 of the largest exponent, summed exactly by three
+// 32-bit reductions; each rounding is 2^-6 of the largest value's last bit.  A
+// float64 addition holds its scheduler for ~78 cycles and a shuffle tree is five of them in a row; this is ~60 integer
+// instructions.  Infinities, NaN and subnormal maxima take the tree.
+__device__ __forceinline__ double warp_sum_int(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const int ex = (int)(b >> 52) & 0x7ff;
+  const int mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)ex);
+  if (mx == 0x7ff || mx < 64) return warp_sum(v);
+  unsigned long long m = ex ? ((b & 0xfffffffffffffULL) | (1ULL << 52)) << 5 : 0ULL;
+  const int sh = mx - ex;
+  m = sh < 60 ? (m + ((1ULL << sh) >> 1)) >> sh : 0ULL;
+  const long long sg = (long long)b >> 63;
+  const long long x = ((long long)m ^ sg) - sg;
+  const unsigned s0 = __reduce_add_sync(0xffffffffu, (unsigned)x & 0x3ffffffu);
+  const unsigned s1 = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 26) & 0x3ffffffu);
+  const int s2 = __reduce_add_sync(0xffffffffu, (int)(x >> 52));
+  const long long t = ((long long)s2 << 52) + ((long long)s1 << 26) + (long long)s0;
+  if (t == 0) return 0.0;
+  const unsigned long long neg = (unsigned long long)(t >> 63);
+  unsigned long long a = ((unsigned long long)t ^ neg) - neg;
+  const int lz = __clzll((long long)a);
+  a <<= lz;                                   // leading bit at 63: value a 2^(mx - 1023 - 57 - lz)
+  const unsigned long long low = a & 0x7ff;
+  a >>= 11;
+  a += low > 0x400 || (low == 0x400 && (a & 1));
+  // a in [2^52, 2^53]: its leading bit (or the carry) adds one to the exponent field below
+  const long long e = mx + 5 - lz;            // exponent field - 1 of the result; mx >= 64 keeps it positive
+  const long long out = (long long)(((unsigned long long)e << 52) + a);
+  if (e >= 0x7fe) return warp_sum(v);
+  return __longlong_as_double((long long)(neg << 63) | out);
+}
+
 // Element (r, c) of the Hermitian matrix whose upper triangle is a (column-major, leading dim lda).
 __device__ __forceinline__ double2 herm_at(const double2* __restrict__ a, int lda, int r, int c) {
   if (r <= c) {
@@ -126,6 +159,14 @@ __device__ __forceinline__ int split_chunk(int m, int q) {
   return (c + 31) & ~31;
 }
 
+// 2 x and x / 2 through the exponent field (a value too small for that halves to zero)
+__device__ __forceinline__ double times2(double x) {
+  return biased_exp(x) == 0 ? x + x : __hiloint2double(__double2hiint(x) + (1 << 20), __double2loint(x));
+}
+__device__ __forceinline__ double half_of(double x) {
+  return biased_exp(x) < 2 ? 0.0 : __hiloint2double(__double2hiint(x) - (1 << 20), __double2loint(x));
+}
+
 __device__ __forceinline__ double2 cmulc2(double2 a, double2 b) {   // a * conj(b)
   return make_double2(fma(a.x, b.x, a.y * b.y), fma(a.y, b.x, -a.x * b.y));
 }
@@ -156,18 +197,19 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_eh_tridiag(TriArgs p) {
   double2* cA = rows + (size_t)Rmax * n;   // [Rmax] A_r, B_r, Q_r of the own rows
   double2* cB = cA + Rmax;
   double2* cQ = cB + Rmax;
-  double2* pacc = cQ + Rmax;               // [4 Rmax] quarter (or whole-row) sums with conj(u)
+  double2* cP = cQ + Rmax;                 // [Rmax] P_r
+  double2* pacc = cP + Rmax;               // [4 Rmax] quarter (or whole-row) sums with conj(u)
   double2* pa1 = pacc + 4 * Rmax;          // [Rmax] element at column j+1 of each row
   __shared__ double red[NW];
-  __shared__ double2 alpha_sh, tau_sh, scale_sh, tcs_sh, cts_sh;
-  __shared__ double beta_sh, s2_sh;
+  __shared__ double2 alpha_sh, tau_sh, scale_sh;
+  __shared__ double beta_sh, prod_sh[7];
 
   for (int lr = 0; lr < R; ++lr) {
     const int r = g + lr * G;
     for (int c = tid; c < n; c += kTriThreads) rows[(size_t)lr * n + c] = herm_at(p.a, p.lda, r, c);
   }
   double2 scP = make_double2(0.0, 0.0);
-  double tauAbs2 = 0.0;   // |tau_{j-1}|^2
+  double tauAbs2 = 0.0;   // |tau_{j-1}|^2 / 2
   int first = 0;          // the own rows r > j are lr = first .. R-1
   int jmodG = 0;          // j mod G: this CTA owns row j when jmodG == g
   for (int j = 0; j < n; ++j, jmodG = jmodG + 1 == G ? 0 : jmodG + 1) {
@@ -212,8 +254,8 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_eh_tridiag(TriArgs p) {
           if (j > 0) yP[c] = ya[k];
         }
       }
-      if (j > 0) {
-        hh = 0.5 * tauAbs2 * sv;
+      if (j > 0 && (j + wid * 32 < n || wid == 4)) {   // the warps that use them
+        hh = tauAbs2 * sv;
         Pj = make_double2(fma(-hh, B.x, A.x), fma(-hh, B.y, A.y));
       }
     }
@@ -224,7 +266,7 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_eh_tridiag(TriArgs p) {
     for (int c = j + tid; c < n; c += kTriThreads) {
       double2 a = uC[c];
       if (c == j) {
-        dj = a.x - (Ej - 2.0 * hh);
+        dj = a.x;   // its update is made where it is stored
       } else {
         if (j > 0) a = rank2_sub(a, Pj, make_double2(uP[c].x, -uP[c].y), Qj, yP[c]);
         uC[c] = a;
@@ -233,19 +275,21 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_eh_tridiag(TriArgs p) {
       }
     }
     if (j == n - 1) {
-      if (g == 0 && tid == 0) p.d[j] = dj;
+      if (g == 0 && tid == 0) p.d[j] = dj - (Ej - 2.0 * hh);
       break;
     }
-    sig = warp_sum(sig);
+    if (j + wid * 32 < n) sig = warp_sum_int(sig);   // warp-uniform
     if (lane == 0) red[wid] = sig;
+    if (wid == 4 && j > 0)   // P of the own rows, a lane each
+      for (int i = lane; i < Ra; i += 32) {
+        const int lr = first + i;
+        cP[lr] = make_double2(fma(-hh, cB[lr].x, cA[lr].x), fma(-hh, cB[lr].y, cA[lr].y));
+      }
     __syncthreads();
     // (C) the chain warp: beta, tau, scale of column j;  all warps: own rows r > j, in parts
     if (wid == kChainWarp) {
-      double sg = lane < NW ? red[lane] : 0.0;
-      sg += __shfl_xor_sync(0xffffffffu, sg, 4);
-      sg += __shfl_xor_sync(0xffffffffu, sg, 2);
-      sg += __shfl_xor_sync(0xffffffffu, sg, 1);
-      if (lane == 0) {
+      const double sg = warp_sum_int(lane < NW ? red[lane] : 0.0);
+      {   // in every lane: the products of tau and scale below are one lane each
         const double ar = alpha_sh.x, ai = alpha_sh.y;
         double beta;
         double2 tau, scale;
@@ -264,12 +308,19 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_eh_tridiag(TriArgs p) {
           const double iden = recip_nr(fma(dr, dr, ai * ai));
           scale = make_double2(dr * iden, -ai * iden);       // 1 / (alpha - beta)
         }
-        tau_sh = tau;
-        scale_sh = scale;
-        beta_sh = beta;
-        tcs_sh = cmulc2(tau, scale);                                         // tau conj(scale)
-        cts_sh = cmul(make_double2(tau.x, -tau.y), scale);                   // conj(tau) scale
-        s2_sh = 2.0 * fma(scale.x, scale.x, scale.y * scale.y);              // 2 |scale|^2
+        // a b + c d by lane: tau conj(scale), conj(tau) scale, 2 |scale|^2, beta^2, |tau|^2 / 2
+        const double sx = scale.x, sy = scale.y, tx = tau.x, ty = tau.y;
+        const double pa = lane == 4 ? times2(sx) : lane == 5 ? beta : lane == 6 ? half_of(tx) : tx;
+        const double pb = lane == 5 ? beta : lane == 6 ? tx : lane == 1 ? -sy : lane == 3 ? sy : sx;
+        const double pc = lane == 4 ? times2(sy) : lane == 5 ? 0.0 : lane == 6 ? half_of(ty) : lane == 3 ? -ty : ty;
+        const double pd = lane == 6 ? ty : lane == 0 || lane == 2 || lane == 4 ? sy : sx;
+        const double pr = fma(pa, pb, pc * pd);
+        if (lane == 0) {
+          tau_sh = tau;
+          scale_sh = scale;
+          beta_sh = beta;
+        }
+        if (lane < 7) prod_sh[lane] = pr;
       }
     }
     if (Ra > 0) {
@@ -299,8 +350,7 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_eh_tridiag(TriArgs p) {
         const int lr = first + i;
         const int r = g + lr * G;
         double2* row = rows + (size_t)lr * n;
-        const double2 P = make_double2(fma(-hh, cB[lr].x, cA[lr].x), fma(-hh, cB[lr].y, cA[lr].y));
-        const double2 Q = cQ[lr];
+        const double2 P = cP[lr], Q = cQ[lr];
         double ax = 0.0, ay = 0.0, bx = 0.0, by = 0.0;
         double2 a1 = make_double2(0.0, 0.0);
         for (int c = c0 + lane; c < c1; c += 64) {
@@ -333,8 +383,12 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_eh_tridiag(TriArgs p) {
             if (two) p.rnext[(j & 1) * n + c2] = b;
           }
         }
-        ax = warp_sum(ax + bx);
-        ay = warp_sum(ay + by);
+        if (c1 - c0 > 32) {
+          ax += bx;
+          ay += by;
+        }
+        ax = warp_sum_int(ax);
+        ay = warp_sum_int(ay);
         if (lane == 0) {
           pacc[i * 4 + k] = make_double2(ax, ay);
           if (k == 0) pa1[i] = a1;
@@ -347,8 +401,8 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_eh_tridiag(TriArgs p) {
     //     the owner of row j stores v_j; CTA 0 the outputs of column j
     const double2 tauC = tau_sh, scC = scale_sh;
     const double2 cscC = make_double2(scC.x, -scC.y);
-    const double2 tcs = tcs_sh, cts = cts_sh;
-    const double s2 = s2_sh;
+    const double2 tcs = make_double2(prod_sh[0], prod_sh[1]), cts = make_double2(prod_sh[2], prod_sh[3]);
+    const double s2 = prod_sh[4];
     // the own rows' y_j (lanes of warps 0 and 1 over the rows) and the coefficients of column j's
     // update for row lr: A = tau y conj(scale), B = 2 v conj(scale), Q = conj(tau) v
     auto row_y = [&](int i) {
@@ -377,13 +431,13 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_eh_tridiag(TriArgs p) {
         sp += r == j + 1 ? y.x
                          : fma(uC[r].x, fma(cscC.x, y.x, -cscC.y * y.y), -uC[r].y * fma(cscC.x, y.y, cscC.y * y.x));
       }
-      sp = warp_sum(sp);
+      sp = warp_sum_int(sp);
       if (lane == 0) {
         atomicAdd(&p.sacc[j & 3], sp);
         if (g == 0) {
-          p.d[j] = dj;
+          p.d[j] = dj - (Ej - 2.0 * hh);
           p.e[j] = beta_sh;
-          p.e2[j] = beta_sh * beta_sh;
+          p.e2[j] = prod_sh[5];
           p.tau[j] = tauC;
           p.vscale[j] = scC;
         }
@@ -414,7 +468,7 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_eh_tridiag(TriArgs p) {
         cQ[lr] = Q;
       }
     }
-    tauAbs2 = fma(tauC.x, tauC.x, tauC.y * tauC.y);
+    tauAbs2 = prod_sh[6];
     scP = scC;
     if (!grid_wait(p.bar, (unsigned)(G * (j + 1)), p.err)) return;
   }
