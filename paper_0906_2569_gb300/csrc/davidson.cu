@@ -1147,6 +1147,11 @@ struct MixedOps {
     int rc = apply_device(c, ik, w.in64, w.out64, N);
     final_precision_end(c);
     if (rc) return rc;
+    if (c.final_fp64 && w.mmax >= 2 * N) {   // the float32 basis is free now: room for N float64 rows
+      auto D = [](void* q) { return static_cast<double*>(q); };
+      rc = ritz_refine(c, N, npw, false, D(w.in64), D(w.out64), D(w.hsub), D(w.phi32), D(w.hphi32));
+      if (rc) return rc;
+    }
     HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k_rayleigh<<<N, 1024, 0, c.stream>>>(npw, w.in64, w.out64, w.eps, w.rnorm)));
     DCK(cudaMemcpyAsync(ev.data(), w.eps, sizeof(double) * N, cudaMemcpyDeviceToHost, c.stream), "eig copy");
     DCK(cudaMemcpyAsync(rn.data(), w.rnorm, sizeof(double) * N, cudaMemcpyDeviceToHost, c.stream), "norm copy");

@@ -1232,6 +1232,10 @@ int GammaDavidson<T>::run(int N, double tol, int maxiter, double2* psio, double*
                                 N, true);
     final_precision_end(c);
     if (rc) return rc;
+    if (c.final_fp64 && mmax >= 2 * N) {   // the float32 basis is free now: room for N float64 rows
+      rc = ritz_refine(c, N, n2, true, w.x64, w.hx64, w.hsub, static_cast<double*>(w.phi), static_cast<double*>(w.hphi));
+      if (rc) return rc;
+    }
     HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k_g_rayleigh<<<N, 512, 0, c.stream>>>(n2, w.x64, w.hx64, w.eps, w.rnorm)));
     GCK(cudaMemcpyAsync(ev.data(), w.eps, sizeof(double) * N, cudaMemcpyDeviceToHost, c.stream), "eig copy");
     GCK(cudaMemcpyAsync(rn.data(), w.rnorm, sizeof(double) * N, cudaMemcpyDeviceToHost, c.stream), "norm copy");

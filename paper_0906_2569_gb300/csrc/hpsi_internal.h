@@ -365,9 +365,12 @@ int gamma_slices_w(Context& c, const Problem& p, const void* x, bool x32, int nb
 int gamma_slices_add(Context& c, const Problem& p, const double* w, double* out, int nbnd, bool* ok);
 // Subspace products of float64 blocks of rows [.][npw] (subspace_fp64.cu): out[i + j ldo] = <a_i|b_j>, and
 // out_j = (accumulate ? out_j : 0) + sign sum_i coef[i + j ldc] a_i (out may be none of the a_i).  Work in ws.part and ws.mixed.
-int fp64_inner(Context& c, const double2* a, int m, const double2* b, int n, int npw, double2* out, int ldo);
+int fp64_inner(Context& c, const double2* a, int m, const double2* b, int n, int npw, double2* out, int ldo,
+               int ld = 0);
 int fp64_outer(Context& c, const double2* a, int k, const double2* coef, int ldc, int n, int npw, double sign,
-               bool accumulate, double2* out);
+               bool accumulate, double2* out, int ld = 0);
+// Rotation of n nearly converged Ritz vectors by the first-order eigenvectors of their float64 H and overlap matrices
+int ritz_refine(Context& c, int n, int len, bool real, double* x, double* hx, double* small, double* tx, double* thx);
 // Their form on the tensor cores, for complex or real rows of len entries; *ok = false: no room for the digit planes
 int slices_inner(Context& c, const double* a, int m, const double* b, int n, int len, bool real, double* out, int ldo,
                  bool* ok);

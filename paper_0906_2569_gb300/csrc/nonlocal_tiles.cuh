@@ -33,7 +33,8 @@ constexpr int CB_SMEM = (CB_TP + CB_TB) * (CB_TK + 1);   // double2 entries of s
 template <int TP>
 __device__ __forceinline__ void calbec_tile_t(int npw, int nproj, int nb, int kchunk, const double2* __restrict__ beta,
                                               const double2* __restrict__ psi, double2* __restrict__ part, int tp,
-                                              int tb, int split, double2* sm) {
+                                              int tb, int split, double2* sm, int ld = 0) {
+  const int row = ld ? ld : npw;               // elements from one row to the next
   constexpr int TX = TP < 16 ? TP : 16;        // threads along the projectors
   constexpr int TY = 256 / TX;                 // threads along the bands
   constexpr int PI = TP / TX, BJ = CB_TB / TY; // outputs per thread
@@ -52,12 +53,12 @@ __device__ __forceinline__ void calbec_tile_t(int npw, int nproj, int nb, int kc
     for (int i = threadIdx.x; i < TP * CB_TK; i += 256) {
       const int r = i / CB_TK, cc = i % CB_TK;
       const int g = g0 + cc;
-      sb[r][cc] = (p0 + r < nproj && g < gend) ? beta[(size_t)(p0 + r) * npw + g] : make_double2(0.0, 0.0);
+      sb[r][cc] = (p0 + r < nproj && g < gend) ? beta[(size_t)(p0 + r) * row + g] : make_double2(0.0, 0.0);
     }
     for (int i = threadIdx.x; i < CB_TB * CB_TK; i += 256) {
       const int r = i / CB_TK, cc = i % CB_TK;
       const int g = g0 + cc;
-      sp[r][cc] = (b0 + r < nb && g < gend) ? psi[(size_t)(b0 + r) * npw + g] : make_double2(0.0, 0.0);
+      sp[r][cc] = (b0 + r < nb && g < gend) ? psi[(size_t)(b0 + r) * row + g] : make_double2(0.0, 0.0);
     }
     __syncthreads();
     // a float64 instruction costs the same for one lane as for 32, so a warp whose bands are all padding skips the sum

@@ -21,10 +21,10 @@ namespace {
 #include "nonlocal_tiles.cuh"
 
 template <int TP>
-__global__ void __launch_bounds__(256) k_sub_inner(int npw, int m, int n, int kchunk, const double2* __restrict__ a,
+__global__ void __launch_bounds__(256) k_sub_inner(int npw, int ld, int m, int n, int kchunk, const double2* __restrict__ a,
                                                    const double2* __restrict__ b, double2* __restrict__ part) {
   __shared__ double2 sm[CB_SMEM];
-  calbec_tile_t<TP>(npw, m, n, kchunk, a, b, part, blockIdx.x, blockIdx.y, blockIdx.z, sm);
+  calbec_tile_t<TP>(npw, m, n, kchunk, a, b, part, blockIdx.x, blockIdx.y, blockIdx.z, sm, ld);
 }
 
 // out[i + j ldo] = sum of the splits of part[split][j][i]
@@ -45,7 +45,7 @@ constexpr int SO_G = 32, SO_B = 4, SO_K = 16;
 
 // out[j][g] = (acc ? out[j][g] : 0) + sign sum_i a[i][g] c[i + j ldc]: one output per thread, so that a few thousand plane
 // waves by a few rows still occupy every scheduler
-__global__ void __launch_bounds__(SO_G* SO_B) k_sub_outer(int npw, int k, int n, double sign, int acc,
+__global__ void __launch_bounds__(SO_G* SO_B) k_sub_outer(int npw, int ld, int k, int n, double sign, int acc,
                                                           const double2* __restrict__ a, const double2* __restrict__ c,
                                                           int ldc, double2* __restrict__ out) {
   __shared__ double2 sa[SO_K][SO_G], sc[SO_B][SO_K];
@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(SO_G* SO_B) k_sub_outer(int npw, int k, int n,
   double2 s = make_double2(0.0, 0.0);
   for (int i0 = 0; i0 < k; i0 += SO_K) {
     const int ni = min(SO_K, k - i0);
-    for (int i = ty; i < ni; i += SO_B) sa[i][tx] = g < npw ? a[(size_t)(i0 + i) * npw + g] : make_double2(0.0, 0.0);
+    for (int i = ty; i < ni; i += SO_B) sa[i][tx] = g < npw ? a[(size_t)(i0 + i) * ld + g] : make_double2(0.0, 0.0);
     if (threadIdx.x < SO_B * SO_K) {
       const int jj = threadIdx.x / SO_K, i = threadIdx.x % SO_K;
       double2 v = make_double2(0.0, 0.0);
@@ -68,16 +68,88 @@ __global__ void __launch_bounds__(SO_G* SO_B) k_sub_outer(int npw, int k, int n,
     __syncthreads();
   }
   if (g < npw && j < n) {
-    double2* o = out + (size_t)j * npw + g;
+    double2* o = out + (size_t)j * ld + g;
     *o = acc ? make_double2(o->x + s.x, o->y + s.y) : s;
+  }
+}
+
+// K[i + j n]: the first-order anti-Hermitian mixing of x_i and x_j in the eigenvectors of (H, S), where H_ij = <x_i|H x_j> is
+// nearly diagonal and S nearly the identity; zero where it would be above 3e-4 (near degeneracy).  The Hermitian part of H
+// alone: the rounding of h x in its float32 local term is not symmetric, and would come back as a lost
+// orthogonality over the gap.
+template <int CW>
+__global__ void __launch_bounds__(256) k_ritz_mix(int n, const double* __restrict__ H, const double* __restrict__ S,
+                                                  double* __restrict__ K) {
+  const size_t t = (size_t)blockIdx.x * 256 + threadIdx.x;
+  if (t >= (size_t)n * n) return;
+  const int i = (int)(t % n), j = (int)(t / n);
+  const size_t di = CW * (size_t)i * (n + 1), dj = CW * (size_t)j * (n + 1), u = CW * ((size_t)i * n + j);
+  const double ei = H[di] / S[di], ej = H[dj] / S[dj], g = ej - ei, em = 0.5 * (ei + ej);
+  double v[CW], top = 0.0;
+  for (int k = 0; k < CW; ++k) {
+    v[k] = 0.5 * (H[CW * t + k] + (k == 0 ? H[u] : -H[u + k])) - em * S[CW * t + k];
+    top = fmax(top, fabs(v[k]));
+  }
+  const bool apart = i != j && top <= 3e-4 * fabs(g) && g != 0.0;
+  for (int k = 0; k < CW; ++k) K[CW * t + k] = apart ? v[k] / g : 0.0;
+}
+// C = (1 + K + K^2 / 2 - (S - 1) / 2), column j over the norm of x_j: orthonormal to the third order of K
+template <int CW>
+__global__ void __launch_bounds__(256) k_ritz_rotation(int n, const double* __restrict__ K, const double* __restrict__ S,
+                                                       double* __restrict__ C) {
+  const size_t t = (size_t)blockIdx.x * 256 + threadIdx.x;
+  if (t >= (size_t)n * n) return;
+  const int i = (int)(t % n), j = (int)(t / n);
+  double q[2] = {0.0, 0.0};
+  for (int l = 0; l < n; ++l) {
+    const size_t a = CW * ((size_t)l * n + i), b = CW * ((size_t)j * n + l);
+    q[0] = fma(K[a], K[b], q[0]);
+    if (CW == 2) {
+      q[0] = fma(-K[a + 1], K[b + 1], q[0]);
+      q[1] = fma(K[a], K[b + 1], fma(K[a + 1], K[b], q[1]));
+    }
+  }
+  const double norm = 1.0 / sqrt(S[CW * (size_t)j * (n + 1)]);
+  for (int k = 0; k < CW; ++k) {
+    const double one = i == j && k == 0 ? 1.0 : 0.0;
+    C[CW * t + k] = norm * (one + K[CW * t + k] + 0.5 * q[k] - (i == j ? 0.0 : 0.5 * S[CW * t + k]));
   }
 }
 
 }  // namespace
 
-int fp64_inner(Context& c, const double2* a, int m, const double2* b, int n, int npw, double2* out, int ldo) {
+// The vectors of a float32 basis carry rounding noise that the Rayleigh-Ritz step turns into mixing of neighbours, noise
+// over their gap (1e-5 at a gap of 1e-3 Ha): most of the vectors' error, and the part that varies between equally accurate
+// forms of H|psi>.  x and h x are at hand in float64 for the quotients, so the mixing inside the block is taken out to first
+// order: two N x N products and two rotations as digit products (32 vectors of 2.4e3 plane waves: 0.2 of 28 ms).
+// small: 3 N^2, tx and thx: N rows of len (complex or real).  Without room for the digits x stays as it is.
+int ritz_refine(Context& c, int n, int len, bool real, double* x, double* hx, double* small, double* tx, double* thx) {
+  if (n < 2) return HPSI_OK;
+  const size_t nn = (size_t)n * n * (real ? 1 : 2), bytes = sizeof(double) * (real ? 1 : 2) * (size_t)n * len;
+  double *H = small, *S = small + nn, *K = S + nn;
+  bool ok = false;
+  int rc = slices_inner(c, x, n, hx, n, len, real, H, n, &ok);
+  if (!rc && ok) rc = slices_inner(c, x, n, x, n, len, real, S, n, &ok);
+  if (rc || !ok) return rc;
+  const unsigned grid = (unsigned)(((size_t)n * n + 255) / 256);
+  if (real) HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k_ritz_mix<1><<<grid, 256, 0, c.stream>>>(n, H, S, K)));
+  else HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k_ritz_mix<2><<<grid, 256, 0, c.stream>>>(n, H, S, K)));
+  double* C = H;
+  if (real) HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k_ritz_rotation<1><<<grid, 256, 0, c.stream>>>(n, K, S, C)));
+  else HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k_ritz_rotation<2><<<grid, 256, 0, c.stream>>>(n, K, S, C)));
+  rc = slices_outer(c, x, n, C, n, n, len, real, 1.0, false, tx, &ok);
+  if (!rc && ok) rc = slices_outer(c, hx, n, C, n, n, len, real, 1.0, false, thx, &ok);
+  if (rc || !ok) return rc;
+  cudaError_t e = cudaMemcpyAsync(x, tx, bytes, cudaMemcpyDeviceToDevice, c.stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(hx, thx, bytes, cudaMemcpyDeviceToDevice, c.stream);
+  if (e != cudaSuccess) return cuda_fail(c, e, "refinement of the Ritz vectors");
+  return HPSI_OK;
+}
+
+int fp64_inner(Context& c, const double2* a, int m, const double2* b, int n, int npw, double2* out, int ldo, int ld) {
   if (m < 1 || n < 1) return HPSI_OK;
-  if ((double)m * n * npw >= kDigitMacs) {
+  if (ld == 0) ld = npw;
+  if (ld == npw && (double)m * n * npw >= kDigitMacs) {
     bool ok = false;
     const int rc = slices_inner(c, reinterpret_cast<const double*>(a), m, reinterpret_cast<const double*>(b), n, npw, false,
                                 reinterpret_cast<double*>(out), ldo, &ok);
@@ -93,7 +165,7 @@ int fp64_inner(Context& c, const double2* a, int m, const double2* b, int n, int
   if (rc) return rc;
   double2* part = static_cast<double2*>(c.ws.part);
   const dim3 grid((m + tp - 1) / tp, (n + CB_TB - 1) / CB_TB, ns);
-  auto go = [&](auto k) { HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k<<<grid, 256, 0, c.stream>>>(npw, m, n, kc, a, b, part))); };
+  auto go = [&](auto k) { HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k<<<grid, 256, 0, c.stream>>>(npw, ld, m, n, kc, a, b, part))); };
   if (tp == 8) go(k_sub_inner<8>);
   else go(k_sub_inner<CB_TP>);
   HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k_sub_reduce<<<(m * n + 127) / 128, 128, 0, c.stream>>>(m, n, ns, part, out, ldo)));
@@ -103,9 +175,10 @@ int fp64_inner(Context& c, const double2* a, int m, const double2* b, int n, int
 }
 
 int fp64_outer(Context& c, const double2* a, int k, const double2* coef, int ldc, int n, int npw, double sign,
-               bool accumulate, double2* out) {
+               bool accumulate, double2* out, int ld) {
   if (n < 1) return HPSI_OK;
-  if ((double)k * n * npw >= kDigitMacs) {
+  if (ld == 0) ld = npw;
+  if (ld == npw && (double)k * n * npw >= kDigitMacs) {
     bool ok = false;
     const int rc = slices_outer(c, reinterpret_cast<const double*>(a), k, reinterpret_cast<const double*>(coef), ldc, n, npw,
                                 false, sign, accumulate, reinterpret_cast<double*>(out), &ok);
@@ -113,7 +186,7 @@ int fp64_outer(Context& c, const double2* a, int k, const double2* coef, int ldc
   }
   HPSI_LAUNCH(c, HPSI_K_DAVIDSON,
               (k_sub_outer<<<dim3((npw + SO_G - 1) / SO_G, (n + SO_B - 1) / SO_B), SO_G * SO_B, 0, c.stream>>>(
-                  npw, k, n, sign, accumulate ? 1 : 0, a, coef, ldc, out)));
+                  npw, ld, k, n, sign, accumulate ? 1 : 0, a, coef, ldc, out)));
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "subspace combinations");
   return HPSI_OK;

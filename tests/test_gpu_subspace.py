@@ -47,3 +47,33 @@ def test_solve_block_sizes(lib, nbnd, real):
     assert np.max(np.abs(v.conj() @ v.T - np.eye(nbnd))) < 1e-12
     hv = oracle.hamiltonian.hpsi(p.lattice, k, m, p.fft, vr, beta, d, v)
     assert np.max(np.linalg.norm(hv - eig[:, None] * v, axis=1)) < 1e-8 + 1e-12
+
+
+@pytest.mark.parametrize("nbnd,real", [(2, True), (33, True), (240, True), (2, False), (33, False), (130, False)])
+def test_mixed_vectors_refined(lib, nbnd, real):
+    """The float32 basis's vectors leave the solver refined in float64: rows of a float32 block are orthogonal to ~3e-7, refined ones
+    to second order in the mixing taken out (1e-5 noise over gap), summed over the block: 1e-10 a band."""
+    import torch
+    from paper_0906_2569_gb300 import binding as B
+    p = workloads.config3(nbnd)
+    k = p.kpts[0]
+    m = B.hpsi_gsphere(p.lattice, p.ecut, k)
+    npw = len(m)
+    vr = workloads.vloc_r(p.lattice, p.atoms, p.fft)
+    ctx = B.hpsi_setup(p.lattice, p.ecut, [k], p.fft, vr, [workloads.beta(p.lattice, p.atoms, k, m)],
+                       workloads.dmat(len(p.atoms)), B.HPSI_MIXED, torch.cuda.current_stream().cuda_stream)
+    psi = workloads.psi0(p.lattice, k, m, nbnd, p.psi_seed)
+    if real:
+        psi = psi[:, npw // 2:].copy()
+        psi[:, 0] = psi[:, 0].real
+    x = torch.from_numpy(psi).cuda()
+    eig, _, res, _ = (B.davidson_solve_gamma if real else B.davidson_solve)(ctx, 0, x, 1e-5, 200)
+    ctx.close()
+    ref = np.asarray(json.load(open(GOLDEN))["c3"]["eigenvalues"])[:nbnd]
+    assert np.max(np.abs(eig - ref)) < 1e-6
+    assert np.max(res) < 1e-5
+    v = x.cpu().numpy()
+    if real:
+        v = np.concatenate([v[:, 1:][:, ::-1].conj(), v], axis=1)
+    o = v.conj() @ v.T
+    assert np.max(np.abs(o - np.diag(np.diag(o)))) < 1e-10 * max(nbnd, 10)
