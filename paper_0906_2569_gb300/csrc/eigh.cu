@@ -151,7 +151,7 @@ __device__ int sturm_count32(int n, const float* d, const float* e2, float sigma
 //     bracket then shrinks to the estimate's error, two or three rounds in all.  A round of that kind that gains less
 //     than a factor 32 is followed by an even one.
 // Four warps while the chip has an SM for each eigenvalue, two while it has half a one: a scheduler carries one warp.
-// 640 rows, 160 wanted: 1.09 -> 0.3 ms; up to 64 rows, 16 wanted: 97 -> 41 us.
+// 640 rows, 160 wanted: 1.09 -> 0.39 ms; up to 64 rows, 16 wanted: 97 -> 41 us.
 constexpr int kBisWarps = 4;
 __global__ void __launch_bounds__(32 * kBisWarps) k_eh_bisect(int n, const double* __restrict__ d,
                                                               const double* __restrict__ e,

@@ -13,7 +13,7 @@
 // What bounds it: instruction issue (a codelet's ~10 float32 instructions a value and stage, a load, a store and their
 // addresses) and the barriers between stages.  Measured with 160 bands on 90^3: planes 729 -> 594 us, z kernels 295 ->
 // 240 us against register codelets with a fixed line group per warp (24 to 30 of 32 lanes busy, cubic boxes of
-// 20 edges only); 81^3, which had only the generic kernels, H|psi> 8.2 -> 1.0 ms.
+// 20 edges only; the others had the generic kernels).
 //
 // The raw form takes float32 psi and gives the local term alone in float32, [nb][npw] both: the Gamma form packs two
 // real bands into one complex one in float32 and adds the kinetic term itself (gamma.cu).

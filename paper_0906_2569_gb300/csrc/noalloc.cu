@@ -6,8 +6,8 @@
 // asynchronous stream pipeline.  This entry point computes the same H|psi> as hpsi_apply, but
 // every intermediate (the plane and stick buffers of the FFTs, the partial sums of <beta|psi>
 // and D<beta|psi>) lives in one fixed array compiled into the library.  Bands are processed in
-// chunks that fit the array.  The local term runs on the register-codelet kernels where the box
-// has them (with the plan chosen at setup or by an earlier hpsi_apply), else on the generic ones;
+// chunks that fit the array.  The local term runs on the two-codelet kernels where the box has
+// them (fixed point in float64, float32 in a mixed context), else on the generic ones;
 // the nonlocal term runs on the float64 kernels at either precision (they need no buffers beyond
 // the array).
 #include <cuda_runtime.h>
