@@ -337,9 +337,10 @@ struct FastLaunch {
     }
     const int nz = bt.off_z[bt.nitems], np = bt.off_p[bt.nitems];
     auto warps = [](int items) { return (items + 31) / 32 * 32; };
-    // z: one round of a stage's items; planes: plane_shape's block, or one round where there is a CTA per SM at most
+    // z: one round of a stage's items; planes: plane_shape's block, or one round where there is a CTA per SM at most;
+    // never more than this instance's launch bound, which another item's radix may have set (any block size serves)
     const int bz = std::max(128, std::min(512, warps(items_z)));
-    const int bp = np <= c.sm_count ? std::max(block, std::min(kPlaneThreads<MAXR>, warps(items_p))) : block;
+    const int bp = std::min(kPlaneThreads<MAXR>, np <= c.sm_count ? std::max(block, warps(items_p)) : block);
     HPSI_LAUNCH(c, HPSI_K_INV_ZY, (k_zinv<MAXR><<<nz, bz, smem_z, c.stream>>>(bt)));
     HPSI_LAUNCH(c, HPSI_K_XVX_Y, (k_plane<MAXR><<<np, bp, smem_p, c.stream>>>(bt)));
     HPSI_LAUNCH(c, HPSI_K_FWD_Z, (k_zfwd<MAXR><<<nz, bz, smem_z, c.stream>>>(bt)));

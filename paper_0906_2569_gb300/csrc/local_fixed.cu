@@ -545,8 +545,10 @@ struct FxLaunch {
       attr = true;
     }
     const int nz = bt.off_z[bt.nitems], np = bt.off_p[bt.nitems];
-    // plane_shape's block, or one round of a stage's items where there is a CTA per SM at most
-    const int plane = np <= c.sm_count ? std::max(block, std::min(kFxThreads<MAXR>, items / 32 * 32)) : block;
+    // plane_shape's block, or one round of a stage's items where there is a CTA per SM at most; never more than this
+    // instance's launch bound, which another item's radix may have set (any block size serves: items are dealt over it)
+    const int want = np <= c.sm_count ? std::max(block, items / 32 * 32) : block;
+    const int plane = std::min(kFxThreads<MAXR>, want);
     HPSI_LAUNCH(c, HPSI_K_INV_ZY, (k_fx_zinv<MAXR><<<nz, 256, smem_z, c.stream>>>(bt)));
     HPSI_LAUNCH(c, HPSI_K_XVX_Y, (k_fx_plane<MAXR><<<np, plane, smem_p, c.stream>>>(bt)));
     HPSI_LAUNCH(c, HPSI_K_FWD_Z, (k_fx_zfwd<MAXR><<<nz, 256, smem_z, c.stream>>>(bt)));
