@@ -19,6 +19,21 @@ int fail(Context& c, int code, const std::string& msg) {
   return code;
 }
 
+cudaError_t allow_smem(const Context& c, std::atomic<unsigned long long>& devices,
+                       std::initializer_list<const void*> kernels) {
+  const unsigned long long bit = c.device < 64 ? 1ULL << c.device : 0ULL;
+  if (devices.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  for (const void* k : kernels) {
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, k);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(c.smem_optin - fa.sharedSizeBytes));
+    if (e != cudaSuccess) return e;
+  }
+  devices.fetch_or(bit, std::memory_order_release);
+  return cudaSuccess;
+}
+
 int cuda_fail(Context& c, cudaError_t e, const char* what) {
   c.err = std::string(what) + ": " + cudaGetErrorString(e);
   return HPSI_ECUDA;

@@ -856,10 +856,9 @@ int invit_all(Context& c, EighState& s, int n, int nwant, int iters) {
                                                                           s.info + 1, iters)));
   HPSI_LAUNCH(c, HPSI_K_EIGH, (k_eh_invit_finish<<<nwant, 128, 0, c.stream>>>(n, s.invs, s.Z)));
   const size_t ismem = sizeof(double) * 7 * (size_t)n + (size_t)n + 16;
-  if (ismem > 48 * 1024) {
-    const cudaError_t err = cudaFuncSetAttribute(k_eh_invit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ismem);
-    if (err != cudaSuccess) return cuda_fail(c, err, "inverse iteration: smem attribute");
-  }
+  static std::atomic<unsigned long long> devices{0};
+  const cudaError_t err = allow_smem(c, devices, {(const void*)k_eh_invit});
+  if (err != cudaSuccess) return cuda_fail(c, err, "inverse iteration: smem attribute");
   HPSI_LAUNCH(c, HPSI_K_EIGH,
               (k_eh_invit<<<nwant, 32, ismem, c.stream>>>(n, s.d, s.e, nwant, s.lam, s.Z, s.info + 1, 1, iters)));
   return HPSI_OK;
@@ -981,7 +980,8 @@ int eigh_lowest(Context& c, const double2* a, int lda, int n, int nwant, double*
   // 1. tridiagonal reduction (cooperative)
   const int G = tri_ctas(c, n);
   const size_t smem = tri_smem(n, G);
-  err = cudaFuncSetAttribute(k_eh_tridiag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static std::atomic<unsigned long long> devices{0};
+  err = allow_smem(c, devices, {(const void*)k_eh_tridiag});
   if (err != cudaSuccess) return cuda_fail(c, err, "eigh_lowest: smem attribute");
   err = cudaMemsetAsync(s->bar, 0, sizeof(unsigned int) * 64, c.stream);
   if (err == cudaSuccess) err = cudaMemsetAsync(s->vref, 0, sizeof(double2) * (size_t)(n + kWY) * n, c.stream);
@@ -1039,8 +1039,6 @@ int eigh_lowest(Context& c, const double2* a, int lda, int n, int nwant, double*
                                   (long long)kWY * n, Zc(s->vref + 1), n, (long long)kWY * n, &zzero, Zc(s->wgram),
                                   kWY, (long long)kWY * kWY, K) != CUBLAS_STATUS_SUCCESS)
       return fail(c, HPSI_ECUDA, "eigh_lowest: reflector Gram matrices failed");
-    err = cudaFuncSetAttribute(k_eh_tfactor, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrsvSmem);
-    if (err != cudaSuccess) return cuda_fail(c, err, "eigh_lowest: smem attribute");
     HPSI_LAUNCH(c, HPSI_K_EIGH,
                 (k_eh_tfactor<<<dim3(kWY / 4, K), 128, kTrsvSmem, c.stream>>>(n - 1, s->wgram, s->tau, s->tfac)));
     for (int k = K - 1; k >= 0; --k) {
@@ -1110,7 +1108,8 @@ int eigh_lowest_real(Context& c, const double* a, int lda, int n, int nwant, dou
   const int G = tri_ctas(c, n);
   const size_t smem = tri_smem_r(n, G);
   const void* tri_kernel = df ? (const void*)k_eh_tridiag_df : (const void*)k_eh_tridiag_r;
-  err = cudaFuncSetAttribute(tri_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static std::atomic<unsigned long long> devices{0};
+  err = allow_smem(c, devices, {(const void*)k_eh_tridiag_df, (const void*)k_eh_tridiag_r});
   if (err != cudaSuccess) return cuda_fail(c, err, "eigh_lowest_real: smem attribute");
   err = cudaMemsetAsync(s->bar, 0, sizeof(unsigned int) * 64, c.stream);
   if (err == cudaSuccess) err = cudaMemsetAsync(vref, 0, sizeof(double) * (size_t)(n + kWY) * n, c.stream);

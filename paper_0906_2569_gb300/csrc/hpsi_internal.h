@@ -4,7 +4,9 @@
 #include <cublas_v2.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <atomic>
 #include <cstdint>
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -384,6 +386,11 @@ int gamma_dscale_fp64(Context& c, const Problem& p, int nb, int nsplit, const do
 // ---- context helpers (api.cpp) ----
 int ensure_buffer(Context& c, void** ptr, size_t* have, size_t need);
 int fail(Context& c, int code, const std::string& msg);
+// Lets kernels use all of the device's opt-in shared memory, once per device; `devices` is the call site's record of those
+// done.  The attribute belongs to the device's copy of a kernel and every context sets the same value, so that
+// threads with contexts of their own never lower it under one another's launches.
+cudaError_t allow_smem(const Context& c, std::atomic<unsigned long long>& devices,
+                       std::initializer_list<const void*> kernels);
 int cuda_fail(Context& c, cudaError_t e, const char* what);
 int apply_device(Context& c, int ik, const double2* psi, double2* hpsi, int nbnd);
 int check_device_error(Context& c);   // synchronizes; HPSI_ETIMEOUT if a bounded wait expired

@@ -327,14 +327,9 @@ struct FastLaunch {
     smem_p = std::max(smem_p, f.smem_p);
   }
   template <int MAXR> int run_t(Context& c) {
-    static bool attr = false;
-    if (!attr) {
-      const int mx = (int)c.smem_optin - 64;
-      cudaFuncSetAttribute(k_zinv<MAXR>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-      cudaFuncSetAttribute(k_plane<MAXR>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-      cudaFuncSetAttribute(k_zfwd<MAXR>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-      attr = true;
-    }
+    static std::atomic<unsigned long long> devices{0};
+    cudaError_t e = allow_smem(c, devices, {(const void*)k_zinv<MAXR>, (const void*)k_plane<MAXR>, (const void*)k_zfwd<MAXR>});
+    if (e != cudaSuccess) return cuda_fail(c, e, "fast local kernels");
     const int nz = bt.off_z[bt.nitems], np = bt.off_p[bt.nitems];
     auto warps = [](int items) { return (items + 31) / 32 * 32; };
     // z: one round of a stage's items; planes: plane_shape's block, or one round where there is a CTA per SM at most;
@@ -344,7 +339,7 @@ struct FastLaunch {
     HPSI_LAUNCH(c, HPSI_K_INV_ZY, (k_zinv<MAXR><<<nz, bz, smem_z, c.stream>>>(bt)));
     HPSI_LAUNCH(c, HPSI_K_XVX_Y, (k_plane<MAXR><<<np, bp, smem_p, c.stream>>>(bt)));
     HPSI_LAUNCH(c, HPSI_K_FWD_Z, (k_zfwd<MAXR><<<nz, bz, smem_z, c.stream>>>(bt)));
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "fast local kernels launch");
     return HPSI_OK;
   }
@@ -353,9 +348,10 @@ struct FastLaunch {
     const void* kern = (const void*)k_hpsi_batch<MAXR>;
     size_t dyn = std::max(smem_z, smem_p);
     if (nl.nitems > 0) dyn = std::max(dyn, sizeof(double2) * (size_t)std::max(CB_SMEM, AV_SMEM));
+    static std::atomic<unsigned long long> devices{0};
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || fa.sharedSizeBytes + dyn > c.smem_optin ||
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) {
+        allow_smem(c, devices, {kern}) != cudaSuccess) {
       cudaGetLastError();
       return HPSI_OK;
     }
@@ -426,7 +422,7 @@ int float_potential(Context& c, int slot, const LineAxis ax[3], int kernel_class
 int local_fast_apply(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd, void* Zt, void* Yb,
                      int nbb) {
   if (cur_prec(c) == HPSI_FP64) return local_fixed_apply(c, p, psi, hpsi, nbnd, Zt, Yb, nbb);
-  static FastLaunch fl;   // host staging of the parameter block (calls are not thread-safe by contract)
+  static thread_local FastLaunch fl;   // host staging of the parameter block: threads use contexts of their own at the same time
   for (int b0 = 0; b0 < nbnd; b0 += nbb) {
     fl.reset();
     fl.add(c, p, psi + (size_t)b0 * p.npw, hpsi + (size_t)b0 * p.npw, std::min(nbb, nbnd - b0), Zt, Yb);
@@ -437,7 +433,7 @@ int local_fast_apply(Context& c, const Problem& p, const double2* psi, double2* 
 }
 
 int local_fast_apply_raw(Context& c, const Problem& p, const float2* f, float2* F, int nbnd, void* Zt, void* Yb, int nbb) {
-  static FastLaunch fl;
+  static thread_local FastLaunch fl;
   for (int b0 = 0; b0 < nbnd; b0 += nbb) {
     fl.reset();
     fl.add(c, p, f + (size_t)b0 * p.npw, F + (size_t)b0 * p.npw, std::min(nbb, nbnd - b0), Zt, Yb, true);
@@ -451,7 +447,7 @@ int local_fast_apply_raw(Context& c, const Problem& p, const float2* f, float2* 
 int local_fast_apply_multi(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
                            double2* const* hpsi, void* const* zt, void* const* yb) {
   if (cur_prec(c) == HPSI_FP64) return local_fixed_apply_multi(c, nitem, prob, nbnd, psi, hpsi, zt, yb);
-  static FastLaunch fl;
+  static thread_local FastLaunch fl;
   for (int i0 = 0; i0 < nitem; i0 += kMaxLocalItems) {
     fl.reset();
     for (int i = i0; i < std::min(nitem, i0 + kMaxLocalItems); ++i)
@@ -475,8 +471,8 @@ int local_batch_persistent(Context& c, int nitem, const int* prob, const int* nb
     if (!local_fast_ok(p, pr) || p.n[0] != c.probs[prob[0]].n[0] || nbnd[i] < 1) return HPSI_OK;
   }
   if (pr == HPSI_FP64) return local_fixed_persistent(c, nitem, prob, nbnd, psi, hpsi, zt, yb, with_nl, done);
-  static FastLaunch fl;
-  static NlBatch nl;
+  static thread_local FastLaunch fl;
+  static thread_local NlBatch nl;
   fl.reset();
   for (int i = 0; i < nitem; ++i) fl.add(c, c.probs[prob[i]], psi[i], hpsi[i], nbnd[i], zt[i], yb[i]);
   nl.nitems = 0;

@@ -536,14 +536,9 @@ struct FxLaunch {
     maxr = items = 0;
   }
   template <int MAXR> int run_t(Context& c) {
-    static bool attr = false;
-    if (!attr) {
-      const int mx = (int)c.smem_optin - 64;
-      cudaFuncSetAttribute(k_fx_zinv<MAXR>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-      cudaFuncSetAttribute(k_fx_plane<MAXR>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-      cudaFuncSetAttribute(k_fx_zfwd<MAXR>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-      attr = true;
-    }
+    static std::atomic<unsigned long long> devices{0};
+    cudaError_t e = allow_smem(c, devices, {(const void*)k_fx_zinv<MAXR>, (const void*)k_fx_plane<MAXR>, (const void*)k_fx_zfwd<MAXR>});
+    if (e != cudaSuccess) return cuda_fail(c, e, "fixed-point local kernels");
     const int nz = bt.off_z[bt.nitems], np = bt.off_p[bt.nitems];
     // plane_shape's block, or one round of a stage's items where there is a CTA per SM at most; never more than this
     // instance's launch bound, which another item's radix may have set (any block size serves: items are dealt over it)
@@ -552,7 +547,7 @@ struct FxLaunch {
     HPSI_LAUNCH(c, HPSI_K_INV_ZY, (k_fx_zinv<MAXR><<<nz, 256, smem_z, c.stream>>>(bt)));
     HPSI_LAUNCH(c, HPSI_K_XVX_Y, (k_fx_plane<MAXR><<<np, plane, smem_p, c.stream>>>(bt)));
     HPSI_LAUNCH(c, HPSI_K_FWD_Z, (k_fx_zfwd<MAXR><<<nz, 256, smem_z, c.stream>>>(bt)));
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "fixed-point local kernels launch");
     return HPSI_OK;
   }
@@ -561,9 +556,10 @@ struct FxLaunch {
     const void* kern = (const void*)k_fx_batch<MAXR>;
     size_t dyn = std::max(smem_z, smem_p);
     if (nl.nitems > 0) dyn = std::max(dyn, sizeof(double2) * (size_t)std::max(CB_SMEM, AV_SMEM));
+    static std::atomic<unsigned long long> devices{0};
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || fa.sharedSizeBytes + dyn > c.smem_optin ||
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) {
+        allow_smem(c, devices, {kern}) != cudaSuccess) {
       cudaGetLastError();
       return HPSI_OK;
     }
@@ -723,7 +719,7 @@ int fixed_potential(Context& c, int slot, const LineAxis ax[3], int kernel_class
 
 int local_fixed_apply(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd, void* Zt, void* Yb,
                       int nbb) {
-  static FxLaunch fl;   // host staging of the parameter block (calls are not thread-safe by contract)
+  static thread_local FxLaunch fl;   // host staging of the parameter block: threads use contexts of their own at the same time
   const int rv = ensure_fixed_potential(c, p.vslot, p.fixed.ax);
   if (rv) return rv;
   for (int b0 = 0; b0 < nbnd; b0 += nbb) {
@@ -737,7 +733,7 @@ int local_fixed_apply(Context& c, const Problem& p, const double2* psi, double2*
 
 int local_fixed_apply_multi(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
                             double2* const* hpsi, void* const* zt, void* const* yb) {
-  static FxLaunch fl;
+  static thread_local FxLaunch fl;
   for (int i0 = 0; i0 < nitem; i0 += kMaxLocalItems) {
     fl.reset();
     for (int i = i0; i < std::min(nitem, i0 + kMaxLocalItems); ++i)
@@ -750,8 +746,8 @@ int local_fixed_apply_multi(Context& c, int nitem, const int* prob, const int* n
 
 int local_fixed_persistent(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
                            double2* const* hpsi, void* const* zt, void* const* yb, bool with_nl, bool* done) {
-  static FxLaunch fl;
-  static NlBatch nl;
+  static thread_local FxLaunch fl;
+  static thread_local NlBatch nl;
   fl.reset();
   for (int i = 0; i < nitem; ++i) fl.add(c, c.probs[prob[i]], psi[i], hpsi[i], nbnd[i], zt[i], yb[i]);
   nl.nitems = 0;

@@ -200,9 +200,9 @@ int local_density(Context& c, const Problem& p, const double2* psi, int nbnd, co
   int rc = ensure_buffer(c, &c.ws.X, &c.ws.xbytes, xneed);
   if (rc) return rc;
   const size_t s0 = local_smem_bytes(p, HPSI_FP64, 0), s1 = local_smem_bytes(p, HPSI_FP64, 1);
-  const int mx = (int)c.smem_optin;
-  cudaFuncSetAttribute(k_inv_zy<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_x_density, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  static std::atomic<unsigned long long> devices{0};
+  cudaError_t e = allow_smem(c, devices, {(const void*)k_inv_zy<double>, (const void*)k_x_density});
+  if (e != cudaSuccess) return cuda_fail(c, e, "density kernels");
   LocalArgs a;
   a.n1 = p.n[0]; a.n2 = p.n[1]; a.n3 = p.n[2];
   a.npw = p.npw; a.npl = p.npl; a.nst = p.nst; a.ns_max = p.ns_max;
@@ -217,7 +217,7 @@ int local_density(Context& c, const Problem& p, const double2* psi, int nbnd, co
     HPSI_LAUNCH(c, HPSI_K_SCF, (k_inv_zy<double><<<dim3(p.npl, nb), 256, s0, c.stream>>>(a)));
     HPSI_LAUNCH(c, HPSI_K_SCF, (k_x_density<<<p.n[2], 256, s1, c.stream>>>(a, wb + b0, rho)));
   }
-  cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "density kernels launch");
   return HPSI_OK;
 }
@@ -270,15 +270,9 @@ static int local_apply_t(Context& c, const Problem& p, const double2* psi, doubl
   if (rc) return rc;
   const size_t s0 = local_smem_bytes(p, cur_prec(c), 0), s1 = local_smem_bytes(p, cur_prec(c), 1),
                s2 = local_smem_bytes(p, cur_prec(c), 2);
-  static bool attr_done[2] = {false, false};
-  const int slot = sizeof(T) == 8 ? 0 : 1;
-  if (!attr_done[slot]) {
-    const int mx = (int)c.smem_optin;
-    cudaFuncSetAttribute(k_inv_zy<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    cudaFuncSetAttribute(k_xvx_y<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    cudaFuncSetAttribute(k_fwd_z<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    attr_done[slot] = true;
-  }
+  static std::atomic<unsigned long long> devices{0};
+  cudaError_t e = allow_smem(c, devices, {(const void*)k_inv_zy<T>, (const void*)k_xvx_y<T>, (const void*)k_fwd_z<T>});
+  if (e != cudaSuccess) return cuda_fail(c, e, "local-potential kernels");
   LocalArgs a;
   a.n1 = p.n[0]; a.n2 = p.n[1]; a.n3 = p.n[2];
   a.npw = p.npw; a.npl = p.npl; a.nst = p.nst; a.ns_max = p.ns_max;
@@ -296,7 +290,7 @@ static int local_apply_t(Context& c, const Problem& p, const double2* psi, doubl
     HPSI_LAUNCH(c, HPSI_K_XVX_Y, (k_xvx_y<T><<<dim3(p.n[2], nb), 256, s1, c.stream>>>(a)));
     HPSI_LAUNCH(c, HPSI_K_FWD_Z, (k_fwd_z<T><<<dim3(p.npl, nb), 256, s2, c.stream>>>(a)));
   }
-  cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "local-potential kernels launch");
   return HPSI_OK;
 }
@@ -316,10 +310,9 @@ size_t local_scratch_per_band(const Problem& p, int precision) {
 template <typename T>
 static int local_apply_into_t(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd, void* X,
                               void* Y, int nbb) {
-  const int mx = (int)c.smem_optin;
-  cudaFuncSetAttribute(k_inv_zy<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xvx_y<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_fwd_z<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  static std::atomic<unsigned long long> devices{0};
+  cudaError_t e = allow_smem(c, devices, {(const void*)k_inv_zy<T>, (const void*)k_xvx_y<T>, (const void*)k_fwd_z<T>});
+  if (e != cudaSuccess) return cuda_fail(c, e, "local-potential kernels");
   const size_t s0 = local_smem_bytes(p, cur_prec(c), 0), s1 = local_smem_bytes(p, cur_prec(c), 1),
                s2 = local_smem_bytes(p, cur_prec(c), 2);
   LocalArgs a;
@@ -339,7 +332,7 @@ static int local_apply_into_t(Context& c, const Problem& p, const double2* psi, 
     HPSI_LAUNCH(c, HPSI_K_XVX_Y, (k_xvx_y<T><<<dim3(p.n[2], nb), 256, s1, c.stream>>>(a)));
     HPSI_LAUNCH(c, HPSI_K_FWD_Z, (k_fwd_z<T><<<dim3(p.npl, nb), 256, s2, c.stream>>>(a)));
   }
-  cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "local-potential kernels launch");
   return HPSI_OK;
 }

@@ -536,7 +536,7 @@ int nonlocal_batch_fp64(Context& c, int nitem, const int* prob, const int* nbnd,
   int rc = ensure_buffer(c, &c.ws.part, &c.ws.partbytes, total);
   if (rc) return rc;
   unsigned char* base = static_cast<unsigned char*>(c.ws.part);
-  static NlBatch bt;   // host staging of the parameter block (calls are not thread-safe by contract)
+  static thread_local NlBatch bt;   // host staging of the parameter block: threads use contexts of their own at the same time
   for (size_t g0 = 0; g0 < items.size(); g0 += kNlBatch) {
     const int n = (int)std::min<size_t>(kNlBatch, items.size() - g0);
     bt.nitems = n;

@@ -407,11 +407,9 @@ int slice_gemm(Context& c, const __nv_bfloat16* A, const int* ea, int M, const _
   int rc = slice_map(c, &ma, A, M, kpad, SM_);
   if (!rc) rc = slice_map(c, &mb, B, N, kpad, SN);
   if (rc) return rc;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_slice_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, kSliceSmem);
-    attr = true;
-  }
+  static std::atomic<unsigned long long> devices{0};
+  const cudaError_t e = allow_smem(c, devices, {(const void*)k_slice_gemm});
+  if (e != cudaSuccess) return cuda_fail(c, e, "digit products");
   SliceArgs a;
   a.M = M;
   a.N = N;

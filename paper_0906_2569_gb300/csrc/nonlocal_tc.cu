@@ -26,7 +26,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "convert.cuh"
 #include "hpsi_internal.h"
@@ -35,15 +34,13 @@
 namespace hpsi {
 
 int tma_encoder(Context& c, PFN_cuTensorMapEncodeTiled_v12000* fn) {
-  static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
+  static const PFN_cuTensorMapEncodeTiled_v12000 encode = [] {
     void* f = nullptr;
     cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f);
-  });
+    const bool ok = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) ==
+                        cudaSuccess && q == cudaDriverEntryPointSuccess;
+    return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(ok ? f : nullptr);
+  }();
   if (!encode) return fail(c, HPSI_ECUDA, "cuTensorMapEncodeTiled is not available");
   *fn = encode;
   return HPSI_OK;
@@ -592,11 +589,9 @@ int launch_gemm(Context& c, const void* A, int M, const void* B, int N, int kpad
   a.mode = mode;
   a.part = part;
   a.err = c.d_err;
-  static bool attr[4] = {false, false, false, false};
-  if (!attr[NT]) {
-    cudaFuncSetAttribute(k_tc_gemm<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<NT>::smem);
-    attr[NT] = true;
-  }
+  static std::atomic<unsigned long long> devices{0};
+  const cudaError_t ea = allow_smem(c, devices, {(const void*)k_tc_gemm<NT>});
+  if (ea != cudaSuccess) return cuda_fail(c, ea, "tensor-core GEMM");
   dim3 grid((N + TBN - 1) / TBN, (M + TBM - 1) / TBM, nsplit);
   HPSI_LAUNCH(c, kernel_class,
               (k_tc_gemm<NT><<<grid, 128, TcCfg<NT>::smem, c.stream>>>(ma[0], ma[1], ma[2], mb[0], mb[1], mb[2], a)));
