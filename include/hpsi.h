@@ -147,9 +147,11 @@ enum hpsi_option {
                                  The results are identical; the separate launches, replayed from a
                                  CUDA graph, are faster since each kernel runs at its own occupancy */
   HPSI_OPT_BATCH_NL = 25      /* hpsi_apply_batch in a mixed context: the nonlocal term.  0 (default):
-                                 in float64 on the CUDA cores, one launch per kernel class over all
-                                 items, when every item has at most 64 projectors, else 1.  1: the
-                                 tensor-core form per item.  2: always the float64 batched form */
+                                 in float64 when every item has at most 64 projectors (one launch per
+                                 kernel class over all items; an item with more than 16 projectors
+                                 and 6e6 multiply-adds a contraction, or one of a few items with many
+                                 projectors, by itself), else 1.  1: the tensor-core form per item.
+                                 2: always the float64 form */
 };
 
 /* Kernel classes reported by hpsi_kernel_stats. */
@@ -319,9 +321,10 @@ HPSI_API int davidson_solve_gamma(hpsi_ctx* ctx, int ik, int nbnd, double tol, i
  * hpsi_apply_batch -- H psi for several problems (k-points or cells) in one launch sequence:
  * for i < nitem: hpsi_out[i] = H(prob[i]) psi_in[i] with nbnd[i] bands.  Device pointers only.
  * Items whose box has the two-codelet kernels share one launch of each local-potential
- * kernel (32 items each, whatever their boxes), and the nonlocal term follows: one launch
- * per kernel class over all items in float64, which a mixed context also takes when every item has
- * at most 64 projectors (HPSI_OPT_BATCH_NL), else the tensor-core form per item.  With
+ * kernel (32 items each, whatever their boxes), and the nonlocal term follows: in float64 one launch
+ * per kernel class over all items but the large ones (HPSI_OPT_BATCH_NL), which a mixed context also takes when
+ * every item has at most 64 projectors, else the mixed tensor-core form per item.  In a float64 context an item of up
+ * to 16 projectors, and a large one, gets the bits of hpsi_apply; others agree with it to rounding.  With
  * HPSI_OPT_PERSISTENT = 1, and every item on those kernels, each box edge (<= 32 items) is instead
  * one persistent cooperative launch whose CTAs take tiles from per-phase work lists: the
  * z-scatter/inverse transforms, the plane transforms with x V, the forward transforms and gather,

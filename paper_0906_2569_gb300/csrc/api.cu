@@ -604,6 +604,7 @@ static int batch_apply_items(Context& c, int nitem, const int* prob, const int* 
     if (local_fast_ok(p, cur_prec(c)) && !c.force_generic) fast.push_back(i);
     else slow.push_back(i);
   }
+  const int nbatch = (int)(fast.size() + slow.size());
   std::stable_sort(fast.begin(), fast.end(),
                    [&](int x, int y) { return c.probs[prob[x]].n[0] < c.probs[prob[y]].n[0]; });
   std::vector<size_t> off(fast.size());
@@ -637,7 +638,7 @@ static int batch_apply_items(Context& c, int nitem, const int* prob, const int* 
     if (c.persistent && slow.empty()) {
       // (items large enough for the tensor-core contractions take those, as in the separate launches)
       bool with_nl = nl_prec(c) == HPSI_FP64;
-      for (size_t j = 0; with_nl && j < fast.size(); ++j) with_nl = !nonlocal_slices_use(c.probs[fp[j]], fn[j]);
+      for (size_t j = 0; with_nl && j < fast.size(); ++j) with_nl = !batch_slices_use(c.probs[fp[j]], fn[j], nbatch);
       const int nf = (int)fast.size();
       for (int g0 = 0; g0 < nf;) {
         const Problem& q = c.probs[fp[g0]];
@@ -653,15 +654,20 @@ static int batch_apply_items(Context& c, int nitem, const int* prob, const int* 
                                       zt.data() + g0, yb.data() + g0);
           if (rc) return rc;
           if (with_nl) {
-            rc = nonlocal_batch_fp64(c, n, fp.data() + g0, fn.data() + g0, fi.data() + g0, fo.data() + g0);
+            rc = nonlocal_batch_fp64(c, n, fp.data() + g0, fn.data() + g0, fi.data() + g0, fo.data() + g0,
+                                     nbatch);
             if (rc) return rc;
           }
         }
         g0 = g1;
       }
+      if (!with_nl && nl_prec(c) == HPSI_FP64) {
+        rc = nonlocal_batch_fp64(c, nitem, prob, nbnd, psi, hpsi, nbatch);
+        if (rc) return rc;
+      }
       for (int i = 0; i < nitem; ++i) {
         if (nbnd[i] == 0) continue;
-        if (!with_nl) {
+        if (nl_prec(c) != HPSI_FP64) {
           rc = nonlocal_apply(c, c.probs[prob[i]], psi[i], hpsi[i], nbnd[i]);
           if (rc) return rc;
         }
@@ -676,10 +682,10 @@ static int batch_apply_items(Context& c, int nitem, const int* prob, const int* 
     int rc = local_apply(c, c.probs[prob[i]], psi[i], hpsi[i], nbnd[i]);
     if (rc) return rc;
   }
-  // the nonlocal term: in float64 all items share one launch per kernel class; the tensor-core
-  // form runs per item
+  // the nonlocal term: in float64 all items but the large ones share one launch per kernel class; the mixed
+  // tensor-core form runs per item
   if (nl_prec(c) == HPSI_FP64) {
-    int rc = nonlocal_batch_fp64(c, nitem, prob, nbnd, psi, hpsi);
+    int rc = nonlocal_batch_fp64(c, nitem, prob, nbnd, psi, hpsi, nbatch);
     if (rc) return rc;
   }
   for (int i = 0; i < nitem; ++i) {
@@ -705,8 +711,8 @@ int pointer_kind(const void* ptr) {
   return 0;
 }
 
-// In a mixed context, whether the batch's nonlocal term runs in float64 on the CUDA cores, one launch
-// per kernel class over all items (HPSI_OPT_BATCH_NL): the tensor-core form works on tiles of 128
+// In a mixed context, whether the batch's nonlocal term runs in float64, one launch per kernel class over all items
+// but the large ones (HPSI_OPT_BATCH_NL, batch_slices_use): the tensor-core form works on tiles of 128
 // projector rows, and with a few projectors per item its per-item launches are mostly empty tiles.
 static bool batch_nl64(const Context& c, int nitem, const int* prob, const int* nbnd) {
   if (c.precision != HPSI_MIXED || nl_prec(c) != HPSI_MIXED || c.batch_nl == 1) return false;

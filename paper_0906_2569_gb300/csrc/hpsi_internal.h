@@ -354,12 +354,14 @@ void nonlocal_fp64_plan(const Context& c, const Problem& p, int nbnd, int* nspli
 int nonlocal_fp64_into(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd, void* scratch,
                        size_t capacity);
 // The float64 nonlocal term of several problems' band blocks, one launch per kernel class
+// The items of a batch (some or all of its nbatch items with bands): one launch per kernel class, large items one by one
 int nonlocal_batch_fp64(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
-                        double2* const* hpsi);
+                        double2* const* hpsi, int nbatch);
 
 // The float64 contractions as exact integer products on the tensor cores (nonlocal_slices.cu); *ok = false: no room for
 // the projectors' digits, the caller takes the CUDA-core kernels.
 bool nonlocal_slices_use(const Problem& p, int nbnd);
+bool batch_slices_use(const Problem& p, int nbnd, int nitem);   // the same for an item of a batch of nitem
 int slices_w(Context& c, const Problem& p, const double2* psi, int nbnd, double2* w, bool* ok);
 int slices_add(Context& c, const Problem& p, const double2* w, double2* hpsi, int nbnd, bool* ok);
 bool gamma_slices_use(const Problem& p, int nbnd);

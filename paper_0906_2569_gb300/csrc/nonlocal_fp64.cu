@@ -510,11 +510,11 @@ int nonlocal_fp64_into(Context& c, const Problem& p, const double2* psi, double2
 
 // The float64 nonlocal term of several items in one launch per kernel class (groups of kNlBatch).
 int nonlocal_batch_fp64(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
-                        double2* const* hpsi) {
+                        double2* const* hpsi, int nbatch) {
   std::vector<int> items;
   for (int i = 0; i < nitem; ++i)
     if (nbnd[i] > 0 && c.probs[prob[i]].nproj > 0) {
-      if (nonlocal_slices_use(c.probs[prob[i]], nbnd[i])) {   // large items one by one on the tensor cores
+      if (batch_slices_use(c.probs[prob[i]], nbnd[i], nbatch)) {   // large items one by one on the tensor cores
         const int rc = nonlocal_apply_fp64(c, c.probs[prob[i]], psi[i], hpsi[i], nbnd[i]);
         if (rc) return rc;
       } else {

@@ -480,6 +480,16 @@ bool nonlocal_slices_use(const Problem& p, int nbnd) {
   return p.nproj > 16 && nbnd > 0 && !p.slices[0].no_room && !p.slices[1].no_room;
 }
 
+// Items of a batch of nitem take this form one by one, about ten launches and 45 us each, where the tiles run over all items
+// at once.  It is the faster one from about 6e6 multiply-adds an item, and for a few items of many projectors, where the
+// tiles' chain over the projectors (1.7 us each for 16 bands and more) is longer.  Measured, tiles against this form, 16
+// items: P = 17, 1503 plane waves, 8 bands 240 / 1123 us; P = 32, 1503, 24 bands 634 / 1411; P = 64, 3911, 24 bands 2115 /
+// 2125; P = 128, 1503, 64 bands 3528 / 2229; 2 items: P = 32, 1503, 24 bands 180 / 189; P = 96, 1503, 24 bands 280 / 213.
+bool batch_slices_use(const Problem& p, int nbnd, int nitem) {
+  return nonlocal_slices_use(p, nbnd) &&
+         ((double)p.nproj * p.npw * nbnd >= 6.0e6 || (nbnd >= 16 && p.nproj > 26 * nitem));
+}
+
 // Digit planes of `rows` rows of `len` doubles (src) in the workspace at `at`; returns the planes and row exponents.
 template <typename R>
 static int slice_rows(Context& c, const R* src, int rows, int len, int kpad, int dup, int scaled, unsigned char* at,
