@@ -139,8 +139,28 @@ __global__ void __launch_bounds__(256) k_gamma_pack_raw(int npw, int nb, const S
   }
 }
 
-// Unpack the raw local term L f of a pair and add the kinetic term (float64 results: in float64, one FMA a component)
-// and the nonlocal term's float32 partial sums nl32 [ns32][nb][nr] in real-basis coordinates (null: none).
+// Sums of float32 numbers as two floats, h + l: 2^-47 of the largest summand or better, on the float32 pipes (Knuth's TwoSum).
+__device__ __forceinline__ float2 pair_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), z = __fsub_rn(s, a);
+  return make_float2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z)));
+}
+__device__ __forceinline__ float2 pair_add(float2 a, float2 b) {
+  const float2 t = pair_sum(a.x, b.x);
+  return make_float2(t.x, __fadd_rn(t.y, __fadd_rn(a.y, b.y)));
+}
+__device__ __forceinline__ float2 pair_times(float2 a, float ch, float cl) {   // a (ch + cl)
+  const float p = __fmul_rn(a.x, ch);
+  return make_float2(p, __fmaf_rn(a.x, ch, -p) + __fmaf_rn(a.x, cl, a.y * ch));
+}
+// kg x + (a.x + a.y) in float64 (an infinite or NaN a.x stands alone)
+__device__ __forceinline__ double pair_fma(double kg, double x, float2 a) {
+  return fma(kg, x, f32_to_f64(a.x)) + f32_to_f64(fabsf(a.x) <= 3.402823466e38f ? a.y : 0.f);
+}
+
+// Unpack the raw local term L f of a pair and add the kinetic term and the nonlocal term's float32 partial sums nl32
+// [ns32][nb][nr] in real-basis coordinates (null: none).  Float64 results: the bands' combinations, the sqrt2 factors and
+// the sums over the partials to 2^-47 as pairs of floats, the kinetic term and the last sum in float64.  Float32
+// results: in float32, the kinetic term as one FMA chain.
 template <typename S>
 __global__ void __launch_bounds__(256) k_gamma_unpack_raw(int npw, int nb, const float2* __restrict__ F, int scaled,
                                                           const double* __restrict__ kin, const S* __restrict__ x,
@@ -151,34 +171,35 @@ __global__ void __launch_bounds__(256) k_gamma_unpack_raw(int npw, int nb, const
   const float2* Fq = F + (size_t)q * npw;
   for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < nh; h += gridDim.x * blockDim.x) {
     const float2 fp = Fq[i0 + h], fm = Fq[i0 - h];
-    // conj(F(-G)) = (fm.x, -fm.y)
-    float2 ya = make_float2(0.5f * (fp.x + fm.x), 0.5f * (fp.y - fm.y));
-    float2 yb = make_float2(0.5f * (fp.y + fm.y), -0.5f * (fp.x - fm.x));
-    if (scaled && h > 0) {
-      ya.x *= (float)kSqrt2; ya.y *= (float)kSqrt2;
-      yb.x *= (float)kSqrt2; yb.y *= (float)kSqrt2;
-    }
-    if (nl32) {
-      const float sn = (!scaled && h > 0) ? (float)kInvSqrt2 : 1.f;
-      float2 na = make_float2(0.f, 0.f), nc = na;
-      const size_t ia = (size_t)a * nr + 2 * h, ib = (size_t)b * nr + 2 * h;
-      for (int sp = 0; sp < ns32; ++sp) {
-        const float2 va = *reinterpret_cast<const float2*>(nl32 + sp * plane + ia);
-        na.x += va.x;
-        na.y += va.y;
-        if (b < nb) {
-          const float2 vb = *reinterpret_cast<const float2*>(nl32 + sp * plane + ib);
-          nc.x += vb.x;
-          nc.y += vb.y;
-        }
-      }
-      ya.x = fmaf(sn, na.x, ya.x);
-      ya.y = fmaf(sn, na.y, ya.y);
-      yb.x = fmaf(sn, nc.x, yb.x);
-      yb.y = fmaf(sn, nc.y, yb.y);
-    }
+    const size_t ia = (size_t)a * nr + 2 * h, ib = (size_t)b * nr + 2 * h;
+    const bool up = scaled && h > 0, down = !scaled && h > 0;   // of the local, and of the nonlocal term by sqrt2
     const double kg = kin[i0 + h];
+    // conj(F(-G)) = (fm.x, -fm.y)
     if constexpr (sizeof(S) == sizeof(float2)) {
+      float2 ya = make_float2(0.5f * (fp.x + fm.x), 0.5f * (fp.y - fm.y));
+      float2 yb = make_float2(0.5f * (fp.y + fm.y), -0.5f * (fp.x - fm.x));
+      if (up) {
+        ya.x *= (float)kSqrt2; ya.y *= (float)kSqrt2;
+        yb.x *= (float)kSqrt2; yb.y *= (float)kSqrt2;
+      }
+      if (nl32) {
+        const float sn = down ? (float)kInvSqrt2 : 1.f;
+        float2 na = make_float2(0.f, 0.f), nc = na;
+        for (int sp = 0; sp < ns32; ++sp) {
+          const float2 va = *reinterpret_cast<const float2*>(nl32 + sp * plane + ia);
+          na.x += va.x;
+          na.y += va.y;
+          if (b < nb) {
+            const float2 vb = *reinterpret_cast<const float2*>(nl32 + sp * plane + ib);
+            nc.x += vb.x;
+            nc.y += vb.y;
+          }
+        }
+        ya.x = fmaf(sn, na.x, ya.x);
+        ya.y = fmaf(sn, na.y, ya.y);
+        yb.x = fmaf(sn, nc.x, yb.x);
+        yb.y = fmaf(sn, nc.y, yb.y);
+      }
       // kin as two floats: the product and the sum round once
       const float2 k2 = f64_split(kg);
       const float2 xa = x[(size_t)a * nh + h];
@@ -190,13 +211,40 @@ __global__ void __launch_bounds__(256) k_gamma_unpack_raw(int npw, int nb, const
                                             h ? fmaf(k2.x, xb.y, fmaf(k2.y, xb.y, yb.y)) : yb.y);
       }
     } else {
+      constexpr float rh = (float)kSqrt2, rl = (float)(kSqrt2 - (double)rh);
+      constexpr float ih = (float)kInvSqrt2, il = (float)(kInvSqrt2 - (double)ih);
+      // twice the local terms (the halving of h and l is exact)
+      float2 v[4] = {pair_sum(fp.x, fm.x), pair_sum(fp.y, -fm.y), pair_sum(fp.y, fm.y), pair_sum(fm.x, -fp.x)};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        v[i] = make_float2(0.5f * v[i].x, 0.5f * v[i].y);
+        if (up) v[i] = pair_times(v[i], rh, rl);
+      }
+      if (nl32) {
+        float2 n[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) n[i] = make_float2(0.f, 0.f);
+        for (int sp = 0; sp < ns32; ++sp) {
+          const float2 va = *reinterpret_cast<const float2*>(nl32 + sp * plane + ia);
+          n[0] = pair_add(n[0], make_float2(va.x, 0.f));
+          n[1] = pair_add(n[1], make_float2(va.y, 0.f));
+          if (b < nb) {
+            const float2 vb = *reinterpret_cast<const float2*>(nl32 + sp * plane + ib);
+            n[2] = pair_add(n[2], make_float2(vb.x, 0.f));
+            n[3] = pair_add(n[3], make_float2(vb.y, 0.f));
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (down) n[i] = pair_times(n[i], ih, il);
+          v[i] = pair_add(v[i], n[i]);
+        }
+      }
       const double2 xa = ld2(x + (size_t)a * nh + h);
-      st2(y + (size_t)a * nh + h, make_double2(fma(kg, xa.x, f32_to_f64(ya.x)),
-                                               h ? fma(kg, xa.y, f32_to_f64(ya.y)) : f32_to_f64(ya.y)));
+      st2(y + (size_t)a * nh + h, make_double2(pair_fma(kg, xa.x, v[0]), pair_fma(kg, h ? xa.y : 0.0, v[1])));
       if (b < nb) {
         const double2 xb = ld2(x + (size_t)b * nh + h);
-        st2(y + (size_t)b * nh + h, make_double2(fma(kg, xb.x, f32_to_f64(yb.x)),
-                                                 h ? fma(kg, xb.y, f32_to_f64(yb.y)) : f32_to_f64(yb.y)));
+        st2(y + (size_t)b * nh + h, make_double2(pair_fma(kg, xb.x, v[2]), pair_fma(kg, h ? xb.y : 0.0, v[3])));
       }
     }
   }
