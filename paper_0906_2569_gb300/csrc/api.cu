@@ -252,6 +252,8 @@ static int plan_for(Context& c, int n, FftPlan* out) {
   for (int pr = 0; pr < npr; ++pr) {
     std::vector<int> lines;
     line_tables(n, pr, lines, &ftw[pr], &cells[pr], &tt.axis[pr]);
+    if (pr == HPSI_MIXED && !lines.empty())
+      tt.axis[pr].gain = line_gain(tt.axis[pr], reinterpret_cast<const float2*>(lines.data() + ftw[pr]));
     at[pr] = all.size();
     all.insert(all.end(), lines.begin(), lines.end());
     while (all.size() % 4) all.push_back(0);   // the fixed-point twiddles are read as int4

@@ -50,6 +50,7 @@ struct FxTw;
 struct LineAxis {
   int n = 0, r1 = 0, r2 = 0, s2 = 0;
   int twiddled = 0;
+  double gain = 1.0;              // float32: the two transforms' mean diagonal over n (line_gain)
   const FxTw* fxtw = nullptr;     // e^{2 pi i j / n} in fixed point and in float32 (Cooley-Tukey form only)
   const float2* ftw = nullptr;
   const int* cell = nullptr;      // cell of every index before the inverse transform, and
@@ -310,6 +311,7 @@ size_t local_scratch_per_band(const Problem& p, int precision);
 // Bytes of one buffer of stick rows of nb bands (the fast paths keep two); the fixed-point path keeps its block
 // exponents behind the rows.
 size_t local_row_bytes(const Problem& p, int precision, int nb);
+double line_gain(const LineAxis& ax, const float2* tw);
 void line_tables(int n, int precision, std::vector<int>& table, size_t* ftw, size_t* cells, LineAxis* ax);
 // Columns per x chunk and threads per CTA of a plane kernel (line_tiles.cpp): `base` + cw `col` bytes of shared memory a CTA,
 // `threads` resident threads an SM at most; *cw = 0 if nothing fits.

@@ -20,6 +20,8 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <utility>
+#include <vector>
 
 #include "convert.cuh"
 #include "float_fft.cuh"
@@ -267,14 +269,14 @@ __global__ void __launch_bounds__(256) k_hpsi_batch(const __grid_constant__ Fast
   if (nl.nitems > 0) nonlocal_phases(nl, pc.bar, pc.err, G, 3, reinterpret_cast<double2*>(smem_raw));
 }
 
-// V[j3][j2][j1] -> [j3][slot of j1][slot of j2] in float32, times 1/N_r
-__global__ void k_fast_v(LineAxis a1, LineAxis a2, int n3, double inv_nr, const double* __restrict__ v,
+// V[j3][j2][j1] -> [j3][slot of j1][slot of j2] in float32, times 1/N_r (and line_gain's correction)
+__global__ void k_fast_v(LineAxis a1, LineAxis a2, int n3, double scale, const double* __restrict__ v,
                          float* __restrict__ out) {
   const size_t n = (size_t)a1.n * a2.n * n3;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     const int j1 = (int)(i % a1.n), j2 = (int)(i / a1.n % a2.n);
     const size_t j3 = i / ((size_t)a1.n * a2.n);
-    out[(j3 * a1.n + a1.slot[j1]) * a2.n + a2.slot[j2]] = (float)(v[i] * inv_nr);
+    out[(j3 * a1.n + a1.slot[j1]) * a2.n + a2.slot[j2]] = (float)(v[i] * scale);
   }
 }
 
@@ -408,11 +410,59 @@ void float_plan(Problem& p, size_t smem_optin) {
   f.ok = f.smem_z <= smem_optin - 1024;
 }
 
+// The float32 constants of the codelets and twiddles are up to 2^-25 off, the same on every line, so the two transforms of a
+// line make an operator that is not n times the identity but off by up to 6e-8 of it (81 points; the 9-point codelet's
+// rotations): an error in <psi|V|psi> that does not average out as the other roundings do.  This is that operator's
+// mean diagonal over n, with the same constants in double, by which V is divided: what stays is a tenth of it
+// (eigenvalues on 36^3 and 45^3 boxes: 5.4e-8 and 5.9e-8 -> 6e-9 Ha from the constants; of mixed solves there in
+// all 7.0e-8 and 1.1e-7 -> 1.7e-8 and 5.1e-8).
+double line_gain(const LineAxis& ax, const float2* tw) {
+  const int n = ax.n, r1 = ax.r1, r2 = ax.r2;
+  std::vector<double2> w(n);
+  auto stage = [&](int r, int items, int first, int step, bool twiddled) {   // item i: cells i first + a step
+    for (int i = 0; i < items; ++i) {
+      double2 v[16];
+      for (int a = 0; a < r; ++a) v[a] = w[i * first + a * step];
+      switch (r) {
+        case 2: FfDft<2>::run(v); break;
+        case 3: FfDft<3>::run(v); break;
+        case 4: FfDft<4>::run(v); break;
+        case 5: FfDft<5>::run(v); break;
+        case 6: FfDft<6>::run(v); break;
+        case 8: FfDft<8>::run(v); break;
+        case 9: FfDft<9>::run(v); break;
+        case 10: FfDft<10>::run(v); break;
+        case 12: FfDft<12>::run(v); break;
+        case 15: FfDft<15>::run(v); break;
+        default: FfDft<16>::run(v);
+      }
+      for (int a = 0; a < r; ++a) {
+        if (twiddled && a > 0) v[a] = ff_mul(v[a], tw[i * a].x, tw[i * a].y);
+        w[i * first + a * step] = v[a];
+      }
+    }
+  };
+  double sum = 0.0;
+  for (int a = 0; a < r1; ++a)
+    for (int t = 0; t < r2; ++t) {
+      std::fill(w.begin(), w.end(), make_double2(0.0, 0.0));
+      w[a * r2 + t].x = 1.0;
+      stage(r1, r2, 1, r2, ax.twiddled);
+      stage(r2, r1, r2, 1, false);
+      for (double2& v : w) std::swap(v.x, v.y);   // the opposite sign, as in plane_tile
+      stage(r2, r1, r2, 1, ax.twiddled);
+      stage(r1, r2, 1, r2, false);
+      sum += w[a * r2 + t].y;
+    }
+  return sum / ((double)n * n);
+}
+
 // V / N_r in float32 in slot order (vbufs[slot + 3]) from the float64 V.
 int float_potential(Context& c, int slot, const LineAxis ax[3], int kernel_class) {
   const size_t nr = (size_t)ax[0].n * ax[1].n * ax[2].n;
+  const double scale = 1.0 / ((double)nr * ax[0].gain * ax[1].gain * ax[2].gain);
   HPSI_LAUNCH(c, kernel_class, (k_fast_v<<<(int)std::min<size_t>(4 * c.sm_count, (nr + 255) / 256), 256, 0, c.stream>>>(
-                                   ax[0], ax[1], ax[2].n, 1.0 / (double)nr, static_cast<const double*>(c.vbufs[slot]),
+                                   ax[0], ax[1], ax[2].n, scale, static_cast<const double*>(c.vbufs[slot]),
                                    static_cast<float*>(c.vbufs[slot + 3]))));
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "float32 potential");
