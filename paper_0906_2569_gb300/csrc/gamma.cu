@@ -152,17 +152,17 @@ __device__ __forceinline__ float2 pair_times(float2 a, float ch, float cl) {   /
   const float p = __fmul_rn(a.x, ch);
   return make_float2(p, __fmaf_rn(a.x, ch, -p) + __fmaf_rn(a.x, cl, a.y * ch));
 }
-// kg x + (a.x + a.y) in float64 (an infinite or NaN a.x stands alone)
-__device__ __forceinline__ double pair_fma(double kg, double x, float2 a) {
-  return fma(kg, x, f32_to_f64(a.x)) + f32_to_f64(fabsf(a.x) <= 3.402823466e38f ? a.y : 0.f);
+// kg x + (a.x + a.y) 2^-sh in float64 (an infinite or NaN a.x stands alone)
+__device__ __forceinline__ double pair_fma(double kg, double x, float2 a, int sh) {
+  return fma(kg, x, f32_to_f64(a.x, sh)) + f32_to_f64(fabsf(a.x) <= 3.402823466e38f ? a.y : 0.f, sh);
 }
 
-// Unpack the raw local term L f of a pair and add the kinetic term and the nonlocal term's float32 partial sums nl32
+// Unpack 2^sh times the raw local term L f of a pair and add the kinetic term and the nonlocal term's float32 partial sums nl32
 // [ns32][nb][nr] in real-basis coordinates (null: none).  Float64 results: the bands' combinations, the sqrt2 factors and
 // the sums over the partials to 2^-47 as pairs of floats, the kinetic term and the last sum in float64.  Float32
 // results: in float32, the kinetic term as one FMA chain.
 template <typename S>
-__global__ void __launch_bounds__(256) k_gamma_unpack_raw(int npw, int nb, const float2* __restrict__ F, int scaled,
+__global__ void __launch_bounds__(256) k_gamma_unpack_raw(int npw, int nb, const float2* __restrict__ F, int sh, int scaled,
                                                           const double* __restrict__ kin, const S* __restrict__ x,
                                                           const float* __restrict__ nl32, int ns32, S* __restrict__ y) {
   const int nh = (npw + 1) / 2, i0 = nh - 1;
@@ -176,8 +176,9 @@ __global__ void __launch_bounds__(256) k_gamma_unpack_raw(int npw, int nb, const
     const double kg = kin[i0 + h];
     // conj(F(-G)) = (fm.x, -fm.y)
     if constexpr (sizeof(S) == sizeof(float2)) {
-      float2 ya = make_float2(0.5f * (fp.x + fm.x), 0.5f * (fp.y - fm.y));
-      float2 yb = make_float2(0.5f * (fp.y + fm.y), -0.5f * (fp.x - fm.x));
+      const float half = __uint_as_float((unsigned)(126 - sh) << 23);
+      float2 ya = make_float2(half * (fp.x + fm.x), half * (fp.y - fm.y));
+      float2 yb = make_float2(half * (fp.y + fm.y), -half * (fp.x - fm.x));
       if (up) {
         ya.x *= (float)kSqrt2; ya.y *= (float)kSqrt2;
         yb.x *= (float)kSqrt2; yb.y *= (float)kSqrt2;
@@ -213,6 +214,7 @@ __global__ void __launch_bounds__(256) k_gamma_unpack_raw(int npw, int nb, const
     } else {
       constexpr float rh = (float)kSqrt2, rl = (float)(kSqrt2 - (double)rh);
       constexpr float ih = (float)kInvSqrt2, il = (float)(kInvSqrt2 - (double)ih);
+      const float pow2 = __uint_as_float((unsigned)(127 + sh) << 23);
       // twice the local terms (the halving of h and l is exact)
       float2 v[4] = {pair_sum(fp.x, fm.x), pair_sum(fp.y, -fm.y), pair_sum(fp.y, fm.y), pair_sum(fm.x, -fp.x)};
 #pragma unroll
@@ -237,14 +239,14 @@ __global__ void __launch_bounds__(256) k_gamma_unpack_raw(int npw, int nb, const
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           if (down) n[i] = pair_times(n[i], ih, il);
-          v[i] = pair_add(v[i], n[i]);
+          v[i] = pair_add(v[i], make_float2(n[i].x * pow2, n[i].y * pow2));
         }
       }
       const double2 xa = ld2(x + (size_t)a * nh + h);
-      st2(y + (size_t)a * nh + h, make_double2(pair_fma(kg, xa.x, v[0]), pair_fma(kg, h ? xa.y : 0.0, v[1])));
+      st2(y + (size_t)a * nh + h, make_double2(pair_fma(kg, xa.x, v[0], sh), pair_fma(kg, h ? xa.y : 0.0, v[1], sh)));
       if (b < nb) {
         const double2 xb = ld2(x + (size_t)b * nh + h);
-        st2(y + (size_t)b * nh + h, make_double2(pair_fma(kg, xb.x, v[2]), pair_fma(kg, h ? xb.y : 0.0, v[3])));
+        st2(y + (size_t)b * nh + h, make_double2(pair_fma(kg, xb.x, v[2], sh), pair_fma(kg, h ? xb.y : 0.0, v[3], sh)));
       }
     }
   }
@@ -509,8 +511,8 @@ static int gamma_apply_t(Context& c, int ik, const S* x, S* y, int nb, bool scal
   const dim3 gu(grid_x((p.npw + 1) / 2), npairs);
   if (raw)
     HPSI_LAUNCH(c, HPSI_K_GAMMA, (k_gamma_unpack_raw<S><<<gu, 256, 0, c.stream>>>(
-                                     p.npw, nb, static_cast<const float2*>(c.ws.gout), scaled ? 1 : 0, p.d_kin, x, nl32,
-                                     ns32, y)));
+                                     p.npw, nb, static_cast<const float2*>(c.ws.gout), p.fast.sh, scaled ? 1 : 0, p.d_kin, x,
+                                     nl32, ns32, y)));
   else
     HPSI_LAUNCH(c, HPSI_K_GAMMA, (k_gamma_unpack<S><<<gu, 256, 0, c.stream>>>(p.npw, nb, F, scaled ? 1 : 0, nl64, nl32,
                                                                               ns32, y)));

@@ -76,6 +76,7 @@ struct SlicePlanes {
 // Tile sizes of a problem's float32 local term (local_fast.cu).
 struct FloatPlan {
   bool ok = false;
+  int sh = 0;                     // the kernels' V is V 2^sh / N_r, 2^sh the power of two below N_r
   LineAxis ax[3];
   int cw = 0, nch = 0, block = 0;
   size_t smem_z = 0, smem_p = 0;
@@ -184,7 +185,7 @@ struct Context {
   std::vector<Problem> probs;
   std::vector<TwiddleTable> tw;
   std::vector<void*> vbufs;            // owned V buffers, four per slot: float64, float32, fixed point (then its
-                                       // scale), float32 / N_r in slot order (the last two may be null)
+                                       // scale), float32 2^sh / N_r in slot order (the last two may be null)
   Workspace ws;
   std::string err;
   double opt_tau = 0.1;                // Davidson: |<k+G|H|k+G> - eps| is kept >= tau (Ha)
@@ -333,7 +334,7 @@ int local_fixed_persistent(Context& c, int nitem, const int* prob, const int* nb
                            double2* const* hpsi, void* const* zt, void* const* yb, bool with_nl, bool* done);
 int local_fast_apply(Context& c, const Problem& p, const double2* psi, double2* hpsi, int nbnd, void* Zt, void* Yb,
                      int nbb);
-// The local term alone (no kinetic part) of float32 bands in float32; needs local_fast_ok in float32.
+// 2^(p.fast.sh) times the local term alone (no kinetic part) of float32 bands in float32; needs local_fast_ok in float32.
 int local_raw_apply(Context& c, const Problem& p, const float2* f, float2* F, int nbnd);
 int local_fast_apply_raw(Context& c, const Problem& p, const float2* f, float2* F, int nbnd, void* Zt, void* Yb, int nbb);
 int local_fast_apply_multi(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,

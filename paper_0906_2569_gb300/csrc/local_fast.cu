@@ -5,7 +5,8 @@
 //   k_plane  per (z-plane, band): the plane [m1-plane][j2] in shared memory; inverse y, then in chunks of columns
 //            inverse x, x V, forward x keeping the m1-planes, then forward y keeping the sticks -> Y[b][j3][stick].
 //   k_zfwd   per (chunk of sticks, band): forward z-transform, keep the sphere, add the kinetic term |k+G|^2/2 psi(G)
-//            in float64 (1/N_r is in the float32 copy of V).
+//            in float64 (1/N_r is in the float32 copy of V but for a power of two, which would take values of small bands below
+//            float32's range before the forward transform sums them).
 // The transforms are the in-place two-stage form of line_stages.cuh: a stage's items are dealt over all threads of the CTA,
 // coprime factors need no twiddles, and one kernel (run-time radix switch) serves every box, cubic or not.
 // psi is read, and H psi written, by integer conversions (convert.cuh), since a cast costs as much as a float64 FMA.
@@ -15,11 +16,12 @@
 // 240 us against register codelets with a fixed line group per warp (24 to 30 of 32 lanes busy, cubic boxes of
 // 20 edges only; the others had the generic kernels).
 //
-// The raw form takes float32 psi and gives the local term alone in float32, [nb][npw] both: the Gamma form packs two
+// The raw form takes float32 psi and gives 2^sh times the local term alone in float32, [nb][npw] both: the Gamma form packs two
 // real bands into one complex one in float32 and adds the kinetic term itself (gamma.cu).
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <utility>
 #include <vector>
 
@@ -46,6 +48,7 @@ struct FastItem {
   LineAxis ax[3];
   int cw, nch;                 // columns per x chunk, z chunks
   int raw;
+  int sh;                      // V holds 2^sh / N_r: results times 2^-sh
   const int *soff, *zoff, *zbeg;   // Problem's lookup tables
   const int* xmap;             // [n1]: plane of ix or -1
   const void* psi;             // double2 (raw: float2) [nb][npw]
@@ -53,7 +56,7 @@ struct FastItem {
   const double* kin;
   float2* Zt;                  // [nb][n3][nst]
   float2* Yb;
-  const float* V;              // [n3][slot of j1][slot of j2], V / N_r
+  const float* V;              // [n3][slot of j1][slot of j2], V 2^sh / N_r
 };
 
 // Every launch takes its items by value (the parameter block is 32 KB on sm_70 and later).
@@ -210,7 +213,7 @@ __device__ __forceinline__ void zfwd_tile(const FastItem& a, int ch, int b, unsi
     staged_loop(ng, [&](int i) { return In{ps[i], a.kin[g0 + i], a.zoff[g0 + i]}; },
                 [&](int i, In q) {
                   const float2 v = L[q.at];   // swapped
-                  out[i] = make_double2(fma(q.kg, q.x.x, f32_to_f64(v.y)), fma(q.kg, q.x.y, f32_to_f64(v.x)));
+                  out[i] = make_double2(fma(q.kg, q.x.x, f32_to_f64(v.y, a.sh)), fma(q.kg, q.x.y, f32_to_f64(v.x, a.sh)));
                 });
   }
 }
@@ -269,7 +272,10 @@ __global__ void __launch_bounds__(256) k_hpsi_batch(const __grid_constant__ Fast
   if (nl.nitems > 0) nonlocal_phases(nl, pc.bar, pc.err, G, 3, reinterpret_cast<double2*>(smem_raw));
 }
 
-// V[j3][j2][j1] -> [j3][slot of j1][slot of j2] in float32, times 1/N_r (and line_gain's correction)
+// floor(log2 N_r)
+inline int scale_bits(const int n[3]) { return std::ilogb((double)n[0] * n[1] * n[2]); }
+
+// V[j3][j2][j1] -> [j3][slot of j1][slot of j2] in float32, times 2^scale_bits / N_r (and line_gain's correction)
 __global__ void k_fast_v(LineAxis a1, LineAxis a2, int n3, double scale, const double* __restrict__ v,
                          float* __restrict__ out) {
   const size_t n = (size_t)a1.n * a2.n * n3;
@@ -309,6 +315,7 @@ struct FastLaunch {
     it.cw = f.cw;
     it.nch = f.nch;
     it.raw = raw;
+    it.sh = f.sh;
     it.soff = p.tab[HPSI_MIXED].soff;
     it.zoff = p.tab[HPSI_MIXED].zoff;
     it.zbeg = p.tab[HPSI_MIXED].zbeg;
@@ -407,6 +414,7 @@ void float_plan(Problem& p, size_t smem_optin) {
               &f.cw, &f.block);
   if (f.cw == 0) return;
   f.smem_p = base + col * f.cw;
+  f.sh = scale_bits(p.n);
   f.ok = f.smem_z <= smem_optin - 1024;
 }
 
@@ -457,10 +465,11 @@ double line_gain(const LineAxis& ax, const float2* tw) {
   return sum / ((double)n * n);
 }
 
-// V / N_r in float32 in slot order (vbufs[slot + 3]) from the float64 V.
+// V 2^sh / N_r in float32 in slot order (vbufs[slot + 3]) from the float64 V.
 int float_potential(Context& c, int slot, const LineAxis ax[3], int kernel_class) {
   const size_t nr = (size_t)ax[0].n * ax[1].n * ax[2].n;
-  const double scale = 1.0 / ((double)nr * ax[0].gain * ax[1].gain * ax[2].gain);
+  const int n[3] = {ax[0].n, ax[1].n, ax[2].n};
+  const double scale = std::ldexp(1.0, scale_bits(n)) / ((double)nr * ax[0].gain * ax[1].gain * ax[2].gain);
   HPSI_LAUNCH(c, kernel_class, (k_fast_v<<<(int)std::min<size_t>(4 * c.sm_count, (nr + 255) / 256), 256, 0, c.stream>>>(
                                    ax[0], ax[1], ax[2].n, scale, static_cast<const double*>(c.vbufs[slot]),
                                    static_cast<float*>(c.vbufs[slot + 3]))));
