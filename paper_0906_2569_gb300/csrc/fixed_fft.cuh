@@ -340,13 +340,12 @@ struct FxShift {
   }
 };
 
-// A float64 from its bits as the integer m 2^(E - e0), E its exponent field and m its 53-bit significand (that is,
-// x 2^(1075 - e0)), rounded; zero and subnormal x give 0.
+// A float64 from its bits as the integer m 2^(E - e0), E its exponent field (1 for a subnormal x) and m its significand
+// (that is, x 2^(1075 - e0)), rounded.
 __host__ __device__ __forceinline__ long long fx_from_bits(long long bits, int e0) {
   const int ex = (int)((bits >> 52) & 0x7ff);
-  if (ex == 0) return 0;
-  const long long m = (bits & 0xfffffffffffffLL) | 0x10000000000000LL;
-  const int sh = ex - e0;
+  const long long m = (bits & 0xfffffffffffffLL) | (ex ? 0x10000000000000LL : 0LL);
+  const int sh = (ex ? ex : 1) - e0;
   const long long q = sh >= 0 ? m << sh : (sh < -60 ? 0 : (m + (1LL << (-sh - 1))) >> -sh);
   return bits < 0 ? -q : q;
 }

@@ -140,18 +140,20 @@ __device__ __forceinline__ void fx_zinv_tile(const FxItem& a, int ch, int b, uns
   for (int i = threadIdx.x; i < n * ld; i += blockDim.x) L[i] = {0, 0};
   __syncthreads();
   // float64 bits into their places, and the largest exponent field
-  unsigned hi = 0;
+  unsigned hi = 0, any = 0;
   staged_loop(ng, [&](int i) { return FxPlaced{ps[i], a.zoff[g0 + i]}; },
               [&](int, FxPlaced q) {
                 hi = max(hi, max((unsigned)(q.v.x >> 32) & 0x7fffffffu, (unsigned)(q.v.y >> 32) & 0x7fffffffu));
+                any |= (unsigned)q.v.x | (unsigned)q.v.y;
                 L[q.at] = q.v;
               });
-  hi = __reduce_max_sync(0xffffffffu, hi);
-  if (lane == 0) atomicMax(&sh->emax, (int)(hi >> 20));
+  hi = __reduce_max_sync(0xffffffffu, max(hi, any != 0 ? 1u : 0u));
+  if (lane == 0) atomicMax(&sh->emax, (int)hi);
   __syncthreads();
-  const int emax = sh->emax;
+  hi = (unsigned)sh->emax;
+  const int emax = max(1, (int)(hi >> 20));   // subnormal numbers have exponent 1
   if (threadIdx.x == 0)
-    a.Ez[(size_t)b * a.nch + ch] = emax == 0x7ff ? kFxNan : emax == 0 ? kFxZero : emax - 1022 - 63 + a.hz;
+    a.Ez[(size_t)b * a.nch + ch] = emax == 0x7ff ? kFxNan : hi == 0 ? kFxZero : emax - 1022 - 63 + a.hz;
   if (emax == 0x7ff) return;   // (every thread) the plane kernel reads the exponent only
   // |x| < 2^(emax - 1022), so q = x 2^(63 - hz - (emax - 1022)) stays below 2^(63 - hz).  The bits become integers as the
   // first stage reads them (a cell without a G holds the bits of zero).
@@ -375,11 +377,16 @@ __device__ __forceinline__ void fx_zfwd_tile(const FxItem& a, int ch, int b, uns
     line_stage1<FixArith, MAXR, true>(a.ax[2], ns, tw, lines);
     __syncthreads();
   }
-  // 2^e / N_r: by its exponent field where that stays a normal number
+  // f = 2^e / N_r by its exponent field; where that would leave the normal numbers, f g with g = 2^-+1000: the results,
+  // 2^62 larger, may well be normal
   const int fe = (int)(__double_as_longlong(a.inv_nr) >> 52) + e;
-  const double f = bad                     ? __longlong_as_double(0x7ff8000000000000LL)
-                   : fe > 0 && fe < 0x7ff ? __longlong_as_double(__double_as_longlong(a.inv_nr) + ((long long)e << 52))
-                                          : ldexp(a.inv_nr, e);
+  const int shift = fe <= 0 ? 1000 : fe >= 0x7ff ? -1000 : 0;
+  const double f = bad                                    ? __longlong_as_double(0x7ff8000000000000LL)
+                   : fe + shift > 0 && fe + shift < 0x7ff ? __longlong_as_double(__double_as_longlong(a.inv_nr) +
+                                                                                 ((long long)(e + shift) << 52))
+                   : fe > 0                               ? INFINITY
+                                                          : 0.0;
+  const double g = __longlong_as_double((long long)(1023 - shift) << 52);
   struct Out {
     double2 x;
     double kg;
@@ -387,12 +394,18 @@ __device__ __forceinline__ void fx_zfwd_tile(const FxItem& a, int ch, int b, uns
   };
   const double2* ps = a.psi + (size_t)b * a.npw + g0;
   double2* out = a.hpsi + (size_t)b * a.npw + g0;
-  staged_loop(ng, [&](int i) { return Out{ps[i], a.kin[g0 + i], a.zoff[g0 + i]}; },
-              [&](int i, Out q) {
-                longlong2 v = {0, 0};
-                if (!bad) v = L[q.at];   // swapped
-                out[i] = make_double2(fma(q.kg, q.x.x, (double)v.y * f), fma(q.kg, q.x.y, (double)v.x * f));
-              });
+  auto load = [&](int i) { return Out{ps[i], a.kin[g0 + i], a.zoff[g0 + i]}; };
+  if (shift == 0 || bad)
+    staged_loop(ng, load, [&](int i, Out q) {
+      longlong2 v = {0, 0};
+      if (!bad) v = L[q.at];   // swapped
+      out[i] = make_double2(fma(q.kg, q.x.x, (double)v.y * f), fma(q.kg, q.x.y, (double)v.x * f));
+    });
+  else
+    staged_loop(ng, load, [&](int i, Out q) {
+      const longlong2 v = L[q.at];
+      out[i] = make_double2(fma(q.kg, q.x.x, (double)v.y * f * g), fma(q.kg, q.x.y, (double)v.x * f * g));
+    });
 }
 
 template <int MAXR>
@@ -469,9 +482,9 @@ __global__ void k_fx_vmax(size_t n, const double* __restrict__ v, unsigned long 
 // V[j3][j2][j1] -> [j3][slot of j1][slot of j2] as V 2^(62 - vexp), |V| < 2^vexp
 __global__ void k_fx_v(LineAxis a1, LineAxis a2, int n3, const double* __restrict__ v,
                        const unsigned long long* __restrict__ vmax, long long* __restrict__ out, int* __restrict__ vexp) {
-  const int emax = (int)(*vmax >> 52);
+  const int emax = max(1, (int)(*vmax >> 52));
   const size_t n = (size_t)a1.n * a2.n * n3;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *vexp = emax == 0x7ff ? kFxNan : emax == 0 ? 0 : emax - 1022;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *vexp = emax == 0x7ff ? kFxNan : *vmax == 0 ? 0 : emax - 1022;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     const int j1 = (int)(i % a1.n), j2 = (int)(i / a1.n % a2.n);
     const size_t j3 = i / ((size_t)a1.n * a2.n);

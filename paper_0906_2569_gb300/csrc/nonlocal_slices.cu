@@ -240,12 +240,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 // ---- digits -----------------------------------------------------------------------------------
 
 // exponent e of a row whose largest exponent field is f: |x| < 2^e (kRowNan: a non-finite entry)
-__device__ __forceinline__ int row_exponent(int f) { return f == 0x7ff ? kRowNan : f == 0 ? 0 : f - 1022; }
+__device__ __forceinline__ int row_exponent(int f) { return f == 0x7ff ? kRowNan : max(f, 1) - 1022; }
 
 // The digits of x 2^(62 - e), e the row's exponent from field f, most significant in the top byte, the lower seven
 // biased by 128 (so that all are plain bytes)
 __device__ __forceinline__ unsigned long long digits_of(double x, int f) {
-  const long long X = f == 0x7ff ? 0 : fx_from_bits(__double_as_longlong(x), f - 9);
+  const long long X = f == 0x7ff ? 0 : fx_from_bits(__double_as_longlong(x), max(f, 1) - 9);
   return (unsigned long long)X + 0x0080808080808080ULL;
 }
 // bf16 pattern of digit s, s > 0: byte - 128; s = 0: the signed top byte
