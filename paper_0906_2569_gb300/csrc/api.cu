@@ -103,8 +103,18 @@ int check_device_error(Context& c) {
   return HPSI_OK;
 }
 
-int ensure_buffer(Context& c, void** ptr, size_t* have, size_t need) {
-  if (need <= *have && *ptr) return HPSI_OK;
+cudaError_t device_malloc(Context& c, void** ptr, size_t bytes) {
+  cudaError_t e = cudaMalloc(ptr, bytes);
+  if (e == cudaErrorMemoryAllocation && release_slices(c)) {
+    cudaGetLastError();
+    e = cudaMalloc(ptr, bytes);
+  }
+  if (e != cudaSuccess) *ptr = nullptr;
+  return e;
+}
+
+bool try_buffer(Context& c, void** ptr, size_t* have, size_t need) {
+  if (need <= *have && *ptr) return true;
   c.ws.epoch++;
   if (*ptr) {
     cudaStreamSynchronize(c.stream);
@@ -112,14 +122,19 @@ int ensure_buffer(Context& c, void** ptr, size_t* have, size_t need) {
     *ptr = nullptr;
     *have = 0;
   }
-  cudaError_t e = cudaMalloc(ptr, std::max<size_t>(need, 256));
-  if (e != cudaSuccess) {
+  if (cudaMalloc(ptr, std::max<size_t>(need, 256)) != cudaSuccess) {
     cudaGetLastError();
     *ptr = nullptr;
-    return fail(c, HPSI_ENOMEM, "device allocation of " + std::to_string(need) + " bytes failed");
+    return false;
   }
   *have = std::max<size_t>(need, 256);
-  return HPSI_OK;
+  return true;
+}
+
+int ensure_buffer(Context& c, void** ptr, size_t* have, size_t need) {
+  if (try_buffer(c, ptr, have, need)) return HPSI_OK;
+  if (release_slices(c) && try_buffer(c, ptr, have, need)) return HPSI_OK;
+  return fail(c, HPSI_ENOMEM, "device allocation of " + std::to_string(need) + " bytes failed");
 }
 
 // <k+G|H|k+G> = |k+G|^2/2 + mean(V) + sum_{(p,q) in D} Re(beta_p(G) D_pq conj(beta_q(G)))
@@ -148,7 +163,7 @@ static int upload(Context& c, T** dst, const T* src, size_t n) {
     *dst = nullptr;
     return HPSI_OK;
   }
-  cudaError_t e = cudaMalloc((void**)dst, n * sizeof(T));
+  cudaError_t e = device_malloc(c, (void**)dst, n * sizeof(T));
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(c, HPSI_ENOMEM, "device allocation failed during setup");
@@ -212,7 +227,7 @@ static int upload_potential(Context& c, const int n[3], const double* vr, int* s
 int ensure_fixed_potential(Context& c, int slot, const LineAxis ax[3]) {
   if (c.vbufs[slot + 2]) return HPSI_OK;
   const size_t nr = (size_t)ax[0].n * ax[1].n * ax[2].n;
-  if (cudaMalloc(&c.vbufs[slot + 2], sizeof(long long) * nr + kFixedScaleBytes) != cudaSuccess) {
+  if (device_malloc(c, &c.vbufs[slot + 2], sizeof(long long) * nr + kFixedScaleBytes) != cudaSuccess) {
     cudaGetLastError();
     c.vbufs[slot + 2] = nullptr;
     return fail(c, HPSI_ENOMEM, "device allocation of the fixed-point potential failed");
@@ -222,7 +237,7 @@ int ensure_fixed_potential(Context& c, int slot, const LineAxis ax[3]) {
 
 static int ensure_float_potential(Context& c, int slot, const LineAxis ax[3]) {
   if (c.vbufs[slot + 3]) return HPSI_OK;
-  if (cudaMalloc(&c.vbufs[slot + 3], sizeof(float) * (size_t)ax[0].n * ax[1].n * ax[2].n) != cudaSuccess) {
+  if (device_malloc(c, &c.vbufs[slot + 3], sizeof(float) * (size_t)ax[0].n * ax[1].n * ax[2].n) != cudaSuccess) {
     cudaGetLastError();
     return fail(c, HPSI_ENOMEM, "device allocation failed during setup");
   }
@@ -485,7 +500,7 @@ static int finish_problem(Context& c, Problem& p, const double* vr, int vslot_sh
     if ((rc = upload(c, &p.d_rowptr, rowptr.data(), rowptr.size()))) return rc;
   }
   p.gamma_ok = gamma_applies(p, beta, dmat, &p.gamma_why);
-  cudaError_t e = cudaMalloc((void**)&p.d_hdiag, sizeof(double) * std::max(1, p.npw));
+  cudaError_t e = device_malloc(c, (void**)&p.d_hdiag, sizeof(double) * std::max(1, p.npw));
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(c, HPSI_ENOMEM, "device allocation failed during setup");
@@ -531,7 +546,7 @@ static void free_problem(Problem& p) {
   cudaFree(p.d_dvalr);
   cudaFree(p.d_betar_bf);
   cudaFree(p.d_betar_df);
-  for (SlicePlanes& s : p.slices) cudaFree(s.digits);
+  for (SlicePlanes& s : p.slices) cudaFree(s.owned);
 }
 
 static void free_context(Context& c) {

@@ -243,10 +243,10 @@ int ensure_cg(Context& c, int npw, int nbnd, CgState** out) {
     s->npw = std::max(npw, s->npw);
     s->nbnd = std::max(nbnd, s->nbnd);
     s->p2_ik = -1;
-    bool ok = cudaMalloc((void**)&s->work, sizeof(double2) * 6 * (size_t)s->npw) == cudaSuccess &&
-              cudaMalloc((void**)&s->coef, sizeof(double2) * (size_t)s->nbnd) == cudaSuccess &&
-              cudaMalloc((void**)&s->p2, sizeof(double) * (size_t)s->npw) == cudaSuccess &&
-              cudaMalloc((void**)&s->sc, sizeof(CgScalars)) == cudaSuccess;
+    bool ok = device_malloc(c, (void**)&s->work, sizeof(double2) * 6 * (size_t)s->npw) == cudaSuccess &&
+              device_malloc(c, (void**)&s->coef, sizeof(double2) * (size_t)s->nbnd) == cudaSuccess &&
+              device_malloc(c, (void**)&s->p2, sizeof(double) * (size_t)s->npw) == cudaSuccess &&
+              device_malloc(c, (void**)&s->sc, sizeof(CgScalars)) == cudaSuccess;
     if (!ok) {
       cudaGetLastError();
       return fail(c, HPSI_ENOMEM, "cg_solve: workspace allocation failed");

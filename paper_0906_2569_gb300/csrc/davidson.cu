@@ -287,7 +287,7 @@ static int alloc_work(Context& c, DavHandles& h, int npw, int nbnd, bool mixed) 
   w.mmax = mmax;
   w.mixed = mixed;
   auto al = [&](void** p, size_t bytes) -> bool {
-    if (cudaMalloc(p, std::max<size_t>(bytes, 256)) != cudaSuccess) {
+    if (device_malloc(c, p, std::max<size_t>(bytes, 256)) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
@@ -718,7 +718,7 @@ static int tall_gemm32(Context& c, DavHandles& h, int npw, int nb, int k, const 
     cudaFree(w.part32);
     w.part32 = nullptr;
     w.part_cap = 0;
-    if (cudaMalloc((void**)&w.part32, sizeof(float2) * need) != cudaSuccess) {
+    if (device_malloc(c, (void**)&w.part32, sizeof(float2) * need) != cudaSuccess) {
       cudaGetLastError();
       return fail(c, HPSI_ENOMEM, "davidson_solve: chunk-product allocation failed");
     }

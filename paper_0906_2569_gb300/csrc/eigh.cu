@@ -802,7 +802,7 @@ int grow(Context& c, EighState& s, int n, int nwant) {
   s.wcap = wcap0;
   const int N = std::max(n, s.ncap), W = std::max(nwant, s.wcap);
   bool ok = true;
-  auto al = [&](void** q, size_t bytes) { ok = ok && cudaMalloc(q, std::max<size_t>(bytes, 16)) == cudaSuccess; };
+  auto al = [&](void** q, size_t bytes) { ok = ok && device_malloc(c, q, std::max<size_t>(bytes, 16)) == cudaSuccess; };
   al((void**)&s.d, sizeof(double) * N);
   al((void**)&s.e, sizeof(double) * N);
   al((void**)&s.e2, sizeof(double) * N);
@@ -846,7 +846,7 @@ int invit_all(Context& c, EighState& s, int n, int nwant, int iters) {
     cudaFree(s.invs);
     s.invs = nullptr;
     s.invcap = 0;
-    if (cudaMalloc((void**)&s.invs, need) != cudaSuccess) {
+    if (device_malloc(c, (void**)&s.invs, need) != cudaSuccess) {
       cudaGetLastError();
       return fail(c, HPSI_ENOMEM, "inverse-iteration scratch allocation failed");
     }
@@ -885,9 +885,9 @@ int eigh_zheevdx(Context& c, EighState& s, const double2* a, int lda, int n, int
   if (n > s.zcap) {
     free_zheevdx(s);
     int lw = 0, meig = 0;
-    if (cudaMalloc((void**)&s.acopy, sizeof(double2) * (size_t)n * n) != cudaSuccess ||
-        cudaMalloc((void**)&s.wfull, sizeof(double) * n) != cudaSuccess ||
-        cudaMalloc((void**)&s.zinfo, sizeof(int)) != cudaSuccess) {
+    if (device_malloc(c, (void**)&s.acopy, sizeof(double2) * (size_t)n * n) != cudaSuccess ||
+        device_malloc(c, (void**)&s.wfull, sizeof(double) * n) != cudaSuccess ||
+        device_malloc(c, (void**)&s.zinfo, sizeof(int)) != cudaSuccess) {
       free_zheevdx(s);
       return fail(c, HPSI_ENOMEM, "eigensolver: zheevdx workspace allocation failed");
     }
@@ -898,7 +898,7 @@ int eigh_zheevdx(Context& c, EighState& s, const double2* a, int lda, int n, int
       return fail(c, HPSI_ECUDA, "eigensolver: zheevdx buffer size failed");
     }
     s.zlwork = std::max(lw, 1);
-    if (cudaMalloc((void**)&s.zwork, sizeof(double2) * s.zlwork) != cudaSuccess) {
+    if (device_malloc(c, (void**)&s.zwork, sizeof(double2) * s.zlwork) != cudaSuccess) {
       free_zheevdx(s);
       return fail(c, HPSI_ENOMEM, "eigensolver: zheevdx workspace allocation failed");
     }

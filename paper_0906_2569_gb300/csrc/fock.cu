@@ -193,7 +193,7 @@ static int fock_alloc(Context& c, const Problem& p, int nocc, FockWork** out) {
   if (w->nr == nr && w->nocc >= nocc && w->npw == p.npw) return HPSI_OK;
   free_fock(*w);
   auto al = [&](void** q, size_t bytes) -> bool {
-    if (cudaMalloc(q, std::max<size_t>(bytes, 256)) != cudaSuccess) {
+    if (device_malloc(c, q, std::max<size_t>(bytes, 256)) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }

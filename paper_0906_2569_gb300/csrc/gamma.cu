@@ -404,9 +404,9 @@ int gamma_nl_prepare(Context& c, Problem& p) {
     }
     const int nr = 2 * ((p.npw + 1) / 2);
     double2* dw = nullptr;
-    if (cudaMalloc((void**)&p.d_betar, sizeof(double) * (size_t)P * nr) != cudaSuccess ||
-        cudaMalloc((void**)&p.d_dvalr, sizeof(double) * (size_t)std::max(1, p.nnz)) != cudaSuccess ||
-        cudaMalloc((void**)&dw, sizeof(double2) * P) != cudaSuccess) {
+    if (device_malloc(c, (void**)&p.d_betar, sizeof(double) * (size_t)P * nr) != cudaSuccess ||
+        device_malloc(c, (void**)&p.d_dvalr, sizeof(double) * (size_t)std::max(1, p.nnz)) != cudaSuccess ||
+        device_malloc(c, (void**)&dw, sizeof(double2) * P) != cudaSuccess) {
       cudaGetLastError();
       cudaFree(p.d_betar);
       cudaFree(p.d_dvalr);
@@ -923,7 +923,7 @@ int GammaDavidson<T>::alloc(int N) {
   w.kmax = std::max(N, mmax / 2);
   const size_t n2 = 2 * (size_t)w.nh, v = sizeof(T) * n2, nt = std::max(N, w.kmax);
   auto al = [&](void** p, size_t bytes) -> bool {
-    if (cudaMalloc(p, std::max<size_t>(bytes, 256)) != cudaSuccess) {
+    if (device_malloc(c, p, std::max<size_t>(bytes, 256)) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }

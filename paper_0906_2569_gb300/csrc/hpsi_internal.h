@@ -70,7 +70,8 @@ struct SlicePlanes {
   void* digits = nullptr;
   int* exps = nullptr;
   int kpad = 0;
-  bool no_room = false;   // the device had no memory for them
+  void* owned = nullptr;  // the allocation, of these planes or of both of a pair
+  bool no_room = false;   // the device had no memory for them, or needed it back
 };
 
 // Tile sizes of a problem's float32 local term (local_fast.cu).
@@ -389,7 +390,13 @@ int dscale_fp64(Context& c, const Problem& p, int nb, int nsplit, double2* part,
 int gamma_dscale_fp64(Context& c, const Problem& p, int nb, int nsplit, const double* part, double* w);
 
 // ---- context helpers (api.cpp) ----
+// A workspace of at least `need` bytes.  The projectors' digit planes can be done without: where the device is out of
+// memory, ensure_buffer and device_malloc release them and try again; try_buffer, for the digit products themselves, does
+// not (false: no room, *ptr null).
 int ensure_buffer(Context& c, void** ptr, size_t* have, size_t need);
+bool try_buffer(Context& c, void** ptr, size_t* have, size_t need);
+cudaError_t device_malloc(Context& c, void** ptr, size_t bytes);
+bool release_slices(Context& c);   // false: there were none
 int fail(Context& c, int code, const std::string& msg);
 // Lets kernels use all of the device's opt-in shared memory, once per device; `devices` is the call site's record of those
 // done.  The attribute belongs to the device's copy of a kernel and every context sets the same value, so that

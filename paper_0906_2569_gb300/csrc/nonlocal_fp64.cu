@@ -275,7 +275,7 @@ int gamma_prepare_df(Context& c, Problem& p) {
   if (p.nproj == 0 || p.d_betar_df) return HPSI_OK;
   const int nr = 2 * ((p.npw + 1) / 2);
   const size_t n = (size_t)p.nproj * nr;
-  if (cudaMalloc((void**)&p.d_betar_df, sizeof(float2) * n) != cudaSuccess) {
+  if (device_malloc(c, (void**)&p.d_betar_df, sizeof(float2) * n) != cudaSuccess) {
     cudaGetLastError();
     p.d_betar_df = nullptr;
     return fail(c, HPSI_ENOMEM, "device allocation of the Gamma-form double-float projectors failed");

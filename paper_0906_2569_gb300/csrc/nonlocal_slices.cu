@@ -431,41 +431,63 @@ int slice_gemm(Context& c, const __nv_bfloat16* A, const int* ea, int M, const _
 }  // namespace
 
 // Digit planes of the projectors, made on first use: which = 0: calbec's A, 1: add_vuspsi's A (complex form); 2, 3: the
-// same of the Gamma form.  *ok = false, and nothing wrong, when the device has no room (the float64 CUDA-core kernels
-// serve then).
+// same of the Gamma form.  They take twice the projectors' memory each; a float64 context, which needs both, makes them
+// together.  *ok = false, and nothing wrong, when the device has no room (the float64 CUDA-core kernels serve then, for the
+// life of the context; the other planes of the pair are not kept either).
 static int slice_planes(Context& c, const Problem& p, int which, bool* ok) {
-  SlicePlanes& s = p.slices[which];
-  *ok = s.digits != nullptr;
-  if (s.digits || s.no_room) return HPSI_OK;
-  const bool real = which >= 2, add = which & 1;
+  *ok = p.slices[which].digits != nullptr;
+  const int first = which & ~1;
+  if (*ok || p.slices[first].no_room) return HPSI_OK;
+  const bool real = which >= 2, both = c.precision == HPSI_FP64;
   const int P = p.nproj, len = real ? 2 * ((p.npw + 1) / 2) : 2 * p.npw;   // doubles of a projector
   const int cols = real ? len : p.npw;
-  const size_t rows = add ? cols : P;
-  const int kpad = pad32(add ? (real ? P : 2 * P) : len);
-  const size_t bytes = al256(sizeof(__nv_bfloat16) * kDigits * rows * kpad);
-  const size_t ints = rows + P;   // row exponents, and room for the rows' exponent fields
-  if (cudaMalloc(&s.digits, bytes + sizeof(int) * ints) != cudaSuccess) {
+  size_t rows[2], at[2] = {0, 0}, ints[2], total = 0;
+  int kpad[2];
+  for (int i = 0; i < 2; ++i) {
+    rows[i] = i ? cols : P;
+    kpad[i] = pad32(i ? (real ? P : 2 * P) : len);
+    ints[i] = al256(sizeof(__nv_bfloat16) * kDigits * rows[i] * kpad[i]);   // then row exponents, and room for the
+    if (!both && first + i != which) continue;                              // rows' exponent fields
+    at[i] = total;
+    total += ints[i] + al256(sizeof(int) * (rows[i] + P));
+  }
+  void* mem = nullptr;
+  if (cudaMalloc(&mem, total) != cudaSuccess) {
     cudaGetLastError();
-    s.digits = nullptr;
-    s.no_room = true;
+    for (int i = 0; i < 2; ++i) {
+      SlicePlanes& s = p.slices[first + i];
+      if (s.owned) {
+        cudaStreamSynchronize(c.stream);
+        cudaFree(s.owned);
+        c.ws.epoch++;   // captured batches refer to them
+      }
+      s = SlicePlanes();
+      s.no_room = true;
+    }
     return HPSI_OK;
   }
-  s.exps = reinterpret_cast<int*>(static_cast<unsigned char*>(s.digits) + bytes);
-  s.kpad = kpad;
+  p.slices[which].owned = mem;
   const double* beta = real ? p.d_betar : reinterpret_cast<const double*>(p.d_beta);
-  __nv_bfloat16* d = static_cast<__nv_bfloat16*>(s.digits);
-  if (add) {
-    const int grid = (cols + 31) / 32;
-    if (real) HPSI_LAUNCH(c, HPSI_K_SPLIT, (k_digits_transposed<1><<<grid, 256, 0, c.stream>>>(P, cols, kpad, beta, d, s.exps)));
-    else HPSI_LAUNCH(c, HPSI_K_SPLIT, (k_digits_transposed<2><<<grid, 256, 0, c.stream>>>(P, cols, kpad, beta, d, s.exps)));
-  } else {
-    int* field = s.exps + rows;
-    cudaError_t e = cudaMemsetAsync(field, 0, sizeof(int) * P, c.stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "projector digit setup");
-    const dim3 grid(std::max(1, std::min(64, kpad / 512)), std::min(P, 65535));
-    HPSI_LAUNCH(c, HPSI_K_SPLIT, (k_row_field<double><<<grid, 256, 0, c.stream>>>(P, len, 1, beta, field)));
-    HPSI_LAUNCH(c, HPSI_K_SPLIT,
-                (k_digits<double><<<grid, 256, 0, c.stream>>>(P, len, kpad, 0, 1, beta, field, d, s.exps)));
+  for (int i = 0; i < 2; ++i) {
+    if (!both && first + i != which) continue;
+    SlicePlanes& s = p.slices[first + i];
+    s.digits = static_cast<unsigned char*>(mem) + at[i];
+    s.exps = reinterpret_cast<int*>(static_cast<unsigned char*>(s.digits) + ints[i]);
+    s.kpad = kpad[i];
+    __nv_bfloat16* d = static_cast<__nv_bfloat16*>(s.digits);
+    if (i) {
+      const int grid = (cols + 31) / 32;
+      if (real) HPSI_LAUNCH(c, HPSI_K_SPLIT, (k_digits_transposed<1><<<grid, 256, 0, c.stream>>>(P, cols, kpad[i], beta, d, s.exps)));
+      else HPSI_LAUNCH(c, HPSI_K_SPLIT, (k_digits_transposed<2><<<grid, 256, 0, c.stream>>>(P, cols, kpad[i], beta, d, s.exps)));
+    } else {
+      int* field = s.exps + rows[i];
+      cudaError_t e = cudaMemsetAsync(field, 0, sizeof(int) * P, c.stream);
+      if (e != cudaSuccess) return cuda_fail(c, e, "projector digit setup");
+      const dim3 grid(std::max(1, std::min(64, kpad[i] / 512)), std::min(P, 65535));
+      HPSI_LAUNCH(c, HPSI_K_SPLIT, (k_row_field<double><<<grid, 256, 0, c.stream>>>(P, len, 1, beta, field)));
+      HPSI_LAUNCH(c, HPSI_K_SPLIT,
+                  (k_digits<double><<<grid, 256, 0, c.stream>>>(P, len, kpad[i], 0, 1, beta, field, d, s.exps)));
+    }
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "projector digit setup");
@@ -473,11 +495,31 @@ static int slice_planes(Context& c, const Problem& p, int which, bool* ok) {
   return HPSI_OK;
 }
 
+bool release_slices(Context& c) {
+  bool any = false;
+  for (Problem& p : c.probs)
+    for (SlicePlanes& s : p.slices) any = any || s.owned;
+  if (!any) return false;
+  cudaStreamSynchronize(c.stream);
+  for (Problem& p : c.probs)
+    for (int first : {0, 2}) {
+      bool had = false;
+      for (int i = 0; i < 2; ++i) {
+        had = had || p.slices[first + i].digits;
+        cudaFree(p.slices[first + i].owned);
+        p.slices[first + i] = SlicePlanes();
+      }
+      p.slices[first].no_room = p.slices[first + 1].no_room = had;
+    }
+  c.ws.epoch++;   // captured batches refer to them
+  return true;
+}
+
 // Complex form: above 16 projectors.  Below, the CUDA-core kernels' float64 work is microseconds, they run over a whole
 // batch in one launch, and the persistent batch and hpsi_apply give the same bits.  Measured (H|psi>, CUDA-core against
 // this form): P = 32, 1503 plane waves, 4 bands 249 -> 94 us; P = 256, 6031, 64 bands 1982 -> 400 us.
 bool nonlocal_slices_use(const Problem& p, int nbnd) {
-  return p.nproj > 16 && nbnd > 0 && !p.slices[0].no_room && !p.slices[1].no_room;
+  return p.nproj > 16 && nbnd > 0 && !p.slices[0].no_room;
 }
 
 // Items of a batch of nitem take this form one by one, about ten launches and 45 us each, where the tiles run over all items
@@ -525,20 +567,29 @@ static int slice_band_block(int nbnd, size_t per_band) {
   return (nbnd + passes - 1) / passes;
 }
 
+// Workspaces of the projections: the digit planes of nbk bands and the K-splits' partial sums of every block (cw = 2: complex)
+static bool slice_room(Context& c, int P, int nbnd, int nbk, int cw, int kpad, int dup) {
+  size_t part = 0;
+  for (int nb : {std::min(nbk, nbnd), nbnd % nbk}) {
+    int per = 0;
+    if (nb > 0) part = std::max(part, sizeof(double) * cw * (size_t)slice_splits(c, P, cw * nb, kpad / SK, &per) * nb * P);
+  }
+  return try_buffer(c, &c.ws.mixed, &c.ws.mixedbytes, slice_rows_bytes(nbk, kpad, dup)) &&
+         try_buffer(c, &c.ws.part, &c.ws.partbytes, part);
+}
+
 // w = D <beta|psi> for nb bands (complex form) into w; *ok as slice_planes
 int slices_w(Context& c, const Problem& p, const double2* psi, int nbnd, double2* w, bool* ok) {
   int rc = slice_planes(c, p, 0, ok);
   if (rc || !*ok) return rc;
   const SlicePlanes& s = p.slices[0];
   const int P = p.nproj, nbk = slice_band_block(nbnd, slice_rows_bytes(1, s.kpad, 1));
-  rc = ensure_buffer(c, &c.ws.mixed, &c.ws.mixedbytes, slice_rows_bytes(nbk, s.kpad, 1));
-  if (rc) return rc;
+  *ok = slice_room(c, P, nbnd, nbk, 2, s.kpad, 1);
+  if (!*ok) return HPSI_OK;
   for (int b0 = 0; b0 < nbnd; b0 += nbk) {
     const int nb = std::min(nbk, nbnd - b0);
     int per = 0;
     const int ns = slice_splits(c, P, 2 * nb, s.kpad / SK, &per);
-    rc = ensure_buffer(c, &c.ws.part, &c.ws.partbytes, sizeof(double2) * (size_t)ns * nb * P);
-    if (rc) return rc;
     __nv_bfloat16* d = nullptr;
     int* e = nullptr;
     rc = slice_rows(c, reinterpret_cast<const double*>(psi + (size_t)b0 * p.npw), nb, 2 * p.npw, s.kpad, 1, 1,
@@ -558,8 +609,8 @@ int slices_add(Context& c, const Problem& p, const double2* w, double2* hpsi, in
   int rc = slice_planes(c, p, 1, ok);
   if (rc || !*ok) return rc;
   const SlicePlanes& s = p.slices[1];
-  rc = ensure_buffer(c, &c.ws.mixed, &c.ws.mixedbytes, slice_rows_bytes(nbnd, s.kpad, 1));
-  if (rc) return rc;
+  *ok = try_buffer(c, &c.ws.mixed, &c.ws.mixedbytes, slice_rows_bytes(nbnd, s.kpad, 1));
+  if (!*ok) return HPSI_OK;
   __nv_bfloat16* d = nullptr;
   int* e = nullptr;
   rc = slice_rows(c, reinterpret_cast<const double*>(w), nbnd, 2 * p.nproj, s.kpad, 2, 1,
@@ -573,7 +624,7 @@ int slices_add(Context& c, const Problem& p, const double2* w, double2* hpsi, in
 // Gamma form: always (the smallest measured, P = 4, 1503 plane waves, 4 bands: 108 -> 97 us; P = 256, 30047, 64 bands:
 // 2478 -> 860 us)
 bool gamma_slices_use(const Problem& p, int nbnd) {
-  return p.nproj > 0 && nbnd > 0 && !p.slices[2].no_room && !p.slices[3].no_room;
+  return p.nproj > 0 && nbnd > 0 && !p.slices[2].no_room;
 }
 
 template <typename R>
@@ -582,14 +633,12 @@ static int gamma_slices_w_t(Context& c, const Problem& p, const R* x, int nbnd, 
   if (rc || !*ok) return rc;
   const SlicePlanes& s = p.slices[2];
   const int P = p.nproj, nr = 2 * ((p.npw + 1) / 2), nbk = slice_band_block(nbnd, slice_rows_bytes(1, s.kpad, 0));
-  rc = ensure_buffer(c, &c.ws.mixed, &c.ws.mixedbytes, slice_rows_bytes(nbk, s.kpad, 0));
-  if (rc) return rc;
+  *ok = slice_room(c, P, nbnd, nbk, 1, s.kpad, 0);
+  if (!*ok) return HPSI_OK;
   for (int b0 = 0; b0 < nbnd; b0 += nbk) {
     const int nb = std::min(nbk, nbnd - b0);
     int per = 0;
     const int ns = slice_splits(c, P, nb, s.kpad / SK, &per);
-    rc = ensure_buffer(c, &c.ws.part, &c.ws.partbytes, sizeof(double) * (size_t)ns * nb * P);
-    if (rc) return rc;
     __nv_bfloat16* d = nullptr;
     int* e = nullptr;
     rc = slice_rows(c, x + (size_t)b0 * nr, nb, nr, s.kpad, 0, scaled ? 1 : 0, static_cast<unsigned char*>(c.ws.mixed),
@@ -614,8 +663,8 @@ int gamma_slices_add(Context& c, const Problem& p, const double* w, double* out,
   if (rc || !*ok) return rc;
   const SlicePlanes& s = p.slices[3];
   const int nr = 2 * ((p.npw + 1) / 2);
-  rc = ensure_buffer(c, &c.ws.mixed, &c.ws.mixedbytes, slice_rows_bytes(nbnd, s.kpad, 0));
-  if (rc) return rc;
+  *ok = try_buffer(c, &c.ws.mixed, &c.ws.mixedbytes, slice_rows_bytes(nbnd, s.kpad, 0));
+  if (!*ok) return HPSI_OK;
   __nv_bfloat16* d = nullptr;
   int* e = nullptr;
   rc = slice_rows(c, w, nbnd, p.nproj, s.kpad, 0, 1, static_cast<unsigned char*>(c.ws.mixed), &d, &e);
@@ -646,7 +695,7 @@ static __global__ void __launch_bounds__(256) k_pack_coef(int k, int n, double s
 static int few_ctas(const Context& c, size_t n) { return (int)std::min<size_t>(8 * c.sm_count, (n + 255) / 256); }
 
 // out[i + j ldo] = <a_i|b_j> for complex (CW = 2) or real (1) rows of len entries; *ok = false: no room for the digit planes
-// (nothing was done)
+// (out is to be written anew)
 template <int CW>
 static int slices_inner_t(Context& c, const double* a, int m, const double* b, int n, int len, double* out, int ldo,
                           bool* ok) {
@@ -656,9 +705,8 @@ static int slices_inner_t(Context& c, const double* a, int m, const double* b, i
   const int kpad = pad32(CW * len);
   const int nbk = slice_band_block(n, slice_rows_bytes(1, kpad, dup)), mbk = slice_band_block(m, slice_rows_bytes(1, kpad, 0));
   const size_t bb = slice_rows_bytes(nbk, kpad, dup), ab = slice_rows_bytes(mbk, kpad, 0);
-  int rc = ensure_buffer(c, &c.ws.mixed, &c.ws.mixedbytes, ab + bb);
-  if (rc == HPSI_ENOMEM) return HPSI_OK;
-  if (rc) return rc;
+  if (!try_buffer(c, &c.ws.mixed, &c.ws.mixedbytes, ab + bb)) return HPSI_OK;
+  int rc = HPSI_OK;
   unsigned char* w0 = static_cast<unsigned char*>(c.ws.mixed);
   for (int j0 = 0; j0 < n; j0 += nbk) {
     const int nj = std::min(nbk, n - j0);
@@ -672,8 +720,7 @@ static int slices_inner_t(Context& c, const double* a, int m, const double* b, i
       if (rc) return rc;
       int per = 0;
       const int ns = slice_splits(c, mi, CW * nj, kpad / SK, &per);
-      rc = ensure_buffer(c, &c.ws.part, &c.ws.partbytes, sizeof(V) * (size_t)ns * mi * nj);
-      if (rc) return rc;
+      if (!try_buffer(c, &c.ws.part, &c.ws.partbytes, sizeof(V) * (size_t)ns * mi * nj)) return HPSI_OK;
       double* part = static_cast<double*>(c.ws.part);
       rc = slice_gemm(c, da, ea, mi, db, eb, CW * nj, kpad, ns, per, CW == 2, false, part, CW * (size_t)mi * nj, mi,
                       HPSI_K_DAVIDSON);
@@ -704,9 +751,8 @@ static int slices_outer_t(Context& c, const double* a, int k, const double* coef
   const size_t eb_ = al256(sizeof(int) * (size_t)len);
   const size_t ab = al256(sizeof(__nv_bfloat16) * kDigits * (size_t)len * kpad0) + eb_;
   const size_t bb = slice_rows_bytes(n, kpad0, dup), cb = al256(sizeof(double) * CW * (size_t)n * kbk);
-  int rc = ensure_buffer(c, &c.ws.mixed, &c.ws.mixedbytes, ab + bb + cb);
-  if (rc == HPSI_ENOMEM) return HPSI_OK;
-  if (rc) return rc;
+  if (!try_buffer(c, &c.ws.mixed, &c.ws.mixedbytes, ab + bb + cb)) return HPSI_OK;
+  int rc = HPSI_OK;
   unsigned char* w0 = static_cast<unsigned char*>(c.ws.mixed);
   __nv_bfloat16* da = reinterpret_cast<__nv_bfloat16*>(w0);
   int* ea = reinterpret_cast<int*>(w0 + ab - eb_);

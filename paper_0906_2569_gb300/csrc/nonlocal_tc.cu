@@ -603,7 +603,7 @@ int prepare_t(Context& c, Problem& p) {
   const int P = p.nproj, npw = p.npw;
   const int kc = round_up(2 * npw, TBK), ka = round_up(2 * P, TBK);
   const size_t cal = (size_t)NT * P * kc, add = (size_t)NT * 2 * npw * ka;
-  cudaError_t e = cudaMalloc((void**)&p.d_beta_bf, sizeof(__nv_bfloat16) * (cal + add));
+  cudaError_t e = device_malloc(c, (void**)&p.d_beta_bf, sizeof(__nv_bfloat16) * (cal + add));
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(c, HPSI_ENOMEM, "device allocation of the bf16 projector terms failed");
@@ -732,7 +732,7 @@ int gamma_prepare_t(Context& c, Problem& p) {
   const int P = p.nproj, nh = (p.npw + 1) / 2, nr = 2 * nh;
   const int kc = round_up(nr, TBK), ka = round_up(P, TBK);
   const size_t cal = (size_t)NT * P * kc, add = (size_t)NT * nr * ka;
-  cudaError_t e = cudaMalloc((void**)&p.d_betar_bf, sizeof(__nv_bfloat16) * (cal + add));
+  cudaError_t e = device_malloc(c, (void**)&p.d_betar_bf, sizeof(__nv_bfloat16) * (cal + add));
   if (e != cudaSuccess) {
     cudaGetLastError();
     p.d_betar_bf = nullptr;
@@ -950,7 +950,7 @@ int tc_inner32(Context& c, TcInner& t, bool cache_a, int rows_cap, const float2*
     cudaFree(t.ws);
     t.ws = nullptr;
     t.wsbytes = 0;
-    if (cudaMalloc(&t.ws, abytes + bbytes + pbytes) != cudaSuccess) {
+    if (device_malloc(c, &t.ws, abytes + bbytes + pbytes) != cudaSuccess) {
       cudaGetLastError();
       return fail(c, HPSI_ENOMEM, "tensor-core inner-product workspace allocation failed");
     }
@@ -969,7 +969,7 @@ int tc_inner32(Context& c, TcInner& t, bool cache_a, int rows_cap, const float2*
         cudaFree(t.terms);
         t.terms = nullptr;
         t.caprows = 0;
-        if (cudaMalloc(&t.terms, sizeof(__nv_bfloat16) * NT * (size_t)cap * kc) != cudaSuccess) {
+        if (device_malloc(c, &t.terms, sizeof(__nv_bfloat16) * NT * (size_t)cap * kc) != cudaSuccess) {
           cudaGetLastError();
           return fail(c, HPSI_ENOMEM, "tensor-core basis split allocation failed");
         }

@@ -275,7 +275,7 @@ int Scf::alloc(int nmix, int nbnd) {
   if (w->nr != nr_ || w->nmix != nmix) {
     free_scf(*w);
     auto al = [&](void** p, size_t bytes) -> bool {
-      if (cudaMalloc(p, std::max<size_t>(bytes, 256)) != cudaSuccess) {
+      if (device_malloc(c, p, std::max<size_t>(bytes, 256)) != cudaSuccess) {
         cudaGetLastError();
         return false;
       }
@@ -298,7 +298,7 @@ int Scf::alloc(int nmix, int nbnd) {
     cudaFree(w->occ);
     w->occ = nullptr;
     w->occ_cap = 0;
-    if (cudaMalloc((void**)&w->occ, sizeof(double) * nbnd) != cudaSuccess) {
+    if (device_malloc(c, (void**)&w->occ, sizeof(double) * nbnd) != cudaSuccess) {
       cudaGetLastError();
       return fail(c, HPSI_ENOMEM, "hpsi_scf: device allocation failed");
     }

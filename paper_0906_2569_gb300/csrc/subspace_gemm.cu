@@ -137,7 +137,7 @@ int SplitBasis::ensure(Context& c, const float2* src, int ld, int cols) {
     for (auto& t : terms) cudaFree(t);
     terms[0] = terms[1] = terms[2] = nullptr;
     for (auto& t : terms)
-      if (cudaMalloc((void**)&t, sizeof(__nv_bfloat16) * need) != cudaSuccess)
+      if (device_malloc(c, (void**)&t, sizeof(__nv_bfloat16) * need) != cudaSuccess)
         return fail(c, HPSI_ENOMEM, "bf16 basis split allocation failed");
     cap = need;
     valid = 0;
@@ -166,14 +166,14 @@ int SubspaceGemm::grow(Context& c, size_t bterms, size_t pfloats) {
     for (auto& t : bt) cudaFree(t);
     bt[0] = bt[1] = bt[2] = nullptr;
     for (auto& t : bt)
-      if (cudaMalloc((void**)&t, sizeof(__nv_bfloat16) * bterms) != cudaSuccess)
+      if (device_malloc(c, (void**)&t, sizeof(__nv_bfloat16) * bterms) != cudaSuccess)
         return fail(c, HPSI_ENOMEM, "bf16 operand split allocation failed");
     bcap = bterms;
   }
   if (pfloats > pcap) {
     cudaFree(P);
     P = nullptr;
-    if (cudaMalloc((void**)&P, sizeof(float) * pfloats) != cudaSuccess)
+    if (device_malloc(c, (void**)&P, sizeof(float) * pfloats) != cudaSuccess)
       return fail(c, HPSI_ENOMEM, "subspace GEMM workspace allocation failed");
     pcap = pfloats;
   }
