@@ -384,7 +384,7 @@ int slices_inner(Context& c, const double* a, int m, const double* b, int n, int
                  bool* ok);
 int slices_outer(Context& c, const double* a, int k, const double* coef, int ldc, int n, int len, bool real, double sign,
                  bool accumulate, double* out, bool* ok);
-constexpr double kDigitMacs = 2.0e7;   // complex multiply-adds from which that form is taken (real: four times as many)
+constexpr double kDigitMacs = 2.0e7;   // complex multiply-adds from which fp64_inner and fp64_outer take that form
 // w = D (sum of the splits' partial <beta|psi>), complex and Gamma form
 int dscale_fp64(Context& c, const Problem& p, int nb, int nsplit, double2* part, double2* w);
 int gamma_dscale_fp64(Context& c, const Problem& p, int nb, int nsplit, const double* part, double* w);

@@ -1,4 +1,4 @@
-// The float64 nonlocal contractions (paper Sec. 3: becp = <beta|psi>, hpsi += beta w) on the tensor cores, exactly.
+// The float64 nonlocal contractions (paper Sec. 3: becp = <beta|psi>, hpsi += beta w) on the tensor cores.
 //
 // GB300's float64 pipe runs at ~1 TFLOP/s, its bf16 tensor cores at ~1900.  A float64 row scaled by a power of two
 // is a 63-bit integer X = x 2^(62 - e), |x| < 2^e, and an integer has digits: X = sum_s v_s 256^(7-s) with eight
@@ -6,13 +6,17 @@
 // fixed point).  A product of two digits has 14 bits, and sums of 1024 of them are integers below 2^24, which a float32
 // accumulator adds without rounding.  So
 //     sum_k a_k b_k = 2^(ea + eb - 124) sum_l 256^(14-l) sum_{i+j=l} sum_k v_i(a_k) v_j(b_k)
-// is taken level by level (l = i + j <= 7: 36 digit products; what is left out is below 2^-63 of the largest terms)
-// with one accumulator per level, emptied into 64-bit integers every 128 values of k (level 7 then holds
-// 8 x 128 products, its limit).  The sums are exact; rounding happens once, when a total becomes a float64.
+// is taken level by level (l = i + j <= 7: 36 of the 64 digit products) with one accumulator per level, emptied into 64-bit
+// integers every 128 values of k (level 7 then holds 8 x 128 products, its limit).  The sums of the 36 products are exact.
+// The 28 left out are at most 7 x 2^14 x 256^6, 2^-59 of 2^(ea + eb), for each k (random digits: 2^-62).  A K-split's total
+// is rounded once, to float64.
 //
-// Error is that of the 63-bit inputs, relative to the rows' largest entries; a chain of float64 FMAs over tens of
-// thousands of terms rounds more.  Against 80-bit or longer arithmetic the nonlocal term of 256 projectors and 36785 plane
-// waves errs by 1.51e-15 of its norm (the FMA kernels: 2.06e-15), of which most is the final float64 sum.
+// So the error is relative to the rows' largest entries, 2^-59 to 2^-62 of them a term, where a chain of float64 FMAs errs by
+// 2^-53 of each term and partial sum.  An entry below 2^-10 of its row's largest has fewer than a float64's 53 bits, and one
+// below 2^-62 none: for a projector that vanishes where psi is largest the chain may be the more accurate one.  On orbitals
+// and projectors the digits are: a chain over tens of thousands of terms rounds more.  Against 128-bit arithmetic the nonlocal
+// term of 256 projectors and 36785 plane waves errs by 1.49e-15 of its norm (the FMA kernels: 2.16e-15; Gamma form 2.23e-15
+// and 2.49e-15), of which most is the final float64 sum.
 //
 // Measured on that case with 160 bands: calbec + add_vuspsi 20.0 -> 1.01 ms (0.86 PFLOP/s of digit products, 0.45 of
 // the measured bf16 rate: the accumulators hold all of TMEM, so they are emptied while the tensor cores wait), the
