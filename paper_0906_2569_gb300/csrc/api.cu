@@ -281,8 +281,7 @@ static int plan_for(Context& c, int n, FftPlan* out) {
     if (tt.cells[pr].empty()) continue;
     ax.fxtw = reinterpret_cast<const FxTw*>(tt.tables + at[pr]);
     ax.ftw = reinterpret_cast<const float2*>(tt.tables + at[pr] + ftw[pr]);
-    ax.cell = tt.tables + at[pr] + cells[pr];
-    ax.slot = ax.cell + n;
+    ax.slot = tt.tables + at[pr] + cells[pr] + n;
   }
   tt.plan.tw64 = tt.d64;
   tt.plan.tw32 = tt.d32;

@@ -53,8 +53,7 @@ struct LineAxis {
   double gain = 1.0;              // float32: the two transforms' mean diagonal over n (line_gain)
   const FxTw* fxtw = nullptr;     // e^{2 pi i j / n} in fixed point and in float32 (Cooley-Tukey form only)
   const float2* ftw = nullptr;
-  const int* cell = nullptr;      // cell of every index before the inverse transform, and
-  const int* slot = nullptr;      // after it
+  const int* slot = nullptr;      // cell of every index after the inverse transform
 };
 // Tile sizes and growth bounds (bits) of a problem's fixed-point local term.
 struct FixedPlan {
