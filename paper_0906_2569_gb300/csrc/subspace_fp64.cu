@@ -73,10 +73,11 @@ __global__ void __launch_bounds__(SO_G* SO_B) k_sub_outer(int npw, int ld, int k
   }
 }
 
-// K[i + j n]: the first-order anti-Hermitian mixing of x_i and x_j in the eigenvectors of (H, S), where H_ij = <x_i|H x_j> is
-// nearly diagonal and S nearly the identity; zero where it would be above 3e-4 (near degeneracy).  The Hermitian part of H
-// alone: the rounding of h x in its float32 local term is not symmetric, and would come back as a lost
-// orthogonality over the gap.
+// K[i + j n]: the anti-Hermitian generator of the mixing of x_i and x_j in the eigenvectors of (H, S), where H_ij =
+// <x_i|H x_j> is nearly diagonal and S nearly the identity: the angle of each pair's own 2 x 2 problem, which is exact for a
+// pair that is close and first order between others; zero where it would be above 0.03 (degenerate to
+// float32 accuracy).  The Hermitian part of H alone: the rounding of h x in its float32 local term is not symmetric, and
+// would come back as a lost orthogonality over the gap.
 template <int CW>
 __global__ void __launch_bounds__(256) k_ritz_mix(int n, const double* __restrict__ H, const double* __restrict__ S,
                                                   double* __restrict__ K) {
@@ -85,48 +86,54 @@ __global__ void __launch_bounds__(256) k_ritz_mix(int n, const double* __restric
   const int i = (int)(t % n), j = (int)(t / n);
   const size_t di = CW * (size_t)i * (n + 1), dj = CW * (size_t)j * (n + 1), u = CW * ((size_t)i * n + j);
   const double ei = H[di] / S[di], ej = H[dj] / S[dj], g = ej - ei, em = 0.5 * (ei + ej);
-  double v[CW], top = 0.0;
+  double v[CW], a2 = 0.0;
   for (int k = 0; k < CW; ++k) {
     v[k] = 0.5 * (H[CW * t + k] + (k == 0 ? H[u] : -H[u + k])) - em * S[CW * t + k];
-    top = fmax(top, fabs(v[k]));
+    a2 = fma(v[k], v[k], a2);
   }
-  const bool apart = i != j && top <= 3e-4 * fabs(g) && g != 0.0;
-  for (int k = 0; k < CW; ++k) K[CW * t + k] = apart ? v[k] / g : 0.0;
+  const double a = sqrt(a2);
+  const bool apart = i != j && a > 0.0 && a <= 0.03 * fabs(g);
+  const double f = apart ? 0.5 * atan(2.0 * a / g) / a : 0.0;
+  for (int k = 0; k < CW; ++k) K[CW * t + k] = v[k] * f;
 }
-// C = (1 + K + K^2 / 2 - (S - 1) / 2), column j over the norm of x_j: orthonormal to the third order of K
+// out = one + alpha A (bone + bscale B) (n x n); orth: A stands for the first-order S^-1/2 of the overlaps S that it holds
 template <int CW>
-__global__ void __launch_bounds__(256) k_ritz_rotation(int n, const double* __restrict__ K, const double* __restrict__ S,
-                                                       double* __restrict__ C) {
+__global__ void __launch_bounds__(256) k_small_product(int n, double one, double alpha, const double* __restrict__ A,
+                                                       bool orth, double bone, double bscale, const double* __restrict__ B,
+                                                       double* __restrict__ out) {
   const size_t t = (size_t)blockIdx.x * 256 + threadIdx.x;
   if (t >= (size_t)n * n) return;
   const int i = (int)(t % n), j = (int)(t / n);
   double q[2] = {0.0, 0.0};
   for (int l = 0; l < n; ++l) {
     const size_t a = CW * ((size_t)l * n + i), b = CW * ((size_t)j * n + l);
-    q[0] = fma(K[a], K[b], q[0]);
+    double x = A[a], y = CW == 2 ? A[a + CW - 1] : 0.0;
+    if (orth) {
+      x = l == i ? 1.0 / sqrt(x) : -0.5 * x;
+      y = l == i ? 0.0 : -0.5 * y;
+    }
+    const double u = fma(bscale, B[b], l == j ? bone : 0.0);
+    q[0] = fma(x, u, q[0]);
     if (CW == 2) {
-      q[0] = fma(-K[a + 1], K[b + 1], q[0]);
-      q[1] = fma(K[a], K[b + 1], fma(K[a + 1], K[b], q[1]));
+      const double w = bscale * B[b + CW - 1];
+      q[0] = fma(-y, w, q[0]);
+      q[1] = fma(x, w, fma(y, u, q[1]));
     }
   }
-  const double norm = 1.0 / sqrt(S[CW * (size_t)j * (n + 1)]);
-  for (int k = 0; k < CW; ++k) {
-    const double one = i == j && k == 0 ? 1.0 : 0.0;
-    C[CW * t + k] = norm * (one + K[CW * t + k] + 0.5 * q[k] - (i == j ? 0.0 : 0.5 * S[CW * t + k]));
-  }
+  for (int k = 0; k < CW; ++k) out[CW * t + k] = fma(alpha, q[k], i == j && k == 0 ? one : 0.0);
 }
 
 }  // namespace
 
 // The vectors of a float32 basis carry rounding noise that the Rayleigh-Ritz step turns into mixing of neighbours, noise
 // over their gap (1e-5 at a gap of 1e-3 Ha): most of the vectors' error, and the part that varies between equally accurate
-// forms of H|psi>.  x and h x are at hand in float64 for the quotients, so the mixing inside the block is taken out to first
-// order: two N x N products and two rotations as digit products (32 vectors of 2.4e3 plane waves: 0.2 of 28 ms).
-// small: 3 N^2, tx and thx: N rows of len (complex or real).  Without room for the digits x stays as it is.
+// forms of H|psi>.  x and h x are at hand in float64 for the quotients, so the mixing inside the block is taken out: two N x N
+// products, C = S^-1/2 exp(K) (S^-1/2 to first order, the exponential to fourth) and two rotations as digit products.
+// small: 4 N^2, tx and thx: N rows of len (complex or real).  Without room for the digits x stays as it is.
 int ritz_refine(Context& c, int n, int len, bool real, double* x, double* hx, double* small, double* tx, double* thx) {
   if (n < 2) return HPSI_OK;
   const size_t nn = (size_t)n * n * (real ? 1 : 2), bytes = sizeof(double) * (real ? 1 : 2) * (size_t)n * len;
-  double *H = small, *S = small + nn, *K = S + nn;
+  double *H = small, *S = small + nn, *K = S + nn, *T = K + nn;
   bool ok = false;
   int rc = slices_inner(c, x, n, hx, n, len, real, H, n, &ok);
   if (!rc && ok) rc = slices_inner(c, x, n, x, n, len, real, S, n, &ok);
@@ -134,9 +141,18 @@ int ritz_refine(Context& c, int n, int len, bool real, double* x, double* hx, do
   const unsigned grid = (unsigned)(((size_t)n * n + 255) / 256);
   if (real) HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k_ritz_mix<1><<<grid, 256, 0, c.stream>>>(n, H, S, K)));
   else HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k_ritz_mix<2><<<grid, 256, 0, c.stream>>>(n, H, S, K)));
+  auto product = [&](double one, double alpha, const double* A, bool orth, double bone, double bscale, const double* B,
+                     double* out) {
+    auto go = [&](auto k) { HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k<<<grid, 256, 0, c.stream>>>(n, one, alpha, A, orth, bone, bscale, B, out))); };
+    if (real) go(k_small_product<1>);
+    else go(k_small_product<2>);
+  };
+  // exp(K) = 1 + K (1 + K / 2 (1 + K / 3 (1 + K / 4))); H is free from here on
+  product(1.0, 1.0 / 3.0, K, false, 1.0, 0.25, K, T);
+  product(1.0, 0.5, K, false, 0.0, 1.0, T, H);
+  product(1.0, 1.0, K, false, 0.0, 1.0, H, T);
   double* C = H;
-  if (real) HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k_ritz_rotation<1><<<grid, 256, 0, c.stream>>>(n, K, S, C)));
-  else HPSI_LAUNCH(c, HPSI_K_DAVIDSON, (k_ritz_rotation<2><<<grid, 256, 0, c.stream>>>(n, K, S, C)));
+  product(0.0, 1.0, S, true, 0.0, 1.0, T, C);
   rc = slices_outer(c, x, n, C, n, n, len, real, 1.0, false, tx, &ok);
   if (!rc && ok) rc = slices_outer(c, hx, n, C, n, n, len, real, 1.0, false, thx, &ok);
   if (rc || !ok) return rc;
