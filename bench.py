@@ -47,14 +47,12 @@ FP32_ALU_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12  # 152 SMs x 128 FP32 lanes x F
 # DRAM bytes (read + write) per unit measured by ncu for a kernel class, keyed by (kernel, precision)
 # with the hash of its source files at capture time; a mismatch reports null.  Units: a band of
 # the kernel's launch for the H|psi> classes, a matrix element for the reduction.
-#   calbec fp64: k_calbec64, 160-band launch, 270.83 MB read + 7.20 MB write
-#   tridiag: k_eh_tridiag, one n = 640 launch, 3.372 MB read + 0.030 MB write
-#   tridiag_real: k_eh_tridiag_r, one n = 1536 launch, 9.580 MB read + 2.8 KB write
+#   tridiag: k_eh_tridiag, one n = 640 launch, 3.384 MB read + 2.8 KB write
+#   tridiag_real: k_eh_tridiag_r, one n = 1536 launch, 9.583 MB read + 25.9 KB write
 NCU_TRAFFIC = {
-    ("tridiag", -1): (("eigh_tridiag.cuh",), "7b3ca0b96a01", (3367936 + 31488) / 640 ** 2),
-    ("tridiag_real", -1): (("eigh_tridiag_real.cuh",), "9dff8d240ee0", (9579520 + 2816) / 1536 ** 2),
+    ("tridiag", -1): (("eigh_tridiag.cuh",), "5d4d8f12e825", (3383808 + 2816) / 640 ** 2),
+    ("tridiag_real", -1): (("eigh_tridiag_real.cuh",), "eb02e14b7d06", (9583104 + 25856) / 1536 ** 2),
     ("tridiag_df", -1): (("eigh_tridiag_df.cuh",), "d822de855785", (9583104 + 8704) / 1536 ** 2),
-    ("calbec", 0): (("nonlocal_fp64.cu",), "dc474a4712d7", (270.831104e6 + 7.199488e6) / 160),
 }
 
 

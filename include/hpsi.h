@@ -72,7 +72,7 @@ enum hpsi_option {
                                  projections <beta|psi> and D, the local term at the working precision
                                  and add_vuspsi on the tensor cores with one K-step per float32
                                  partial (the projections' error enters the quotients at first
-                                 order; ~5e-8 Ha on the 144^3 cell); 1: with the float64 H (~3e-9 Ha);
+                                 order; ~2e-8 Ha on the 144^3 cell); 1: with the float64 H (~3e-9 Ha);
                                  0: with the mixed H (~2e-6 Ha) */
   HPSI_OPT_BASIS = 8,         /* davidson_solve: the reduced basis grows to this many times N
                                  vectors (2: the basic 2N form, 3 or 4) before a restart; 0
@@ -143,8 +143,8 @@ enum hpsi_option {
                                  eigenvector GEMMs) */
   HPSI_OPT_PERSISTENT = 24,   /* hpsi_apply_batch: 1: one persistent cooperative launch per box edge
                                  (<= 32 items each) when every item has the two-codelet
-                                 kernels; 0 (default): one launch per kernel class and box edge.
-                                 The results are identical; the separate launches, replayed from a
+                                 kernels; 0 (default): one launch per kernel class, whatever the boxes
+                                 (<= 32 items each).  The results are identical; the separate launches, replayed from a
                                  CUDA graph, are faster since each kernel runs at its own occupancy */
   HPSI_OPT_BATCH_NL = 25      /* hpsi_apply_batch in a mixed context: the nonlocal term.  0 (default):
                                  in float64 when every item has at most 64 projectors (one launch per
@@ -156,13 +156,13 @@ enum hpsi_option {
 
 /* Kernel classes reported by hpsi_kernel_stats. */
 enum hpsi_kernel {
-  HPSI_K_INV_ZY = 0,   /* scatter + inverse z and y transforms per m1-plane */
-  HPSI_K_XVX_Y = 1,    /* inverse x, x V(r), forward x, forward y per z-plane */
-  HPSI_K_FWD_Z = 2,    /* forward z, gather, kinetic term per m1-plane */
+  HPSI_K_INV_ZY = 0,   /* scatter + inverse z transform per chunk of sticks (generic kernels: z and y per m1-plane) */
+  HPSI_K_XVX_Y = 1,    /* inverse y and x, x V(r), forward x and y per z-plane (generic: inverse y in the class above) */
+  HPSI_K_FWD_Z = 2,    /* forward z, gather, kinetic term per chunk of sticks (generic: per m1-plane) */
   HPSI_K_CALBEC = 3,   /* <beta|psi> (split-K partial sums) */
   HPSI_K_DSCALE = 4,   /* reduction of the partials and D <beta|psi> */
   HPSI_K_ADDVUS = 5,   /* hpsi += beta (D <beta|psi>) */
-  HPSI_K_SPLIT = 6,    /* mixed path: bf16 operand splitting */
+  HPSI_K_SPLIT = 6,    /* operands of the tensor cores: bf16 terms (mixed), integer digits (float64) */
   HPSI_K_DAVIDSON = 7, /* Davidson residual / preconditioner / helper kernels */
   HPSI_K_EIGH = 8,     /* reduced eigenproblem: multisection, inverse iteration,
                           back-transformation helpers */

@@ -606,11 +606,10 @@ int apply_device(Context& c, int ik, const double2* psi, double2* hpsi, int nbnd
   return nonlocal_apply(c, p, psi, hpsi, nbnd);
 }
 
-// All items at once.  Problems whose box has the fast kernels share, per box edge, one persistent
-// cooperative launch (the three FFT phases and, when the nonlocal term is float64, its three phases
-// too), or, with HPSI_OPT_PERSISTENT off or when another item takes the generic path, one launch per
-// kernel and box edge; their stick rows live side by side in one workspace.  The tensor-core
-// nonlocal term follows per item.
+// All items at once.  Problems whose box has the fast kernels share one launch per kernel (32 items each), or, with
+// HPSI_OPT_PERSISTENT and none on the generic path, one persistent cooperative launch per box edge (the three FFT
+// phases and, when the nonlocal term is float64 and no item is large, its three phases too); their stick rows live
+// side by side in one workspace.  The mixed tensor-core nonlocal term follows per item.
 static int batch_apply_items(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
                              double2* const* hpsi) {
   std::vector<int> fast, slow;

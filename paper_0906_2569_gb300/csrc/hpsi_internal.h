@@ -361,7 +361,7 @@ int nonlocal_fp64_into(Context& c, const Problem& p, const double2* psi, double2
 int nonlocal_batch_fp64(Context& c, int nitem, const int* prob, const int* nbnd, const double2* const* psi,
                         double2* const* hpsi, int nbatch);
 
-// The float64 contractions as exact integer products on the tensor cores (nonlocal_slices.cu); *ok = false: no room for
+// The float64 contractions as integer digit products on the tensor cores (nonlocal_slices.cu); *ok = false: no room for
 // the projectors' digits, the caller takes the CUDA-core kernels.
 bool nonlocal_slices_use(const Problem& p, int nbnd);
 bool batch_slices_use(const Problem& p, int nbnd, int nitem);   // the same for an item of a batch of nitem

@@ -427,8 +427,9 @@ void float_plan(Problem& p, size_t smem_optin) {
 double line_gain(const LineAxis& ax, const float2* tw) {
   const int n = ax.n, r1 = ax.r1, r2 = ax.r2;
   std::vector<double2> w(n);
-  auto stage = [&](int r, int items, int first, int step, bool twiddled) {   // item i: cells i first + a step
-    for (int i = 0; i < items; ++i) {
+  // items from .. to - 1 of a stage, item i in the cells i first + a step
+  auto stage = [&](int r, int from, int to, int first, int step, bool twiddled) {
+    for (int i = from; i < to; ++i) {
       double2 v[16];
       for (int a = 0; a < r; ++a) v[a] = w[i * first + a * step];
       switch (r) {
@@ -455,11 +456,11 @@ double line_gain(const LineAxis& ax, const float2* tw) {
     for (int t = 0; t < r2; ++t) {
       std::fill(w.begin(), w.end(), make_double2(0.0, 0.0));
       w[a * r2 + t].x = 1.0;
-      stage(r1, r2, 1, r2, ax.twiddled);
-      stage(r2, r1, r2, 1, false);
+      stage(r1, t, t + 1, 1, r2, ax.twiddled);   // the others are zero
+      stage(r2, 0, r1, r2, 1, false);
       for (double2& v : w) std::swap(v.x, v.y);   // the opposite sign, as in plane_tile
-      stage(r2, r1, r2, 1, ax.twiddled);
-      stage(r1, r2, 1, r2, false);
+      stage(r2, 0, r1, r2, 1, ax.twiddled);
+      stage(r1, t, t + 1, 1, r2, false);          // the diagonal is in this one
       sum += w[a * r2 + t].y;
     }
   return sum / ((double)n * n);

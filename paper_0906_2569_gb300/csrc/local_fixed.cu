@@ -18,8 +18,8 @@
 // radices are run-time switches over the same codelets, since a codelet is hundreds of instructions.
 //
 // What bounds it: instruction issue and the latency of the multiplications (an add is 2 instructions, a 64-bit
-// multiplication by a constant ~9).  Measured on the 90^3 box with 160 bands: plane kernel 19.35 -> 3.2 ms, z
-// kernels 1.07 + 1.17 -> 0.33 + 0.46 ms against float64 register codelets; 32 cells of 25^3 to 50^3: 9.6 -> 1.41 ms
+// multiplication by a constant ~9); 27 bands of 90^3: 56% of issue cycles, ALU pipe 51%, DRAM 2%.  Measured on the 90^3
+// box with 160 bands: plane kernel 19.35 -> 2.6 ms, z kernels 1.07 + 1.17 -> 0.28 + 0.30 ms against float64 register codelets; 32 cells of 25^3 to 50^3: 9.6 -> 1.41 ms
 // (planes); 27 x 30 x 32: 428 -> 31 us against the float64 Stockham kernels.  Error of the local term against 128-bit
 // arithmetic: below the float64 kernels' at every edge tried (16 to 135), by 5 to 40%.
 #include <cuda_runtime.h>

@@ -3,7 +3,7 @@
 //   w[b][p]    = sum_q D_pq becp[b][q]                                          (D-scale, CSR of D)
 //   hpsi_b(G) += sum_p beta_p(G) w[b][p]                                        (add_vuspsi)
 // On GB300 float64 runs at ~1.2 TFLOP/s on the CUDA cores (the FP64 MMA path is not faster).  Large blocks go to
-// the tensor cores as exact integer products (nonlocal_slices.cu); here are the small ones:
+// the tensor cores as integer digit products (nonlocal_slices.cu); here are the small ones:
 // plain shared-memory-tiled complex GEMMs whose inner loop is DFMA-bound; calbec
 // (P x nb outputs, K = npw) splits K across CTAs and reduces the partials deterministically in
 // the D-scale kernel.

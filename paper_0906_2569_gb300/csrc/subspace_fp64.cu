@@ -3,9 +3,9 @@
 // GEMMs of float64 leave most of the chip idle (16 x 64 rows of 1503: 104 us where the FMAs are 12 us of
 // the float64 pipe).  Two forms each:
 //   small   CUDA-core FMAs: inner products with K split over CTAs, combinations with one output per thread;
-//   large   exact digit products on the tensor cores (nonlocal_slices.cu).
+//   large   digit products on the tensor cores (nonlocal_slices.cu).
 // The line between them, kDigitMacs, is ~170 us of the float64 pipe and ~80 us as digits (their planes are made on each
-// call).  davidson_solve in float64: 16 bands of 1503 plane waves 43 -> 25 ms; 160 bands of 36785, where every product is large,
+// call).  davidson_solve in float64: 16 bands of 1503 plane waves 43 -> 27 ms; 160 bands of 36785, where every product is large,
 // 6.5 -> 0.91 s.
 #include <cuda_runtime.h>
 
