@@ -214,7 +214,8 @@ __global__ void __launch_bounds__(256) k_gamma_unpack_raw(int npw, int nb, const
     } else {
       constexpr float rh = (float)kSqrt2, rl = (float)(kSqrt2 - (double)rh);
       constexpr float ih = (float)kInvSqrt2, il = (float)(kInvSqrt2 - (double)ih);
-      const float pow2 = __uint_as_float((unsigned)(127 + sh) << 23);
+      const float pow2 = __uint_as_float((unsigned)(127 + sh) << 23), back = __uint_as_float((unsigned)(127 - sh) << 23);
+      int e[4] = {sh, sh, sh, sh};   // powers of two of v
       // twice the local terms (the halving of h and l is exact)
       float2 v[4] = {pair_sum(fp.x, fm.x), pair_sum(fp.y, -fm.y), pair_sum(fp.y, fm.y), pair_sum(fm.x, -fp.x)};
 #pragma unroll
@@ -239,14 +240,17 @@ __global__ void __launch_bounds__(256) k_gamma_unpack_raw(int npw, int nb, const
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           if (down) n[i] = pair_times(n[i], ih, il);
-          v[i] = pair_add(v[i], make_float2(n[i].x * pow2, n[i].y * pow2));
+          const bool big = fabsf(n[i].x) > 0x1p100f;   // times 2^sh it might leave float32
+          const float fv = big ? back : 1.f, fn = big ? 1.f : pow2;
+          v[i] = pair_add(make_float2(v[i].x * fv, v[i].y * fv), make_float2(n[i].x * fn, n[i].y * fn));
+          if (big) e[i] = 0;
         }
       }
       const double2 xa = ld2(x + (size_t)a * nh + h);
-      st2(y + (size_t)a * nh + h, make_double2(pair_fma(kg, xa.x, v[0], sh), pair_fma(kg, h ? xa.y : 0.0, v[1], sh)));
+      st2(y + (size_t)a * nh + h, make_double2(pair_fma(kg, xa.x, v[0], e[0]), pair_fma(kg, h ? xa.y : 0.0, v[1], e[1])));
       if (b < nb) {
         const double2 xb = ld2(x + (size_t)b * nh + h);
-        st2(y + (size_t)b * nh + h, make_double2(pair_fma(kg, xb.x, v[2], sh), pair_fma(kg, h ? xb.y : 0.0, v[3], sh)));
+        st2(y + (size_t)b * nh + h, make_double2(pair_fma(kg, xb.x, v[2], e[2]), pair_fma(kg, h ? xb.y : 0.0, v[3], e[3])));
       }
     }
   }

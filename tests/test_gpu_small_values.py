@@ -46,6 +46,21 @@ def test_mixed_local_term_of_small_bands(lib, gamma):
     assert err[0] < 1e-6 and err[1] <= 2.0 * err[0]
 
 
+@pytest.mark.parametrize("e", [0, 90, 118])
+def test_mixed_gamma_nonlocal_of_large_bands(lib, e):
+    """Bands of up to 2^118: the nonlocal term of the Gamma form alone (V = 0) stays in float32's range and scales with the
+    band (all its operands and sums are floating-point numbers of eight exponent bits)."""
+    lat, ecut, n = np.diag([8.0, 8.0, 8.0]), 8.0, 20
+    from paper_0906_2569_gb300 import binding as B
+    m = B.hpsi_gsphere(lat, ecut, np.zeros(3))
+    beta = workloads.beta(lat, np.random.default_rng(1).random((5, 3)) @ lat, np.zeros(3), m)
+    psi = workloads.random_block(len(m), 3, 3)[:, len(m) // 2:].copy()
+    psi[:, 0] = psi[:, 0].real
+    args = (lat, ecut, (n, n, n), np.zeros((n, n, n)), [beta], workloads.dmat(5), B.HPSI_MIXED)
+    one, large = _apply(*args, psi, True), _apply(*args, psi * 2.0 ** e, True) * 2.0 ** -e
+    assert np.linalg.norm(large - one) <= 1e-6 * np.linalg.norm(one)
+
+
 def _float64_case(gamma, nproj=20):
     from paper_0906_2569_gb300 import binding as B
     lat, ecut, n = np.diag([8.0, 8.0, 8.0]), 8.0, 20
