@@ -107,11 +107,7 @@ __global__ void __launch_bounds__(256) k_small_product(int n, double one, double
   double q[2] = {0.0, 0.0};
   for (int l = 0; l < n; ++l) {
     const size_t a = CW * ((size_t)l * n + i), b = CW * ((size_t)j * n + l);
-    double x = A[a], y = CW == 2 ? A[a + CW - 1] : 0.0;
-    if (orth) {
-      x = l == i ? 1.0 / sqrt(x) : -0.5 * x;
-      y = l == i ? 0.0 : -0.5 * y;
-    }
+    const double x = A[a], y = CW == 2 ? A[a + CW - 1] : 0.0;
     const double u = fma(bscale, B[b], l == j ? bone : 0.0);
     q[0] = fma(x, u, q[0]);
     if (CW == 2) {
@@ -119,6 +115,11 @@ __global__ void __launch_bounds__(256) k_small_product(int n, double one, double
       q[0] = fma(-y, w, q[0]);
       q[1] = fma(x, w, fma(y, u, q[1]));
     }
+  }
+  if (orth) {   // 1 / sqrt(S_ii) and -S_il / 2
+    const double d = A[CW * (size_t)i * (n + 1)], f = 1.0 / sqrt(d) + 0.5 * d;
+    for (int k = 0; k < CW; ++k)
+      q[k] = fma(-0.5, q[k], f * fma(bscale, B[CW * t + k], i == j && k == 0 ? bone : 0.0));
   }
   for (int k = 0; k < CW; ++k) out[CW * t + k] = fma(alpha, q[k], i == j && k == 0 ? one : 0.0);
 }
