@@ -256,8 +256,8 @@ HPSI_API int hpsi_nproj(const hpsi_ctx* ctx, int ik);
  * owns and returns after the result has been copied back).  Mixed host/device pairs are
  * HPSI_EINVAL.  The library allocates its device workspace on first use and keeps it.
  * The nonlocal term in float64 of a problem with more than 16 projectors (Gamma form: with any) runs on the tensor cores
- * as integer digits, to 2^-61 of the largest entry of each projector and band (hpsi_apply_noalloc and small
- * items of a batch: float64 on the CUDA cores).  The first such application makes the projectors' digits, which take four
+ * as integer digits; its error is relative to the largest entries of each projector and band, at most 2^-59 of
+ * their product for each plane wave (hpsi_apply_noalloc and small items of a batch: float64 on the CUDA cores).  The first such application makes the projectors' digits, which take four
  * times the projectors' memory for the life of the context (and the bands' up to 1 GB of workspace); where the device has no
  * room, or another workspace of the context needs the memory, the context goes on with the float64 kernels.
  */

@@ -21,9 +21,9 @@ __device__ __forceinline__ float f64_to_f32(double x) {
 }
 __device__ __forceinline__ float2 f64_to_f32(double2 x) { return make_float2(f64_to_f32(x.x), f64_to_f32(x.y)); }
 
-// (double)f 2^-sh for 0 <= sh < 64, exact but for subnormal f, which give zero (2^-126 of what a float32 result stands
-// beside; its producers, tensor cores on bf16 terms and float32 transforms, lose as much); without a branch, since one
-// around the cast costs 2% of H|psi> for 160 bands of 1503 plane waves
+// (double)f 2^-sh for 0 <= sh < 64, exact but for subnormal f, which give zero: what produces such values here (tensor cores
+// on bf16 terms, float32 transforms whose results are 2^sh times what they stand for) has lost as much before.
+// Without a branch: one around the cast costs 2% of H|psi> for 160 bands of 1503 plane waves.
 __device__ __forceinline__ double f32_to_f64(float f, int sh = 0) {
   const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
   unsigned hi = (a >> 3) + (a >= 0x7f800000u ? 0x70000000u : 0x38000000u - ((unsigned)sh << 20));   // infinity, NaN: all ones
